@@ -272,7 +272,7 @@ int gwfa_align_batch_device(gwfa_engine *e, uint32_t n_queries, const uint32_t *
  * but its scratch is one fixed 32 MiB device array inside the library (present
  * on every GPU that loads it, until the process exits), carved into
  * floor((32 MiB - 256 B) / slab) CTA slabs of 2^log2_tiles hash tiles each
- * (log2_tiles 0 = 15: five CTAs in exact mode, two with pruning).  There is
+ * (log2_tiles 0 = 15: six CTAs in exact mode, three with pruning).  There is
  * no overflow tier: a query needing more than 3/4 of its slab gets status
  * GWFA_ERR_CAPACITY.  log2_tiles outside [8, 24] (other than 0) is
  * GWFA_ERR_INVALID; a valid log2_tiles whose slab does not fit the array is
@@ -307,8 +307,9 @@ uint32_t gwfa_engine_last_launches(const gwfa_engine *e);
  * Per-query statistics of later batch calls on this engine (NULL = off): the
  * kernels write 8 uint64 per query id into d_stats (device memory of
  * n_queries * 8 words, owned by the caller, valid until replaced): time spent in
- * GwfExtend and in GwfExpand (ns, measured by the CTA), extension rounds,
- * tiles extended, tiles expanded, largest expanded-tile count of a score, tiles
+ * GwfExpand and GwfExtend along vertices, and in the arc spills of GwfExtend (ns,
+ * measured by the CTA), extension rounds, tiles visited, tiles listed for the next
+ * score, largest tile count of a score, tiles
  * claimed in the hash, and the number of scores.  These are the wavefront sizes
  * the learned cost model trains on.
  */

@@ -53,9 +53,10 @@ def _time(engine: Engine, batch: DeviceBatch, max_lag: int, reps: int) -> float:
 
 def _tier0_bytes(threads_ctas: int, log2: int, prune: bool) -> int:
     """Approximate device bytes of a tier of CTAs with 2^log2-tile slabs: per tile a
-    hash line (64 / 128 bytes), a touched entry, three 16-byte list entries and one
-    frontier snapshot (64 / 128 bytes); pruning adds the spill requests and T."""
-    per_tile = (64 + 4 + 48 + 64) if not prune else (128 + 4 + 48 + 128 + 20 + 16)
+    record (64 / 128 bytes), two hash entries, its hash position and stamp, two list
+    entries and the spill requests (32 bytes); pruning adds the keys, trace words, T and
+    the insertion and free lists."""
+    per_tile = 152 if not prune else 328
     return threads_ctas * (per_tile << log2)
 
 

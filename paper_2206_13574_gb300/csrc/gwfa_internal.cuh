@@ -39,65 +39,76 @@ struct DevGraph {
     uint32_t nv;
 };
 
-// List entry: tile slot, vertex, tile index kb (diagonals 8kb .. 8kb+7).
-struct __align__(16) LEnt {
-    uint32_t slot;
-    uint32_t v;
-    int32_t kb;
-    uint32_t pad;
-};
-// Extended-frontier header: slot | live-lane mask << 24, vertex, kb, |v|.
-struct __align__(16) EHdr {
-    uint32_t slot_mask;
-    uint32_t v;
-    int32_t kb;
-    uint32_t lv;
-};
-constexpr uint32_t kMaxLog2Tiles = 24;   // slot must fit the 24 low bits of EHdr
+constexpr uint32_t kMaxLog2Tiles = 24;
 
-// Hash slot of one tile, one 64-byte line in exact mode (128 in pruning mode):
-// key (v << 32 | kb, all ones = empty), the two lane-mask words of the phase
-// parities, and the 8 offsets; in pruning mode also the 8 trace indices (Alg. 5)
-// of the diagonals, used with traceback.  A tile visit touches a single line.
-template <class T>
-struct alignas(sizeof(T) == 4 ? 64 : 128) SlotT {
-    unsigned long long key;
-    uint32_t reg[2];
-    T vals[kTile];
-    uint32_t trace[sizeof(T) == 4 ? 1 : kTile];
+// Hash entry: the tile's key (v << 32 | kb, all ones = empty) and its record.
+struct alignas(16) TabEnt {
+    unsigned long long key, idx;
 };
-// Extended-frontier entry: header + snapshot of the 8 offsets (and, in pruning
-// mode, of their trace indices) after extension.
-template <class T>
-struct alignas(sizeof(T) == 4 ? 64 : 128) EEntT {
-    EHdr hdr;
-    T vals[kTile];
-    uint32_t trace[sizeof(T) == 4 ? 1 : kTile];
+// Tile record: the 8 offsets, and per side (0 left, 1 right) the candidate that the
+// neighbour tile's edge diagonal hands over (by parity of the score that takes it, -1 =
+// none), the neighbour's record once linked, and kb.  64 bytes in exact mode, 128 in
+// pruning mode; a query's records are dense, in order of first use.
+//   exact mode:   offset j << 1 | in Q, absent = -2; border words j;
+//   pruning mode: (j << 32 | tag << 30 | base), absent = -1; border words j << 32 | base.
+template <class T> struct RecT;
+template <> struct alignas(64) RecT<int> {
+    int vals[kTile];
+    struct alignas(16) {
+        int in[2];
+        uint32_t link;
+        int kb;
+    } side[2];
+};
+template <> struct alignas(128) RecT<long long> {
+    long long vals[kTile];
+    struct alignas(16) {
+        long long in[2];
+        uint32_t link;
+        int kb;
+        uint32_t counted, pad;   // side 1: the tile holds a diagonal (load limit)
+    } side[2];
+};
+// Trace indices (Alg. 5) of a record's diagonals and border words, used with traceback.
+struct alignas(64) TraceRec {
+    uint32_t tr[kTile];
+    uint32_t in[2][2];
+    uint32_t pad[4];
 };
 
-// Per-CTA slab layout (all arrays 256-byte aligned), cap = 2^log2 tiles.
+// 16-byte chunk `part` of an empty record.
+__host__ __device__ inline uint4 empty_chunk(bool prune, uint32_t part) {
+    const uint32_t o = 0xFFFFFFFFu, z = prune && (part == 5 || part == 7) ? 0u : o;
+    const uint32_t a = !prune && part < 2 ? 0xFFFFFFFEu : o;
+    return prune ? make_uint4(o, o, z, z) : make_uint4(a, a, a, a);
+}
+
+// Per-CTA slab layout (all arrays 256-byte aligned), cap = 2^log2 tiles: the hash (twice
+// as many entries as tiles), the records, the hash position of each record and its list
+// stamp -- these start all ones / empty -- then the two tile lists and the spill lists.
 struct SlabLayout {
-    uint64_t slots, touched, qlist, slist0, slist1, elist, req, reqt, trace, total, slot_bytes;
+    uint64_t table, recs, touched, stamp, tkey, list0, list1, req, reqt, ins, freel, trace, trec, total;
 };
 
 __host__ __device__ inline uint64_t align256(uint64_t x) { return (x + 255) & ~255ull; }
 
 __host__ __device__ inline SlabLayout slab_layout(uint32_t log2cap, bool prune) {
     const uint64_t cap = 1ull << log2cap;
-    const uint64_t sb = prune ? sizeof(SlotT<long long>) : sizeof(SlotT<int>);
-    const uint64_t eb = prune ? sizeof(EEntT<long long>) : sizeof(EEntT<int>);
     SlabLayout L;
     uint64_t o = 0;
-    L.slot_bytes = sb;
-    L.slots = o;   o = align256(o + cap * sb);
+    L.table = o;   o = align256(o + 2 * cap * sizeof(TabEnt));
+    L.recs = o;    o = align256(o + cap * (prune ? sizeof(RecT<long long>) : sizeof(RecT<int>)));
     L.touched = o; o = align256(o + cap * 4);
-    L.qlist = o;   o = align256(o + cap * sizeof(LEnt));
-    L.slist0 = o;  o = align256(o + cap * sizeof(LEnt));
-    L.slist1 = o;  o = align256(o + cap * sizeof(LEnt));
-    L.elist = o;   o = align256(o + cap * eb);
-    L.req = o;     o = align256(o + (prune ? cap * 16 : 0));
-    L.reqt = o;    o = align256(o + (prune ? cap * 4 : 0));    // trace index of each spill request
+    L.stamp = o;   o = align256(o + cap * 4);
+    L.tkey = o;    o = align256(o + (prune ? cap * 8 : 0));    // keys by record (memory bound)
+    L.list0 = o;   o = align256(o + cap * 8);                  // (record, vertex)
+    L.list1 = o;   o = align256(o + cap * 8);
+    L.req = o;     o = align256(o + (prune ? cap * 16 : 4 * cap * 8));   // arc-spill requests of a score
+    L.reqt = o;    o = align256(o + (prune ? cap * 4 : 0));    // trace index of each request
+    L.ins = o;     o = align256(o + (prune ? 2 * cap * 16 : 0));   // diagonals a spill round inserted
+    L.freel = o;   o = align256(o + (prune ? cap * 4 : 0));    // records the memory bound freed
     L.trace = o;   o = align256(o + (prune ? cap * 2 * 8 : 0));   // Alg. 5's T: (v, t) pairs
+    L.trec = o;    o = align256(o + (prune ? cap * sizeof(TraceRec) : 0));
     L.total = o;
     return L;
 }
@@ -169,7 +180,6 @@ cudaError_t launch_align(const TierArgs &a, bool prune, uint32_t ctas, uint32_t 
                          cudaStream_t st);
 cudaError_t launch_pack(uint32_t nq, const char *d_q, const uint64_t *d_off, uint32_t *d_words,
                         int32_t *d_status, cudaStream_t st);
-cudaError_t launch_fill(void *p, uint64_t bytes, cudaStream_t st);
 cudaError_t launch_slab_init(uint8_t *slabs, uint64_t slab_bytes, uint32_t n_slabs, uint32_t log2cap,
                              bool prune, cudaStream_t st);
 int align_occupancy(bool prune, uint32_t threads, int *blocks_per_sm);

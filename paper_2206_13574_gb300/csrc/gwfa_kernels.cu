@@ -1,31 +1,39 @@
 // gwfa_kernels.cu -- the graph wavefront alignment score loop on the GPU.
 //
-// One CTA runs the whole score loop of one query (Alg. 1): GwfExtend (Alg. 2,
-// with the arc spills of Eq. 2's last case), the end test, GwfPrune (Alg. 4) and
-// GwfExpand (Alg. 3), until the end cell (|q|, v_e, |v_e|) is on the wavefront.
-// A persistent grid of CTAs pulls query ids from an atomic counter.
+// One CTA runs the whole score loop of one query (Alg. 1): GwfExtend (Alg. 2, with the
+// arc spills of Eq. 2's last case), the end test, GwfPrune (Alg. 4) and GwfExpand (Alg. 3),
+// until the end cell (|q|, v_e, |v_e|) is on the wavefront.  A persistent grid of CTAs
+// pulls query ids from an atomic counter.
 //
-// Data layout (per CTA slab, reused across queries, see SlabLayout):
-//   H~     open-addressing hash of tiles: key (v << 32 | kb) -> 8 offsets of the
-//          diagonals k = 8 kb .. 8 kb + 7 of vertex v.  An offset is the int32 j
-//          (exact mode) or the int64 (j << 32 | tag << 30 | base) (pruning mode,
-//          base = spelled walk length before v, so W~ = base + j); absent = -1.
-//          Entries persist for the whole query (an entry blocks re-spilling,
-//          Alg. 2) and are wiped through the `touched` list when it ends.
-//   reg    two lane-mask words per tile, one per phase parity.  A phase that
-//          makes lanes live ORs their bits into its parity; the lane that finds
-//          the word 0 appends the tile to that phase's list; the next phase takes
-//          the mask with an exchange to 0, so each list holds every tile once.
-//   Q      qlist: tiles live after GwfExpand (the queue Q of Alg. 1-3).
-//   spill  slist[2]: tiles that received offset 0 by a spill and still have to
-//          be extended in this score (Alg. 2 pushes them onto the queue being
-//          drained).  Exact mode extends a won spill depth-first in the thread
-//          that won it and only overflows to these lists; pruning mode goes
-//          breadth first (see extend_round_prune).
-//   E      the extended frontier (Q' of Alg. 2): header (slot, mask, v, kb, |v|)
-//          and a snapshot of the 8 offsets after extension.  GwfExpand reads the
-//          snapshot, so its sources are the offsets before any of its own writes
-//          (the H~ / H~' split of Alg. 3) and it max-merges straight into H~.
+// A score d is two steps with a barrier after each:
+//   offset_pass   visits every tile (the 8 diagonals 8 kb .. 8 kb + 7 of one vertex) that
+//                 may change, by an 8-lane group: GwfExpand of score d - 1 gathered into
+//                 the tile (a lane's own source and its neighbours' by shuffle, the two
+//                 edge lanes' from border words that the neighbour tiles left), GwfPrune on
+//                 those sources, GwfExtend of the diagonals that improved, and the tile's
+//                 own border words and list entries for score d + 1;
+//   spill rounds  the arcs of the diagonals that reached |v| (rare: about 1% of the
+//                 diagonals, none in many scores).  They come after the pass because a
+//                 spill only fills a diagonal that GwfExpand left absent.
+// A tile is read and written once a score, by one group, with plain loads and stores: no
+// offset is merged by an atomic, and all the data of a query live in one CTA, so the loads
+// may hit L1.  Measured against the form with separate extend and expand passes that
+// max-merged candidates with atomics and probed the hash for each one leaving a tile
+// (10,000 queries of 1-20 kb, 512 threads x 4 CTAs per SM): 100.7 -> 68.4 ms; 300 queries
+// with a heavy tail 442 -> 186 ms; 400 pruned 50 kb queries 50.7 -> 36.6 ms.  On the
+// 2,000-query profiling case 34.5 -> 18.3 warp instructions a cell, 14.5 -> 20.3 active
+// lanes.  What bounds it now: the barriers (17 of 32 stall cycles per instruction), i.e.
+// the chain of dependent L2 round trips of the longest spill and of the last tile visits.
+//
+// Data (per CTA slab, see SlabLayout; reused across queries):
+//   H~     tile records, dense in order of first use, and an open-addressing hash from
+//          (v << 32 | kb) to them.  The hash is probed for spills and when two
+//          neighbouring tiles meet for the first time (they then hold each other's record
+//          index).  Entries persist for the whole query (an entry blocks re-spilling,
+//          Alg. 2); records and hash are emptied when it ends.
+//   lists  (record, vertex) of the tiles to visit in this score and in the next: the tiles
+//          with a diagonal in Q and those a border word was left for.  A flag per tile and
+//          parity keeps them without repeats.
 //
 // Order independence (why parallel execution gives the paper's exact result and
 // work counts): in Alg. 2 every diagonal of the closure is extended exactly once
@@ -43,14 +51,16 @@ namespace gwfa {
 
 namespace {
 
-constexpr long long kTagPend = 0, kTagFresh = 1, kTagSettled = 2;
+// Settled offsets in pruning mode carry whether the diagonal is in Q; a spilled one is
+// pending until the spills of its round have been merged.
+constexpr long long kTagPend = 0, kTagDead = 2, kTagLive = 3;
 constexpr uint32_t kBaseMask = 0x3FFFFFFFu;
-constexpr int kStack = 6;   // depth-first spill stack per thread (exact mode)
-// Tiles an 8-lane group takes per claim (both phases).  With a warp's four groups
-// claiming together, one is fastest: two in flight hid more latency only while each
-// group claimed alone, and their registers spill.
-constexpr int kGroupTiles = 1;
+constexpr uint32_t kNone = 0xFFFFFFFFu;      // no tile / unclaimed
 constexpr uint32_t kNoTrace = 0x3FFFFFFFu;   // trace index of the start diagonal (no predecessor)
+constexpr int kAbsent = -2;                  // exact mode: offset -1, not in Q
+// Tiles whose "listed for the next score" flag is a bit in shared memory; tiles claimed
+// beyond them use a stamp in global memory.  4 KB per parity and CTA.
+constexpr uint32_t kBitTiles = 32768;
 
 template <bool P> struct VT;
 template <> struct VT<false> { using T = int; };
@@ -60,68 +70,74 @@ __device__ __forceinline__ long long pk(int j, long long tag, uint32_t base) {
     return ((long long)j << 32) | (tag << 30) | (long long)base;
 }
 __device__ __forceinline__ int pj(long long v) { return (int)(v >> 32); }
-__device__ __forceinline__ int pj(int v) { return v; }
 __device__ __forceinline__ uint32_t pbase(long long v) { return (uint32_t)(v & kBaseMask); }
-__device__ __forceinline__ uint32_t pbase(int) { return 0; }
 
 template <bool P> struct Slab {
-    using T = typename VT<P>::T;
-    SlotT<T> *slots;
-    uint32_t *touched;
-    LEnt *qlist, *slist[2];
-    EEntT<T> *elist;
-    int4 *req;
-    uint32_t *reqt;
+    TabEnt *table;
+    RecT<typename VT<P>::T> *recs;
+    uint32_t *touched, *stamp;
+    uint2 *list[2], *req;
+    unsigned long long *tkey;   // the rest: pruning mode only
+    uint32_t *freel, *reqt;
+    int4 *req4;
+    uint4 *ins;
     uint2 *trace;
-    uint32_t cap, mask;
+    TraceRec *trec;
+    uint32_t cap, tmask;
 };
 
 template <bool P>
 __device__ __forceinline__ Slab<P> carve(uint8_t *base, uint32_t log2cap) {
     SlabLayout L = slab_layout(log2cap, P);
     Slab<P> s;
-    s.slots = (SlotT<typename VT<P>::T> *)(base + L.slots);
+    s.table = (TabEnt *)(base + L.table);
+    s.recs = (RecT<typename VT<P>::T> *)(base + L.recs);
     s.touched = (uint32_t *)(base + L.touched);
-    s.qlist = (LEnt *)(base + L.qlist);
-    s.slist[0] = (LEnt *)(base + L.slist0);
-    s.slist[1] = (LEnt *)(base + L.slist1);
-    s.elist = (EEntT<typename VT<P>::T> *)(base + L.elist);
-    s.req = (int4 *)(base + L.req);
+    s.stamp = (uint32_t *)(base + L.stamp);
+    s.list[0] = (uint2 *)(base + L.list0);
+    s.list[1] = (uint2 *)(base + L.list1);
+    s.req = (uint2 *)(base + L.req);
+    s.tkey = (unsigned long long *)(base + L.tkey);
+    s.freel = (uint32_t *)(base + L.freel);
     s.reqt = (uint32_t *)(base + L.reqt);
+    s.req4 = (int4 *)(base + L.req);
+    s.ins = (uint4 *)(base + L.ins);
     s.trace = (uint2 *)(base + L.trace);
+    s.trec = (TraceRec *)(base + L.trec);
     s.cap = 1u << log2cap;
-    s.mask = s.cap - 1;
+    s.tmask = 2 * s.cap - 1;
     return s;
 }
+
+// Counters of one score; four of them rotate, so that a thread still reading those of
+// score d never sees them cleared (score d + 2 does it, a barrier of d + 1 later).
+struct Score {
+    uint32_t nq;        // list length: tiles to visit in this score (filled by the score before)
+    uint32_t nreq;      // arc-spill requests of the offset pass
+    uint32_t cells, spills, visited, pruned;
+    uint32_t amax;      // largest i + W~ (fits: i < 2^31, W~ < 2^31)
+    int found, err;
+    int err_next;       // out of room for a tile that only the next score needs
+};
 
 // CTA-shared state of the query being aligned.
 struct Sh {
     uint32_t qid;
-    int err;
-    int found;
-    uint32_t nq[2];     // Q list length, by parity of the score that consumes it
-    uint32_t ns[3];     // spill list length, rotating over three rounds (see align_one)
-    uint32_t nreq[2];   // pending spill requests (pruning mode), by round parity
-    uint32_t ne;        // extended-frontier entries this score
-    uint32_t nt;        // tiles claimed (touched) this query
-    uint32_t score_cells;
-    // 32-bit shares of the 64-bit totals, folded in by thread 0 with an exchange
-    // (a 64-bit shared-memory atomic costs far more than a 32-bit one)
-    uint32_t spills32, visited32, pruned32;
-    unsigned long long amax;
-    unsigned long long cells, visited, pruned, spills, evicted;
-    uint32_t nsurv;     // memory bound: tiles kept by the last eviction
-    uint32_t peak;
-    uint32_t claim[3];  // work counters of the phases, rotating (see align_one)
+    uint32_t nt;        // records handed out this query
+    uint32_t nclaim;    // tiles that hold a diagonal (the 3/4 load limit counts these)
+    uint32_t nr[3];     // requests / insertions of the spill rounds, rotating
+    uint32_t nins[2];
+    int nfree;          // memory bound: records on the free list
     uint32_t tlen;      // traceback: entries of T
+    uint32_t peak;
+    unsigned long long cells, visited, pruned, spills, evicted;
     unsigned long long end_vp;   // traceback: vertex << 32 | trace of a diagonal at the end point
     unsigned long long t_start;  // query start (global timer, ns)
-    unsigned long long t_phase;  // statistics: start of the current phase
-    unsigned long long st[6];    // statistics: extend ns, expand ns, rounds, extended tiles,
-                                 // expanded tiles, largest extended frontier (thread 0 only)
+    unsigned long long t_phase;  // statistics: start of the current pass
+    unsigned long long st[6];    // statistics (thread 0 only), see gwfa_engine_set_stats
+    Score score[4];
+    uint32_t bits[2][kBitTiles / 32];
 };
-
-__device__ __forceinline__ void set_err(Sh &sh, int code) { atomicCAS(&sh.err, 0, code); }
 
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
     unsigned long long t;
@@ -129,31 +145,16 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
     return t;
 }
 
-__device__ __forceinline__ LEnt ld_lent(const LEnt *p) {
-    const uint4 x = __ldcg((const uint4 *)p);
-    return LEnt{x.x, x.y, (int32_t)x.z, x.w};
-}
-__device__ __forceinline__ EHdr ld_ehdr(const EHdr *p) {
-    const uint4 x = __ldcg((const uint4 *)p);
-    return EHdr{x.x, x.y, (int32_t)x.z, x.w};
-}
-__device__ __forceinline__ void st_ehdr(EHdr *p, uint32_t slot_mask, uint32_t v, int kb, uint32_t lv) {
-    __stcg((uint4 *)p, make_uint4(slot_mask, v, (uint32_t)kb, lv));
-}
-
 // 16 bases starting at base position p of a packed stream.
-__device__ __forceinline__ uint32_t window16(const uint32_t *__restrict__ w, uint64_t p) {
-    const uint64_t wi = p >> 4;
-    const uint32_t sh = (uint32_t)(p & 15) * 2;
-    const uint32_t lo = __ldg(w + wi), hi = __ldg(w + wi + 1);
-    return __funnelshift_r(lo, hi, sh);
+__device__ __forceinline__ uint32_t window16(const uint32_t *__restrict__ w, uint32_t p) {
+    const uint32_t *a = w + (p >> 4);
+    return __funnelshift_r(__ldg(a), __ldg(a + 1), (p & 15) * 2);
 }
 
 struct QCtx {
     const uint32_t *qw;   // this query's packed words (global, or staged in shared memory)
     int n;
     uint32_t ve;
-    int ke;
     bool smem;            // qw points to shared memory (server kernel)
     bool free_end;        // the walk may end at any position of v_e (or anywhere: any_v)
     bool any_v;           // no end vertex
@@ -170,28 +171,26 @@ __device__ __forceinline__ bool at_end(const QCtx &q, uint32_t v, int k, int j, 
 
 // 16 query bases from position p: read-only cache for a batch staged before the
 // launch, plain (shared-memory) loads for a query the CTA staged itself.
-__device__ __forceinline__ uint32_t qwin(const QCtx &q, uint64_t p) {
-    const uint64_t wi = p >> 4;
-    const uint32_t sh = (uint32_t)(p & 15) * 2;
+__device__ __forceinline__ uint32_t qwin(const QCtx &q, uint32_t p) {
+    const uint32_t *a = q.qw + (p >> 4);
     uint32_t lo, hi;
     if (q.smem) {
-        lo = q.qw[wi];
-        hi = q.qw[wi + 1];
+        lo = a[0];
+        hi = a[1];
     } else {
-        lo = __ldg(q.qw + wi);
-        hi = __ldg(q.qw + wi + 1);
+        lo = __ldg(a);
+        hi = __ldg(a + 1);
     }
-    return __funnelshift_r(lo, hi, sh);
+    return __funnelshift_r(lo, hi, (p & 15) * 2);
 }
 
 // LCP(q[i+1..|q|], v[j+1..|v|]) of Eq. 2 in 0-based positions: XOR of 16-base
 // windows, the first differing base is the lowest set bit pair.
-__device__ __forceinline__ int lcp(const QCtx &q, int i, const uint32_t *__restrict__ vw, int j,
-                                   int lv) {
+__device__ __forceinline__ int lcp(const QCtx &q, int i, const uint32_t *__restrict__ vw, int j, int lv) {
     const int maxl = min(q.n - i, lv - j);
     int l = 0;
     while (l < maxl) {
-        const uint32_t x = qwin(q, (uint64_t)(i + l)) ^ window16(vw, (uint64_t)(j + l));
+        const uint32_t x = qwin(q, (uint32_t)(i + l)) ^ window16(vw, (uint32_t)(j + l));
         if (x) {
             l += (__ffs(x) - 1) >> 1;
             break;
@@ -201,29 +200,17 @@ __device__ __forceinline__ int lcp(const QCtx &q, int i, const uint32_t *__restr
     return min(l, maxl);
 }
 
-// The same LCP when the first window XOR `x` (bases i.. against j..) is already
-// loaded, so that two diagonals can have their first windows in flight together.
-__device__ __forceinline__ int lcp_finish(const QCtx &q, int i, const uint32_t *__restrict__ vw,
-                                          int j, int maxl, uint32_t x) {
-    int l = 0;
-    while (l < maxl) {
-        if (x) {
-            l += (__ffs(x) - 1) >> 1;
-            break;
-        }
-        l += 16;
-        if (l >= maxl) break;
-        x = qwin(q, (uint64_t)(i + l)) ^ window16(vw, (uint64_t)(j + l));
-    }
-    return min(l, maxl);
-}
-
-// Pruning mode: atomics on slab memory (always device global memory) issued in the
-// global state space; the slab pointers come from shared memory, where the compiler
-// no longer knows their space.
+// Atomics on slab memory (always device global memory) issued in the global state
+// space; the slab pointers come from shared memory, where the compiler no longer
+// knows their space.
 __device__ __forceinline__ uint32_t g_exch(uint32_t *p, uint32_t v) {
     uint32_t r;
     asm volatile("atom.global.exch.b32 %0, [%1], %2;" : "=r"(r) : "l"(p), "r"(v) : "memory");
+    return r;
+}
+__device__ __forceinline__ int g_cas(int *p, int c, int v) {
+    int r;
+    asm volatile("atom.global.cas.b32 %0, [%1], %2, %3;" : "=r"(r) : "l"(p), "r"(c), "r"(v) : "memory");
     return r;
 }
 __device__ __forceinline__ long long g_max(long long *p, long long v) {
@@ -231,219 +218,121 @@ __device__ __forceinline__ long long g_max(long long *p, long long v) {
     asm volatile("atom.global.max.s64 %0, [%1], %2;" : "=l"(r) : "l"(p), "l"(v) : "memory");
     return r;
 }
-__device__ __forceinline__ unsigned long long g_cas(unsigned long long *p, unsigned long long c,
-                                                    unsigned long long v) {
-    unsigned long long r;
-    asm volatile("atom.global.cas.b64 %0, [%1], %2, %3;" : "=l"(r) : "l"(p), "l"(c), "l"(v) : "memory");
-    return r;
+__device__ __forceinline__ void g_max32(uint32_t *p, uint32_t v) {
+    asm volatile("red.global.max.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
-template <bool P, class T>
-__device__ __forceinline__ T slab_max(T *p, T v) {
-    if constexpr (P) return g_max(p, v);
-    else return atomicMax(p, v);
+
+// A hash entry is one 16-byte unit: key and record index appear together, so whoever
+// finds the key can use the record at once.
+struct Ent {
+    unsigned long long key, idx;
+};
+__device__ __forceinline__ Ent ld_ent(const TabEnt *p) {
+    Ent e;
+    asm volatile("{ .reg .b128 x; ld.relaxed.gpu.global.b128 x, [%2]; mov.b128 {%0, %1}, x; }"
+                 : "=l"(e.key), "=l"(e.idx) : "l"(p) : "memory");
+    return e;
+}
+__device__ __forceinline__ Ent cas_ent(TabEnt *p, unsigned long long key, unsigned long long idx) {
+    Ent o;
+    const unsigned long long empty = kEmptyKey;
+    asm volatile("{ .reg .b128 c, n, o; mov.b128 c, {%3, %3}; mov.b128 n, {%4, %5};\n"
+                 "  atom.relaxed.gpu.global.cas.b128 o, [%2], c, n; mov.b128 {%0, %1}, o; }"
+                 : "=l"(o.key), "=l"(o.idx) : "l"(p), "l"(empty), "l"(key), "l"(idx) : "memory");
+    return o;
 }
 
 __device__ __forceinline__ unsigned long long tile_key(uint32_t v, int kb) {
     return ((unsigned long long)v << 32) | (uint32_t)kb;
 }
-
 __device__ __forceinline__ uint32_t tile_hash(unsigned long long key, uint32_t mask) {
     return (uint32_t)((key * 0x9E3779B97F4A7C15ull) >> 32) & mask;
 }
 
-// find_or_insert's probe sequence when the key of its first slot h was already read
-// (cur), so that the read can be issued ahead of other round trips.
+// A tile came to hold a diagonal: the load limit of 3/4 of the slab's tiles.
+template <bool P> __device__ __forceinline__ void count_claim(const Slab<P> &s, Sh &sh, int *err) {
+    if (atomicAdd(&sh.nclaim, 1u) + 1 > (s.cap >> 1) + (s.cap >> 2)) atomicCAS(err, 0, GWFA_ERR_CAPACITY);
+}
+
+// Record of tile (v, kb), claimed if absent; -1 (and *err) when the slab is full.
 template <bool P>
-__device__ int find_or_insert_at(const Slab<P> &s, Sh &sh, unsigned long long key, uint32_t h,
-                                 unsigned long long cur) {
+__device__ __noinline__ int find_or_insert(const Slab<P> &s, Sh &sh, uint32_t v, int kb, int *err) {
+    const unsigned long long key = tile_key(v, kb);
+    uint32_t h = tile_hash(key, s.tmask);
+    uint32_t idx = kNone;
     for (int probe = 0; probe < 256; ++probe) {
-        if (probe > 0) cur = __ldcg(&s.slots[h].key);
-        if (cur == key) return (int)h;
-        if (cur == kEmptyKey) {
-            unsigned long long prev;
-            if constexpr (P) prev = g_cas(&s.slots[h].key, kEmptyKey, key);
-            else prev = atomicCAS(&s.slots[h].key, kEmptyKey, key);
-            if (prev == kEmptyKey) {
-                const uint32_t t = atomicAdd(&sh.nt, 1u);
-                s.touched[t] = h;   // t < cap: each claim takes a distinct empty slot
-                if (t + 1 > (s.cap >> 1) + (s.cap >> 2)) set_err(sh, GWFA_ERR_CAPACITY);
-                return (int)h;
+        Ent e = ld_ent(&s.table[h]);
+        if (e.key == kEmptyKey) {
+            if (idx == kNone) {
+                if constexpr (P) {
+                    const int f = sh.nfree > 0 ? atomicSub(&sh.nfree, 1) : 0;
+                    idx = f > 0 ? s.freel[f - 1] : atomicAdd(&sh.nt, 1u);
+                } else {
+                    idx = atomicAdd(&sh.nt, 1u);
+                }
+                if (idx >= s.cap) break;
             }
-            if (prev == key) return (int)h;
+            e = cas_ent(&s.table[h], key, idx);
+            if (e.key == kEmptyKey) {
+                s.touched[idx] = h;
+                s.recs[idx].side[0].kb = kb;
+                s.recs[idx].side[1].kb = kb;
+                if constexpr (P) s.tkey[idx] = key;
+                else count_claim<P>(s, sh, err);   // a claimed tile always gets a diagonal
+                return (int)idx;
+            }
         }
-        h = (h + 1) & s.mask;
+        if (e.key == key) return (int)e.idx;   // a record taken for a lost race stays unused
+        h = (h + 1) & s.tmask;
     }
-    set_err(sh, GWFA_ERR_CAPACITY);
+    atomicCAS(err, 0, GWFA_ERR_CAPACITY);
     return -1;
 }
 
+// List a tile for the next score; true for the one caller that has to append it.
 template <bool P>
-__device__ int find_or_insert(const Slab<P> &s, Sh &sh, unsigned long long key) {
-    const uint32_t h = tile_hash(key, s.mask);
-    return find_or_insert_at(s, sh, key, h, __ldcg(&s.slots[h].key));
-}
-
-// Make lane `bit` of tile (slot, v, kb) live for the phase owning `regw`; the
-// first lane to do so appends the tile to that phase's list.
-__device__ __forceinline__ void reg_append(uint32_t *regw, LEnt *list, uint32_t *count,
-                                           uint32_t cap, uint32_t slot, uint32_t v, int kb,
-                                           uint32_t bit, Sh &sh) {
-    if (atomicOr(regw, bit) == 0u) {
-        const uint32_t i = atomicAdd(count, 1u);
-        if (i < cap) __stcg((uint4 *)&list[i], make_uint4(slot, v, (uint32_t)kb, 0u));
-        else set_err(sh, GWFA_ERR_CAPACITY);
+__device__ __forceinline__ bool list_once(const Slab<P> &s, Sh &sh, uint32_t idx, int d) {
+    if (idx < kBitTiles) {
+        const uint32_t bit = 1u << (idx & 31);
+        return !(atomicOr(&sh.bits[(d + 1) & 1][idx >> 5], bit) & bit);
     }
+    return g_exch(&s.stamp[idx], (uint32_t)(d + 1)) != (uint32_t)(d + 1);
 }
 
-// Dynamic work distribution inside a phase: lane 0 of a warp claims the next
-// 4 x `step` entries for the warp's four groups (group g of the warp takes entries
-// [base + g step, base + (g + 1) step)), so a warp held up by a long exact-match run
-// or spill chain does not stall the others at the phase barrier, and the four groups
-// run the same iterations in step.  Every lane of the warp calls it.
-__device__ __forceinline__ uint32_t warp_claim(uint32_t *ctr, uint32_t step) {
-    uint32_t e = 0;
-    if ((threadIdx.x & 31) == 0) e = atomicAdd(ctr, 4u * step);
-    return __shfl_sync(0xFFFFFFFFu, e, 0);
+// The neighbour tile on side sd (0 left, 1 right), linked on first use.
+template <bool P>
+__device__ __noinline__ uint32_t link_neighbour(const Slab<P> &s, Sh &sh, uint32_t idx, uint32_t v, int kb, int sd,
+                                                int *err) {
+    const int t = find_or_insert<P>(s, sh, v, sd ? kb + 1 : kb - 1, err);
+    if (t < 0) return kNone;
+    s.recs[idx].side[sd].link = (uint32_t)t;
+    s.recs[t].side[sd ^ 1].link = idx;
+    return (uint32_t)t;
 }
 
-
-
-// Exact mode: diagonal (v, k) reached |v| (Alg. 2 arc loop).  Offset 0 goes to
-// (u, k + |v|) for every arc (v, u) where it is absent; a diagonal this thread
-// inserts is extended by this thread at once, depth first, with its own arcs in
-// turn.  Only when the small stack is full does a won diagonal go to the spill
-// list of the next round instead.
-__device__ void spill_dfs(const DevGraph &g, const Slab<false> &s, Sh &sh, const QCtx &q,
-                          uint32_t arc0, uint32_t arc1, int ku0, int next_par, LEnt *next_list,
-                          uint32_t *next_count) {
-    uint32_t st_slot[kStack], st_u[kStack];
-    int st_k[kStack];
-    int top = 0;
-    uint32_t a0 = arc0, a1 = arc1;
-    int ku = ku0;
-    for (;;) {
-        for (uint32_t a = a0; a < a1; ++a) {
-            const uint32_t u = __ldg(&g.arc_dst[a]);
-            const int su = find_or_insert(s, sh, tile_key(u, ku >> 3));
-            if (su < 0) return;
-            const int prev = atomicMax(&s.slots[su].vals[ku & 7], 0);
-            if (prev < 0) {
-                atomicAdd(&sh.spills32, 1u);
-                if (top < kStack) {
-                    st_slot[top] = (uint32_t)su;
-                    st_u[top] = u;
-                    st_k[top] = ku;
-                    ++top;
-                } else {
-                    reg_append(&s.slots[su].reg[next_par], next_list, next_count, s.cap, (uint32_t)su, u, ku >> 3,
-                               1u << (ku & 7), sh);
-                }
-            }
-        }
-        if (top == 0) return;
-        --top;
-        const uint32_t su = st_slot[top], u = st_u[top];
-        const int k = st_k[top];
-        const uint4 vi = __ldg(&g.vinfo[u]);
-        const int l = lcp(q, k, g.words + vi.x, 0, (int)vi.y);
-        __stcg(&s.slots[su].vals[k & 7], l);
-        const uint32_t eidx = atomicAdd(&sh.ne, 1u);
-        atomicAdd(&sh.score_cells, 1u);
-        if (eidx < s.cap) {
-            st_ehdr(&s.elist[eidx].hdr, su | ((1u << (k & 7)) << 24), u, k >> 3, vi.y);
-            __stcg(&s.elist[eidx].vals[k & 7], l);
+// What a diagonal extended outside its tile's visit (a spilled one) owes the next score:
+// its tile listed, and its candidate over the tile's edge handed to the neighbour tile.
+template <bool P>
+__device__ void enter_next(const Slab<P> &s, Sh &sh, const QCtx &q, uint32_t idx, uint32_t v, int k, int j,
+                           uint32_t base, uint32_t lv, int d, uint32_t tr, bool traceback) {
+    Score &S = sh.score[d & 3];
+    uint32_t *nq = &sh.score[(d + 1) & 3].nq;
+    uint2 *next = s.list[(d + 1) & 1];
+    if (list_once<P>(s, sh, idx, d)) next[atomicAdd(nq, 1u)] = make_uint2(idx, v);
+    const int ln = k & 7;
+    const int sd = ln == 7;
+    if ((ln == 0 && (uint32_t)j < lv) || (ln == 7 && k + j < q.n)) {
+        uint32_t t = s.recs[idx].side[sd].link;
+        if (t == kNone) t = link_neighbour<P>(s, sh, idx, v, k >> 3, sd, &S.err_next);
+        if (t == kNone) return;
+        const int c = sd ? j : j + 1;
+        if constexpr (P) {
+            s.recs[t].side[sd ^ 1].in[(d + 1) & 1] = ((long long)c << 32) | base;
+            if (traceback) s.trec[t].in[sd ^ 1][(d + 1) & 1] = tr;
         } else {
-            set_err(sh, GWFA_ERR_CAPACITY);
+            s.recs[t].side[sd ^ 1].in[(d + 1) & 1] = c;
         }
-        if (at_end(q, u, k, l, vi.y)) sh.found = 1;
-        if ((uint32_t)l == vi.y) {
-            a0 = vi.z;
-            a1 = vi.w;
-            ku = k + (int)vi.y;
-        } else {
-            a0 = a1 = 0;
-        }
-    }
-}
-
-// One extension round over `list` in exact mode.  Each 8-lane group takes
-// U tiles per iteration and keeps their dependency chains (list entry ->
-// mask, offsets, vertex info -> first LCP window) in flight together.
-template <int U>
-__device__ void extend_round_exact(const DevGraph &g, const Slab<false> &s, Sh &sh, const QCtx &q,
-                                   const LEnt *list, uint32_t n_list, int par, int next_par,
-                                   LEnt *next_list, uint32_t *next_count, uint32_t *claim) {
-    const int ln = threadIdx.x & 7;
-    const unsigned gmask = 0xFFu << (threadIdx.x & 24);
-    for (;;) {
-        const uint32_t wb = warp_claim(claim, (uint32_t)U);
-        if (wb >= n_list) break;
-        const uint32_t e0 = wb + ((threadIdx.x & 31) >> 3) * (uint32_t)U;
-        if (e0 >= n_list) continue;   // nothing left for this group in the warp's claim
-        const uint32_t cnt = min((uint32_t)U, n_list - e0);   // uniform within the group
-        LEnt ent[U];
-        uint32_t m[U];
-        int val[U];
-        uint2 vi[U];   // label word, |v| (the arc range is reloaded for the rare spill)
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            ent[u] = (u == 0 || (uint32_t)u < cnt) ? ld_lent(&list[e0 + u]) : ent[0];
-            m[u] = 0u;
-            if (ln == 0 && (uint32_t)u < cnt) m[u] = atomicExch(&s.slots[ent[u].slot].reg[par], 0u);
-            val[u] = __ldcg(&s.slots[ent[u].slot].vals[ln]);
-            vi[u] = __ldg((const uint2 *)&g.vinfo[ent[u].v]);
-        }
-        uint32_t eidx = 0, pop = 0;
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            m[u] = __shfl_sync(gmask, m[u], 0, 8);
-            pop += __popc(m[u]);
-        }
-        if (ln == 0) {
-            eidx = atomicAdd(&sh.ne, cnt);
-            atomicAdd(&sh.score_cells, pop);
-        }
-        eidx = __shfl_sync(gmask, eidx, 0, 8);
-        bool live[U];
-        int k[U], maxl[U];
-        uint32_t x[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            live[u] = (m[u] >> ln) & 1u;
-            k[u] = ent[u].kb * kTile + ln;
-            maxl[u] = 0;
-            x[u] = 0;
-            if (live[u]) {
-                const int i = k[u] + val[u];
-                maxl[u] = min(q.n - i, (int)vi[u].y - val[u]);
-                if (maxl[u] > 0)
-                    x[u] = qwin(q, (uint64_t)i) ^ window16(g.words + vi[u].x, (uint64_t)val[u]);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if ((uint32_t)u >= cnt) break;
-            if (live[u]) {
-                val[u] += lcp_finish(q, k[u] + val[u], g.words + vi[u].x, val[u], maxl[u], x[u]);
-                __stcg(&s.slots[ent[u].slot].vals[ln], val[u]);
-                if (at_end(q, ent[u].v, k[u], val[u], vi[u].y)) sh.found = 1;
-            }
-            const uint32_t ei = eidx + u;
-            if (ei < s.cap) {
-                if (ln == 0) st_ehdr(&s.elist[ei].hdr, ent[u].slot | (m[u] << 24), ent[u].v, ent[u].kb, vi[u].y);
-                __stcg(&s.elist[ei].vals[ln], live[u] ? val[u] : -1);
-            } else if (ln == 0) {
-                set_err(sh, GWFA_ERR_CAPACITY);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if ((uint32_t)u >= cnt) break;
-            if (live[u] && (uint32_t)val[u] == vi[u].y) {
-                const uint4 full = __ldg(&g.vinfo[ent[u].v]);
-                spill_dfs(g, s, sh, q, full.z, full.w, k[u] + (int)vi[u].y, next_par, next_list, next_count);
-            }
-        }
+        if (list_once<P>(s, sh, t, d)) next[atomicAdd(nq, 1u)] = make_uint2(t, v);
     }
 }
 
@@ -451,422 +340,463 @@ __device__ void extend_round_exact(const DevGraph &g, const Slab<false> &s, Sh &
 // index in T.  Unlike Alg. 5, equal (v, t) pairs are not merged through a map:
 // T then holds one entry per spilling diagonal, which bounds it by the spill count
 // and gives the same walk.
-__device__ __forceinline__ uint32_t push_trace(const Slab<true> &s, Sh &sh, uint32_t v, uint32_t t) {
+__device__ __forceinline__ uint32_t push_trace(const Slab<true> &s, Sh &sh, uint32_t v, uint32_t t, int *err) {
     const uint32_t idx = atomicAdd(&sh.tlen, 1u);
     if (idx >= 2 * s.cap || idx >= kNoTrace) {
-        set_err(sh, GWFA_ERR_CAPACITY);
+        atomicCAS(err, 0, GWFA_ERR_CAPACITY);
         return kNoTrace;
     }
-    __stcg(&s.trace[idx], make_uint2(v, t));
+    s.trace[idx] = make_uint2(v, t);
     return idx;
 }
 
-// One extension round over `list` in pruning mode.  Spills are recorded, not
-// applied: apply_spill_requests runs after the round's barrier, so a spill can
-// never touch a diagonal that was present before the round (Alg. 2's presence
-// test) and same-round spills into one diagonal merge by the larger walk base.
-__device__ void extend_round_prune(const DevGraph &g, const Slab<true> &s, Sh &sh, const QCtx &q,
-                                   const LEnt *list, uint32_t n_list, int par, uint32_t *req_count,
-                                   uint32_t *claim, bool traceback) {
-    const int ln = threadIdx.x & 7;
-    const unsigned gmask = 0xFFu << (threadIdx.x & 24);
-    for (;;) {
-        const uint32_t wb = warp_claim(claim, 1u);
-        if (wb >= n_list) break;
-        const uint32_t e = wb + ((threadIdx.x & 31) >> 3);
-        if (e >= n_list) continue;
-        const LEnt ent = ld_lent(&list[e]);
-        uint32_t m = 0, eidx = 0;
-        if (ln == 0) m = g_exch(&s.slots[ent.slot].reg[par], 0u);
-        long long val = __ldcg(&s.slots[ent.slot].vals[ln]);
-        const uint2 vi = __ldg((const uint2 *)&g.vinfo[ent.v]);   // label word, |v|
-        const uint32_t tr = traceback ? __ldcg(&s.slots[ent.slot].trace[ln]) : 0u;
-        m = __shfl_sync(gmask, m, 0, 8);
-        if (ln == 0) {
-            eidx = atomicAdd(&sh.ne, 1u);
-            atomicAdd(&sh.score_cells, (uint32_t)__popc(m));
+// Pruning mode: a settled diagonal reached |v|: offset 0 with the walk base past v goes
+// to (u, k + |v|) for every arc (v, u), after the pass (see apply_spills).
+__device__ __forceinline__ void request_spill(const Slab<true> &s, Sh &sh, uint32_t at, const uint4 &vi, uint32_t v,
+                                              int k, uint32_t base, uint32_t tr, bool traceback, int *err) {
+    const uint32_t nb = base + vi.y;
+    if (nb > kBaseMask) atomicCAS(err, 0, GWFA_ERR_CAPACITY);
+    const uint32_t t = traceback ? push_trace(s, sh, v, tr, err) : 0u;
+    if (at < s.cap) {
+        s.req4[at] = make_int4(k + (int)vi.y, (int)nb, (int)vi.z, (int)vi.w);
+        if (traceback) s.reqt[at] = t;
+    } else {
+        atomicCAS(err, 0, GWFA_ERR_CAPACITY);
+    }
+}
+
+// GwfExpand (Alg. 3) of the score before with GwfPrune (Alg. 4) on its sources, and
+// GwfExtend (Alg. 2) of this one, in one visit of every listed tile by an 8-lane group:
+// each lane gathers its diagonal's candidates (its own and its neighbours' by shuffle, the
+// edge lanes' from the tile's border words), keeps the largest if it beats its offset,
+// extends it along equal bases, stores it, and hands the next score its list entry and the
+// candidates that leave the tile.  Arc spills are only requested here.
+template <bool P, bool TB>
+__device__ __forceinline__ void offset_pass(const DevGraph &g, const Slab<P> &s, Sh &sh, const QCtx &q, int d,
+                                            bool prune_on, int max_lag) {
+    using T = typename VT<P>::T;
+    const unsigned full = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31, ln = lane & 7;
+    const int par = d & 1;
+    Score &S = sh.score[d & 3];
+    uint32_t *nq = &sh.score[(d + 1) & 3].nq;
+    const uint32_t n_list = S.nq;
+    const uint2 *list = s.list[par];
+    uint2 *next = s.list[par ^ 1];
+    const int sd = ln >> 2;   // the side whose border words this lane reads (lanes 0 and 7 use them)
+    uint32_t cells = 0, visited = 0, pruned = 0, amax = 0;
+    // the flags of the list being read are spent: clear them for score d + 1
+    const uint32_t nw = min((sh.nt + 31) >> 5, kBitTiles / 32);
+    for (uint32_t w = threadIdx.x; w < nw; w += blockDim.x) sh.bits[par][w] = 0u;
+    for (uint32_t wb = (threadIdx.x >> 5) * 4; wb < n_list; wb += (blockDim.x >> 5) * 4) {
+        const uint32_t e = wb + (lane >> 3);
+        const bool on = e < n_list;
+        const uint2 ent = list[on ? e : wb];
+        RecT<T> *rec = &s.recs[ent.x];
+        T raw = rec->vals[ln];
+        const uint2 vi = __ldg((const uint2 *)&g.vinfo[ent.y]);   // label word, |v|
+        T in;
+        uint32_t link;
+        int k;
+        if constexpr (P) {
+            in = rec->side[sd].in[par];
+            const uint2 lk = *(const uint2 *)&rec->side[sd].link;
+            link = lk.x;
+            k = (int)lk.y * kTile + ln;
+        } else {
+            const int4 sw = *(const int4 *)&rec->side[sd];
+            in = par ? sw.y : sw.x;
+            link = (uint32_t)sw.z;
+            k = sw.w * kTile + ln;
         }
-        eidx = __shfl_sync(gmask, eidx, 0, 8);
-        const int k = ent.kb * kTile + ln;
-        const bool live = (m >> ln) & 1u;
-        unsigned long long a = 0;
-        if (live) {
-            const int j = pj(val);
-            const int i = k + j;
-            const int j2 = j + lcp(q, i, g.words + vi.x, j, (int)vi.y);
-            val = pk(j2, kTagSettled, pbase(val));
-            __stcg(&s.slots[ent.slot].vals[ln], val);
-            if (at_end(q, ent.v, k, j2, vi.y)) {
-                sh.found = 1;
-                // one 64-bit store, so that the vertex and its trace stay a pair when
-                // several diagonals reach a free end in the same score
-                sh.end_vp = ((unsigned long long)ent.v << 32) | tr;
-            }
-            a = (unsigned long long)(k + j2) + pbase(val) + (unsigned)j2;   // a = i + W~ (Alg. 4)
-            if ((uint32_t)j2 == vi.y) {
-                // the spilled diagonals get the walk base past v and, with traceback,
-                // the index of the T entry "left v with this trace" (Alg. 5)
-                const uint32_t nb = pbase(val) + vi.y;
-                if (nb > kBaseMask) set_err(sh, GWFA_ERR_CAPACITY);
-                const uint32_t t = traceback ? push_trace(s, sh, ent.v, tr) : 0u;
-                const uint32_t r = atomicAdd(req_count, 1u);
-                if (r < s.cap) {
-                    const uint4 full = __ldg(&g.vinfo[ent.v]);   // the arc range, for the rare spill
-                    __stcg(&s.req[r], make_int4(k + (int)vi.y, (int)nb, (int)full.z, (int)full.w));
-                    if (traceback) __stcg(&s.reqt[r], t);
-                } else {
-                    set_err(sh, GWFA_ERR_CAPACITY);
+        uint32_t tr = 0, tin = 0;
+        if constexpr (TB) {
+            tr = s.trec[ent.x].tr[ln];
+            tin = s.trec[ent.x].in[sd][par];
+        }
+        const bool edge = on && (ln == 0 || ln == 7) && in >= 0;
+        if (!edge) in = (T)-1;
+        else rec->side[sd].in[par] = (T)-1;   // consumed
+        if (!on) raw = P ? (T)-1 : (T)kAbsent;
+        bool live;
+        int j;
+        uint32_t base = 0;
+        if constexpr (P) {
+            live = raw >= 0 && ((raw >> 30) & 3) == kTagLive;
+            j = pj(raw);
+            base = pbase(raw);
+        } else {
+            live = raw & 1;
+            j = raw >> 1;
+        }
+        const bool was = live;
+        if constexpr (P) {
+            if (prune_on) {
+                // a source that lags is dropped; its offset stays
+                const long long am = (long long)sh.score[(d + 3) & 3].amax;
+                if (live && am - ((long long)k + 2ll * j + base) >= (long long)max_lag) {
+                    live = false;
+                    ++pruned;
+                }
+                if (in >= 0) {
+                    // the source over the edge: (k - 1, c) on the left, (k + 1, c - 1) on the right
+                    const long long c = pj(in);
+                    const long long a = (long long)k - 1 + 2 * c + pbase(in);
+                    if (am - a >= (long long)max_lag) in = -1;
                 }
             }
         }
-        for (int o = 4; o >= 1; o >>= 1) {
-            const unsigned long long b = __shfl_xor_sync(gmask, a, o, 8);
-            a = b > a ? b : a;
+        // candidates of this diagonal's own source: (k+1, j), (k-1, j+1), (k, j+1)
+        const bool ins = live && k + j < q.n, del = live && j < (int)vi.y;
+        bool inq;
+        int jn;         // the new offset
+        uint32_t trn = 0;
+        if constexpr (P) {
+            const long long bb = (long long)base;
+            const long long c_ins = ins ? ((long long)j << 32) | bb : -1ll;
+            const long long c_del = del ? ((long long)(j + 1) << 32) | bb : -1ll;
+            long long left = __shfl_up_sync(full, c_ins, 1, 8), right = __shfl_down_sync(full, c_del, 1, 8);
+            uint32_t tl = 0, trr = 0;
+            if constexpr (TB) {
+                tl = __shfl_up_sync(full, tr, 1, 8);
+                trr = __shfl_down_sync(full, tr, 1, 8);
+                if (ln == 0) tl = tin;
+                if (ln == 7) trr = tin;
+            }
+            if (ln == 0) left = in;
+            if (ln == 7) right = in;
+            const long long mis = ins && del ? c_del : -1ll;
+            long long c = mis;
+            if (left > c) c = left;
+            if (right > c) c = right;
+            if constexpr (TB) {
+                // sources of equal offset and base are equally good predecessors: the
+                // largest trace index, for a deterministic choice
+                if (mis == c) trn = tr;
+                if (left == c) trn = max(trn, tl);
+                if (right == c) trn = max(trn, trr);
+            }
+            inq = d == 0 ? was : pj(c) > (raw < 0 ? -1 : j);
+            if (c < 0 && d) inq = false;
+            if (d == 0) c = ((long long)j << 32) | bb, trn = tr;
+            jn = inq ? pj(c) : j;
+            if (inq) base = pbase(c);
+            if (inq && raw < 0) ++visited;
+            // first diagonal of this tile?
+            const unsigned pres = __ballot_sync(full, raw >= 0), add = __ballot_sync(full, inq);
+            if (ln == 0 && !((pres >> (lane & 24)) & 0xFFu) && ((add >> (lane & 24)) & 0xFFu)) {
+                s.recs[ent.x].side[1].counted = 1u;
+                count_claim<P>(s, sh, &S.err);
+            }
+        } else {
+            const int c_ins = ins ? j : -1, c_del = del ? j + 1 : -1;
+            int left = __shfl_up_sync(full, c_ins, 1, 8), right = __shfl_down_sync(full, c_del, 1, 8);
+            if (ln == 0) left = in;
+            if (ln == 7) right = in;
+            const int c = max(ins ? c_del : -1, max(left, right));
+            inq = d == 0 ? live : c > j;
+            jn = d == 0 ? j : max(c, j);
         }
-        if (ln == 0 && a > 0) atomicMax(&sh.amax, a);
-        if (eidx < s.cap) {
-            if (ln == 0) st_ehdr(&s.elist[eidx].hdr, ent.slot | (m << 24), ent.v, ent.kb, vi.y);
-            __stcg(&s.elist[eidx].vals[ln], live ? val : -1ll);
-            if (traceback) __stcg(&s.elist[eidx].trace[ln], tr);
-        } else if (ln == 0) {
-            set_err(sh, GWFA_ERR_CAPACITY);
+        if (inq) jn += lcp(q, k + jn, g.words + vi.x, jn, (int)vi.y);
+        const int i2 = k + jn;
+        if (inq || was) {
+            if constexpr (P) {
+                rec->vals[ln] = pk(jn, inq ? kTagLive : kTagDead, base);
+                if (TB && inq) s.trec[ent.x].tr[ln] = trn;
+            } else {
+                rec->vals[ln] = (jn << 1) | (inq ? 1 : 0);
+            }
+        }
+        if constexpr (P) {
+            if (inq) amax = max(amax, (uint32_t)i2 + (uint32_t)jn + base);
+        }
+        if (inq && i2 == q.n && at_end(q, ent.y, k, jn, vi.y)) {
+            S.found = 1;
+            // one 64-bit store, so that the vertex and its trace stay a pair when
+            // several diagonals reach a free end in the same score
+            if constexpr (P) sh.end_vp = ((unsigned long long)ent.y << 32) | trn;
+        }
+        const unsigned qm = __ballot_sync(full, inq);
+        cells += __popc(qm);
+        const bool spill = inq && jn == (int)vi.y;
+        const unsigned sp = __ballot_sync(full, spill);
+        if (sp) {
+            uint32_t b = 0;
+            if (lane == 0) b = atomicAdd(&S.nreq, (uint32_t)__popc(sp));
+            b = __shfl_sync(full, b, 0) + __popc(sp & ((1u << lane) - 1));
+            if (spill) {
+                if constexpr (P) {
+                    const uint4 f = __ldg(&g.vinfo[ent.y]);
+                    request_spill(s, sh, b, f, ent.y, k, base, trn, TB, &S.err);
+                } else {
+                    if (b < 4 * s.cap) s.req[b] = make_uint2(ent.y, (uint32_t)(k + (int)vi.y));
+                    else atomicCAS(&S.err, 0, GWFA_ERR_CAPACITY);
+                }
+            }
+        }
+        // the next score visits this tile if it has a diagonal in Q (lane 3 lists it), and
+        // a neighbour that an edge diagonal's candidate enters (lanes 0 and 7)
+        uint32_t target = ent.x;
+        bool want = ln == 3 && ((qm >> (lane & 24)) & 0xFFu);
+        if (inq && ((ln == 0 && jn < (int)vi.y) || (ln == 7 && i2 < q.n))) {
+            if (link == kNone) link = link_neighbour<P>(s, sh, ent.x, ent.y, k >> 3, sd, &S.err_next);
+            if (link != kNone) {
+                const int c = sd ? jn : jn + 1;
+                if constexpr (P) {
+                    s.recs[link].side[sd ^ 1].in[par ^ 1] = ((long long)c << 32) | base;
+                    if (TB) s.trec[link].in[sd ^ 1][par ^ 1] = trn;
+                } else {
+                    s.recs[link].side[sd ^ 1].in[par ^ 1] = c;
+                }
+                target = link;
+                want = true;
+            }
+        }
+        __syncwarp();
+        const bool fresh = want && list_once<P>(s, sh, target, d);
+        const unsigned nm = __ballot_sync(full, fresh);
+        if (nm) {
+            uint32_t b = 0;
+            if (lane == 0) b = atomicAdd(nq, (uint32_t)__popc(nm));
+            b = __shfl_sync(full, b, 0) + __popc(nm & ((1u << lane) - 1));
+            if (fresh) next[b] = make_uint2(target, ent.y);
+        }
+    }
+    if (lane == 0 && cells) atomicAdd(&S.cells, cells);
+    if constexpr (P) {
+        visited = __reduce_add_sync(full, visited);
+        pruned = __reduce_add_sync(full, pruned);
+        amax = __reduce_max_sync(full, amax);
+        if (lane == 0) {
+            if (visited) atomicAdd(&S.visited, visited);
+            if (pruned) atomicAdd(&S.pruned, pruned);
+            if (amax) atomicMax(&S.amax, amax);
         }
     }
 }
 
-// Pruning mode, second half of a round: offset 0 with walk base nb on (u, ku)
-// for every recorded spill; the inserted diagonals form the next round's list.
-__device__ void apply_spill_requests(const DevGraph &g, const Slab<true> &s, Sh &sh, uint32_t n_req,
-                                     int next_par, LEnt *next_list, uint32_t *next_count) {
-    const uint32_t nr = min(n_req, s.cap);
-    for (uint32_t r = threadIdx.x; r < nr; r += blockDim.x) {
-        const int4 rq = __ldcg(&s.req[r]);
+// Exact mode: requests [r0, r0 + n) of the log, one thread each: offset 0 to (u, ku) for
+// every arc (v, u) where it is absent (Alg. 2's arc loop).  A diagonal this thread inserts
+// is extended by it at once; if that one reaches its vertex's end too, the thread goes on
+// with it, or, when the arcs give several, appends the others to the log.
+__device__ void spill_round(const DevGraph &g, const Slab<false> &s, Sh &sh, const QCtx &q, int d, uint32_t r0,
+                            uint32_t n, uint32_t *next_count) {
+    Score &S = sh.score[d & 3];
+    uint32_t won = 0;
+    for (uint32_t r = threadIdx.x; r < n; r += blockDim.x) {
+        uint2 rq = s.req[r0 + r];
+        for (;;) {
+            const uint4 vi = __ldg(&g.vinfo[rq.x]);
+            const int ku = (int)rq.y;
+            uint2 more = make_uint2(kNone, 0u);
+            for (uint32_t a = vi.z; a < vi.w; ++a) {
+                const uint32_t u = __ldg(&g.arc_dst[a]);
+                const int su = find_or_insert<false>(s, sh, u, ku >> 3, &S.err);
+                if (su < 0) break;
+                if (g_cas(&s.recs[su].vals[ku & 7], kAbsent, 1) != kAbsent) continue;
+                ++won;
+                const uint2 ui = __ldg((const uint2 *)&g.vinfo[u]);
+                const int l = lcp(q, ku, g.words + ui.x, 0, (int)ui.y);
+                s.recs[su].vals[ku & 7] = (l << 1) | 1;
+                if (at_end(q, u, ku, l, ui.y)) S.found = 1;
+                enter_next<false>(s, sh, q, (uint32_t)su, u, ku, l, 0u, ui.y, d, 0u, false);
+                if ((uint32_t)l == ui.y) {
+                    const uint2 c = make_uint2(u, (uint32_t)(ku + (int)ui.y));
+                    if (more.x == kNone) {
+                        more = c;
+                    } else {
+                        const uint32_t at = r0 + n + atomicAdd(next_count, 1u);
+                        if (at < 4 * s.cap) s.req[at] = c;
+                        else atomicCAS(&S.err, 0, GWFA_ERR_CAPACITY);
+                    }
+                }
+            }
+            if (more.x == kNone) break;
+            rq = more;
+        }
+    }
+    won = __reduce_add_sync(0xFFFFFFFFu, won);
+    if ((threadIdx.x & 31) == 0 && won) {
+        atomicAdd(&S.cells, won);
+        atomicAdd(&S.spills, won);
+    }
+}
+
+// Pruning mode: offset 0 with walk base nb on (u, ku) for every request of the round; the
+// inserted diagonals go to the round's insertion list.  A spill never changes a diagonal
+// that was present before the round (Alg. 2's presence test: a settled offset of 0 is
+// larger than any pending one), and spills of one round into one diagonal merge by the
+// larger walk base.
+__device__ void apply_spills(const DevGraph &g, const Slab<true> &s, Sh &sh, int d, uint32_t n, uint32_t *n_ins,
+                             bool traceback) {
+    Score &S = sh.score[d & 3];
+    uint32_t won = 0;
+    for (uint32_t r = threadIdx.x; r < min(n, s.cap); r += blockDim.x) {
+        const int4 rq = s.req4[r];
         const int ku = rq.x;
         const long long cand = pk(0, kTagPend, (uint32_t)rq.y);
         for (uint32_t a = (uint32_t)rq.z; a < (uint32_t)rq.w; ++a) {
             const uint32_t u = __ldg(&g.arc_dst[a]);
-            const int su = find_or_insert(s, sh, tile_key(u, ku >> 3));
-            if (su < 0) return;
-            const long long prev = g_max(&s.slots[su].vals[ku & 7], cand);
-            if (prev < 0) {
-                atomicAdd(&sh.visited32, 1u);
-                atomicAdd(&sh.spills32, 1u);
-                __stcg(&s.slots[su].trace[ku & 7], 0u);   // set by resolve_spill_traces
-                reg_append(&s.slots[su].reg[next_par], next_list, next_count, s.cap, (uint32_t)su, u, ku >> 3,
-                           1u << (ku & 7), sh);
-            }
+            const int su = find_or_insert<true>(s, sh, u, ku >> 3, &S.err);
+            if (su < 0) break;
+            if (g_max(&s.recs[su].vals[ku & 7], cand) >= 0) continue;
+            ++won;
+            if (traceback) s.trec[su].tr[ku & 7] = 0u;   // set by resolve_spill_traces
+            if (!g_exch(&s.recs[su].side[1].counted, 1u)) count_claim<true>(s, sh, &S.err);
+            const uint32_t i = atomicAdd(n_ins, 1u);
+            if (i < 2 * s.cap) s.ins[i] = make_uint4((uint32_t)su, u, (uint32_t)ku, 0u);
+            else atomicCAS(&S.err, 0, GWFA_ERR_CAPACITY);
         }
+    }
+    won = __reduce_add_sync(0xFFFFFFFFu, won);
+    if ((threadIdx.x & 31) == 0 && won) {
+        atomicAdd(&S.cells, won);
+        atomicAdd(&S.spills, won);
+        atomicAdd(&S.visited, won);
     }
 }
 
-// Traceback with pruning: after apply_spill_requests (and a barrier) every diagonal
-// a spill inserted in this round holds the largest base among its spills, still
-// tagged pending; each request whose base is that one offers its T index and the
-// largest index wins (any of them is a walk of that base, so the choice only has to
-// be deterministic).
-__device__ void resolve_spill_traces(const DevGraph &g, const Slab<true> &s, Sh &sh, uint32_t n_req) {
-    const uint32_t nr = min(n_req, s.cap);
-    for (uint32_t r = threadIdx.x; r < nr; r += blockDim.x) {
-        const int4 rq = __ldcg(&s.req[r]);
+// Traceback with pruning, after apply_spills (and a barrier): every diagonal a spill
+// inserted in this round holds the largest base among its spills, still tagged pending;
+// each request whose base is that one offers its T index and the largest index wins (any
+// of them is a walk of that base, so the choice only has to be deterministic).
+__device__ void resolve_spill_traces(const DevGraph &g, const Slab<true> &s, Sh &sh, int d, uint32_t n) {
+    for (uint32_t r = threadIdx.x; r < min(n, s.cap); r += blockDim.x) {
+        const int4 rq = s.req4[r];
         const int ku = rq.x;
         const long long cand = pk(0, kTagPend, (uint32_t)rq.y);
-        const uint32_t t = __ldcg(&s.reqt[r]);
         for (uint32_t a = (uint32_t)rq.z; a < (uint32_t)rq.w; ++a) {
-            const int su = find_or_insert(s, sh, tile_key(__ldg(&g.arc_dst[a]), ku >> 3));
+            const int su = find_or_insert<true>(s, sh, __ldg(&g.arc_dst[a]), ku >> 3, &sh.score[d & 3].err);
             if (su < 0) return;
-            if (__ldcg(&s.slots[su].vals[ku & 7]) == cand) atomicMax(&s.slots[su].trace[ku & 7], t);
+            if (s.recs[su].vals[ku & 7] == cand) g_max32(&s.trec[su].tr[ku & 7], s.reqt[r]);
         }
     }
 }
 
-// Pruning mode: the merge of `cand` replaced `prev` and was the first of this
-// GwfExpand to do so (every offset is settled when GwfExpand starts, so the first
-// fresh value is the first change).
-__device__ __forceinline__ bool first_fresh(long long prev, long long cand) {
-    return cand > prev && ((prev >> 30) & 3) != kTagFresh;
-}
-
-// Offer value `cand` to lane `ln` of tile (slot, v, kb): GwfExpand's max-merge
-// into H~; the lane joins the next Q if its offset strictly improved.
-template <bool P>
-__device__ __forceinline__ void offer_done(const Slab<P> &s, Sh &sh, uint32_t slot, uint32_t v, int kb,
-                                           int ln, typename VT<P>::T cand, typename VT<P>::T prev, int par,
-                                           uint32_t *qcount, bool traceback) {
-    if constexpr (P) {
-        if (prev < 0) atomicAdd(&sh.visited32, 1u);
-        if (traceback && first_fresh(prev, cand)) __stcg(&s.slots[slot].trace[ln], 0u);
+// Pruning mode: extend the diagonals inserted by the round; those that reach their
+// vertex's end request the next round's spills.
+__device__ void extend_spilled(const DevGraph &g, const Slab<true> &s, Sh &sh, const QCtx &q, int d, uint32_t n,
+                               uint32_t *n_req, bool traceback) {
+    Score &S = sh.score[d & 3];
+    uint32_t amax = 0;
+    for (uint32_t r = threadIdx.x; r < min(n, 2 * s.cap); r += blockDim.x) {
+        const uint4 in = s.ins[r];
+        const int k = (int)in.z;
+        const uint4 vi = __ldg(&g.vinfo[in.y]);
+        const uint32_t base = pbase(s.recs[in.x].vals[k & 7]);
+        const uint32_t tr = traceback ? s.trec[in.x].tr[k & 7] : 0u;
+        const int j = lcp(q, k, g.words + vi.x, 0, (int)vi.y);
+        s.recs[in.x].vals[k & 7] = pk(j, kTagLive, base);
+        amax = max(amax, (uint32_t)(k + j) + (uint32_t)j + base);
+        if (at_end(q, in.y, k, j, vi.y)) {
+            S.found = 1;
+            sh.end_vp = ((unsigned long long)in.y << 32) | tr;
+        }
+        enter_next<true>(s, sh, q, in.x, in.y, k, j, base, vi.y, d, tr, traceback);
+        if ((uint32_t)j == vi.y)
+            request_spill(s, sh, atomicAdd(n_req, 1u), vi, in.y, k, base, tr, traceback, &S.err);
     }
-    if (pj(prev) < pj(cand)) reg_append(&s.slots[slot].reg[par], s.qlist, qcount, s.cap, slot, v, kb, 1u << ln, sh);
+    amax = __reduce_max_sync(0xFFFFFFFFu, amax);
+    if ((threadIdx.x & 31) == 0 && amax) atomicMax(&S.amax, amax);
 }
 
-template <bool P>
-__device__ __forceinline__ void offer(const Slab<P> &s, Sh &sh, uint32_t slot, uint32_t v, int kb,
-                                      int ln, typename VT<P>::T cand, int par, uint32_t *qcount, bool traceback) {
-    const typename VT<P>::T prev = slab_max<P>(&s.slots[slot].vals[ln], cand);
-    offer_done<P>(s, sh, slot, v, kb, ln, cand, prev, par, qcount, traceback);
-}
-
-// GwfExpand (Alg. 3) over the extended frontier, with GwfPrune (Alg. 4) applied
-// to the sources on the way in.  U snapshot entries per group and
-// iteration: their candidate max-merges are issued together before any registration.
-template <bool P, int U>
-__device__ void expand_all(const Slab<P> &s, Sh &sh, const QCtx &q, uint32_t n_e, bool prune_on,
-                           long long amax, int max_lag, int par, uint32_t *qcount, uint32_t *claim,
-                           bool traceback) {
-    using T = typename VT<P>::T;
-    const int ln = threadIdx.x & 7;
-    const unsigned gmask = 0xFFu << (threadIdx.x & 24);
-    const uint32_t ne = min(n_e, s.cap);
-    for (;;) {
-        const uint32_t wb = warp_claim(claim, (uint32_t)U);
-        if (wb >= ne) break;
-        const uint32_t base = wb + ((threadIdx.x & 31) >> 3) * (uint32_t)U;
-        if (base >= ne) continue;
-        bool valid[U], ins[U], del[U];
-        EHdr h[U];
-        T c_ins[U], c_del[U], cand[U], prev[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint32_t e = base + u;
-            valid[u] = e < ne;
-            h[u] = EHdr{0u, 0u, 0, 0u};
-            T val = (T)-1;
-            if (valid[u]) {
-                h[u] = ld_ehdr(&s.elist[e].hdr);
-                val = __ldcg(&s.elist[e].vals[ln]);
-            }
-            const uint32_t m = h[u].slot_mask >> 24;
-            bool act = valid[u] && ((m >> ln) & 1u);
-            const int k = h[u].kb * kTile + ln;
-            const int j = act ? pj(val) : 0;
-            const int i = k + j;
-            const uint32_t b = pbase(val);
-            if (P && act && prune_on) {
-                const long long a = (long long)i + (long long)b + j;
-                if (amax - a >= (long long)max_lag) {
-                    act = false;
-                    atomicAdd(&sh.pruned32, 1u);
-                }
-            }
-            ins[u] = act && i < q.n;                 // (k+1, j)
-            del[u] = act && j < (int)h[u].lv;        // (k-1, j+1)
-            const bool mis = ins[u] && j < (int)h[u].lv;   // (k, j+1)
-            T c_mis;
-            if constexpr (P) {
-                c_ins[u] = ins[u] ? pk(j, kTagFresh, b) : -1ll;
-                c_del[u] = del[u] ? pk(j + 1, kTagFresh, b) : -1ll;
-                c_mis = mis ? pk(j + 1, kTagFresh, b) : -1ll;
-            } else {
-                c_ins[u] = ins[u] ? j : -1;
-                c_del[u] = del[u] ? j + 1 : -1;
-                c_mis = mis ? j + 1 : -1;
-            }
-            T from_left = __shfl_up_sync(gmask, c_ins[u], 1, 8);
-            T from_right = __shfl_down_sync(gmask, c_del[u], 1, 8);
-            if (ln == 0) from_left = (T)-1;
-            if (ln == 7) from_right = (T)-1;
-            cand[u] = c_mis;
-            if (from_left > cand[u]) cand[u] = from_left;
-            if (from_right > cand[u]) cand[u] = from_right;
-        }
-        // the neighbour tile a boundary lane leaves for (insertion from lane 7, deletion
-        // from lane 0): its first hash read goes out before this tile's merges
-        unsigned long long nkey[U], ncur[U];
-        uint32_t nh[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const bool out = valid[u] && ((ln == 7 && ins[u]) || (ln == 0 && del[u]));
-            nkey[u] = tile_key(h[u].v, h[u].kb + (ln == 7 ? 1 : -1));
-            nh[u] = tile_hash(nkey[u], s.mask);
-            ncur[u] = out ? __ldcg(&s.slots[nh[u]].key) : 0ull;
-        }
-        // a boundary lane whose early read found the neighbour tile merges into it
-        // together with this tile's merges
-        bool near[U];
-        T nprev[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            prev[u] = (T)0x7FFFFFFF;
-            if (valid[u] && cand[u] >= 0)
-                prev[u] = slab_max<P>(&s.slots[h[u].slot_mask & 0xFFFFFFu].vals[ln], cand[u]);
-            near[u] = ncur[u] == nkey[u] && valid[u] && ((ln == 7 && ins[u]) || (ln == 0 && del[u]));
-            nprev[u] = 0;
-            if (near[u]) nprev[u] = slab_max<P>(&s.slots[nh[u]].vals[7 - ln], ln == 7 ? c_ins[u] : c_del[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (!(valid[u] && cand[u] >= 0)) continue;
-            if constexpr (P) {
-                if (prev[u] < 0) atomicAdd(&sh.visited32, 1u);   // exact mode counts at query end
-            }
-            if constexpr (P) {
-                if (traceback && first_fresh(prev[u], cand[u]))
-                    __stcg(&s.slots[h[u].slot_mask & 0xFFFFFFu].trace[ln], 0u);
-            }
-            if (pj(prev[u]) < pj(cand[u]))
-                reg_append(&s.slots[h[u].slot_mask & 0xFFFFFFu].reg[par], s.qlist, qcount, s.cap,
-                           h[u].slot_mask & 0xFFFFFFu, h[u].v,
-                           h[u].kb, 1u << ln, sh);
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (valid[u] && ln == 7 && ins[u]) {   // insertion leaves the tile: (v, 8(kb+1))
-                if (near[u]) {
-                    offer_done<P>(s, sh, nh[u], h[u].v, h[u].kb + 1, 0, c_ins[u], nprev[u], par, qcount, traceback);
-                } else {
-                    const int t = find_or_insert_at(s, sh, nkey[u], nh[u], ncur[u]);
-                    if (t >= 0) offer<P>(s, sh, (uint32_t)t, h[u].v, h[u].kb + 1, 0, c_ins[u], par, qcount, traceback);
-                }
-            }
-            if (valid[u] && ln == 0 && del[u]) {   // deletion leaves the tile: (v, 8 kb - 1)
-                if (near[u]) {
-                    offer_done<P>(s, sh, nh[u], h[u].v, h[u].kb - 1, 7, c_del[u], nprev[u], par, qcount, traceback);
-                } else {
-                    const int t = find_or_insert_at(s, sh, nkey[u], nh[u], ncur[u]);
-                    if (t >= 0) offer<P>(s, sh, (uint32_t)t, h[u].v, h[u].kb - 1, 7, c_del[u], par, qcount, traceback);
-                }
-            }
-        }
-    }
-}
-
-// Traceback with pruning, after GwfExpand's merge (and a barrier): every diagonal
-// the merge raised holds the largest candidate (offset, base), tagged fresh; each
-// candidate equal to it offers the trace index of its source, and the largest
-// index wins (sources of equal offset and base are equally good predecessors).
-// The candidates and the pruning of their sources are recomputed as in expand_all.
-__device__ void resolve_expand_traces(const Slab<true> &s, Sh &sh, const QCtx &q, uint32_t n_e, bool prune_on,
-                                      long long amax, int max_lag, uint32_t *claim) {
-    const int ln = threadIdx.x & 7;
-    const unsigned gmask = 0xFFu << (threadIdx.x & 24);
-    const uint32_t ne = min(n_e, s.cap);
-    for (;;) {
-        const uint32_t wb = warp_claim(claim, 1u);
-        if (wb >= ne) break;
-        const uint32_t e = wb + ((threadIdx.x & 31) >> 3);
-        if (e >= ne) continue;
-        const EHdr h = ld_ehdr(&s.elist[e].hdr);
-        const long long val = __ldcg(&s.elist[e].vals[ln]);
-        const uint32_t tr = __ldcg(&s.elist[e].trace[ln]);
-        const uint32_t slot = h.slot_mask & 0xFFFFFFu;
-        bool act = (h.slot_mask >> (24 + ln)) & 1u;
-        const int k = h.kb * kTile + ln;
-        const int j = act ? pj(val) : 0;
-        const int i = k + j;
-        const uint32_t b = pbase(val);
-        if (act && prune_on && amax - ((long long)i + (long long)b + j) >= (long long)max_lag) act = false;
-        const bool ins = act && i < q.n;
-        const bool del = act && j < (int)h.lv;
-        const bool mis = ins && j < (int)h.lv;
-        const long long c_ins = ins ? pk(j, kTagFresh, b) : -1ll;
-        const long long c_del = del ? pk(j + 1, kTagFresh, b) : -1ll;
-        long long from_left = __shfl_up_sync(gmask, c_ins, 1, 8);
-        long long from_right = __shfl_down_sync(gmask, c_del, 1, 8);
-        const uint32_t t_left = __shfl_up_sync(gmask, tr, 1, 8);
-        const uint32_t t_right = __shfl_down_sync(gmask, tr, 1, 8);
-        if (ln == 0) from_left = -1;
-        if (ln == 7) from_right = -1;
-        if (mis || from_left >= 0 || from_right >= 0) {
-            const long long cur = __ldcg(&s.slots[slot].vals[ln]);
-            if (mis && cur == pk(j + 1, kTagFresh, b)) atomicMax(&s.slots[slot].trace[ln], tr);
-            if (from_left >= 0 && cur == from_left) atomicMax(&s.slots[slot].trace[ln], t_left);
-            if (from_right >= 0 && cur == from_right) atomicMax(&s.slots[slot].trace[ln], t_right);
-        }
-        if (ln == 7 && ins) {   // insertion left the tile: (v, 8(kb+1)), lane 0
-            const int t = find_or_insert(s, sh, tile_key(h.v, h.kb + 1));
-            if (t >= 0 && __ldcg(&s.slots[t].vals[0]) == c_ins) atomicMax(&s.slots[t].trace[0], tr);
-        }
-        if (ln == 0 && del) {   // deletion left the tile: (v, 8 kb - 1), lane 7
-            const int t = find_or_insert(s, sh, tile_key(h.v, h.kb - 1));
-            if (t >= 0 && __ldcg(&s.slots[t].vals[7]) == c_del) atomicMax(&s.slots[t].trace[7], tr);
-        }
-    }
-}
-
-template <bool P>
-__device__ void wipe_touched(const Slab<P> &s, uint32_t nt) {
-    using T = typename VT<P>::T;
-    nt = min(nt, s.cap);
-    for (uint32_t t = threadIdx.x; t < nt * kTile; t += blockDim.x) {
-        const uint32_t slot = __ldcg(&s.touched[t / kTile]);
-        __stcg(&s.slots[slot].vals[t % kTile], (T)-1);
-        if (t % kTile == 0) {
-            __stcg(&s.slots[slot].key, kEmptyKey);
-            __stcg((unsigned long long *)s.slots[slot].reg, 0ull);
-        }
-    }
-}
-
-// Memory bound on H~ (pruning mode, called every evict_every scores right after
-// GwfExpand): the lanes in the new Q (registered in parity `par`) and those whose
-// anti-diagonal a = i + W~ lags this score's a_max by less than `lag` are kept, the
-// others are removed (sh.evicted).  The tiles with a kept lane are staged in the
-// frontier-snapshot list, which is free between scores; the table is wiped through
-// the touched list and they are inserted again, and Q is rebuilt with their new
-// slots.  A removed diagonal may be inserted again later, like any absent one.
-__device__ void evict_behind(const Slab<true> &s, Sh &sh, long long amax, int lag, int par,
-                             uint32_t *qcount) {
+// Empty the records and hash entries of a query; in exact mode, which never removes a
+// diagonal from H~, also count the diagonals they hold (the visited ones).
+template <bool P> __device__ void wipe(const Slab<P> &s, Sh &sh) {
     const uint32_t nt = min(sh.nt, s.cap);
-    if (threadIdx.x == 0) sh.nsurv = 0;
-    __syncthreads();
-    unsigned long long ev = 0;
+    uint32_t c = 0;
+    constexpr uint32_t kChunks = sizeof(RecT<typename VT<P>::T>) / 16, kValChunks = sizeof(typename VT<P>::T) / 2;
+    for (uint32_t t = threadIdx.x; t < nt * kChunks; t += blockDim.x) {
+        const uint32_t part = t % kChunks;
+        uint4 *p = (uint4 *)s.recs + t;
+        if constexpr (!P) {
+            if (part < kValChunks) {
+                const int4 v = *(const int4 *)p;
+                c += (v.x >= 0) + (v.y >= 0) + (v.z >= 0) + (v.w >= 0);
+            }
+        }
+        *p = empty_chunk(P, part);
+        if (part == 0) {
+            const uint32_t i = t / kChunks, h = s.touched[i];
+            if (h != kNone) {
+                *(uint4 *)&s.table[h] = make_uint4(~0u, ~0u, ~0u, ~0u);
+                s.touched[i] = kNone;
+            }
+            if (i >= kBitTiles) s.stamp[i] = kNone;
+            if constexpr (P) s.tkey[i] = kEmptyKey;
+        }
+    }
+    if constexpr (!P) {
+        c = __reduce_add_sync(0xFFFFFFFFu, c);
+        if ((threadIdx.x & 31) == 0 && c) atomicAdd(&sh.visited, (unsigned long long)c);
+    }
+}
+
+// Memory bound on H~ (pruning mode, called every evict_every scores between the offset
+// pass and the arc spills, so right after GwfExpand as far as the entries outside Q are
+// concerned): the diagonals in Q and those whose anti-diagonal a = i + W~ lags the score
+// before's a_max by less than `lag` are kept, the others are removed (sh.evicted).  The
+// hash is rebuilt from the tiles that still hold a diagonal or are listed for the next
+// score; the records of the others go to the free list.  Records never move, so lists,
+// flags and border words stay valid; the links between neighbours, which could point to a
+// freed record, are dropped and found again on use.  A removed diagonal may be inserted
+// again later, like any absent one.
+__device__ void evict_behind(const Slab<true> &s, Sh &sh, long long amax, int lag, int d) {
+    const uint32_t nt = min(sh.nt, s.cap);
     for (uint32_t t = threadIdx.x; t < nt; t += blockDim.x) {
-        const uint32_t slot = __ldcg(&s.touched[t]);
-        const unsigned long long key = __ldcg(&s.slots[slot].key);
-        const uint32_t regw = __ldcg(&s.slots[slot].reg[par]);
+        const uint32_t h = s.touched[t];
+        if (h != kNone) *(uint4 *)&s.table[h] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    }
+    if (threadIdx.x == 0) {
+        sh.nclaim = 0;
+        if (sh.nfree < 0) sh.nfree = 0;
+    }
+    __syncthreads();
+    uint32_t ev = 0;
+    for (uint32_t t = threadIdx.x; t < nt; t += blockDim.x) {
+        const unsigned long long key = s.tkey[t];
+        if (key == kEmptyKey) continue;   // free, or never used
         const int kb = (int)(uint32_t)(key & 0xFFFFFFFFull);
-        long long v8[kTile];
-        uint32_t keep = 0;
+        bool any = false;
 #pragma unroll
         for (int ln = 0; ln < kTile; ++ln) {
-            v8[ln] = __ldcg(&s.slots[slot].vals[ln]);
-            if (v8[ln] < 0) continue;
-            const int j = pj(v8[ln]);
-            const long long a = (long long)(kb * kTile + ln) + 2ll * j + (long long)pbase(v8[ln]);
-            if (((regw >> ln) & 1u) || amax - a < (long long)lag) keep |= 1u << ln;
-            else ++ev;
+            const long long v = s.recs[t].vals[ln];
+            if (v < 0) continue;
+            const long long a = (long long)(kb * kTile + ln) + 2ll * pj(v) + (long long)pbase(v);
+            if (((v >> 30) & 3) == kTagLive || amax - a < (long long)lag) {
+                any = true;
+            } else {
+                s.recs[t].vals[ln] = -1ll;
+                ++ev;
+            }
         }
-        if (keep) {
-            const uint32_t i = atomicAdd(&sh.nsurv, 1u);   // i < nt <= cap
-            st_ehdr(&s.elist[i].hdr, regw, (uint32_t)(key >> 32), kb, 0u);
-#pragma unroll
-            for (int ln = 0; ln < kTile; ++ln)
-                __stcg(&s.elist[i].vals[ln], ((keep >> ln) & 1u) ? v8[ln] : -1ll);
-        }
-    }
-    if (ev) atomicAdd(&sh.evicted, ev);
-    __syncthreads();
-    wipe_touched<true>(s, nt);
-    if (threadIdx.x == 0) {
-        sh.nt = 0;
-        *qcount = 0;
-    }
-    __syncthreads();
-    const uint32_t ns = sh.nsurv;
-    for (uint32_t i = threadIdx.x; i < ns; i += blockDim.x) {
-        const EHdr h = ld_ehdr(&s.elist[i].hdr);
-        const int slot = find_or_insert(s, sh, tile_key(h.v, h.kb));
-        if (slot < 0) continue;
-#pragma unroll
-        for (int ln = 0; ln < kTile; ++ln) __stcg(&s.slots[slot].vals[ln], __ldcg(&s.elist[i].vals[ln]));
-        if (h.slot_mask) {   // part of the new Q
-            __stcg(&s.slots[slot].reg[par], h.slot_mask);
-            const uint32_t qi = atomicAdd(qcount, 1u);
-            if (qi < s.cap) __stcg((uint4 *)&s.qlist[qi], make_uint4((uint32_t)slot, h.v, (uint32_t)h.kb, 0u));
-            else set_err(sh, GWFA_ERR_CAPACITY);
+        s.recs[t].side[0].link = s.recs[t].side[1].link = kNone;
+        s.recs[t].side[1].counted = any ? 1u : 0u;
+        const bool listed = t < kBitTiles ? (sh.bits[(d + 1) & 1][t >> 5] >> (t & 31)) & 1u
+                                          : s.stamp[t] == (uint32_t)(d + 1);
+        if (any) atomicAdd(&sh.nclaim, 1u);
+        if (any || listed) {
+            uint32_t h = tile_hash(key, s.tmask);
+            while (cas_ent(&s.table[h], key, t).key != kEmptyKey) h = (h + 1) & s.tmask;   // at most half full
+            s.touched[t] = h;
+        } else {
+            s.tkey[t] = kEmptyKey;
+            s.touched[t] = kNone;
+            s.freel[atomicAdd(&sh.nfree, 1)] = t;
         }
     }
+    ev = __reduce_add_sync(0xFFFFFFFFu, ev);
+    if ((threadIdx.x & 31) == 0 && ev) atomicAdd(&sh.evicted, (unsigned long long)ev);
     __syncthreads();
 }
 
 template <bool P>
-__device__ void align_one(const TierArgs &A, const Slab<P> &s, Sh &sh, uint32_t qid) {
+__device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, Sh &sh, uint32_t qid) {
     const DevGraph &g = A.g;
     const uint64_t qo = A.q_off[qid];
-    const int n = (int)(A.q_off[qid + 1] - qo);
     QCtx q;
+    q.n = (int)(A.q_off[qid + 1] - qo);
     q.qw = A.qwords + (qo >> 4) + qid;
-    q.n = n;
     q.smem = A.q_smem != 0;
     const uint32_t vs = A.v_s[qid];
     q.ve = A.v_e[qid];
@@ -885,198 +815,169 @@ __device__ void align_one(const TierArgs &A, const Slab<P> &s, Sh &sh, uint32_t 
         }
         return;
     }
-    q.ke = n - (int)__ldg(&g.vinfo[q.ve]).y;
     // Alg. 1 initialisation: H~_{v_s,0} <- 0, Q <- [(v_s, 0)], d <- 0
     if (threadIdx.x == 0) {
         sh.t_start = globaltimer_ns();
         for (int i = 0; i < 6; ++i) sh.st[i] = 0;
-        sh.err = 0;
-        sh.nt = 0;
+        for (int i = 0; i < 4; ++i) sh.score[i] = Score{};
+        sh.nt = sh.nclaim = 0;
+        sh.nfree = 0;
         sh.cells = sh.visited = sh.pruned = sh.spills = sh.evicted = 0;
-        sh.spills32 = sh.visited32 = sh.pruned32 = 0;
         sh.peak = 0;
-        sh.nq[0] = sh.nq[1] = 0;
-        sh.claim[0] = sh.claim[1] = sh.claim[2] = 0;
         sh.tlen = 0;
         sh.end_vp = ((unsigned long long)q.ve << 32) | kNoTrace;
-        const int slot = find_or_insert(s, sh, tile_key(vs, 0));
-        if (slot >= 0) {
-            typename VT<P>::T v0;
+        const int t = find_or_insert<P>(s, sh, vs, 0, &sh.score[0].err);
+        if (t >= 0) {
             if constexpr (P) {
-                v0 = pk(0, kTagFresh, 0u);
-                s.slots[slot].trace[0] = kNoTrace;
+                s.recs[t].vals[0] = pk(0, kTagLive, 0u);
+                s.recs[t].side[1].counted = 1u;
+                sh.nclaim = 1;
+                if (A.traceback) s.trec[t].tr[0] = kNoTrace;
+                sh.visited = 1;
             } else {
-                v0 = 0;
+                s.recs[t].vals[0] = 1;
             }
-            s.slots[slot].vals[0] = v0;
-            if constexpr (P) sh.visited = 1;
-            reg_append(&s.slots[slot].reg[1], s.qlist, &sh.nq[0], s.cap, (uint32_t)slot, vs, 0, 1u, sh);
+            s.list[0][0] = make_uint2((uint32_t)t, vs);
+            sh.score[0].nq = 1;
         }
     }
+    for (uint32_t w = threadIdx.x; w < kBitTiles / 32; w += blockDim.x) sh.bits[0][w] = sh.bits[1][w] = 0u;
     __syncthreads();
     if (A.ends & GWFA_FREE_START) {
         // free walk start (Sec. 2.1 variant): query position 0 also faces every
         // position j of v_s, i.e. the diagonals (v_s, -j) start with offset j
         const int lvs = (int)__ldg(&g.vinfo[vs]).y;
         const int ntile = (lvs + kTile - 1) / kTile;   // tiles kb = -1 .. -ntile
-        for (int t = threadIdx.x; t < ntile; t += blockDim.x) {
-            const int kb = -1 - t;
-            uint32_t bits = 0;
-            for (int ln = 0; ln < kTile; ++ln)
-                if (kb * kTile + ln >= -lvs) bits |= 1u << ln;
-            const int slot = find_or_insert(s, sh, tile_key(vs, kb));
-            if (slot < 0) continue;
+        for (int i = threadIdx.x; i < ntile; i += blockDim.x) {
+            const int kb = -1 - i;
+            const int t = find_or_insert<P>(s, sh, vs, kb, &sh.score[0].err);
+            if (t < 0) continue;
+            uint32_t cnt = 0;
             for (int ln = 0; ln < kTile; ++ln) {
-                if (!((bits >> ln) & 1u)) continue;
                 const int j = -(kb * kTile + ln);
+                if (j > lvs) continue;
+                ++cnt;
                 if constexpr (P) {
-                    s.slots[slot].vals[ln] = pk(j, kTagFresh, 0u);
-                    s.slots[slot].trace[ln] = kNoTrace;
+                    s.recs[t].vals[ln] = pk(j, kTagLive, 0u);
+                    if (A.traceback) s.trec[t].tr[ln] = kNoTrace;
                 } else {
-                    s.slots[slot].vals[ln] = j;
+                    s.recs[t].vals[ln] = (j << 1) | 1;
                 }
             }
-            if constexpr (P) atomicAdd(&sh.visited, (unsigned long long)__popc(bits));
-            reg_append(&s.slots[slot].reg[1], s.qlist, &sh.nq[0], s.cap, (uint32_t)slot, vs, kb, bits, sh);
+            if constexpr (P) {
+                s.recs[t].side[1].counted = 1u;
+                count_claim<P>(s, sh, &sh.score[0].err);
+                atomicAdd(&sh.visited, (unsigned long long)cnt);
+            }
+            s.list[0][atomicAdd(&sh.score[0].nq, 1u)] = make_uint2((uint32_t)t, vs);
         }
         __syncthreads();
     }
 
-    uint32_t phase = 1;   // parity (phase & 1) of the reg words of the tiles in Q
-    uint32_t cstep = 0;   // processing phases so far: phase number c claims with claim[c % 3]
-    int d = 0;
-    int status = 0;
-    int failed = 0;
-    for (;;) {
-        // ---- GwfExtend (Alg. 2)
+    int d = 0, status = 0;
+    for (;; ++d) {
+        Score &S = sh.score[d & 3];
         if (threadIdx.x == 0) {
-            sh.ne = 0;
-            sh.score_cells = 0;
-            sh.found = 0;
-            sh.amax = 0;
-            sh.ns[1] = 0;
-            sh.nreq[0] = 0;
-            sh.nq[(d + 1) & 1] = 0;
+            sh.score[(d + 2) & 3] = Score{};
+            sh.nr[0] = 0;
+            sh.nins[0] = 0;
+            if (A.stats) sh.t_phase = globaltimer_ns();
+        }
+        // ---- GwfExpand of the last score (Alg. 3, with GwfPrune, Alg. 4) and GwfExtend of this one
+        bool prune_on = false;
+        long long amax = 0;
+        if constexpr (P) {
+            amax = (long long)sh.score[(d + 3) & 3].amax;
+            prune_on = A.max_lag > 0 && amax > (long long)A.max_lag;
+            if (A.traceback) offset_pass<P, true>(g, s, sh, q, d, prune_on, A.max_lag);
+            else offset_pass<P, false>(g, s, sh, q, d, prune_on, A.max_lag);
+        } else {
+            offset_pass<P, false>(g, s, sh, q, d, false, 0);
         }
         __syncthreads();
-        const LEnt *list = s.qlist;
-        uint32_t n_list = min(sh.nq[d & 1], s.cap);
-        if (A.stats && threadIdx.x == 0) sh.t_phase = globaltimer_ns();
-        for (int round = 0;; ++round) {
-            if (A.stats && threadIdx.x == 0) {
-                sh.st[2]++;
-                sh.st[3] += n_list;
-            }
-            const uint32_t next_phase = phase + 1;
-            LEnt *next_list = s.slist[(round + 1) & 1];
-            // round r fills ns[(r+1)%3] and clears ns[(r+2)%3] for round r+1; the
-            // cleared counter was last read before the previous round's barrier
-            uint32_t *next_count = &sh.ns[(round + 1) % 3];
-            // processing phase c claims with claim[c % 3] and clears the two others for
-            // the next phase; both were last used before this phase's barrier
-            if (threadIdx.x == 0) {
-                sh.ns[(round + 2) % 3] = 0;
-                sh.claim[(cstep + 1) % 3] = 0;
-                sh.claim[(cstep + 2) % 3] = 0;
-            }
-            uint32_t *claim = &sh.claim[cstep % 3];
-            ++cstep;
-            if constexpr (P) {
-                extend_round_prune(g, s, sh, q, list, n_list, phase & 1, &sh.nreq[round & 1], claim,
-                                   A.traceback != 0);
-                __syncthreads();
-                if (threadIdx.x == 0) sh.nreq[(round + 1) & 1] = 0;
-                apply_spill_requests(g, s, sh, sh.nreq[round & 1], next_phase & 1, next_list,
-                                     next_count);
-                if (A.traceback) {
-                    __syncthreads();
-                    resolve_spill_traces(g, s, sh, sh.nreq[round & 1]);
-                }
-            } else {
-                extend_round_exact<kGroupTiles>(g, s, sh, q, list, n_list, phase & 1, next_phase & 1,
-                                                next_list, next_count, claim);
-            }
-            // every exit decision comes from a barrier reduction: sh.err may be set by
-            // threads that already run the next phase, so it is never re-read for control
-            failed = __syncthreads_or(sh.err != 0);
-            const uint32_t ns = *next_count;
-            phase = next_phase;
-            if (failed || ns == 0) break;
-            list = next_list;
-            n_list = min(ns, s.cap);
-        }
-        if (threadIdx.x == 0) {
-            sh.cells += sh.score_cells;
-            sh.spills += atomicExch(&sh.spills32, 0u);
-            sh.visited += atomicExch(&sh.visited32, 0u);
-            sh.pruned += atomicExch(&sh.pruned32, 0u);
-            sh.peak = max(sh.peak, sh.score_cells);
-        }
         if (A.stats && threadIdx.x == 0) {
             const unsigned long long t = globaltimer_ns();
             sh.st[0] += t - sh.t_phase;
             sh.t_phase = t;
-            sh.st[4] += sh.ne;
-            sh.st[5] = max(sh.st[5], (unsigned long long)sh.ne);
+            sh.st[2] += 1;
+            sh.st[3] += S.nq;
+            sh.st[4] += sh.score[(d + 1) & 3].nq;
+            sh.st[5] = max(sh.st[5], (unsigned long long)S.nq);
         }
-        if (failed) break;
-        // end test of Alg. 1
-        if (sh.found) break;
-        if (A.max_score >= 0 && d >= A.max_score) { status = GWFA_ERR_SCORE_LIMIT; break; }
-        d = d + 1;
-        // ---- GwfPrune (Alg. 4) folded into the sources of GwfExpand (Alg. 3)
-        const long long amax = (long long)sh.amax;
-        const bool prune_on = P && A.max_lag > 0 && amax > (long long)A.max_lag;
-        phase = phase + 1;
-        if (threadIdx.x == 0) {
-            sh.claim[(cstep + 1) % 3] = 0;
-            sh.claim[(cstep + 2) % 3] = 0;
-        }
-        uint32_t *claim = &sh.claim[cstep % 3];
-        ++cstep;
-        expand_all<P, kGroupTiles>(s, sh, q, sh.ne, prune_on, amax, A.max_lag, phase & 1, &sh.nq[d & 1],
-                                   claim, A.traceback != 0);
-        failed = __syncthreads_or(sh.err != 0);
-        if constexpr (P) {
-            if (A.traceback && !failed) {
-                if (threadIdx.x == 0) {
-                    sh.claim[(cstep + 1) % 3] = 0;
-                    sh.claim[(cstep + 2) % 3] = 0;
-                }
-                uint32_t *rclaim = &sh.claim[cstep % 3];
-                ++cstep;
-                resolve_expand_traces(s, sh, q, sh.ne, prune_on, amax, A.max_lag, rclaim);
-                failed = __syncthreads_or(sh.err != 0);
-            }
-        }
-        if (A.stats && threadIdx.x == 0) sh.st[1] += globaltimer_ns() - sh.t_phase;
-        if (failed) break;
-        if (sh.nq[d & 1] == 0) {
-            status = P && A.max_lag > 0 ? GWFA_ERR_EMPTY_FRONTIER : GWFA_ERR_UNREACHABLE;
+        if (S.cells == 0) {   // GwfExpand left Q empty (or there was no room for v_s)
+            status = S.err ? S.err : P && A.max_lag > 0 ? GWFA_ERR_EMPTY_FRONTIER : GWFA_ERR_UNREACHABLE;
             break;
         }
         if constexpr (P) {
-            if (A.evict_lag > 0 && d % A.evict_every == 0) {
-                evict_behind(s, sh, amax, A.evict_lag, phase & 1, &sh.nq[d & 1]);
-                failed = __syncthreads_or(sh.err != 0);
-                if (failed) break;
+            if (A.evict_lag > 0 && d > 0 && d % A.evict_every == 0) evict_behind(s, sh, amax, A.evict_lag, d);
+        }
+        // ---- arc spills, in rounds until no extended diagonal reaches its vertex's end
+        uint32_t n = S.nreq, r0 = 0;
+        for (int round = 0; n; ++round) {
+            uint32_t *next_count = &sh.nr[round % 3];
+            if (threadIdx.x == 0) sh.nr[(round + 1) % 3] = 0;
+            if constexpr (P) {
+                uint32_t *n_ins = &sh.nins[round & 1];
+                if (threadIdx.x == 0) sh.nins[(round + 1) & 1] = 0;
+                apply_spills(g, s, sh, d, n, n_ins, A.traceback != 0);
+                __syncthreads();
+                if (A.traceback) {
+                    resolve_spill_traces(g, s, sh, d, n);
+                    __syncthreads();
+                }
+                extend_spilled(g, s, sh, q, d, *n_ins, next_count, A.traceback != 0);
+            } else {
+                spill_round(g, s, sh, q, d, r0, n, next_count);
+                r0 += n;
+            }
+            __syncthreads();
+            n = *next_count;
+            if constexpr (!P) n = min(n, r0 < 4 * s.cap ? 4 * s.cap - r0 : 0u);
+            if (A.stats && threadIdx.x == 0 && n) sh.st[2] += 1;
+        }
+        if (threadIdx.x == 0) {
+            sh.cells += S.cells;
+            sh.spills += S.spills;
+            sh.peak = max(sh.peak, S.cells);
+            if constexpr (P) {
+                sh.visited += S.visited;
+                sh.pruned += S.pruned;
+            }
+            if (A.stats) sh.st[1] += globaltimer_ns() - sh.t_phase;
+        }
+        if (S.err) { status = S.err; break; }
+        if (S.found) break;   // end test of Alg. 1
+        if (A.max_score >= 0 && d >= A.max_score) { status = GWFA_ERR_SCORE_LIMIT; break; }
+        if (S.err_next) { status = S.err_next; ++d; break; }
+    }
+    __syncthreads();
+    const uint32_t n_tiles = sh.nclaim;
+    if constexpr (P) {
+        if (threadIdx.x == 0) {
+            const Score &S = sh.score[d & 3];
+            // the diagonals a failing last pass dropped or inserted
+            if (S.cells == 0) {
+                sh.visited += S.visited;
+                sh.pruned += S.pruned;
+            }
+            if (A.traceback && status == 0) {
+                // GwfTraceback (Alg. 6): push the end vertex, then follow T back to the
+                // start and write the walk in order
+                const uint32_t te = push_trace(s, sh, (uint32_t)(sh.end_vp >> 32), (uint32_t)sh.end_vp & 0xFFFFFFFFu,
+                                               &sh.score[0].err);
+                uint32_t len = 0;
+                for (uint32_t t = te; t != kNoTrace && len <= sh.tlen; t = s.trace[t].y) ++len;
+                if (A.path_len) A.path_len[qid] = len;
+                uint32_t pos = len;
+                for (uint32_t t = te; t != kNoTrace && pos > 0; t = s.trace[t].y) {
+                    --pos;
+                    if (A.paths && pos < A.path_cap) A.paths[(uint64_t)qid * A.path_cap + pos] = s.trace[t].x;
+                }
             }
         }
     }
+    wipe<P>(s, sh);
     __syncthreads();
-    if (failed) status = sh.err;   // stable now: every thread has left the processing phases
-    const uint32_t nt = sh.nt;
-    if constexpr (!P) {
-        // exact mode never removes a diagonal from H~, so the visited count is the
-        // number of lanes of the touched tiles that hold an offset
-        const uint32_t ntc = min(nt, s.cap);
-        uint32_t c = 0;
-        for (uint32_t t = threadIdx.x; t < ntc * kTile; t += blockDim.x)
-            c += __ldcg(&s.slots[__ldcg(&s.touched[t / kTile])].vals[t % kTile]) >= 0 ? 1u : 0u;
-        c = __reduce_add_sync(0xFFFFFFFFu, c);
-        if ((threadIdx.x & 31) == 0 && c) atomicAdd(&sh.visited, (unsigned long long)c);
-        __syncthreads();
-    }
     if (threadIdx.x == 0) {
         if (status == GWFA_ERR_CAPACITY && A.retry) {
             const uint32_t r = atomicAdd(A.retry_count, 1u);
@@ -1085,43 +986,24 @@ __device__ void align_one(const TierArgs &A, const Slab<P> &s, Sh &sh, uint32_t 
             gwfa_result r = {};
             r.status = status;
             r.edit_distance = status == 0 ? d : -1;
-            r.is_upper_bound = sh.pruned + sh.pruned32 > 0 ? 1 : 0;
+            r.is_upper_bound = sh.pruned > 0 ? 1 : 0;
             r.n_scores = (uint32_t)(d + 1);
             r.cells = sh.cells;
-            r.visited = sh.visited + sh.visited32;
+            r.visited = sh.visited;
             r.peak_frontier = sh.peak;
-            r.pruned = sh.pruned + sh.pruned32;
-            r.spills = sh.spills + sh.spills32;
+            r.pruned = sh.pruned;
+            r.spills = sh.spills;
             r.evicted = sh.evicted;
-            if constexpr (P) {
-                if (A.traceback && status == 0) {
-                    // GwfTraceback (Alg. 6): push the end vertex, then follow T back to the
-                    // start and write the walk in order
-                    const uint32_t te = push_trace(s, sh, (uint32_t)(sh.end_vp >> 32),
-                                                   (uint32_t)sh.end_vp & 0xFFFFFFFFu);
-                    uint32_t len = 0;
-                    for (uint32_t t = te; t != kNoTrace && len <= sh.tlen; t = __ldcg(&s.trace[t]).y) ++len;
-                    if (A.path_len) A.path_len[qid] = len;
-                    uint32_t pos = len;
-                    for (uint32_t t = te; t != kNoTrace && pos > 0; t = __ldcg(&s.trace[t]).y) {
-                        --pos;
-                        if (A.paths && pos < A.path_cap)
-                            A.paths[(uint64_t)qid * A.path_cap + pos] = __ldcg(&s.trace[t]).x;
-                    }
-                }
-            }
             r.device_us = (uint32_t)min((globaltimer_ns() - sh.t_start) / 1000ull, 0xFFFFFFFFull);
             A.out[qid] = r;
             if (A.stats) {
                 unsigned long long *o = A.stats + (uint64_t)qid * kStatWords;
                 for (int i = 0; i < 6; ++i) o[i] = sh.st[i];
-                o[6] = sh.nt;
+                o[6] = n_tiles;
                 o[7] = (unsigned long long)(d + 1);
             }
         }
     }
-    wipe_touched<P>(s, nt);
-    __syncthreads();
 }
 
 // The persistent loop of a CTA: pull a query id, run its score loop, repeat.
@@ -1310,24 +1192,18 @@ __global__ void pack_kernel(uint32_t nq, const char *__restrict__ q, const uint6
     if (blockIdx.x == 0 && threadIdx.x < 2) words[(off[nq] >> 4) + nq + threadIdx.x] = 0;
 }
 
-__global__ void fill_kernel(uint4 *p, uint64_t n16) {
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n16;
-         i += (uint64_t)gridDim.x * blockDim.x)
-        p[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
-}
-
-// Slabs start empty: slot keys and offsets all ones (empty / absent), lane-mask
-// words 0 (the second 8 bytes of every slot).  Only the hash slots are written:
-// every list of the slab (touched, Q, spills, frontier snapshots, spill requests,
-// T) is written before it is read.
-__global__ void slab_init_kernel(uint8_t *slabs, uint64_t slab_bytes, uint32_t n_slabs,
-                                 uint64_t slots_bytes, uint64_t slot_bytes) {
-    const uint64_t per = slots_bytes / 16, total = per * n_slabs;
+// Slabs start empty: hash entries, claims and stamps all ones, records empty.  The lists
+// of a slab (tile lists, spill requests, insertions, T) are written before they are read.
+__global__ void slab_init_kernel(uint8_t *slabs, uint64_t slab_bytes, uint32_t n_slabs, uint64_t init_bytes,
+                                 uint64_t recs, uint64_t recs_end, bool prune) {
+    const uint64_t per = init_bytes / 16, total = per * n_slabs;
+    const uint32_t rec_chunks = prune ? sizeof(RecT<long long>) / 16 : sizeof(RecT<int>) / 16;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < total;
          i += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t o = (i % per) * 16;   // offset inside the slab's slot region
+        const uint64_t o = (i % per) * 16;   // offset inside the slab
         uint4 *p = (uint4 *)(slabs + (i / per) * slab_bytes + o);
-        *p = o % slot_bytes == 0 ? make_uint4(~0u, ~0u, 0u, 0u) : make_uint4(~0u, ~0u, ~0u, ~0u);
+        *p = o >= recs && o < recs_end ? empty_chunk(prune, (uint32_t)((o - recs) / 16 % rec_chunks))
+                                       : make_uint4(~0u, ~0u, ~0u, ~0u);
     }
 }
 
@@ -1366,24 +1242,14 @@ cudaError_t launch_pack(uint32_t nq, const char *d_q, const uint64_t *d_off, uin
     return cudaGetLastError();
 }
 
-cudaError_t launch_fill(void *p, uint64_t bytes, cudaStream_t st) {
-    const uint64_t n16 = bytes / 16;
-    if (n16 == 0) return cudaSuccess;
-    uint64_t blocks = (n16 + 255) / 256;
-    if (blocks > 4096) blocks = 4096;
-    fill_kernel<<<(unsigned)blocks, 256, 0, st>>>((uint4 *)p, n16);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_slab_init(uint8_t *slabs, uint64_t slab_bytes, uint32_t n_slabs, uint32_t log2cap,
                              bool prune, cudaStream_t st) {
     const SlabLayout L = slab_layout(log2cap, prune);
-    const uint64_t n16 = (L.touched - L.slots) / 16 * n_slabs;
+    const uint64_t n16 = L.list0 / 16 * n_slabs;
     if (n16 == 0) return cudaSuccess;
     uint64_t blocks = (n16 + 255) / 256;
     if (blocks > 8192) blocks = 8192;
-    slab_init_kernel<<<(unsigned)blocks, 256, 0, st>>>(slabs, slab_bytes, n_slabs,
-                                                        L.touched - L.slots, L.slot_bytes);
+    slab_init_kernel<<<(unsigned)blocks, 256, 0, st>>>(slabs, slab_bytes, n_slabs, L.list0, L.recs, L.touched, prune);
     return cudaGetLastError();
 }
 
