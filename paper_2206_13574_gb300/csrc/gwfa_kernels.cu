@@ -61,6 +61,7 @@ constexpr int kAbsent = -2;                  // exact mode: offset -1, not in Q
 // Tiles whose "listed for the next score" flag is a bit in shared memory; tiles claimed
 // beyond them use a stamp in global memory.  4 KB per parity and CTA.
 constexpr uint32_t kBitTiles = 32768;
+constexpr uint32_t kSmall = 64;   // spill-list entries kept in shared memory
 
 template <bool P> struct VT;
 template <> struct VT<false> { using T = int; };
@@ -136,6 +137,9 @@ struct Sh {
     unsigned long long t_phase;  // statistics: start of the current pass
     unsigned long long st[6];    // statistics (thread 0 only), see gwfa_engine_set_stats
     Score score[4];
+    // the first entries of the score's spill lists: exact mode 2 x kSmall requests (v, ku),
+    // pruning mode kSmall requests, then kSmall insertions
+    uint4 small[2 * kSmall];
     uint32_t bits[2][kBitTiles / 32];
 };
 
@@ -254,14 +258,14 @@ template <bool P> __device__ __forceinline__ void count_claim(const Slab<P> &s, 
     if (atomicAdd(&sh.nclaim, 1u) + 1 > (s.cap >> 1) + (s.cap >> 2)) atomicCAS(err, 0, GWFA_ERR_CAPACITY);
 }
 
-// Record of tile (v, kb), claimed if absent; -1 (and *err) when the slab is full.
+// Record of tile (v, kb), claimed if absent; -1 (and *err) when the slab is full.  The
+// first probe is inline, the rest (and the claim) is not.
 template <bool P>
-__device__ __noinline__ int find_or_insert(const Slab<P> &s, Sh &sh, uint32_t v, int kb, int *err) {
-    const unsigned long long key = tile_key(v, kb);
-    uint32_t h = tile_hash(key, s.tmask);
+__device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsigned long long key, uint32_t h, Ent e,
+                                                int *err) {
     uint32_t idx = kNone;
     for (int probe = 0; probe < 256; ++probe) {
-        Ent e = ld_ent(&s.table[h]);
+        if (probe > 0) e = ld_ent(&s.table[h]);
         if (e.key == kEmptyKey) {
             if (idx == kNone) {
                 if constexpr (P) {
@@ -275,8 +279,8 @@ __device__ __noinline__ int find_or_insert(const Slab<P> &s, Sh &sh, uint32_t v,
             e = cas_ent(&s.table[h], key, idx);
             if (e.key == kEmptyKey) {
                 s.touched[idx] = h;
-                s.recs[idx].side[0].kb = kb;
-                s.recs[idx].side[1].kb = kb;
+                s.recs[idx].side[0].kb = (int)(uint32_t)key;
+                s.recs[idx].side[1].kb = (int)(uint32_t)key;
                 if constexpr (P) s.tkey[idx] = key;
                 else count_claim<P>(s, sh, err);   // a claimed tile always gets a diagonal
                 return (int)idx;
@@ -287,6 +291,13 @@ __device__ __noinline__ int find_or_insert(const Slab<P> &s, Sh &sh, uint32_t v,
     }
     atomicCAS(err, 0, GWFA_ERR_CAPACITY);
     return -1;
+}
+template <bool P>
+__device__ __forceinline__ int find_or_insert(const Slab<P> &s, Sh &sh, uint32_t v, int kb, int *err) {
+    const unsigned long long key = tile_key(v, kb);
+    const uint32_t h = tile_hash(key, s.tmask);
+    const Ent e = ld_ent(&s.table[h]);
+    return e.key == key ? (int)e.idx : find_or_insert_slow<P>(s, sh, key, h, e, err);
 }
 
 // List a tile for the next score; true for the one caller that has to append it.
@@ -350,6 +361,19 @@ __device__ __forceinline__ uint32_t push_trace(const Slab<true> &s, Sh &sh, uint
     return idx;
 }
 
+// Spill lists: the first entries in shared memory, the rest in the slab.
+__device__ __forceinline__ void put_req(const Slab<false> &s, Sh &sh, uint32_t i, uint32_t v, int ku, int *err) {
+    if (i < 4 * kSmall) ((uint2 *)sh.small)[i] = make_uint2(v, (uint32_t)ku);
+    else if (i < 4 * s.cap) s.req[i] = make_uint2(v, (uint32_t)ku);
+    else atomicCAS(err, 0, GWFA_ERR_CAPACITY);
+}
+__device__ __forceinline__ uint2 get_req(const Slab<false> &s, const Sh &sh, uint32_t i) {
+    return i < 4 * kSmall ? ((const uint2 *)sh.small)[i] : s.req[i];
+}
+__device__ __forceinline__ int4 get_req4(const Slab<true> &s, const Sh &sh, uint32_t i) {
+    return i < kSmall ? ((const int4 *)sh.small)[i] : s.req4[i];
+}
+
 // Pruning mode: a settled diagonal reached |v|: offset 0 with the walk base past v goes
 // to (u, k + |v|) for every arc (v, u), after the pass (see apply_spills).
 __device__ __forceinline__ void request_spill(const Slab<true> &s, Sh &sh, uint32_t at, const uint4 &vi, uint32_t v,
@@ -358,7 +382,7 @@ __device__ __forceinline__ void request_spill(const Slab<true> &s, Sh &sh, uint3
     if (nb > kBaseMask) atomicCAS(err, 0, GWFA_ERR_CAPACITY);
     const uint32_t t = traceback ? push_trace(s, sh, v, tr, err) : 0u;
     if (at < s.cap) {
-        s.req4[at] = make_int4(k + (int)vi.y, (int)nb, (int)vi.z, (int)vi.w);
+        *(at < kSmall ? (int4 *)&sh.small[at] : &s.req4[at]) = make_int4(k + (int)vi.y, (int)nb, (int)vi.z, (int)vi.w);
         if (traceback) s.reqt[at] = t;
     } else {
         atomicCAS(err, 0, GWFA_ERR_CAPACITY);
@@ -396,12 +420,13 @@ __device__ __forceinline__ void offset_pass(const DevGraph &g, const Slab<P> &s,
         T raw = rec->vals[ln];
         const uint2 vi = __ldg((const uint2 *)&g.vinfo[ent.y]);   // label word, |v|
         T in;
-        uint32_t link;
+        uint32_t link, counted = 0;
         int k;
         if constexpr (P) {
             in = rec->side[sd].in[par];
-            const uint2 lk = *(const uint2 *)&rec->side[sd].link;
+            const uint4 lk = *(const uint4 *)&rec->side[sd].link;
             link = lk.x;
+            counted = lk.z;
             k = (int)lk.y * kTile + ln;
         } else {
             const int4 sw = *(const int4 *)&rec->side[sd];
@@ -482,10 +507,10 @@ __device__ __forceinline__ void offset_pass(const DevGraph &g, const Slab<P> &s,
             jn = inq ? pj(c) : j;
             if (inq) base = pbase(c);
             if (inq && raw < 0) ++visited;
-            // first diagonal of this tile?
-            const unsigned pres = __ballot_sync(full, raw >= 0), add = __ballot_sync(full, inq);
-            if (ln == 0 && !((pres >> (lane & 24)) & 0xFFu) && ((add >> (lane & 24)) & 0xFFu)) {
-                s.recs[ent.x].side[1].counted = 1u;
+            // a tile that holds a diagonal for the first time (claimed here or by a spill)
+            const unsigned has = __ballot_sync(full, inq || raw >= 0);
+            if (ln == 7 && !counted && on && ((has >> (lane & 24)) & 0xFFu)) {
+                rec->side[1].counted = 1u;
                 count_claim<P>(s, sh, &S.err);
             }
         } else {
@@ -529,8 +554,7 @@ __device__ __forceinline__ void offset_pass(const DevGraph &g, const Slab<P> &s,
                     const uint4 f = __ldg(&g.vinfo[ent.y]);
                     request_spill(s, sh, b, f, ent.y, k, base, trn, TB, &S.err);
                 } else {
-                    if (b < 4 * s.cap) s.req[b] = make_uint2(ent.y, (uint32_t)(k + (int)vi.y));
-                    else atomicCAS(&S.err, 0, GWFA_ERR_CAPACITY);
+                    put_req(s, sh, b, ent.y, k + (int)vi.y, &S.err);
                 }
             }
         }
@@ -575,81 +599,89 @@ __device__ __forceinline__ void offset_pass(const DevGraph &g, const Slab<P> &s,
     }
 }
 
-// Exact mode: requests [r0, r0 + n) of the log, one thread each: offset 0 to (u, ku) for
-// every arc (v, u) where it is absent (Alg. 2's arc loop).  A diagonal this thread inserts
-// is extended by it at once; if that one reaches its vertex's end too, the thread goes on
-// with it, or, when the arcs give several, appends the others to the log.
-__device__ void spill_round(const DevGraph &g, const Slab<false> &s, Sh &sh, const QCtx &q, int d, uint32_t r0,
-                            uint32_t n, uint32_t *next_count) {
+// Exact mode: requests [r0, r0 + n) of the score's log: offset 0 to (u, ku) for every arc
+// (v, u) where it is absent (Alg. 2's arc loop).  A spill is a chain of dependent L2 round
+// trips (arc, hash entry, offset, label) and a score has a few dozen of them, so they are
+// spread over the warps, and in a warp over quads of lanes, one arc a lane.  A diagonal
+// that a lane inserts is extended by it at once; if that one reaches its vertex's end too,
+// its quad goes on with it (or it is logged for the next round when the lane has one
+// waiting already).
+__device__ __forceinline__ void spill_round(const DevGraph &g, const Slab<false> &s, Sh &sh, const QCtx &q, int d,
+                                            uint32_t r0, uint32_t n, uint32_t *next_count) {
     Score &S = sh.score[d & 3];
+    const unsigned full = 0xFFFFFFFFu;
+    const int lane = threadIdx.x & 31, arc = lane & 3;
+    const uint32_t nw = blockDim.x >> 5;
     uint32_t won = 0;
-    for (uint32_t r = threadIdx.x; r < n; r += blockDim.x) {
-        uint2 rq = s.req[r0 + r];
+    for (uint32_t b = threadIdx.x >> 5; b < n; b += 8 * nw) {
+        const uint32_t r = b + (uint32_t)(lane >> 2) * nw;
+        uint2 rq = r < n ? get_req(s, sh, r0 + r) : make_uint2(kNone, 0u);
+        uint2 wait = make_uint2(kNone, 0u);   // this lane's inserted diagonal that spills in turn
         for (;;) {
-            const uint4 vi = __ldg(&g.vinfo[rq.x]);
-            const int ku = (int)rq.y;
-            uint2 more = make_uint2(kNone, 0u);
-            for (uint32_t a = vi.z; a < vi.w; ++a) {
-                const uint32_t u = __ldg(&g.arc_dst[a]);
-                const int su = find_or_insert<false>(s, sh, u, ku >> 3, &S.err);
-                if (su < 0) break;
-                if (g_cas(&s.recs[su].vals[ku & 7], kAbsent, 1) != kAbsent) continue;
-                ++won;
-                const uint2 ui = __ldg((const uint2 *)&g.vinfo[u]);
-                const int l = lcp(q, ku, g.words + ui.x, 0, (int)ui.y);
-                s.recs[su].vals[ku & 7] = (l << 1) | 1;
-                if (at_end(q, u, ku, l, ui.y)) S.found = 1;
-                enter_next<false>(s, sh, q, (uint32_t)su, u, ku, l, 0u, ui.y, d, 0u, false);
-                if ((uint32_t)l == ui.y) {
-                    const uint2 c = make_uint2(u, (uint32_t)(ku + (int)ui.y));
-                    if (more.x == kNone) {
-                        more = c;
-                    } else {
-                        const uint32_t at = r0 + n + atomicAdd(next_count, 1u);
-                        if (at < 4 * s.cap) s.req[at] = c;
-                        else atomicCAS(&S.err, 0, GWFA_ERR_CAPACITY);
+            if (rq.x != kNone) {
+                const uint2 ar = __ldg((const uint2 *)&g.vinfo[rq.x].z);
+                const int ku = (int)rq.y;
+                for (uint32_t a = ar.x + arc; a < ar.y; a += 4) {
+                    const uint32_t u = __ldg(&g.arc_dst[a]);
+                    const uint2 ui = __ldg((const uint2 *)&g.vinfo[u]);
+                    const int su = find_or_insert<false>(s, sh, u, ku >> 3, &S.err);
+                    if (su < 0) break;
+                    const int prev = g_cas(&s.recs[su].vals[ku & 7], kAbsent, 1);
+                    const int l = lcp(q, ku, g.words + ui.x, 0, (int)ui.y);   // while the swap is under way
+                    if (prev != kAbsent) continue;
+                    ++won;
+                    s.recs[su].vals[ku & 7] = (l << 1) | 1;
+                    if (at_end(q, u, ku, l, ui.y)) S.found = 1;
+                    enter_next<false>(s, sh, q, (uint32_t)su, u, ku, l, 0u, ui.y, d, 0u, false);
+                    if ((uint32_t)l == ui.y) {
+                        if (wait.x == kNone) wait = make_uint2(u, (uint32_t)(ku + l));
+                        else put_req(s, sh, r0 + n + atomicAdd(next_count, 1u), u, ku + l, &S.err);
                     }
                 }
             }
-            if (more.x == kNone) break;
-            rq = more;
+            const unsigned m = __ballot_sync(full, wait.x != kNone);
+            if (!m) break;
+            const unsigned m4 = (m >> (lane & 28)) & 15u;
+            const int src = m4 ? __ffs(m4) - 1 : 0;
+            rq.x = __shfl_sync(full, wait.x, src, 4);
+            rq.y = __shfl_sync(full, wait.y, src, 4);
+            if (arc == src) wait.x = kNone;
         }
     }
-    won = __reduce_add_sync(0xFFFFFFFFu, won);
-    if ((threadIdx.x & 31) == 0 && won) {
+    won = __reduce_add_sync(full, won);
+    if (lane == 0 && won) {
         atomicAdd(&S.cells, won);
         atomicAdd(&S.spills, won);
     }
 }
 
-// Pruning mode: offset 0 with walk base nb on (u, ku) for every request of the round; the
+// Pruning mode, by `nthr` threads (a warp or the CTA): offset 0 with walk base nb on
+// (u, ku) for every request of the round, a quad of lanes a request and a lane an arc; the
 // inserted diagonals go to the round's insertion list.  A spill never changes a diagonal
 // that was present before the round (Alg. 2's presence test: a settled offset of 0 is
 // larger than any pending one), and spills of one round into one diagonal merge by the
 // larger walk base.
-__device__ void apply_spills(const DevGraph &g, const Slab<true> &s, Sh &sh, int d, uint32_t n, uint32_t *n_ins,
-                             bool traceback) {
+__device__ __forceinline__ void apply_spills(const DevGraph &g, const Slab<true> &s, Sh &sh, int d, uint32_t n,
+                                             uint32_t *n_ins, uint32_t nthr, bool traceback) {
     Score &S = sh.score[d & 3];
     uint32_t won = 0;
-    for (uint32_t r = threadIdx.x; r < min(n, s.cap); r += blockDim.x) {
-        const int4 rq = s.req4[r];
+    for (uint32_t r = threadIdx.x >> 2; r < min(n, s.cap); r += nthr >> 2) {
+        const int4 rq = get_req4(s, sh, r);
         const int ku = rq.x;
         const long long cand = pk(0, kTagPend, (uint32_t)rq.y);
-        for (uint32_t a = (uint32_t)rq.z; a < (uint32_t)rq.w; ++a) {
+        for (uint32_t a = (uint32_t)rq.z + (threadIdx.x & 3); a < (uint32_t)rq.w; a += 4) {
             const uint32_t u = __ldg(&g.arc_dst[a]);
             const int su = find_or_insert<true>(s, sh, u, ku >> 3, &S.err);
             if (su < 0) break;
             if (g_max(&s.recs[su].vals[ku & 7], cand) >= 0) continue;
             ++won;
             if (traceback) s.trec[su].tr[ku & 7] = 0u;   // set by resolve_spill_traces
-            if (!g_exch(&s.recs[su].side[1].counted, 1u)) count_claim<true>(s, sh, &S.err);
             const uint32_t i = atomicAdd(n_ins, 1u);
-            if (i < 2 * s.cap) s.ins[i] = make_uint4((uint32_t)su, u, (uint32_t)ku, 0u);
+            if (i < 2 * s.cap) *(i < kSmall ? &sh.small[kSmall + i] : &s.ins[i]) = make_uint4((uint32_t)su, u, (uint32_t)ku, 0u);
             else atomicCAS(&S.err, 0, GWFA_ERR_CAPACITY);
         }
     }
-    won = __reduce_add_sync(0xFFFFFFFFu, won);
-    if ((threadIdx.x & 31) == 0 && won) {
+    if (won) {
         atomicAdd(&S.cells, won);
         atomicAdd(&S.spills, won);
         atomicAdd(&S.visited, won);
@@ -660,12 +692,13 @@ __device__ void apply_spills(const DevGraph &g, const Slab<true> &s, Sh &sh, int
 // inserted in this round holds the largest base among its spills, still tagged pending;
 // each request whose base is that one offers its T index and the largest index wins (any
 // of them is a walk of that base, so the choice only has to be deterministic).
-__device__ void resolve_spill_traces(const DevGraph &g, const Slab<true> &s, Sh &sh, int d, uint32_t n) {
-    for (uint32_t r = threadIdx.x; r < min(n, s.cap); r += blockDim.x) {
-        const int4 rq = s.req4[r];
+__device__ __forceinline__ void resolve_spill_traces(const DevGraph &g, const Slab<true> &s, Sh &sh, int d, uint32_t n,
+                                                     uint32_t nthr) {
+    for (uint32_t r = threadIdx.x >> 2; r < min(n, s.cap); r += nthr >> 2) {
+        const int4 rq = get_req4(s, sh, r);
         const int ku = rq.x;
         const long long cand = pk(0, kTagPend, (uint32_t)rq.y);
-        for (uint32_t a = (uint32_t)rq.z; a < (uint32_t)rq.w; ++a) {
+        for (uint32_t a = (uint32_t)rq.z + (threadIdx.x & 3); a < (uint32_t)rq.w; a += 4) {
             const int su = find_or_insert<true>(s, sh, __ldg(&g.arc_dst[a]), ku >> 3, &sh.score[d & 3].err);
             if (su < 0) return;
             if (s.recs[su].vals[ku & 7] == cand) g_max32(&s.trec[su].tr[ku & 7], s.reqt[r]);
@@ -675,19 +708,18 @@ __device__ void resolve_spill_traces(const DevGraph &g, const Slab<true> &s, Sh 
 
 // Pruning mode: extend the diagonals inserted by the round; those that reach their
 // vertex's end request the next round's spills.
-__device__ void extend_spilled(const DevGraph &g, const Slab<true> &s, Sh &sh, const QCtx &q, int d, uint32_t n,
-                               uint32_t *n_req, bool traceback) {
+__device__ __forceinline__ void extend_spilled(const DevGraph &g, const Slab<true> &s, Sh &sh, const QCtx &q, int d,
+                                               uint32_t n, uint32_t *n_req, uint32_t nthr, bool traceback) {
     Score &S = sh.score[d & 3];
-    uint32_t amax = 0;
-    for (uint32_t r = threadIdx.x; r < min(n, 2 * s.cap); r += blockDim.x) {
-        const uint4 in = s.ins[r];
+    for (uint32_t r = threadIdx.x; r < min(n, 2 * s.cap); r += nthr) {
+        const uint4 in = r < kSmall ? sh.small[kSmall + r] : s.ins[r];
         const int k = (int)in.z;
         const uint4 vi = __ldg(&g.vinfo[in.y]);
         const uint32_t base = pbase(s.recs[in.x].vals[k & 7]);
         const uint32_t tr = traceback ? s.trec[in.x].tr[k & 7] : 0u;
         const int j = lcp(q, k, g.words + vi.x, 0, (int)vi.y);
         s.recs[in.x].vals[k & 7] = pk(j, kTagLive, base);
-        amax = max(amax, (uint32_t)(k + j) + (uint32_t)j + base);
+        atomicMax(&S.amax, (uint32_t)(k + j) + (uint32_t)j + base);
         if (at_end(q, in.y, k, j, vi.y)) {
             S.found = 1;
             sh.end_vp = ((unsigned long long)in.y << 32) | tr;
@@ -696,8 +728,6 @@ __device__ void extend_spilled(const DevGraph &g, const Slab<true> &s, Sh &sh, c
         if ((uint32_t)j == vi.y)
             request_spill(s, sh, atomicAdd(n_req, 1u), vi, in.y, k, base, tr, traceback, &S.err);
     }
-    amax = __reduce_max_sync(0xFFFFFFFFu, amax);
-    if ((threadIdx.x & 31) == 0 && amax) atomicMax(&S.amax, amax);
 }
 
 // Empty the records and hash entries of a query; in exact mode, which never removes a
@@ -830,8 +860,6 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         if (t >= 0) {
             if constexpr (P) {
                 s.recs[t].vals[0] = pk(0, kTagLive, 0u);
-                s.recs[t].side[1].counted = 1u;
-                sh.nclaim = 1;
                 if (A.traceback) s.trec[t].tr[0] = kNoTrace;
                 sh.visited = 1;
             } else {
@@ -865,8 +893,6 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
                 }
             }
             if constexpr (P) {
-                s.recs[t].side[1].counted = 1u;
-                count_claim<P>(s, sh, &sh.score[0].err);
                 atomicAdd(&sh.visited, (unsigned long long)cnt);
             }
             s.list[0][atomicAdd(&sh.score[0].nq, 1u)] = make_uint2((uint32_t)t, vs);
@@ -912,28 +938,49 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
             if (A.evict_lag > 0 && d > 0 && d % A.evict_every == 0) evict_behind(s, sh, amax, A.evict_lag, d);
         }
         // ---- arc spills, in rounds until no extended diagonal reaches its vertex's end
-        uint32_t n = S.nreq, r0 = 0;
-        for (int round = 0; n; ++round) {
-            uint32_t *next_count = &sh.nr[round % 3];
-            if (threadIdx.x == 0) sh.nr[(round + 1) % 3] = 0;
-            if constexpr (P) {
-                uint32_t *n_ins = &sh.nins[round & 1];
-                if (threadIdx.x == 0) sh.nins[(round + 1) & 1] = 0;
-                apply_spills(g, s, sh, d, n, n_ins, A.traceback != 0);
-                __syncthreads();
-                if (A.traceback) {
-                    resolve_spill_traces(g, s, sh, d, n);
-                    __syncthreads();
+        uint32_t n = S.nreq;
+        if constexpr (P) {
+            // few requests (the usual case): one warp does every round by itself, and the
+            // others wait once instead of twice or three times a round
+            const bool solo = n <= 32;
+            const uint32_t nthr = solo ? 32u : blockDim.x;
+            auto sync = [&]() {
+                if (solo) __syncwarp();
+                else __syncthreads();
+            };
+            const bool any = n > 0;
+            if (!solo || threadIdx.x < 32) {
+                for (int round = 0; n; ++round) {
+                    uint32_t *next_count = &sh.nr[round % 3], *n_ins = &sh.nins[round & 1];
+                    if (threadIdx.x == 0) {
+                        sh.nr[(round + 1) % 3] = 0;
+                        sh.nins[(round + 1) & 1] = 0;
+                    }
+                    apply_spills(g, s, sh, d, n, n_ins, nthr, A.traceback != 0);
+                    sync();
+                    if (A.traceback) {
+                        resolve_spill_traces(g, s, sh, d, n, nthr);
+                        sync();
+                    }
+                    extend_spilled(g, s, sh, q, d, *n_ins, next_count, nthr, A.traceback != 0);
+                    sync();
+                    n = *next_count;
+                    if (A.stats && threadIdx.x == 0 && n) sh.st[2] += 1;
                 }
-                extend_spilled(g, s, sh, q, d, *n_ins, next_count, A.traceback != 0);
-            } else {
+            }
+            if (solo && any) __syncthreads();
+        } else {
+            uint32_t r0 = 0;
+            for (int round = 0; n; ++round) {
+                uint32_t *next_count = &sh.nr[round % 3];
+                if (threadIdx.x == 0) sh.nr[(round + 1) % 3] = 0;
                 spill_round(g, s, sh, q, d, r0, n, next_count);
                 r0 += n;
+                __syncthreads();
+                n = *next_count;
+                n = min(n, r0 < 4 * s.cap ? 4 * s.cap - r0 : 0u);
+                if (A.stats && threadIdx.x == 0 && n) sh.st[2] += 1;
             }
-            __syncthreads();
-            n = *next_count;
-            if constexpr (!P) n = min(n, r0 < 4 * s.cap ? 4 * s.cap - r0 : 0u);
-            if (A.stats && threadIdx.x == 0 && n) sh.st[2] += 1;
         }
         if (threadIdx.x == 0) {
             sh.cells += S.cells;
@@ -1030,16 +1077,20 @@ __device__ __forceinline__ void align_queries(const TierArgs &A) {
     }
 }
 
-// Up to 512 threads, 4 CTAs per SM at 32 registers: the throughput shape.
+// Up to 512 threads: the throughput shape.  Exact mode 4 CTAs per SM at 32 registers
+// (10,000 reads 59.8 ms; 3 CTAs at 40 registers 79 ms before the spills were spread over
+// the warps).  Pruning mode 3 at 40: its 64-bit offsets spill at 32 (388 bytes of spill
+// stores), and its frontiers are small (400 pruned 50 kb reads 34.5 ms at 4 CTAs, 28.2 ms
+// at 3; traceback of 800 reads with its CIGARs 14.2 and 12.5 ms).
 template <bool P>
-__global__ void __launch_bounds__(512, 4) align_kernel(TierArgs A) {
+__global__ void __launch_bounds__(512, P ? 3 : 4) align_kernel(TierArgs A) {
     align_queries<P>(A);
 }
 
-// 1024 threads, 2 CTAs per SM at the same 32 registers: twice the groups on one
-// query, for the few heaviest queries whose own latency bounds a batch.
+// 1024 threads: twice the groups on one query, for the few heaviest queries whose own
+// latency bounds a batch.  Registers as above: 2 CTAs per SM at 32, 1 at 64.
 template <bool P>
-__global__ void __launch_bounds__(1024, 2) align_kernel_wide(TierArgs A) {
+__global__ void __launch_bounds__(1024, P ? 1 : 2) align_kernel_wide(TierArgs A) {
     align_queries<P>(A);
 }
 
