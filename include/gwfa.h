@@ -183,9 +183,10 @@ typedef struct gwfa_engine gwfa_engine;
  *                  n_wide queries of the schedule (gwfa_schedule), so the heaviest
  *                  queries start at once on slabs that fit them instead of forming a
  *                  tail of overflow re-runs; their overflows go to the retry tiers
- *   threads        threads per CTA (multiple of 32, 32..1024; above 512 a CTA
- *                  takes half an SM: for the few heaviest queries, e.g. the huge
- *                  class, whose own latency bounds a batch); 0 = 128
+ *   threads        threads per CTA (multiple of 32, 32..1024; a wide CTA shortens
+ *                  its query, narrow ones run more of them); 0 = 128; 512 (the
+ *                  default configuration) lets the engine choose the width of
+ *                  each batch's CTAs from its queries
  *   max_queries, max_bases  sizes of the engine's staging buffers for the
  *                  host-buffer entry point (grown on demand)
  */
@@ -215,7 +216,8 @@ typedef struct {
     uint32_t n_wide;
 } gwfa_schedule;
 
-/* fills a default configuration for this GPU (3 tiers, 512 threads, no classes) */
+/* fills a default configuration for this GPU (3 tiers, 512 threads = width chosen for
+ * each batch, no classes) */
 int gwfa_engine_default_config(const gwfa_graph *g, int prune, gwfa_engine_config *cfg);
 int gwfa_engine_create(const gwfa_graph *g, const gwfa_engine_config *cfg, gwfa_engine **out);
 int gwfa_engine_destroy(gwfa_engine *e);
@@ -272,7 +274,7 @@ int gwfa_align_batch_device(gwfa_engine *e, uint32_t n_queries, const uint32_t *
  * but its scratch is one fixed 32 MiB device array inside the library (present
  * on every GPU that loads it, until the process exits), carved into
  * floor((32 MiB - 256 B) / slab) CTA slabs of 2^log2_tiles hash tiles each
- * (log2_tiles 0 = 15: six CTAs in exact mode, three with pruning).  There is
+ * (log2_tiles 0 = 15: six CTAs in exact mode, two with pruning).  There is
  * no overflow tier: a query needing more than 3/4 of its slab gets status
  * GWFA_ERR_CAPACITY.  log2_tiles outside [8, 24] (other than 0) is
  * GWFA_ERR_INVALID; a valid log2_tiles whose slab does not fit the array is

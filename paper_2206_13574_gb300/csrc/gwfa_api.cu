@@ -88,6 +88,27 @@ struct Carve {
     }
 };
 
+// The default config's CTA width: the engine chooses it for each batch.
+constexpr uint32_t kAutoThreads = 512;
+
+// Width of tier 0's CTAs for n queries of `len` bases on average (0 = not known on the
+// host), where the configuration leaves it to the engine.  A wide CTA shortens a query, a
+// narrow one wastes fewer warps on small frontiers and at barriers: few queries are bound
+// by their longest, many by throughput, and a frontier grows with the length.  Measured
+// crossings, 1024 -> 512 -> 256 threads (ms at 1024 / 512 / 256): 1-20 kb reads, 6.4 kb on
+// average, n = 1000: 9.6 / 12.3 / 20.3, 1500: 13.9 / 14.6 / 25.7, 2500: 22.5 / 15.9 / 24.5,
+// 4000: 35.8 / 23.9 / 29.1, 7000: 62 / 41.7 / 37.7; 0.5-5 kb, 2.0 kb on average, n = 600:
+// 1.37 / 1.47 / 1.74, 1000: 1.94 / 1.51 / 1.88, 2500: 4.8 / 2.56 / 2.46.
+// Lag pruning keeps the frontier near 0.03 tiles per unit of lag, whatever the length
+// (lag 1000, 1024 / 256 / 128 threads, n = 150: 9.5 / 9.6 / 10.2, 400: 25.7 / 9.8 / 10.8,
+// 1000: 59 / 18.7 / 12.0; lag 4000: 15.6 / 19.5 / 27.2, 41.5 / 21.5 / 26.9, 95 / 39 / 33).
+uint32_t auto_threads(uint64_t n, uint64_t len, int sms, int max_lag) {
+    const uint64_t m = (uint64_t)sms;
+    if (max_lag > 0) return n <= m && max_lag > 2000 ? 1024u : n <= 4 * m ? 256u : 128u;
+    if (len == 0) len = 4000;
+    return n <= m * len / 600 ? 1024u : n <= m * len / 180 ? 512u : gwfa::kNarrow;
+}
+
 uint64_t words_for(uint32_t nq, uint64_t nbases) { return (nbases >> 4) + nq + 2; }
 
 }  // namespace
@@ -328,7 +349,7 @@ static int align_plain(const gwfa_graph *g, const char *h_q, uint32_t n, uint32_
         a.path_len = o.traceback ? d_plen : nullptr;
         a.path_cap = path_cap;
         if (o.traceback) cudaMemsetAsync(d_plen, 0, 4, s);
-        st = cuda_status(gwfa::launch_align(a, prune, 1, 512, s));
+        st = cuda_status(gwfa::launch_align(a, prune, 1, o.max_lag > 0 ? 256 : n < 3000 ? 512 : 1024, s));
         if (st) return st;
         st = cuda_status(cudaMemcpyAsync(out, d_res, sizeof(gwfa_result), cudaMemcpyDeviceToHost, s));
         if (!st && o.traceback) st = cuda_status(cudaMemcpyAsync(path_len, d_plen, 4, cudaMemcpyDeviceToHost, s));
@@ -355,10 +376,9 @@ int gwfa_engine_default_config(const gwfa_graph *g, int prune, gwfa_engine_confi
     int sms = 0, bps = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device) != cudaSuccess)
         return GWFA_ERR_CUDA;
-    // 512-thread CTAs, as many as fit on an SM (the kernel is bound by the latency
-    // of dependent L2 round trips, so resident warps matter more than registers)
-    cfg->threads = 512;
-    if (gwfa::align_occupancy(prune != 0, cfg->threads, &bps) || bps < 1) bps = 1;
+    // width chosen for each batch (tier0_threads); as many narrow CTAs as fit on an SM
+    cfg->threads = kAutoThreads;
+    if (gwfa::align_occupancy(prune != 0, prune ? gwfa::kNarrow / 2 : gwfa::kNarrow, &bps) || bps < 1) bps = 1;
     cfg->wide = {0u, prune ? 18u : 19u, 512u, 0u};   // no concurrent classes by default
     cfg->huge = {0u, 22u, 512u, 0u};
     cfg->n_tiers = 3;
@@ -424,6 +444,7 @@ int gwfa_engine_create(const gwfa_graph *g, const gwfa_engine_config *cfg, gwfa_
     e->g = g;
     e->cfg = *cfg;
     e->cfg.threads = threads;
+    if (cudaDeviceGetAttribute(&e->sms, cudaDevAttrMultiProcessorCount, g->device) != cudaSuccess) e->sms = 1;
     st = cuda_status(cudaStreamCreateWithFlags(&e->stream, cudaStreamNonBlocking));
     for (uint32_t t = 0; !st && t < cfg->n_tiers; ++t) {
         e->slab_bytes[t] = gwfa::slab_layout(cfg->tiers[t].log2_tiles, cfg->prune_slabs != 0).total;
@@ -566,7 +587,7 @@ static TierArgs tier_args(gwfa_engine *e, const uint32_t *d_words, const uint64_
 static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const uint64_t *d_q_off,
                      const uint32_t *d_vs, const uint32_t *d_ve, const uint32_t *d_order,
                      const gwfa_schedule *sched, const int32_t *d_status, const gwfa_opts &o,
-                     gwfa_result *d_out, cudaStream_t s) {
+                     gwfa_result *d_out, uint64_t len, cudaStream_t s) {
     int st = engine_retry_capacity(e, n);
     if (st) return st;
     const uint32_t T = e->cfg.n_tiers;
@@ -596,17 +617,25 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
     // the classes' CTAs and tier 0's must be resident together (tier 0 would
     // otherwise fill every SM slot and the heaviest queries would start only after
     // it): tier 0 gives up the room of the class CTAs it runs beside
-    const uint32_t t0_threads = e->cfg.tiers[0].threads ? e->cfg.tiers[0].threads : e->cfg.threads;
-    uint64_t yield_threads = 0;
+    auto tier_threads = [&](const gwfa_tier &t, uint32_t count) {
+        if (t.threads) return t.threads;
+        return e->cfg.threads != kAutoThreads ? e->cfg.threads : auto_threads(count, len, e->sms, o.max_lag);
+    };
+    auto per_sm = [&](uint32_t threads) {
+        int b = 1;
+        return gwfa::align_occupancy(prune, threads, &b) || b < 1 ? 1u : (uint32_t)b;
+    };
+    const uint32_t t0_threads = tier_threads(e->cfg.tiers[0], n - n_huge - n_wide), t0_per_sm = per_sm(t0_threads);
+    double yield_sms = 0;
     uint32_t cctas[2] = {0, 0};
     for (int c = 0; c < 2; ++c) {
         if (!cls[c].count) continue;
-        const uint32_t th = cls[c].tier->threads ? cls[c].tier->threads : e->cfg.threads;
         cctas[c] = std::min(cls[c].tier->ctas, cls[c].count);
-        yield_threads += (uint64_t)cctas[c] * th;
+        yield_sms += (double)cctas[c] / per_sm(tier_threads(*cls[c].tier, cctas[c]));
     }
-    const uint32_t t0_yield = (uint32_t)((yield_threads + t0_threads - 1) / t0_threads);
-    const uint32_t t0_ctas = e->cfg.tiers[0].ctas > t0_yield ? e->cfg.tiers[0].ctas - t0_yield : 1;
+    const uint32_t t0_max = std::min(e->cfg.tiers[0].ctas, (uint32_t)e->sms * t0_per_sm);
+    const uint32_t t0_yield = (uint32_t)std::ceil(yield_sms * t0_per_sm);
+    const uint32_t t0_ctas = t0_max > t0_yield ? t0_max - t0_yield : 1;
     bool forked = false;
     for (int c = 0; c < 2; ++c) {
         if (!cls[c].count) continue;
@@ -625,7 +654,7 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
         a.slabs = cls[c].slabs;
         a.slab_bytes = cls[c].slab_bytes;
         a.log2cap = cls[c].tier->log2_tiles;
-        const uint32_t th = cls[c].tier->threads ? cls[c].tier->threads : e->cfg.threads;
+        const uint32_t th = tier_threads(*cls[c].tier, cctas[c]);
         st = cuda_status(cudaStreamWaitEvent(cls[c].side, e->ev_fork, 0));
         if (!st) st = cuda_status(gwfa::launch_align(a, prune, cctas[c], th, cls[c].side));
         if (!st) st = cuda_status(cudaEventRecord(cls[c].join, cls[c].side));
@@ -656,7 +685,7 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
         a.slabs = e->slabs[t];
         a.slab_bytes = e->slab_bytes[t];
         a.log2cap = e->cfg.tiers[t].log2_tiles;
-        const uint32_t th = e->cfg.tiers[t].threads ? e->cfg.tiers[t].threads : e->cfg.threads;
+        const uint32_t th = t == 0 ? t0_threads : tier_threads(e->cfg.tiers[t], e->cfg.tiers[t].ctas);
         st = cuda_status(gwfa::launch_align(a, prune, t == 0 ? t0_ctas : e->cfg.tiers[t].ctas, th, s));
         if (st) return st;
         e->last_launches++;
@@ -680,7 +709,7 @@ int gwfa_align_batch_device(gwfa_engine *e, uint32_t n, const uint32_t *d_words,
     if (st) return st;
     // exactly the caller's stream (NULL = the legacy default stream), so the batch is
     // ordered after whatever produced its inputs on that stream
-    return run_tiers(e, n, d_words, d_q_off, d_vs, d_ve, d_order, sched, d_status, o, d_out,
+    return run_tiers(e, n, d_words, d_q_off, d_vs, d_ve, d_order, sched, d_status, o, d_out, 0,
                      (cudaStream_t)stream);
 }
 
@@ -726,7 +755,7 @@ int gwfa_align_batch(gwfa_engine *e, uint32_t n, const char *h_q, const uint64_t
     nvtxRangePushA("alignment tiers");
     if (!st)
         st = run_tiers(e, n, d_words, d_off, d_vs, d_ve, h_order ? d_order : nullptr, sched, d_status, o,
-                       d_out, s);
+                       d_out, nb / n, s);
     nvtxRangePop();
     if (!st) e->last_launches += 1;
     nvtxRangePushA("copy out + wait");

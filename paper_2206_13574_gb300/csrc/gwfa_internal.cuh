@@ -40,6 +40,8 @@ struct DevGraph {
 };
 
 constexpr uint32_t kMaxLog2Tiles = 24;
+constexpr uint32_t kNarrow = 256;   // threads per CTA up to which the narrow kernel runs
+
 
 // Hash entry: the tile's key (v << 32 | kb, all ones = empty) and its record.
 struct alignas(16) TabEnt {
@@ -87,7 +89,7 @@ __host__ __device__ inline uint4 empty_chunk(bool prune, uint32_t part) {
 // as many entries as tiles), the records, the hash position of each record and its list
 // stamp -- these start all ones / empty -- then the two tile lists and the spill lists.
 struct SlabLayout {
-    uint64_t table, recs, touched, stamp, tkey, list0, list1, req, reqt, ins, freel, trace, trec, total;
+    uint64_t table, recs, touched, stamp, tkey, list0, list1, links, req, reqt, ins, freel, trace, trec, total;
 };
 
 __host__ __device__ inline uint64_t align256(uint64_t x) { return (x + 255) & ~255ull; }
@@ -103,6 +105,7 @@ __host__ __device__ inline SlabLayout slab_layout(uint32_t log2cap, bool prune) 
     L.tkey = o;    o = align256(o + (prune ? cap * 8 : 0));    // keys by record (memory bound)
     L.list0 = o;   o = align256(o + cap * 8);                  // (record, vertex)
     L.list1 = o;   o = align256(o + cap * 8);
+    L.links = o;   o = align256(o + 2 * cap * 8);              // neighbours to be linked
     L.req = o;     o = align256(o + (prune ? cap * 16 : 4 * cap * 8));   // arc-spill requests of a score
     L.reqt = o;    o = align256(o + (prune ? cap * 4 : 0));    // trace index of each request
     L.ins = o;     o = align256(o + (prune ? 2 * cap * 16 : 0));   // diagonals a spill round inserted
@@ -134,7 +137,6 @@ struct TierArgs {
     int32_t max_lag;
     int32_t max_score;
     unsigned long long *stats;  // optional, kStatWords per query id (see gwfa_engine_set_stats)
-    int q_smem;                 // query words are in shared memory (server kernel)
     int traceback;              // 64-bit values carry a trace index (Alg. 5-6) instead of a base
     int ends;                   // formulation variant flags (GWFA_FREE_START / _FREE_END / _EXTEND)
     int evict_lag;              // memory bound on H~ (pruning mode): lag behind a_max, 0 = off
@@ -171,6 +173,7 @@ struct ServerArgs {
     unsigned int *idle_votes;      // device: CTAs currently idle for wait_limit polls or more
     uint32_t n_ctas;
     uint32_t ring, slot_words;
+    uint32_t *stage;               // device: slot_words per CTA, the words of its request
     uint32_t wait_limit, sleep_ns;
     int32_t max_lag, max_score;
 };
@@ -184,8 +187,8 @@ cudaError_t launch_slab_init(uint8_t *slabs, uint64_t slab_bytes, uint32_t n_sla
                              bool prune, cudaStream_t st);
 int align_occupancy(bool prune, uint32_t threads, int *blocks_per_sm);
 cudaError_t preload_kernels();
-cudaError_t launch_server(const ServerArgs &a, bool prune, uint32_t ctas, uint32_t threads,
-                          uint32_t smem_bytes, cudaStream_t st);
+cudaError_t launch_server(const ServerArgs &a, bool prune, uint32_t ctas, uint32_t threads, int sms,
+                          cudaStream_t st);
 
 }  // namespace gwfa
 
@@ -233,5 +236,6 @@ struct gwfa_engine {
     unsigned long long *stats = nullptr;
     uint32_t *paths = nullptr, *path_len = nullptr;
     uint32_t path_cap = 0;
+    int sms = 0;
     std::mutex mu;
 };

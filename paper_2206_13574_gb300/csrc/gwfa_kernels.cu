@@ -62,6 +62,7 @@ constexpr int kAbsent = -2;                  // exact mode: offset -1, not in Q
 // beyond them use a stamp in global memory.  4 KB per parity and CTA.
 constexpr uint32_t kBitTiles = 32768;
 constexpr uint32_t kSmall = 64;   // spill-list entries kept in shared memory
+constexpr uint32_t kLink = 128;   // neighbours to be linked, a score's list in shared memory
 
 template <bool P> struct VT;
 template <> struct VT<false> { using T = int; };
@@ -77,7 +78,7 @@ template <bool P> struct Slab {
     TabEnt *table;
     RecT<typename VT<P>::T> *recs;
     uint32_t *touched, *stamp;
-    uint2 *list[2], *req;
+    uint2 *list[2], *req, *links;
     unsigned long long *tkey;   // the rest: pruning mode only
     uint32_t *freel, *reqt;
     int4 *req4;
@@ -98,6 +99,7 @@ __device__ __forceinline__ Slab<P> carve(uint8_t *base, uint32_t log2cap) {
     s.list[0] = (uint2 *)(base + L.list0);
     s.list[1] = (uint2 *)(base + L.list1);
     s.req = (uint2 *)(base + L.req);
+    s.links = (uint2 *)(base + L.links);
     s.tkey = (unsigned long long *)(base + L.tkey);
     s.freel = (uint32_t *)(base + L.freel);
     s.reqt = (uint32_t *)(base + L.reqt);
@@ -118,6 +120,7 @@ struct Score {
     uint32_t cells, spills, visited, pruned;
     uint32_t amax;      // largest i + W~ (fits: i < 2^31, W~ < 2^31)
     int found, err;
+    uint32_t nlink;     // neighbours to be linked after the pass
     int err_next;       // out of room for a tile that only the next score needs
 };
 
@@ -140,6 +143,7 @@ struct Sh {
     // the first entries of the score's spill lists: exact mode 2 x kSmall requests (v, ku),
     // pruning mode kSmall requests, then kSmall insertions
     uint4 small[2 * kSmall];
+    uint2 link[kLink];            // (record | side << 31, vertex)
     uint32_t bits[2][kBitTiles / 32];
 };
 
@@ -156,10 +160,9 @@ __device__ __forceinline__ uint32_t window16(const uint32_t *__restrict__ w, uin
 }
 
 struct QCtx {
-    const uint32_t *qw;   // this query's packed words (global, or staged in shared memory)
+    const uint32_t *qw;   // this query's packed words
     int n;
     uint32_t ve;
-    bool smem;            // qw points to shared memory (server kernel)
     bool free_end;        // the walk may end at any position of v_e (or anywhere: any_v)
     bool any_v;           // no end vertex
 };
@@ -173,19 +176,11 @@ __device__ __forceinline__ bool at_end(const QCtx &q, uint32_t v, int k, int j, 
     return v == q.ve && (q.free_end || (uint32_t)j == lv);
 }
 
-// 16 query bases from position p: read-only cache for a batch staged before the
-// launch, plain (shared-memory) loads for a query the CTA staged itself.
+// 16 query bases from position p.  Plain loads: the server kernel's CTAs write the words
+// of their request themselves.
 __device__ __forceinline__ uint32_t qwin(const QCtx &q, uint32_t p) {
     const uint32_t *a = q.qw + (p >> 4);
-    uint32_t lo, hi;
-    if (q.smem) {
-        lo = a[0];
-        hi = a[1];
-    } else {
-        lo = __ldg(a);
-        hi = __ldg(a + 1);
-    }
-    return __funnelshift_r(lo, hi, (p & 15) * 2);
+    return __funnelshift_r(a[0], a[1], (p & 15) * 2);
 }
 
 // LCP(q[i+1..|q|], v[j+1..|v|]) of Eq. 2 in 0-based positions: XOR of 16-base
@@ -321,12 +316,25 @@ __device__ __noinline__ uint32_t link_neighbour(const Slab<P> &s, Sh &sh, uint32
     return (uint32_t)t;
 }
 
+// Leave the candidate that an edge diagonal at offset j sends over side sd of its tile
+// with the neighbour tile t, for score d + 1.
+template <bool P>
+__device__ __forceinline__ void leave_border(const Slab<P> &s, uint32_t t, int sd, int j, uint32_t base, int d,
+                                             uint32_t tr, bool traceback) {
+    const int c = sd ? j : j + 1;   // (k+1, j) to the right, (k-1, j+1) to the left
+    if constexpr (P) {
+        s.recs[t].side[sd ^ 1].in[(d + 1) & 1] = ((long long)c << 32) | base;
+        if (traceback) s.trec[t].in[sd ^ 1][(d + 1) & 1] = tr;
+    } else {
+        s.recs[t].side[sd ^ 1].in[(d + 1) & 1] = c;
+    }
+}
+
 // What a diagonal extended outside its tile's visit (a spilled one) owes the next score:
 // its tile listed, and its candidate over the tile's edge handed to the neighbour tile.
 template <bool P>
 __device__ void enter_next(const Slab<P> &s, Sh &sh, const QCtx &q, uint32_t idx, uint32_t v, int k, int j,
                            uint32_t base, uint32_t lv, int d, uint32_t tr, bool traceback) {
-    Score &S = sh.score[d & 3];
     uint32_t *nq = &sh.score[(d + 1) & 3].nq;
     uint2 *next = s.list[(d + 1) & 1];
     if (list_once<P>(s, sh, idx, d)) next[atomicAdd(nq, 1u)] = make_uint2(idx, v);
@@ -334,16 +342,33 @@ __device__ void enter_next(const Slab<P> &s, Sh &sh, const QCtx &q, uint32_t idx
     const int sd = ln == 7;
     if ((ln == 0 && (uint32_t)j < lv) || (ln == 7 && k + j < q.n)) {
         uint32_t t = s.recs[idx].side[sd].link;
-        if (t == kNone) t = link_neighbour<P>(s, sh, idx, v, k >> 3, sd, &S.err_next);
+        if (t == kNone) t = link_neighbour<P>(s, sh, idx, v, k >> 3, sd, &sh.score[d & 3].err_next);
         if (t == kNone) return;
-        const int c = sd ? j : j + 1;
-        if constexpr (P) {
-            s.recs[t].side[sd ^ 1].in[(d + 1) & 1] = ((long long)c << 32) | base;
-            if (traceback) s.trec[t].in[sd ^ 1][(d + 1) & 1] = tr;
-        } else {
-            s.recs[t].side[sd ^ 1].in[(d + 1) & 1] = c;
-        }
+        leave_border<P>(s, t, sd, j, base, d, tr, traceback);
         if (list_once<P>(s, sh, t, d)) next[atomicAdd(nq, 1u)] = make_uint2(t, v);
+    }
+}
+
+// The border words of the pass whose neighbour had no link yet, one thread each, from the
+// CTA's last threads down (the spills, done in the same step, start with its first): a
+// hash lookup, often with a claim, is two dependent L2 round trips and more, and in the
+// pass it would hold up the warp's other tiles.
+template <bool P>
+__device__ __forceinline__ void link_pending(const Slab<P> &s, Sh &sh, int d, uint32_t n, bool traceback) {
+    uint32_t *nq = &sh.score[(d + 1) & 3].nq;
+    for (uint32_t i = blockDim.x - 1 - threadIdx.x; i < n; i += blockDim.x) {
+        const uint2 rq = i < kLink ? sh.link[i] : s.links[i];
+        const uint32_t idx = rq.x & 0x7FFFFFFFu;
+        const int sd = (int)(rq.x >> 31), ln = sd ? 7 : 0;
+        const uint32_t t = link_neighbour<P>(s, sh, idx, rq.y, s.recs[idx].side[0].kb, sd, &sh.score[d & 3].err_next);
+        if (t == kNone) continue;
+        if constexpr (P) {
+            const long long v = s.recs[idx].vals[ln];
+            leave_border<P>(s, t, sd, pj(v), pbase(v), d, traceback ? s.trec[idx].tr[ln] : 0u, traceback);
+        } else {
+            leave_border<P>(s, t, sd, s.recs[idx].vals[ln] >> 1, 0u, d, 0u, false);
+        }
+        if (list_once<P>(s, sh, t, d)) s.list[(d + 1) & 1][atomicAdd(nq, 1u)] = make_uint2(t, rq.y);
     }
 }
 
@@ -389,189 +414,246 @@ __device__ __forceinline__ void request_spill(const Slab<true> &s, Sh &sh, uint3
     }
 }
 
+// LCP of two diagonals of one vertex, their first windows loaded together; a diagonal
+// with m = 0 is not extended (its positions are 0, so that the loads stay in bounds).
+__device__ __forceinline__ void lcp2(const QCtx &q, const uint32_t *__restrict__ vw, const int (&i)[2],
+                                     const int (&j)[2], const int (&m)[2], int (&l)[2]) {
+    uint32_t x[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) x[u] = qwin(q, (uint32_t)i[u]) ^ window16(vw, (uint32_t)j[u]);
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+        l[u] = x[u] ? (__ffs(x[u]) - 1) >> 1 : 16;
+        if (!x[u] && m[u] > 16) {
+            do {
+                const uint32_t y = qwin(q, (uint32_t)(i[u] + l[u])) ^ window16(vw, (uint32_t)(j[u] + l[u]));
+                if (y) {
+                    l[u] += (__ffs(y) - 1) >> 1;
+                    break;
+                }
+                l[u] += 16;
+            } while (l[u] < m[u]);
+        }
+        l[u] = min(l[u], m[u]);
+    }
+}
+
 // GwfExpand (Alg. 3) of the score before with GwfPrune (Alg. 4) on its sources, and
-// GwfExtend (Alg. 2) of this one, in one visit of every listed tile by an 8-lane group:
-// each lane gathers its diagonal's candidates (its own and its neighbours' by shuffle, the
-// edge lanes' from the tile's border words), keeps the largest if it beats its offset,
-// extends it along equal bases, stores it, and hands the next score its list entry and the
-// candidates that leave the tile.  Arc spills are only requested here.
+// GwfExtend (Alg. 2) of this one, in one visit of every listed tile by four lanes with two
+// diagonals each: a lane gathers its diagonals' candidates (their own and their
+// neighbours', by shuffle from the next lanes, from the tile's border words at its edges),
+// keeps the largest where it beats the offset, extends those along equal bases, stores
+// them, and hands the next score the tile's list entry and the candidates that leave the
+// tile.  Arc spills, and neighbours met for the first time, are only requested here.
+// The work around the two comparisons of a lane (entry, record, flags, lists) is most of
+// its instructions, so eight tiles share them in a warp.
 template <bool P, bool TB>
 __device__ __forceinline__ void offset_pass(const DevGraph &g, const Slab<P> &s, Sh &sh, const QCtx &q, int d,
                                             bool prune_on, int max_lag) {
     using T = typename VT<P>::T;
     const unsigned full = 0xFFFFFFFFu;
-    const int lane = threadIdx.x & 31, ln = lane & 7;
+    const int lane = threadIdx.x & 31, sub = lane & 3;
     const int par = d & 1;
     Score &S = sh.score[d & 3];
     uint32_t *nq = &sh.score[(d + 1) & 3].nq;
     const uint32_t n_list = S.nq;
-    const uint2 *list = s.list[par];
-    uint2 *next = s.list[par ^ 1];
-    const int sd = ln >> 2;   // the side whose border words this lane reads (lanes 0 and 7 use them)
+    const int sd = sub >> 1;   // the side whose border words this lane reads (lanes 0 and 3 use them)
     uint32_t cells = 0, visited = 0, pruned = 0, amax = 0;
     // the flags of the list being read are spent: clear them for score d + 1
     const uint32_t nw = min((sh.nt + 31) >> 5, kBitTiles / 32);
     for (uint32_t w = threadIdx.x; w < nw; w += blockDim.x) sh.bits[par][w] = 0u;
-    for (uint32_t wb = (threadIdx.x >> 5) * 4; wb < n_list; wb += (blockDim.x >> 5) * 4) {
-        const uint32_t e = wb + (lane >> 3);
+    for (uint32_t wb = (threadIdx.x >> 5) * 8; wb < n_list; wb += (blockDim.x >> 5) * 8) {
+        const uint32_t e = wb + (lane >> 2);
         const bool on = e < n_list;
-        const uint2 ent = list[on ? e : wb];
+        const uint2 ent = s.list[par][on ? e : wb];
         RecT<T> *rec = &s.recs[ent.x];
-        T raw = rec->vals[ln];
         const uint2 vi = __ldg((const uint2 *)&g.vinfo[ent.y]);   // label word, |v|
-        T in;
+        T raw[2], in;
         uint32_t link, counted = 0;
-        int k;
+        int k[2];
         if constexpr (P) {
+            const longlong2 r2 = *(const longlong2 *)&rec->vals[2 * sub];
+            raw[0] = r2.x;
+            raw[1] = r2.y;
             in = rec->side[sd].in[par];
             const uint4 lk = *(const uint4 *)&rec->side[sd].link;
             link = lk.x;
+            k[0] = (int)lk.y * kTile + 2 * sub;
             counted = lk.z;
-            k = (int)lk.y * kTile + ln;
         } else {
+            const int2 r2 = *(const int2 *)&rec->vals[2 * sub];
+            raw[0] = r2.x;
+            raw[1] = r2.y;
             const int4 sw = *(const int4 *)&rec->side[sd];
             in = par ? sw.y : sw.x;
             link = (uint32_t)sw.z;
-            k = sw.w * kTile + ln;
+            k[0] = sw.w * kTile + 2 * sub;
         }
-        uint32_t tr = 0, tin = 0;
+        k[1] = k[0] + 1;
+        uint32_t tr[2] = {0u, 0u}, trn[2] = {0u, 0u}, tin = 0u;
         if constexpr (TB) {
-            tr = s.trec[ent.x].tr[ln];
+            const uint2 t2 = *(const uint2 *)&s.trec[ent.x].tr[2 * sub];
+            tr[0] = t2.x;
+            tr[1] = t2.y;
             tin = s.trec[ent.x].in[sd][par];
         }
-        const bool edge = on && (ln == 0 || ln == 7) && in >= 0;
-        if (!edge) in = (T)-1;
-        else rec->side[sd].in[par] = (T)-1;   // consumed
-        if (!on) raw = P ? (T)-1 : (T)kAbsent;
-        bool live;
-        int j;
-        uint32_t base = 0;
-        if constexpr (P) {
-            live = raw >= 0 && ((raw >> 30) & 3) == kTagLive;
-            j = pj(raw);
-            base = pbase(raw);
-        } else {
-            live = raw & 1;
-            j = raw >> 1;
+        if (on && (sub == 0 || sub == 3) && in >= 0) rec->side[sd].in[par] = (T)-1;   // consumed
+        else in = (T)-1;
+        if (!on) raw[0] = raw[1] = P ? (T)-1 : (T)kAbsent;
+        bool live[2], inq[2];
+        int j[2];
+        uint32_t base[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            base[u] = 0u;
+            if constexpr (P) {
+                live[u] = raw[u] >= 0 && ((raw[u] >> 30) & 3) == kTagLive;
+                j[u] = pj(raw[u]);
+                base[u] = pbase(raw[u]);
+            } else {
+                live[u] = raw[u] & 1;
+                j[u] = raw[u] >> 1;
+            }
         }
-        const bool was = live;
-        if constexpr (P) {
+        if (d == 0) {   // the start diagonals are in Q as they are
+            inq[0] = live[0];
+            inq[1] = live[1];
+            trn[0] = tr[0];
+            trn[1] = tr[1];
+        } else if constexpr (P) {
             if (prune_on) {
-                // a source that lags is dropped; its offset stays
+                // a source that lags is dropped (its offset stays)
                 const long long am = (long long)sh.score[(d + 3) & 3].amax;
-                if (live && am - ((long long)k + 2ll * j + base) >= (long long)max_lag) {
-                    live = false;
-                    ++pruned;
-                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u)
+                    if (live[u] && am - ((long long)k[u] + 2ll * j[u] + base[u]) >= (long long)max_lag) {
+                        live[u] = false;
+                        ++pruned;
+                    }
+                // and so is one over the edge: (k - 1, c) on the left, (k + 1, c - 1) on the right
                 if (in >= 0) {
-                    // the source over the edge: (k - 1, c) on the left, (k + 1, c - 1) on the right
-                    const long long c = pj(in);
-                    const long long a = (long long)k - 1 + 2 * c + pbase(in);
-                    if (am - a >= (long long)max_lag) in = -1;
+                    const long long a = (long long)(sub == 0 ? k[0] : k[1]) - 1 + 2ll * pj(in) + pbase(in);
+                    if (am - a >= (long long)max_lag) in = (T)-1;
                 }
+            }
+            long long c_ins[2], c_del[2], mis[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const bool ins = live[u] && k[u] + j[u] < q.n, del = live[u] && j[u] < (int)vi.y;
+                c_ins[u] = ins ? ((long long)j[u] << 32) | base[u] : -1ll;
+                c_del[u] = del ? ((long long)(j[u] + 1) << 32) | base[u] : -1ll;
+                mis[u] = ins ? c_del[u] : -1ll;
+            }
+            long long left = __shfl_up_sync(full, c_ins[1], 1, 4), right = __shfl_down_sync(full, c_del[0], 1, 4);
+            uint32_t tl = 0u, tn = 0u;
+            if constexpr (TB) {
+                tl = __shfl_up_sync(full, tr[1], 1, 4);
+                tn = __shfl_down_sync(full, tr[0], 1, 4);
+                if (sub == 0) tl = tin;
+                if (sub == 3) tn = tin;
+            }
+            if (sub == 0) left = in;
+            if (sub == 3) right = in;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const long long cl = u ? c_ins[0] : left, cr = u ? right : c_del[1];
+                long long c = mis[u];
+                if (cl > c) c = cl;
+                if (cr > c) c = cr;
+                inq[u] = c >= 0 && pj(c) > j[u];   // j = -1 where absent
+                if constexpr (TB) {
+                    // sources of equal offset and base are equally good predecessors: the
+                    // largest trace index, for a deterministic choice
+                    if (mis[u] == c) trn[u] = tr[u];
+                    if (cl == c) trn[u] = max(trn[u], u ? tr[0] : tl);
+                    if (cr == c) trn[u] = max(trn[u], u ? tn : tr[1]);
+                }
+                if (inq[u]) {
+                    if (raw[u] < 0) ++visited;
+                    j[u] = pj(c);
+                    base[u] = pbase(c);
+                }
+            }
+        } else {
+            int c_ins[2], c_del[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                c_ins[u] = live[u] && k[u] + j[u] < q.n ? j[u] : -1;
+                c_del[u] = live[u] && j[u] < (int)vi.y ? j[u] + 1 : -1;
+            }
+            int left = __shfl_up_sync(full, c_ins[1], 1, 4), right = __shfl_down_sync(full, c_del[0], 1, 4);
+            if (sub == 0) left = in;
+            if (sub == 3) right = in;
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int c = max(c_ins[u] >= 0 ? c_del[u] : -1, u ? max(c_ins[0], right) : max(left, c_del[1]));
+                inq[u] = c > j[u];
+                j[u] = max(c, j[u]);
             }
         }
-        // candidates of this diagonal's own source: (k+1, j), (k-1, j+1), (k, j+1)
-        const bool ins = live && k + j < q.n, del = live && j < (int)vi.y;
-        bool inq;
-        int jn;         // the new offset
-        uint32_t trn = 0;
+        {
+            int i[2], jj[2], m[2], l[2];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                i[u] = inq[u] ? k[u] + j[u] : 0;
+                jj[u] = inq[u] ? j[u] : 0;
+                m[u] = inq[u] ? min(q.n - i[u], (int)vi.y - j[u]) : 0;
+            }
+            lcp2(q, g.words + vi.x, i, jj, m, l);
+            j[0] += l[0];
+            j[1] += l[1];
+        }
         if constexpr (P) {
-            const long long bb = (long long)base;
-            const long long c_ins = ins ? ((long long)j << 32) | bb : -1ll;
-            const long long c_del = del ? ((long long)(j + 1) << 32) | bb : -1ll;
-            long long left = __shfl_up_sync(full, c_ins, 1, 8), right = __shfl_down_sync(full, c_del, 1, 8);
-            uint32_t tl = 0, trr = 0;
-            if constexpr (TB) {
-                tl = __shfl_up_sync(full, tr, 1, 8);
-                trr = __shfl_down_sync(full, tr, 1, 8);
-                if (ln == 0) tl = tin;
-                if (ln == 7) trr = tin;
-            }
-            if (ln == 0) left = in;
-            if (ln == 7) right = in;
-            const long long mis = ins && del ? c_del : -1ll;
-            long long c = mis;
-            if (left > c) c = left;
-            if (right > c) c = right;
-            if constexpr (TB) {
-                // sources of equal offset and base are equally good predecessors: the
-                // largest trace index, for a deterministic choice
-                if (mis == c) trn = tr;
-                if (left == c) trn = max(trn, tl);
-                if (right == c) trn = max(trn, trr);
-            }
-            inq = d == 0 ? was : pj(c) > (raw < 0 ? -1 : j);
-            if (c < 0 && d) inq = false;
-            if (d == 0) c = ((long long)j << 32) | bb, trn = tr;
-            jn = inq ? pj(c) : j;
-            if (inq) base = pbase(c);
-            if (inq && raw < 0) ++visited;
             // a tile that holds a diagonal for the first time (claimed here or by a spill)
-            const unsigned has = __ballot_sync(full, inq || raw >= 0);
-            if (ln == 7 && !counted && on && ((has >> (lane & 24)) & 0xFFu)) {
+            const unsigned has = __ballot_sync(full, inq[0] || inq[1] || raw[0] >= 0 || raw[1] >= 0);
+            if (sub == 3 && !counted && on && ((has >> (lane & 28)) & 15u)) {
                 rec->side[1].counted = 1u;
                 count_claim<P>(s, sh, &S.err);
             }
+            if (on) {
+                longlong2 r2;
+                r2.x = inq[0] || raw[0] >= 0 ? pk(j[0], inq[0] ? kTagLive : kTagDead, base[0]) : -1ll;
+                r2.y = inq[1] || raw[1] >= 0 ? pk(j[1], inq[1] ? kTagLive : kTagDead, base[1]) : -1ll;
+                *(longlong2 *)&rec->vals[2 * sub] = r2;
+                if (TB) *(uint2 *)&s.trec[ent.x].tr[2 * sub] = make_uint2(inq[0] ? trn[0] : tr[0], inq[1] ? trn[1] : tr[1]);
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+                if (inq[u]) amax = max(amax, (uint32_t)(k[u] + j[u]) + (uint32_t)j[u] + base[u]);
         } else {
-            const int c_ins = ins ? j : -1, c_del = del ? j + 1 : -1;
-            int left = __shfl_up_sync(full, c_ins, 1, 8), right = __shfl_down_sync(full, c_del, 1, 8);
-            if (ln == 0) left = in;
-            if (ln == 7) right = in;
-            const int c = max(ins ? c_del : -1, max(left, right));
-            inq = d == 0 ? live : c > j;
-            jn = d == 0 ? j : max(c, j);
+            // right for every diagonal: an absent one keeps -2, one outside Q its offset
+            if (on) *(int2 *)&rec->vals[2 * sub] = make_int2((j[0] << 1) | (inq[0] ? 1 : 0), (j[1] << 1) | (inq[1] ? 1 : 0));
         }
-        if (inq) jn += lcp(q, k + jn, g.words + vi.x, jn, (int)vi.y);
-        const int i2 = k + jn;
-        if (inq || was) {
-            if constexpr (P) {
-                rec->vals[ln] = pk(jn, inq ? kTagLive : kTagDead, base);
-                if (TB && inq) s.trec[ent.x].tr[ln] = trn;
-            } else {
-                rec->vals[ln] = (jn << 1) | (inq ? 1 : 0);
+        bool spill[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            spill[u] = inq[u] && j[u] == (int)vi.y;
+            if (inq[u] && k[u] + j[u] == q.n && at_end(q, ent.y, k[u], j[u], vi.y)) {
+                S.found = 1;
+                // one 64-bit store, so that the vertex and its trace stay a pair when
+                // several diagonals reach a free end in the same score
+                if constexpr (P) sh.end_vp = ((unsigned long long)ent.y << 32) | trn[u];
             }
         }
-        if constexpr (P) {
-            if (inq) amax = max(amax, (uint32_t)i2 + (uint32_t)jn + base);
-        }
-        if (inq && i2 == q.n && at_end(q, ent.y, k, jn, vi.y)) {
-            S.found = 1;
-            // one 64-bit store, so that the vertex and its trace stay a pair when
-            // several diagonals reach a free end in the same score
-            if constexpr (P) sh.end_vp = ((unsigned long long)ent.y << 32) | trn;
-        }
-        const unsigned qm = __ballot_sync(full, inq);
-        cells += __popc(qm);
-        const bool spill = inq && jn == (int)vi.y;
-        const unsigned sp = __ballot_sync(full, spill);
-        if (sp) {
-            uint32_t b = 0;
-            if (lane == 0) b = atomicAdd(&S.nreq, (uint32_t)__popc(sp));
-            b = __shfl_sync(full, b, 0) + __popc(sp & ((1u << lane) - 1));
-            if (spill) {
-                if constexpr (P) {
-                    const uint4 f = __ldg(&g.vinfo[ent.y]);
-                    request_spill(s, sh, b, f, ent.y, k, base, trn, TB, &S.err);
-                } else {
-                    put_req(s, sh, b, ent.y, k + (int)vi.y, &S.err);
-                }
+        const unsigned qm0 = __ballot_sync(full, inq[0]), qm1 = __ballot_sync(full, inq[1]);
+        cells += __popc(qm0) + __popc(qm1);
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+            if (spill[u]) {
+                const uint32_t at = atomicAdd(&S.nreq, 1u);
+                if constexpr (P) request_spill(s, sh, at, __ldg(&g.vinfo[ent.y]), ent.y, k[u], base[u], trn[u], TB, &S.err);
+                else put_req(s, sh, at, ent.y, k[u] + (int)vi.y, &S.err);
             }
-        }
-        // the next score visits this tile if it has a diagonal in Q (lane 3 lists it), and
-        // a neighbour that an edge diagonal's candidate enters (lanes 0 and 7)
+        // the next score visits this tile if it has a diagonal in Q (lane 1 lists it), and
+        // a neighbour that an edge diagonal's candidate enters (lanes 0 and 3)
         uint32_t target = ent.x;
-        bool want = ln == 3 && ((qm >> (lane & 24)) & 0xFFu);
-        if (inq && ((ln == 0 && jn < (int)vi.y) || (ln == 7 && i2 < q.n))) {
-            if (link == kNone) link = link_neighbour<P>(s, sh, ent.x, ent.y, k >> 3, sd, &S.err_next);
-            if (link != kNone) {
-                const int c = sd ? jn : jn + 1;
-                if constexpr (P) {
-                    s.recs[link].side[sd ^ 1].in[par ^ 1] = ((long long)c << 32) | base;
-                    if (TB) s.trec[link].in[sd ^ 1][par ^ 1] = trn;
-                } else {
-                    s.recs[link].side[sd ^ 1].in[par ^ 1] = c;
-                }
+        bool want = sub == 1 && (((qm0 | qm1) >> (lane & 28)) & 15u);
+        if ((sub == 0 && inq[0] && j[0] < (int)vi.y) || (sub == 3 && inq[1] && k[1] + j[1] < q.n)) {
+            if (link == kNone) {
+                const uint32_t i = atomicAdd(&S.nlink, 1u);
+                *(i < kLink ? &sh.link[i] : &s.links[i]) = make_uint2(ent.x | ((uint32_t)sd << 31), ent.y);
+            } else {
+                leave_border<P>(s, link, sd, sd ? j[1] : j[0], sd ? base[1] : base[0], d, sd ? trn[1] : trn[0], TB);
                 target = link;
                 want = true;
             }
@@ -583,7 +665,7 @@ __device__ __forceinline__ void offset_pass(const DevGraph &g, const Slab<P> &s,
             uint32_t b = 0;
             if (lane == 0) b = atomicAdd(nq, (uint32_t)__popc(nm));
             b = __shfl_sync(full, b, 0) + __popc(nm & ((1u << lane) - 1));
-            if (fresh) next[b] = make_uint2(target, ent.y);
+            if (fresh) s.list[par ^ 1][b] = make_uint2(target, ent.y);
         }
     }
     if (lane == 0 && cells) atomicAdd(&S.cells, cells);
@@ -601,27 +683,27 @@ __device__ __forceinline__ void offset_pass(const DevGraph &g, const Slab<P> &s,
 
 // Exact mode: requests [r0, r0 + n) of the score's log: offset 0 to (u, ku) for every arc
 // (v, u) where it is absent (Alg. 2's arc loop).  A spill is a chain of dependent L2 round
-// trips (arc, hash entry, offset, label) and a score has a few dozen of them, so they are
-// spread over the warps, and in a warp over quads of lanes, one arc a lane.  A diagonal
-// that a lane inserts is extended by it at once; if that one reaches its vertex's end too,
-// its quad goes on with it (or it is logged for the next round when the lane has one
-// waiting already).
+// trips (arc, hash entry, offset, label) and a score has a few dozen of them: a pair of
+// lanes takes one, an arc a lane (most vertices have one or two).  Packed into few warps
+// they run in step: with 1, 2, 4 or 8 requests a warp (four lanes each) 10,000 reads take
+// 74.9, 59.6, 52.9 or 48.9 ms, with 16 46.9.  A diagonal that a lane inserts is extended by
+// it at once; if that one reaches its vertex's end too, its pair goes on with it (or it is
+// logged for the next round when the lane has one waiting already).
 __device__ __forceinline__ void spill_round(const DevGraph &g, const Slab<false> &s, Sh &sh, const QCtx &q, int d,
                                             uint32_t r0, uint32_t n, uint32_t *next_count) {
     Score &S = sh.score[d & 3];
     const unsigned full = 0xFFFFFFFFu;
-    const int lane = threadIdx.x & 31, arc = lane & 3;
-    const uint32_t nw = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, arc = lane & 1;
     uint32_t won = 0;
-    for (uint32_t b = threadIdx.x >> 5; b < n; b += 8 * nw) {
-        const uint32_t r = b + (uint32_t)(lane >> 2) * nw;
+    for (uint32_t b = (threadIdx.x >> 5) * 16; b < n; b += blockDim.x >> 1) {
+        const uint32_t r = b + (uint32_t)(lane >> 1);
         uint2 rq = r < n ? get_req(s, sh, r0 + r) : make_uint2(kNone, 0u);
         uint2 wait = make_uint2(kNone, 0u);   // this lane's inserted diagonal that spills in turn
         for (;;) {
             if (rq.x != kNone) {
                 const uint2 ar = __ldg((const uint2 *)&g.vinfo[rq.x].z);
                 const int ku = (int)rq.y;
-                for (uint32_t a = ar.x + arc; a < ar.y; a += 4) {
+                for (uint32_t a = ar.x + arc; a < ar.y; a += 2) {
                     const uint32_t u = __ldg(&g.arc_dst[a]);
                     const uint2 ui = __ldg((const uint2 *)&g.vinfo[u]);
                     const int su = find_or_insert<false>(s, sh, u, ku >> 3, &S.err);
@@ -641,10 +723,10 @@ __device__ __forceinline__ void spill_round(const DevGraph &g, const Slab<false>
             }
             const unsigned m = __ballot_sync(full, wait.x != kNone);
             if (!m) break;
-            const unsigned m4 = (m >> (lane & 28)) & 15u;
-            const int src = m4 ? __ffs(m4) - 1 : 0;
-            rq.x = __shfl_sync(full, wait.x, src, 4);
-            rq.y = __shfl_sync(full, wait.y, src, 4);
+            const unsigned m2 = (m >> (lane & 30)) & 3u;
+            const int src = m2 ? __ffs(m2) - 1 : 0;
+            rq.x = __shfl_sync(full, wait.x, src, 2);
+            rq.y = __shfl_sync(full, wait.y, src, 2);
             if (arc == src) wait.x = kNone;
         }
     }
@@ -827,7 +909,6 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
     QCtx q;
     q.n = (int)(A.q_off[qid + 1] - qo);
     q.qw = A.qwords + (qo >> 4) + qid;
-    q.smem = A.q_smem != 0;
     const uint32_t vs = A.v_s[qid];
     q.ve = A.v_e[qid];
     int pre = 0;
@@ -939,6 +1020,8 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         }
         // ---- arc spills, in rounds until no extended diagonal reaches its vertex's end
         uint32_t n = S.nreq;
+        const uint32_t nl = S.nlink;
+        if (nl) link_pending<P>(s, sh, d, nl, A.traceback != 0);
         if constexpr (P) {
             // few requests (the usual case): one warp does every round by itself, and the
             // others wait once instead of twice or three times a round
@@ -948,7 +1031,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
                 if (solo) __syncwarp();
                 else __syncthreads();
             };
-            const bool any = n > 0;
+            const bool any = n > 0 || nl > 0;
             if (!solo || threadIdx.x < 32) {
                 for (int round = 0; n; ++round) {
                     uint32_t *next_count = &sh.nr[round % 3], *n_ins = &sh.nins[round & 1];
@@ -981,6 +1064,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
                 n = min(n, r0 < 4 * s.cap ? 4 * s.cap - r0 : 0u);
                 if (A.stats && threadIdx.x == 0 && n) sh.st[2] += 1;
             }
+            if (nl && !r0) __syncthreads();
         }
         if (threadIdx.x == 0) {
             sh.cells += S.cells;
@@ -1077,20 +1161,19 @@ __device__ __forceinline__ void align_queries(const TierArgs &A) {
     }
 }
 
-// Up to 512 threads: the throughput shape.  Exact mode 4 CTAs per SM at 32 registers
-// (10,000 reads 59.8 ms; 3 CTAs at 40 registers 79 ms before the spills were spread over
-// the warps).  Pruning mode 3 at 40: its 64-bit offsets spill at 32 (388 bytes of spill
-// stores), and its frontiers are small (400 pruned 50 kb reads 34.5 ms at 4 CTAs, 28.2 ms
-// at 3; traceback of 800 reads with its CIGARs 14.2 and 12.5 ms).
+// Up to kNarrow threads: the throughput shape, 5 CTAs per SM at 48 registers (10,000 reads
+// of 1-20 kb: 48.9 ms, against 55 at 4 with 64, 54 at 6 with 40 and 52 at three CTAs of
+// 512 threads); pruning mode, with 64-bit offsets, 4 at 64 (400 pruned 50 kb reads 24.7 ms,
+// 25.9 at 5 with 48, 28 for eight CTAs of 128).
 template <bool P>
-__global__ void __launch_bounds__(512, P ? 3 : 4) align_kernel(TierArgs A) {
+__global__ void __launch_bounds__(kNarrow, P ? 4 : 5) align_kernel(TierArgs A) {
     align_queries<P>(A);
 }
 
-// 1024 threads: twice the groups on one query, for the few heaviest queries whose own
-// latency bounds a batch.  Registers as above: 2 CTAs per SM at 32, 1 at 64.
+// Up to 1024 threads, 64 registers: more groups on one query, for batches and queries
+// whose own latency is the bound.
 template <bool P>
-__global__ void __launch_bounds__(1024, P ? 1 : 2) align_kernel_wide(TierArgs A) {
+__global__ void __launch_bounds__(1024, 1) align_kernel_wide(TierArgs A) {
     align_queries<P>(A);
 }
 
@@ -1112,9 +1195,11 @@ __device__ __forceinline__ void st_release_sys(unsigned long long *p, unsigned l
 // vote if work comes); the CTAs leave together once every CTA has voted, or after
 // 16 x wait_limit polls in any case, and the host relaunches the kernel when work
 // comes.  Leaving together keeps the full set of CTAs whenever the kernel runs.
-template <bool P>
-__global__ void __launch_bounds__(512, 4) server_kernel(ServerArgs S) {
-    extern __shared__ uint32_t qsm[];   // the request's packed words, staged
+// CTAs per SM are a template parameter: all CTAs must be resident, and with fewer of them
+// a thread has more registers (64, 40 or 32 at 2, 3 or 4).
+template <bool P, int PerSm>
+__global__ void __launch_bounds__(512, PerSm) server_kernel(ServerArgs S) {
+    uint32_t *const qst = S.stage + (uint64_t)blockIdx.x * S.slot_words;   // the request's packed words
     __shared__ Sh sh;
     __shared__ unsigned long long s_ticket;
     __shared__ uint64_t s_qoff[2];
@@ -1179,7 +1264,7 @@ __global__ void __launch_bounds__(512, 4) server_kernel(ServerArgs S) {
         const uint32_t n = __ldcv(&d->n);
         const uint32_t nw = (n + 15) >> 4;
         const uint32_t *src = S.arena[rc] + (uint64_t)slot * S.slot_words;
-        for (uint32_t w = threadIdx.x; w < nw + 2; w += blockDim.x) qsm[w] = w < nw ? __ldcv(src + w) : 0u;
+        for (uint32_t w = threadIdx.x; w < nw + 2; w += blockDim.x) qst[w] = w < nw ? __ldcv(src + w) : 0u;
         if (threadIdx.x == 0) {
             s_qoff[0] = 0;
             s_qoff[1] = n;
@@ -1189,8 +1274,7 @@ __global__ void __launch_bounds__(512, 4) server_kernel(ServerArgs S) {
         __syncthreads();
         TierArgs A{};
         A.g = S.g;
-        A.qwords = qsm;
-        A.q_smem = 1;
+        A.qwords = qst;
         A.q_off = s_qoff;
         A.v_s = &s_vs;
         A.v_e = &s_ve;
@@ -1262,7 +1346,7 @@ __global__ void slab_init_kernel(uint8_t *slabs, uint64_t slab_bytes, uint32_t n
 
 cudaError_t launch_align(const TierArgs &a, bool prune, uint32_t ctas, uint32_t threads,
                          cudaStream_t st) {
-    if (threads > 512) {
+    if (threads > kNarrow) {
         if (prune) align_kernel_wide<true><<<ctas, threads, 0, st>>>(a);
         else align_kernel_wide<false><<<ctas, threads, 0, st>>>(a);
     } else {
@@ -1272,15 +1356,14 @@ cudaError_t launch_align(const TierArgs &a, bool prune, uint32_t ctas, uint32_t 
     return cudaGetLastError();
 }
 
-cudaError_t launch_server(const ServerArgs &a, bool prune, uint32_t ctas, uint32_t threads,
-                          uint32_t smem_bytes, cudaStream_t st) {
-    if (prune) {
-        cudaFuncSetAttribute(server_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-        server_kernel<true><<<ctas, threads, smem_bytes, st>>>(a);
-    } else {
-        cudaFuncSetAttribute(server_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes);
-        server_kernel<false><<<ctas, threads, smem_bytes, st>>>(a);
-    }
+cudaError_t launch_server(const ServerArgs &a, bool prune, uint32_t ctas, uint32_t threads, int sms,
+                          cudaStream_t st) {
+    // the fewest CTAs per SM that hold them all (above 4 per SM narrower ones still fit)
+    const uint32_t per_sm = (ctas + (uint32_t)sms - 1) / (uint32_t)sms;
+    void (*k)(ServerArgs) = per_sm <= 2 ? (prune ? server_kernel<true, 2> : server_kernel<false, 2>)
+                            : per_sm == 3 ? (prune ? server_kernel<true, 3> : server_kernel<false, 3>)
+                                          : (prune ? server_kernel<true, 4> : server_kernel<false, 4>);
+    k<<<ctas, threads, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -1318,10 +1401,9 @@ cudaError_t preload_kernels() {
 }
 
 int align_occupancy(bool prune, uint32_t threads, int *blocks_per_sm) {
-    cudaError_t e = prune
-        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, align_kernel<true>, (int)threads, 0)
-        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, align_kernel<false>, (int)threads, 0);
-    return e == cudaSuccess ? 0 : -1;
+    void (*k)(TierArgs) = threads > kNarrow ? (prune ? align_kernel_wide<true> : align_kernel_wide<false>)
+                                            : (prune ? align_kernel<true> : align_kernel<false>);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, (int)threads, 0) == cudaSuccess ? 0 : -1;
 }
 
 }  // namespace gwfa

@@ -127,5 +127,6 @@ extern "C" int gwfa_align_noalloc(const gwfa_graph *g, uint32_t n_queries, const
     a.log2cap = log2_tiles;
     a.max_lag = o.max_lag;
     a.max_score = o.max_score;
-    return gwfa::launch_align(a, prune, ctas, 512, s) == cudaSuccess ? GWFA_OK : GWFA_ERR_CUDA;
+    // a handful of CTAs: as wide as their frontiers are worth
+    return gwfa::launch_align(a, prune, ctas, prune ? 256 : 1024, s) == cudaSuccess ? GWFA_OK : GWFA_ERR_CUDA;
 }

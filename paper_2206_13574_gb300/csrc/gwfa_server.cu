@@ -59,7 +59,9 @@ struct gwfa_server {
     unsigned long long *d_head = nullptr, *d_timeouts = nullptr;
     unsigned int *d_votes = nullptr;
     gwfa::ServerArgs args{};
-    uint32_t slot_words = 0, smem_bytes = 0;
+    uint32_t slot_words = 0;
+    uint32_t *stage = nullptr;
+    int sms = 1;
     cudaStream_t stream = nullptr;
     bool launched = false;
     std::mutex mu;
@@ -89,7 +91,7 @@ int ensure_running(gwfa_server *sv) {
     const uint32_t ctas = sv->cfg.ctas_small + sv->cfg.ctas_big;
     // a new generation of CTAs starts with no idle votes (stream-ordered after the last)
     int st = sstat(cudaMemsetAsync(sv->d_votes, 0, sizeof(unsigned int), sv->stream));
-    if (!st) st = sstat(gwfa::launch_server(sv->args, sv->prune, ctas, sv->cfg.threads, sv->smem_bytes, sv->stream));
+    if (!st) st = sstat(gwfa::launch_server(sv->args, sv->prune, ctas, sv->cfg.threads, sv->sms, sv->stream));
     if (!st) {
         sv->launched = true;
         sv->n_launches++;
@@ -181,7 +183,7 @@ int gwfa_server_create(const gwfa_graph *g, const gwfa_server_config *cfg, const
     sv->opts = o;
     sv->prune = o.max_lag > 0;
     sv->slot_words = (c.max_query_len + 15) / 16 + 2;
-    sv->smem_bytes = sv->slot_words * 4 + 16;
+    if (cudaDeviceGetAttribute(&sv->sms, cudaDevAttrMultiProcessorCount, g->device) != cudaSuccess) sv->sms = 1;
     sv->busy[0].assign(c.ring_slots, 0);
     sv->busy[1].assign(c.ring_slots, 0);
     // device slabs: class 0 then class 1
@@ -190,6 +192,7 @@ int gwfa_server_create(const gwfa_graph *g, const gwfa_server_config *cfg, const
     sv->big_offset = sv->slab_bytes[0] * c.ctas_small;
     const uint64_t slab_total = sv->big_offset + sv->slab_bytes[1] * c.ctas_big;
     st = sstat(cudaMalloc(&sv->slabs, slab_total));
+    if (!st) st = sstat(cudaMalloc(&sv->stage, (uint64_t)sv->slot_words * 4 * (c.ctas_small + c.ctas_big)));
     if (!st) st = sstat(cudaStreamCreateWithFlags(&sv->stream, cudaStreamNonBlocking));
     if (!st)
         st = sstat(gwfa::launch_slab_init(sv->slabs, sv->slab_bytes[0], c.ctas_small, c.log2_small, sv->prune,
@@ -259,6 +262,7 @@ int gwfa_server_create(const gwfa_graph *g, const gwfa_server_config *cfg, const
     a.n_ctas = c.ctas_small + c.ctas_big;
     a.ring = c.ring_slots;
     a.slot_words = sv->slot_words;
+    a.stage = sv->stage;
     a.sleep_ns = 2000;
     a.wait_limit = std::max<uint32_t>(c.idle_us / 2, 1);
     a.max_lag = o.max_lag;
@@ -385,6 +389,7 @@ int gwfa_server_destroy(gwfa_server *sv) {
         cudaStreamDestroy(sv->stream);
     }
     cudaFree(sv->slabs);
+    cudaFree(sv->stage);
     cudaFree(sv->d_head);
     cudaFree(sv->d_timeouts);
     cudaFree(sv->d_votes);
