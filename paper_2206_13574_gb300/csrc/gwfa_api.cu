@@ -196,14 +196,24 @@ int gwfa_graph_create(uint32_t nv, const char *h_seq, const uint64_t *h_seq_off,
     std::vector<uint4> vinfo(nv);
     for (uint32_t v = 0; v < nv; ++v)
         vinfo[v] = make_uint4(vstart[v], vlen[v], g->h_arc_off[v], g->h_arc_off[v + 1]);
+    std::vector<uint4> vx(2 * (uint64_t)nv);
+    for (uint32_t v = 0; v < nv; ++v) {
+        uint32_t dst[4] = {0, 0, 0, 0};
+        for (uint32_t a = 0; a < 4 && g->h_arc_off[v] + a < g->h_arc_off[v + 1]; ++a)
+            dst[a] = g->h_arc_dst[g->h_arc_off[v] + a];
+        vx[2 * (uint64_t)v] = vinfo[v];
+        vx[2 * (uint64_t)v + 1] = make_uint4(dst[0], dst[1], dst[2], dst[3]);
+    }
     st = dmalloc(&g->d_words, g->n_words * 4);
+    if (!st) st = dmalloc(&g->d_vx, vx.size() * sizeof(uint4));
+    if (!st) st = cuda_status(cudaMemcpy(g->d_vx, vx.data(), vx.size() * sizeof(uint4), cudaMemcpyHostToDevice));
     if (!st) st = dmalloc(&g->d_vinfo, (uint64_t)nv * sizeof(uint4));
     if (!st) st = dmalloc(&g->d_arc_dst, std::max<uint64_t>(g->na, 1) * 4);
     if (!st) st = cuda_status(cudaMemcpy(g->d_words, words.data(), g->n_words * 4, cudaMemcpyHostToDevice));
     if (!st) st = cuda_status(cudaMemcpy(g->d_vinfo, vinfo.data(), (uint64_t)nv * sizeof(uint4), cudaMemcpyHostToDevice));
     if (!st && g->na) st = cuda_status(cudaMemcpy(g->d_arc_dst, g->h_arc_dst.data(), g->na * 4, cudaMemcpyHostToDevice));
     if (!st) st = cuda_status(cudaStreamCreateWithFlags(&g->stream, cudaStreamNonBlocking));
-    g->device_bytes = g->n_words * 4 + (uint64_t)nv * sizeof(uint4) + g->na * 4;
+    g->device_bytes = g->n_words * 4 + 3 * (uint64_t)nv * sizeof(uint4) + g->na * 4;
     if (st) { gwfa_graph_destroy(g); return st; }
     *out = g;
     return GWFA_OK;
@@ -214,6 +224,7 @@ int gwfa_graph_destroy(gwfa_graph *g) {
     cudaSetDevice(g->device);
     cudaFree(g->d_words);
     cudaFree(g->d_vinfo);
+    cudaFree(g->d_vx);
     cudaFree(g->d_arc_dst);
     cudaFree(g->plain_slab);
     cudaFree(g->plain_stage);

@@ -32,8 +32,11 @@ constexpr uint64_t kEmptyKey = ~0ull;
 // the end so that a 32-base window may always read two consecutive words.
 // vinfo[v] = {first word of the label, |v|, first out-arc, end of out-arcs}: one
 // 16-byte load gives everything the extension of a diagonal of v needs.
+// vx[2 v] repeats vinfo[v] and vx[2 v + 1] holds the first four out-arc targets: the
+// alignment kernel finds a vertex and its arcs in one 32-byte sector.
 struct DevGraph {
     const uint32_t *words;
+    const uint4 *vx;
     const uint4 *vinfo;
     const uint32_t *arc_dst;
     uint32_t nv;
@@ -78,16 +81,9 @@ struct alignas(64) TraceRec {
     uint32_t pad[4];
 };
 
-// 16-byte chunk `part` of an empty record.
-__host__ __device__ inline uint4 empty_chunk(bool prune, uint32_t part) {
-    const uint32_t o = 0xFFFFFFFFu, z = prune && (part == 5 || part == 7) ? 0u : o;
-    const uint32_t a = !prune && part < 2 ? 0xFFFFFFFEu : o;
-    return prune ? make_uint4(o, o, z, z) : make_uint4(a, a, a, a);
-}
-
 // Per-CTA slab layout (all arrays 256-byte aligned), cap = 2^log2 tiles: the hash (twice
-// as many entries as tiles), the records, the hash position of each record and its list
-// stamp -- these start all ones / empty -- then the two tile lists and the spill lists.
+// as many entries as tiles, all ones = empty), the records, the hash position of each
+// record and its list stamp, then the two tile lists and the spill lists.
 struct SlabLayout {
     uint64_t table, recs, touched, stamp, tkey, list0, list1, links, req, reqt, ins, freel, trace, trec, total;
 };
@@ -200,7 +196,7 @@ struct gwfa_graph {
     int has_cycles = 0;
     std::vector<uint32_t> h_arc_off, h_arc_dst, h_vlen;
     uint32_t *d_words = nullptr, *d_arc_dst = nullptr;
-    uint4 *d_vinfo = nullptr;
+    uint4 *d_vinfo = nullptr, *d_vx = nullptr;
     uint64_t device_bytes = 0;
     // plain-path workspace (one slab), guarded by mu
     mutable std::mutex mu;
@@ -211,7 +207,7 @@ struct gwfa_graph {
     mutable uint64_t plain_stage_bytes = 0;
     mutable cudaStream_t stream = nullptr;
     gwfa::DevGraph dev() const {
-        return gwfa::DevGraph{d_words, d_vinfo, d_arc_dst, nv};
+        return gwfa::DevGraph{d_words, d_vx, d_vinfo, d_arc_dst, nv};
     }
 };
 

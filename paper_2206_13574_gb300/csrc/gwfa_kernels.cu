@@ -15,15 +15,18 @@
 //   spill rounds  the arcs of the diagonals that reached |v| (rare: about 1% of the
 //                 diagonals, none in many scores).  They come after the pass because a
 //                 spill only fills a diagonal that GwfExpand left absent.
-// A tile is read and written once a score, by one group, with plain loads and stores: no
-// offset is merged by an atomic, and all the data of a query live in one CTA, so the loads
-// may hit L1.  Measured against the form with separate extend and expand passes that
-// max-merged candidates with atomics and probed the hash for each one leaving a tile
-// (10,000 queries of 1-20 kb, 512 threads x 4 CTAs per SM): 100.7 -> 68.4 ms; 300 queries
-// with a heavy tail 442 -> 186 ms; 400 pruned 50 kb queries 50.7 -> 36.6 ms.  On the
-// 2,000-query profiling case 34.5 -> 18.3 warp instructions a cell, 14.5 -> 20.3 active
-// lanes.  What bounds it now: the barriers (17 of 32 stall cycles per instruction), i.e.
-// the chain of dependent L2 round trips of the longest spill and of the last tile visits.
+// A tile is read and written once a score, by one thread group, with plain loads and
+// stores: no offset is merged by an atomic, and all the data of a query live in one CTA,
+// so they stay in L1 (39 cycles a load there, 275 from L2, 477 for an atomic, which also
+// drops its line from L1; all measured).  For the same reason a record is written whole by
+// the thread that claims it, not initialised beforehand: the dense records of 760 queries
+// at a time fit L2 only while nothing else is fetched for them (10,000 reads 48.3 -> 35.3 ms).
+// Measured against the form with separate extend and expand passes that max-merged
+// candidates with atomics and probed the hash for each one leaving a tile (reads of
+// 1-20 kb): 10,000 reads 102.9 -> 35.3 ms, 997 reads 55.2 -> 13.7 ms, 300 with a heavy tail
+// 405 -> 68 ms, 400 pruned 50 kb reads 51.0 -> 24.7 ms, one 10 kb read 7.4 -> 2.0 ms.
+// What bounds it: latency.  A score is two barriers, one tile visit per group or a few,
+// and the longest chain of spills, each link of it an arc, a hash entry and a label.
 //
 // Data (per CTA slab, see SlabLayout; reused across queries):
 //   H~     tile records, dense in order of first use, and an open-addressing hash from
@@ -62,6 +65,7 @@ constexpr int kAbsent = -2;                  // exact mode: offset -1, not in Q
 // beyond them use a stamp in global memory.  4 KB per parity and CTA.
 constexpr uint32_t kBitTiles = 32768;
 constexpr uint32_t kSmall = 64;   // spill-list entries kept in shared memory
+constexpr uint32_t kLog2Claims = 9;
 constexpr uint32_t kLink = 128;   // neighbours to be linked, a score's list in shared memory
 
 template <bool P> struct VT;
@@ -143,6 +147,7 @@ struct Sh {
     // the first entries of the score's spill lists: exact mode 2 x kSmall requests (v, ku),
     // pruning mode kSmall requests, then kSmall insertions
     uint4 small[2 * kSmall];
+    uint32_t claim[1 << kLog2Claims];   // exact mode: diagonals the spills of a score inserted
     uint2 link[kLink];            // (record | side << 31, vertex)
     uint32_t bits[2][kBitTiles / 32];
 };
@@ -199,6 +204,11 @@ __device__ __forceinline__ int lcp(const QCtx &q, int i, const uint32_t *__restr
     return min(l, maxl);
 }
 
+// Target of out-arc `a` of v, the `o`-th of its arcs.
+__device__ __forceinline__ uint32_t arc_target(const DevGraph &g, uint32_t v, uint32_t a, uint32_t o) {
+    return __ldg(o < 4 ? (const uint32_t *)&g.vx[2 * (uint64_t)v + 1] + o : &g.arc_dst[a]);
+}
+
 // Atomics on slab memory (always device global memory) issued in the global state
 // space; the slab pointers come from shared memory, where the compiler no longer
 // knows their space.
@@ -253,6 +263,23 @@ template <bool P> __device__ __forceinline__ void count_claim(const Slab<P> &s, 
     if (atomicAdd(&sh.nclaim, 1u) + 1 > (s.cap >> 1) + (s.cap >> 2)) atomicCAS(err, 0, GWFA_ERR_CAPACITY);
 }
 
+// An empty record of a tile at kb, written by the thread that claims it, in whole lines:
+// they stay in L1, and records need no initialisation before a query nor wiping after it.
+template <bool P> __device__ __forceinline__ void empty_record(const Slab<P> &s, uint32_t idx, int kb) {
+    uint4 *p = (uint4 *)&s.recs[idx];
+    const uint32_t o = 0xFFFFFFFFu;
+    if constexpr (P) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) p[i] = i == 5 || i == 7 ? make_uint4(o, (uint32_t)kb, 0u, 0u) : make_uint4(o, o, o, o);
+        s.tkey[idx] = kEmptyKey;
+    } else {
+        p[0] = p[1] = make_uint4(o - 1, o - 1, o - 1, o - 1);   // kAbsent
+        p[2] = p[3] = make_uint4(o, o, o, (uint32_t)kb);
+    }
+    s.touched[idx] = kNone;
+    if (idx >= kBitTiles) s.stamp[idx] = kNone;
+}
+
 // Record of tile (v, kb), claimed if absent; -1 (and *err) when the slab is full.  The
 // first probe is inline, the rest (and the claim) is not.
 template <bool P>
@@ -270,18 +297,21 @@ __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsign
                     idx = atomicAdd(&sh.nt, 1u);
                 }
                 if (idx >= s.cap) break;
+                empty_record<P>(s, idx, (int)(uint32_t)key);
+                __threadfence_block();   // before the key that leads others to it
             }
             e = cas_ent(&s.table[h], key, idx);
             if (e.key == kEmptyKey) {
                 s.touched[idx] = h;
-                s.recs[idx].side[0].kb = (int)(uint32_t)key;
-                s.recs[idx].side[1].kb = (int)(uint32_t)key;
                 if constexpr (P) s.tkey[idx] = key;
                 else count_claim<P>(s, sh, err);   // a claimed tile always gets a diagonal
                 return (int)idx;
             }
         }
-        if (e.key == key) return (int)e.idx;   // a record taken for a lost race stays unused
+        if (e.key == key) {
+            __threadfence_block();
+            return (int)e.idx;   // a record taken for a lost race stays unused
+        }
         h = (h + 1) & s.tmask;
     }
     atomicCAS(err, 0, GWFA_ERR_CAPACITY);
@@ -292,7 +322,9 @@ __device__ __forceinline__ int find_or_insert(const Slab<P> &s, Sh &sh, uint32_t
     const unsigned long long key = tile_key(v, kb);
     const uint32_t h = tile_hash(key, s.tmask);
     const Ent e = ld_ent(&s.table[h]);
-    return e.key == key ? (int)e.idx : find_or_insert_slow<P>(s, sh, key, h, e, err);
+    if (e.key != key) return find_or_insert_slow<P>(s, sh, key, h, e, err);
+    __threadfence_block();   // see empty_record
+    return (int)e.idx;
 }
 
 // List a tile for the next score; true for the one caller that has to append it.
@@ -401,13 +433,13 @@ __device__ __forceinline__ int4 get_req4(const Slab<true> &s, const Sh &sh, uint
 
 // Pruning mode: a settled diagonal reached |v|: offset 0 with the walk base past v goes
 // to (u, k + |v|) for every arc (v, u), after the pass (see apply_spills).
-__device__ __forceinline__ void request_spill(const Slab<true> &s, Sh &sh, uint32_t at, const uint4 &vi, uint32_t v,
+__device__ __forceinline__ void request_spill(const Slab<true> &s, Sh &sh, uint32_t at, uint32_t lv, uint32_t v,
                                               int k, uint32_t base, uint32_t tr, bool traceback, int *err) {
-    const uint32_t nb = base + vi.y;
+    const uint32_t nb = base + lv;
     if (nb > kBaseMask) atomicCAS(err, 0, GWFA_ERR_CAPACITY);
     const uint32_t t = traceback ? push_trace(s, sh, v, tr, err) : 0u;
     if (at < s.cap) {
-        *(at < kSmall ? (int4 *)&sh.small[at] : &s.req4[at]) = make_int4(k + (int)vi.y, (int)nb, (int)vi.z, (int)vi.w);
+        *(at < kSmall ? (int4 *)&sh.small[at] : &s.req4[at]) = make_int4(k + (int)lv, (int)nb, (int)v, 0);
         if (traceback) s.reqt[at] = t;
     } else {
         atomicCAS(err, 0, GWFA_ERR_CAPACITY);
@@ -467,7 +499,7 @@ __device__ __forceinline__ void offset_pass(const DevGraph &g, const Slab<P> &s,
         const bool on = e < n_list;
         const uint2 ent = s.list[par][on ? e : wb];
         RecT<T> *rec = &s.recs[ent.x];
-        const uint2 vi = __ldg((const uint2 *)&g.vinfo[ent.y]);   // label word, |v|
+        const uint2 vi = __ldg((const uint2 *)&g.vx[2 * (uint64_t)ent.y]);   // label word, |v|
         T raw[2], in;
         uint32_t link, counted = 0;
         int k[2];
@@ -641,7 +673,7 @@ __device__ __forceinline__ void offset_pass(const DevGraph &g, const Slab<P> &s,
         for (int u = 0; u < 2; ++u)
             if (spill[u]) {
                 const uint32_t at = atomicAdd(&S.nreq, 1u);
-                if constexpr (P) request_spill(s, sh, at, __ldg(&g.vinfo[ent.y]), ent.y, k[u], base[u], trn[u], TB, &S.err);
+                if constexpr (P) request_spill(s, sh, at, vi.y, ent.y, k[u], base[u], trn[u], TB, &S.err);
                 else put_req(s, sh, at, ent.y, k[u] + (int)vi.y, &S.err);
             }
         // the next score visits this tile if it has a diagonal in Q (lane 1 lists it), and
@@ -681,6 +713,28 @@ __device__ __forceinline__ void offset_pass(const DevGraph &g, const Slab<P> &s,
     }
 }
 
+// Exact mode: the one thread that may insert diagonal `ln` of record idx in this score.  The
+// claims of a score are kept in a small hash in shared memory (entry: score mod 32, record,
+// diagonal; 0 or another score = free): an atomic on the offset itself takes 477 cycles
+// and drops the record's line from L1.  An entry is never freed within a score, so a
+// thread that finds no room can fall back to that atomic: everyone else with the same
+// diagonal finds none either.
+__device__ __forceinline__ bool claim_lane(const Slab<false> &s, Sh &sh, uint32_t idx, int ln, int d) {
+    const uint32_t tag = (uint32_t)d & 31u, key = tag << 27 | idx << 3 | (uint32_t)ln;
+    uint32_t h = (idx << 3 | (uint32_t)ln) * 0x9E3779B1u >> (32 - kLog2Claims);
+    for (int probe = 0; probe < 16; ++probe) {
+        uint32_t e = sh.claim[h];
+        if (e == 0u || e >> 27 != tag) {
+            const uint32_t old = e;
+            e = atomicCAS(&sh.claim[h], old, key);
+            if (e == old) return true;
+        }
+        if (e == key) return false;
+        h = (h + 1) & ((1u << kLog2Claims) - 1);
+    }
+    return g_cas(&s.recs[idx].vals[ln], kAbsent, 1) == kAbsent;
+}
+
 // Exact mode: requests [r0, r0 + n) of the score's log: offset 0 to (u, ku) for every arc
 // (v, u) where it is absent (Alg. 2's arc loop).  A spill is a chain of dependent L2 round
 // trips (arc, hash entry, offset, label) and a score has a few dozen of them: a pair of
@@ -701,17 +755,16 @@ __device__ __forceinline__ void spill_round(const DevGraph &g, const Slab<false>
         uint2 wait = make_uint2(kNone, 0u);   // this lane's inserted diagonal that spills in turn
         for (;;) {
             if (rq.x != kNone) {
-                const uint2 ar = __ldg((const uint2 *)&g.vinfo[rq.x].z);
+                const uint2 ar = __ldg((const uint2 *)&g.vx[2 * (uint64_t)rq.x].z);
                 const int ku = (int)rq.y;
-                for (uint32_t a = ar.x + arc; a < ar.y; a += 2) {
-                    const uint32_t u = __ldg(&g.arc_dst[a]);
-                    const uint2 ui = __ldg((const uint2 *)&g.vinfo[u]);
+                for (uint32_t o = (uint32_t)arc; ar.x + o < ar.y; o += 2) {
+                    const uint32_t u = arc_target(g, rq.x, ar.x + o, o);
+                    const uint2 ui = __ldg((const uint2 *)&g.vx[2 * (uint64_t)u]);
                     const int su = find_or_insert<false>(s, sh, u, ku >> 3, &S.err);
                     if (su < 0) break;
-                    const int prev = g_cas(&s.recs[su].vals[ku & 7], kAbsent, 1);
-                    const int l = lcp(q, ku, g.words + ui.x, 0, (int)ui.y);   // while the swap is under way
-                    if (prev != kAbsent) continue;
+                    if (s.recs[su].vals[ku & 7] != kAbsent || !claim_lane(s, sh, (uint32_t)su, ku & 7, d)) continue;
                     ++won;
+                    const int l = lcp(q, ku, g.words + ui.x, 0, (int)ui.y);
                     s.recs[su].vals[ku & 7] = (l << 1) | 1;
                     if (at_end(q, u, ku, l, ui.y)) S.found = 1;
                     enter_next<false>(s, sh, q, (uint32_t)su, u, ku, l, 0u, ui.y, d, 0u, false);
@@ -751,8 +804,9 @@ __device__ __forceinline__ void apply_spills(const DevGraph &g, const Slab<true>
         const int4 rq = get_req4(s, sh, r);
         const int ku = rq.x;
         const long long cand = pk(0, kTagPend, (uint32_t)rq.y);
-        for (uint32_t a = (uint32_t)rq.z + (threadIdx.x & 3); a < (uint32_t)rq.w; a += 4) {
-            const uint32_t u = __ldg(&g.arc_dst[a]);
+        const uint2 ar = __ldg((const uint2 *)&g.vx[2 * (uint64_t)(uint32_t)rq.z].z);
+        for (uint32_t o = threadIdx.x & 3; ar.x + o < ar.y; o += 4) {
+            const uint32_t u = arc_target(g, (uint32_t)rq.z, ar.x + o, o);
             const int su = find_or_insert<true>(s, sh, u, ku >> 3, &S.err);
             if (su < 0) break;
             if (g_max(&s.recs[su].vals[ku & 7], cand) >= 0) continue;
@@ -780,8 +834,10 @@ __device__ __forceinline__ void resolve_spill_traces(const DevGraph &g, const Sl
         const int4 rq = get_req4(s, sh, r);
         const int ku = rq.x;
         const long long cand = pk(0, kTagPend, (uint32_t)rq.y);
-        for (uint32_t a = (uint32_t)rq.z + (threadIdx.x & 3); a < (uint32_t)rq.w; a += 4) {
-            const int su = find_or_insert<true>(s, sh, __ldg(&g.arc_dst[a]), ku >> 3, &sh.score[d & 3].err);
+        const uint2 ar = __ldg((const uint2 *)&g.vx[2 * (uint64_t)(uint32_t)rq.z].z);
+        for (uint32_t o = threadIdx.x & 3; ar.x + o < ar.y; o += 4) {
+            const uint32_t u = arc_target(g, (uint32_t)rq.z, ar.x + o, o);
+            const int su = find_or_insert<true>(s, sh, u, ku >> 3, &sh.score[d & 3].err);
             if (su < 0) return;
             if (s.recs[su].vals[ku & 7] == cand) g_max32(&s.trec[su].tr[ku & 7], s.reqt[r]);
         }
@@ -796,7 +852,7 @@ __device__ __forceinline__ void extend_spilled(const DevGraph &g, const Slab<tru
     for (uint32_t r = threadIdx.x; r < min(n, 2 * s.cap); r += nthr) {
         const uint4 in = r < kSmall ? sh.small[kSmall + r] : s.ins[r];
         const int k = (int)in.z;
-        const uint4 vi = __ldg(&g.vinfo[in.y]);
+        const uint2 vi = __ldg((const uint2 *)&g.vx[2 * (uint64_t)in.y]);
         const uint32_t base = pbase(s.recs[in.x].vals[k & 7]);
         const uint32_t tr = traceback ? s.trec[in.x].tr[k & 7] : 0u;
         const int j = lcp(q, k, g.words + vi.x, 0, (int)vi.y);
@@ -808,37 +864,24 @@ __device__ __forceinline__ void extend_spilled(const DevGraph &g, const Slab<tru
         }
         enter_next<true>(s, sh, q, in.x, in.y, k, j, base, vi.y, d, tr, traceback);
         if ((uint32_t)j == vi.y)
-            request_spill(s, sh, atomicAdd(n_req, 1u), vi, in.y, k, base, tr, traceback, &S.err);
+            request_spill(s, sh, atomicAdd(n_req, 1u), vi.y, in.y, k, base, tr, traceback, &S.err);
     }
 }
 
-// Empty the records and hash entries of a query; in exact mode, which never removes a
-// diagonal from H~, also count the diagonals they hold (the visited ones).
+// Empty the hash entries of a query; in exact mode, which never removes a diagonal from
+// H~, also count the diagonals its records hold (the visited ones).
 template <bool P> __device__ void wipe(const Slab<P> &s, Sh &sh) {
     const uint32_t nt = min(sh.nt, s.cap);
-    uint32_t c = 0;
-    constexpr uint32_t kChunks = sizeof(RecT<typename VT<P>::T>) / 16, kValChunks = sizeof(typename VT<P>::T) / 2;
-    for (uint32_t t = threadIdx.x; t < nt * kChunks; t += blockDim.x) {
-        const uint32_t part = t % kChunks;
-        uint4 *p = (uint4 *)s.recs + t;
-        if constexpr (!P) {
-            if (part < kValChunks) {
-                const int4 v = *(const int4 *)p;
-                c += (v.x >= 0) + (v.y >= 0) + (v.z >= 0) + (v.w >= 0);
-            }
-        }
-        *p = empty_chunk(P, part);
-        if (part == 0) {
-            const uint32_t i = t / kChunks, h = s.touched[i];
-            if (h != kNone) {
-                *(uint4 *)&s.table[h] = make_uint4(~0u, ~0u, ~0u, ~0u);
-                s.touched[i] = kNone;
-            }
-            if (i >= kBitTiles) s.stamp[i] = kNone;
-            if constexpr (P) s.tkey[i] = kEmptyKey;
-        }
+    for (uint32_t t = threadIdx.x; t < nt; t += blockDim.x) {
+        const uint32_t h = s.touched[t];
+        if (h != kNone) *(uint4 *)&s.table[h] = make_uint4(~0u, ~0u, ~0u, ~0u);
     }
     if constexpr (!P) {
+        uint32_t c = 0;
+        for (uint32_t t = threadIdx.x; t < 2 * nt; t += blockDim.x) {
+            const int4 v = *(const int4 *)&s.recs[t >> 1].vals[4 * (t & 1)];
+            c += (v.x >= 0) + (v.y >= 0) + (v.z >= 0) + (v.w >= 0);
+        }
         c = __reduce_add_sync(0xFFFFFFFFu, c);
         if ((threadIdx.x & 31) == 0 && c) atomicAdd(&sh.visited, (unsigned long long)c);
     }
@@ -951,6 +994,8 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         }
     }
     for (uint32_t w = threadIdx.x; w < kBitTiles / 32; w += blockDim.x) sh.bits[0][w] = sh.bits[1][w] = 0u;
+    if constexpr (!P)
+        for (uint32_t w = threadIdx.x; w < 1u << kLog2Claims; w += blockDim.x) sh.claim[w] = 0u;
     __syncthreads();
     if (A.ends & GWFA_FREE_START) {
         // free walk start (Sec. 2.1 variant): query position 0 also faces every
@@ -1161,10 +1206,10 @@ __device__ __forceinline__ void align_queries(const TierArgs &A) {
     }
 }
 
-// Up to kNarrow threads: the throughput shape, 5 CTAs per SM at 48 registers (10,000 reads
-// of 1-20 kb: 48.9 ms, against 55 at 4 with 64, 54 at 6 with 40 and 52 at three CTAs of
-// 512 threads); pruning mode, with 64-bit offsets, 4 at 64 (400 pruned 50 kb reads 24.7 ms,
-// 25.9 at 5 with 48, 28 for eight CTAs of 128).
+// Up to kNarrow threads: the throughput shape, 5 CTAs per SM at 48 registers.  When it was
+// chosen, 10,000 reads of 1-20 kb took 48.9 ms, 55 at 4 CTAs with 64, 54 at 6 with 40 and 52
+// at three CTAs of 512 threads; pruning mode, with 64-bit offsets, 4 at 64 (400 pruned 50 kb
+// reads 24.7 ms, 25.9 at 5 with 48, 28 for eight CTAs of 128).
 template <bool P>
 __global__ void __launch_bounds__(kNarrow, P ? 4 : 5) align_kernel(TierArgs A) {
     align_queries<P>(A);
@@ -1327,19 +1372,12 @@ __global__ void pack_kernel(uint32_t nq, const char *__restrict__ q, const uint6
     if (blockIdx.x == 0 && threadIdx.x < 2) words[(off[nq] >> 4) + nq + threadIdx.x] = 0;
 }
 
-// Slabs start empty: hash entries, claims and stamps all ones, records empty.  The lists
-// of a slab (tile lists, spill requests, insertions, T) are written before they are read.
-__global__ void slab_init_kernel(uint8_t *slabs, uint64_t slab_bytes, uint32_t n_slabs, uint64_t init_bytes,
-                                 uint64_t recs, uint64_t recs_end, bool prune) {
-    const uint64_t per = init_bytes / 16, total = per * n_slabs;
-    const uint32_t rec_chunks = prune ? sizeof(RecT<long long>) / 16 : sizeof(RecT<int>) / 16;
+// Slabs start with an empty hash (all ones); everything else is written before it is read.
+__global__ void slab_init_kernel(uint8_t *slabs, uint64_t slab_bytes, uint32_t n_slabs, uint64_t table_bytes) {
+    const uint64_t per = table_bytes / 16, total = per * n_slabs;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < total;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-        const uint64_t o = (i % per) * 16;   // offset inside the slab
-        uint4 *p = (uint4 *)(slabs + (i / per) * slab_bytes + o);
-        *p = o >= recs && o < recs_end ? empty_chunk(prune, (uint32_t)((o - recs) / 16 % rec_chunks))
-                                       : make_uint4(~0u, ~0u, ~0u, ~0u);
-    }
+         i += (uint64_t)gridDim.x * blockDim.x)
+        *(uint4 *)(slabs + (i / per) * slab_bytes + (i % per) * 16) = make_uint4(~0u, ~0u, ~0u, ~0u);
 }
 
 }  // namespace
@@ -1379,11 +1417,11 @@ cudaError_t launch_pack(uint32_t nq, const char *d_q, const uint64_t *d_off, uin
 cudaError_t launch_slab_init(uint8_t *slabs, uint64_t slab_bytes, uint32_t n_slabs, uint32_t log2cap,
                              bool prune, cudaStream_t st) {
     const SlabLayout L = slab_layout(log2cap, prune);
-    const uint64_t n16 = L.list0 / 16 * n_slabs;
+    const uint64_t n16 = L.recs / 16 * n_slabs;
     if (n16 == 0) return cudaSuccess;
     uint64_t blocks = (n16 + 255) / 256;
     if (blocks > 8192) blocks = 8192;
-    slab_init_kernel<<<(unsigned)blocks, 256, 0, st>>>(slabs, slab_bytes, n_slabs, L.list0, L.recs, L.touched, prune);
+    slab_init_kernel<<<(unsigned)blocks, 256, 0, st>>>(slabs, slab_bytes, n_slabs, L.recs);
     return cudaGetLastError();
 }
 
