@@ -23,10 +23,12 @@
 // at a time fit L2 only while nothing else is fetched for them (10,000 reads 48.3 -> 35.3 ms).
 // Measured against the form with separate extend and expand passes that max-merged
 // candidates with atomics and probed the hash for each one leaving a tile (reads of
-// 1-20 kb): 10,000 reads 102.9 -> 35.3 ms, 997 reads 55.2 -> 13.7 ms, 300 with a heavy tail
-// 405 -> 68 ms, 400 pruned 50 kb reads 51.0 -> 24.7 ms, one 10 kb read 7.4 -> 2.0 ms.
-// What bounds it: latency.  A score is two barriers, one tile visit per group or a few,
-// and the longest chain of spills, each link of it an arc, a hash entry and a label.
+// 1-20 kb): 10,000 reads 101 -> 32.2 ms, 997 reads 49 -> 12.9 ms, 300 with a heavy tail
+// 415 -> 64 ms, 400 pruned 50 kb reads 50.7 -> 23.2 ms, one 10 kb read 8.5 -> 2.1 ms.
+// What bounds it: of the ~13,000 cycles a score of one 10 kb read takes, the pass has 5,000
+// (one visit per warp, bound by issue), the second step 7,700: a few warps walk the code
+// of links and spills, one after the other, while the rest wait.  Memory is not it: with
+// all claims in shared memory and the hash entries fetched ahead the step took as long.
 //
 // Data (per CTA slab, see SlabLayout; reused across queries):
 //   H~     tile records, dense in order of first use, and an open-addressing hash from
@@ -204,9 +206,34 @@ __device__ __forceinline__ int lcp(const QCtx &q, int i, const uint32_t *__restr
     return min(l, maxl);
 }
 
+// Loads that are issued where they stand, ahead of a lookup they do not depend on.
+__device__ __forceinline__ uint2 ld_early(const uint4 *p, int half) {
+    uint2 r;
+    asm volatile("ld.global.nc.v2.u32 {%0, %1}, [%2];" : "=r"(r.x), "=r"(r.y) : "l"((const uint2 *)p + half));
+    return r;
+}
+
 // Target of out-arc `a` of v, the `o`-th of its arcs.
 __device__ __forceinline__ uint32_t arc_target(const DevGraph &g, uint32_t v, uint32_t a, uint32_t o) {
     return __ldg(o < 4 ? (const uint32_t *)&g.vx[2 * (uint64_t)v + 1] + o : &g.arc_dst[a]);
+}
+
+// LCP of a spilled diagonal (offset 0, query position i) when the XOR `x` of its first
+// windows is already there.
+__device__ __forceinline__ int lcp0(const QCtx &q, int i, const uint32_t *__restrict__ vw, int lv, uint32_t x) {
+    const int maxl = min(q.n - i, lv);
+    int l = x ? (__ffs(x) - 1) >> 1 : 16;
+    if (!x) {
+        while (l < maxl) {
+            const uint32_t y = qwin(q, (uint32_t)(i + l)) ^ window16(vw, (uint32_t)l);
+            if (y) {
+                l += (__ffs(y) - 1) >> 1;
+                break;
+            }
+            l += 16;
+        }
+    }
+    return min(l, maxl);
 }
 
 // Atomics on slab memory (always device global memory) issued in the global state
@@ -755,16 +782,22 @@ __device__ __forceinline__ void spill_round(const DevGraph &g, const Slab<false>
         uint2 wait = make_uint2(kNone, 0u);   // this lane's inserted diagonal that spills in turn
         for (;;) {
             if (rq.x != kNone) {
-                const uint2 ar = __ldg((const uint2 *)&g.vx[2 * (uint64_t)rq.x].z);
+                const uint4 *vr = &g.vx[2 * (uint64_t)rq.x];
+                const uint2 ar = ld_early(vr, 1);
+                uint32_t u = __ldg((const uint32_t *)(vr + 1) + arc);   // valid where there is such an arc
                 const int ku = (int)rq.y;
                 for (uint32_t o = (uint32_t)arc; ar.x + o < ar.y; o += 2) {
-                    const uint32_t u = arc_target(g, rq.x, ar.x + o, o);
-                    const uint2 ui = __ldg((const uint2 *)&g.vx[2 * (uint64_t)u]);
+                    if (o >= 2) u = arc_target(g, rq.x, ar.x + o, o);
+                    const uint2 ui = ld_early(&g.vx[2 * (uint64_t)u], 0);
                     const int su = find_or_insert<false>(s, sh, u, ku >> 3, &S.err);
                     if (su < 0) break;
-                    if (s.recs[su].vals[ku & 7] != kAbsent || !claim_lane(s, sh, (uint32_t)su, ku & 7, d)) continue;
+                    // the offset and the first windows together; most spills end here, the
+                    // diagonal being there already
+                    const int raw = s.recs[su].vals[ku & 7];
+                    const uint32_t x = qwin(q, (uint32_t)ku) ^ __ldg(g.words + ui.x);
+                    if (raw != kAbsent || !claim_lane(s, sh, (uint32_t)su, ku & 7, d)) continue;
                     ++won;
-                    const int l = lcp(q, ku, g.words + ui.x, 0, (int)ui.y);
+                    const int l = lcp0(q, ku, g.words + ui.x, (int)ui.y, x);
                     s.recs[su].vals[ku & 7] = (l << 1) | 1;
                     if (at_end(q, u, ku, l, ui.y)) S.found = 1;
                     enter_next<false>(s, sh, q, (uint32_t)su, u, ku, l, 0u, ui.y, d, 0u, false);
@@ -842,6 +875,75 @@ __device__ __forceinline__ void resolve_spill_traces(const DevGraph &g, const Sl
             if (s.recs[su].vals[ku & 7] == cand) g_max32(&s.trec[su].tr[ku & 7], s.reqt[r]);
         }
     }
+}
+
+// Pruning mode without traceback, one warp, at most 8 requests of at most four arcs (nearly
+// always so): the whole round in one step, a lane an arc.  Every spill of the round is in
+// this warp, so a match of the lanes finds those into one diagonal (the largest base wins),
+// and the offset needs neither atomic nor second look; the label is compared before it is
+// known who wins.  Returns false, having done nothing, if a vertex has more arcs.
+__device__ __forceinline__ bool spill_step(const DevGraph &g, const Slab<true> &s, Sh &sh, const QCtx &q, int d,
+                                           uint32_t n, uint32_t *n_req) {
+    Score &S = sh.score[d & 3];
+    const unsigned full = 0xFFFFFFFFu;
+    const uint32_t lane = threadIdx.x & 31, r = lane >> 2, arc = lane & 3;
+    int4 rq = make_int4(0, 0, 0, 0);
+    uint2 ar = make_uint2(0u, 0u);
+    uint32_t u = 0;
+    if (r < n) {
+        rq = get_req4(s, sh, r);
+        const uint4 *vr = &g.vx[2 * (uint64_t)(uint32_t)rq.z];
+        ar = ld_early(vr, 1);
+        u = __ldg((const uint32_t *)(vr + 1) + arc);
+    }
+    if (__any_sync(full, ar.y - ar.x > 4)) return false;
+    const int ku = rq.x, ln = ku & 7;
+    int su = -1, j = 0;
+    uint32_t base = (uint32_t)rq.y;
+    uint2 ui = make_uint2(0u, 0u);
+    bool want = ar.x + arc < ar.y;
+    if (want) {
+        ui = ld_early(&g.vx[2 * (uint64_t)u], 0);
+        su = find_or_insert<true>(s, sh, u, ku >> 3, &S.err);
+        want = su >= 0;
+        if (want) {
+            const long long raw = s.recs[su].vals[ln];
+            const uint32_t x = qwin(q, (uint32_t)ku) ^ __ldg(g.words + ui.x);
+            want = raw < 0;
+            if (want) j = lcp0(q, ku, g.words + ui.x, (int)ui.y, x);
+        }
+    }
+    __syncwarp();   // the old offsets are read: now they may be written
+    const unsigned w = __ballot_sync(full, want);
+    if (__popc(w) > 1) {
+        const uint32_t key = want ? (uint32_t)su << 3 | (uint32_t)ln : ~lane;
+        const unsigned peers = __match_any_sync(full, key);
+        for (unsigned m = w; m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            const uint32_t b = __shfl_sync(full, base, l);
+            if (peers >> l & 1u) base = max(base, b);
+        }
+        want = want && (int)lane == __ffs(peers) - 1;
+    }
+    const uint32_t won = (uint32_t)__popc(__ballot_sync(full, want));
+    if (want) {
+        s.recs[su].vals[ln] = pk(j, kTagLive, base);
+        atomicMax(&S.amax, (uint32_t)(ku + j) + (uint32_t)j + base);
+        if (at_end(q, u, ku, j, ui.y)) {
+            S.found = 1;
+            sh.end_vp = (unsigned long long)u << 32;
+        }
+        enter_next<true>(s, sh, q, (uint32_t)su, u, ku, j, base, ui.y, d, 0u, false);
+    }
+    __syncwarp();   // every request of this round is read: the next round's may be written
+    if (want && (uint32_t)j == ui.y)
+        request_spill(s, sh, atomicAdd(n_req, 1u), ui.y, u, ku, base, 0u, false, &S.err);
+    if (lane == 0 && won) {
+        S.cells += won;
+        S.spills += won;
+        S.visited += won;
+    }
+    return true;
 }
 
 // Pruning mode: extend the diagonals inserted by the round; those that reach their
@@ -945,7 +1047,7 @@ __device__ void evict_behind(const Slab<true> &s, Sh &sh, long long amax, int la
     __syncthreads();
 }
 
-template <bool P>
+template <bool P, bool TB>
 __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, Sh &sh, uint32_t qid) {
     const DevGraph &g = A.g;
     const uint64_t qo = A.q_off[qid];
@@ -984,7 +1086,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         if (t >= 0) {
             if constexpr (P) {
                 s.recs[t].vals[0] = pk(0, kTagLive, 0u);
-                if (A.traceback) s.trec[t].tr[0] = kNoTrace;
+                if (TB) s.trec[t].tr[0] = kNoTrace;
                 sh.visited = 1;
             } else {
                 s.recs[t].vals[0] = 1;
@@ -1013,7 +1115,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
                 ++cnt;
                 if constexpr (P) {
                     s.recs[t].vals[ln] = pk(j, kTagLive, 0u);
-                    if (A.traceback) s.trec[t].tr[ln] = kNoTrace;
+                    if (TB) s.trec[t].tr[ln] = kNoTrace;
                 } else {
                     s.recs[t].vals[ln] = (j << 1) | 1;
                 }
@@ -1029,20 +1131,19 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
     int d = 0, status = 0;
     for (;; ++d) {
         Score &S = sh.score[d & 3];
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == blockDim.x - 32) {   // the last warp: the first to run out of tiles
             sh.score[(d + 2) & 3] = Score{};
             sh.nr[0] = 0;
             sh.nins[0] = 0;
-            if (A.stats) sh.t_phase = globaltimer_ns();
         }
+        if (A.stats && threadIdx.x == 0) sh.t_phase = globaltimer_ns();
         // ---- GwfExpand of the last score (Alg. 3, with GwfPrune, Alg. 4) and GwfExtend of this one
         bool prune_on = false;
         long long amax = 0;
         if constexpr (P) {
             amax = (long long)sh.score[(d + 3) & 3].amax;
             prune_on = A.max_lag > 0 && amax > (long long)A.max_lag;
-            if (A.traceback) offset_pass<P, true>(g, s, sh, q, d, prune_on, A.max_lag);
-            else offset_pass<P, false>(g, s, sh, q, d, prune_on, A.max_lag);
+            offset_pass<P, TB>(g, s, sh, q, d, prune_on, A.max_lag);
         } else {
             offset_pass<P, false>(g, s, sh, q, d, false, 0);
         }
@@ -1061,12 +1162,12 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
             break;
         }
         if constexpr (P) {
-            if (A.evict_lag > 0 && d > 0 && d % A.evict_every == 0) evict_behind(s, sh, amax, A.evict_lag, d);
+            if (!TB && A.evict_lag > 0 && d > 0 && d % A.evict_every == 0) evict_behind(s, sh, amax, A.evict_lag, d);
         }
         // ---- arc spills, in rounds until no extended diagonal reaches its vertex's end
         uint32_t n = S.nreq;
         const uint32_t nl = S.nlink;
-        if (nl) link_pending<P>(s, sh, d, nl, A.traceback != 0);
+        if (nl) link_pending<P>(s, sh, d, nl, TB);
         if constexpr (P) {
             // few requests (the usual case): one warp does every round by itself, and the
             // others wait once instead of twice or three times a round
@@ -1084,13 +1185,19 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
                         sh.nr[(round + 1) % 3] = 0;
                         sh.nins[(round + 1) & 1] = 0;
                     }
-                    apply_spills(g, s, sh, d, n, n_ins, nthr, A.traceback != 0);
+                    if (solo && n <= 8 && !TB && spill_step(g, s, sh, q, d, n, next_count)) {
+                        __syncwarp();
+                        n = *next_count;
+                        if (A.stats && threadIdx.x == 0 && n) sh.st[2] += 1;
+                        continue;
+                    }
+                    apply_spills(g, s, sh, d, n, n_ins, nthr, TB);
                     sync();
-                    if (A.traceback) {
+                    if (TB) {
                         resolve_spill_traces(g, s, sh, d, n, nthr);
                         sync();
                     }
-                    extend_spilled(g, s, sh, q, d, *n_ins, next_count, nthr, A.traceback != 0);
+                    extend_spilled(g, s, sh, q, d, *n_ins, next_count, nthr, TB);
                     sync();
                     n = *next_count;
                     if (A.stats && threadIdx.x == 0 && n) sh.st[2] += 1;
@@ -1111,7 +1218,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
             }
             if (nl && !r0) __syncthreads();
         }
-        if (threadIdx.x == 0) {
+        if (threadIdx.x == blockDim.x - 32) {
             sh.cells += S.cells;
             sh.spills += S.spills;
             sh.peak = max(sh.peak, S.cells);
@@ -1119,8 +1226,8 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
                 sh.visited += S.visited;
                 sh.pruned += S.pruned;
             }
-            if (A.stats) sh.st[1] += globaltimer_ns() - sh.t_phase;
         }
+        if (A.stats && threadIdx.x == 0) sh.st[1] += globaltimer_ns() - sh.t_phase;
         if (S.err) { status = S.err; break; }
         if (S.found) break;   // end test of Alg. 1
         if (A.max_score >= 0 && d >= A.max_score) { status = GWFA_ERR_SCORE_LIMIT; break; }
@@ -1136,7 +1243,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
                 sh.visited += S.visited;
                 sh.pruned += S.pruned;
             }
-            if (A.traceback && status == 0) {
+            if (TB && status == 0) {
                 // GwfTraceback (Alg. 6): push the end vertex, then follow T back to the
                 // start and write the walk in order
                 const uint32_t te = push_trace(s, sh, (uint32_t)(sh.end_vp >> 32), (uint32_t)sh.end_vp & 0xFFFFFFFFu,
@@ -1183,7 +1290,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
 }
 
 // The persistent loop of a CTA: pull a query id, run its score loop, repeat.
-template <bool P>
+template <bool P, bool TB>
 __device__ __forceinline__ void align_queries(const TierArgs &A) {
     __shared__ Sh sh;
     // the slab's array pointers are the same for every thread: held once in shared
@@ -1202,24 +1309,27 @@ __device__ __forceinline__ void align_queries(const TierArgs &A) {
         const uint32_t qid = sh.qid;
         __syncthreads();
         if (qid == 0xFFFFFFFFu) break;
-        align_one<P>(A, s, sh, qid);
+        align_one<P, TB>(A, s, sh, qid);
     }
 }
 
-// Up to kNarrow threads: the throughput shape, 5 CTAs per SM at 48 registers.  When it was
-// chosen, 10,000 reads of 1-20 kb took 48.9 ms, 55 at 4 CTAs with 64, 54 at 6 with 40 and 52
-// at three CTAs of 512 threads; pruning mode, with 64-bit offsets, 4 at 64 (400 pruned 50 kb
-// reads 24.7 ms, 25.9 at 5 with 48, 28 for eight CTAs of 128).
-template <bool P>
-__global__ void __launch_bounds__(kNarrow, P ? 4 : 5) align_kernel(TierArgs A) {
-    align_queries<P>(A);
+// Up to kNarrow threads: the throughput shape, 6 CTAs per SM at 40 registers: 10,000 reads of
+// 1-20 kb take 32.0 ms, 34.5 at 5 with 48, 55 at 7 (36 registers spill), 38 for eight CTAs of
+// 192 threads, 35.7 for four of 384.  Pruning mode, with 64-bit offsets, 4 at 64: 400 pruned
+// 50 kb reads 23.3 ms, 24.2 at 5 with 48, 26.5 at 6.  Traceback is a kernel of its own: with
+// the switch at run time the pruning kernel's code was twice as long, and the few warps that
+// do a score's spills are bound by the instructions they fetch (24.5 -> 23.3 ms together
+// with spill_step).
+template <bool P, bool TB>
+__global__ void __launch_bounds__(kNarrow, P ? 4 : 6) align_kernel(TierArgs A) {
+    align_queries<P, TB>(A);
 }
 
 // Up to 1024 threads, 64 registers: more groups on one query, for batches and queries
 // whose own latency is the bound.
-template <bool P>
+template <bool P, bool TB>
 __global__ void __launch_bounds__(1024, 1) align_kernel_wide(TierArgs A) {
-    align_queries<P>(A);
+    align_queries<P, TB>(A);
 }
 
 __device__ __forceinline__ unsigned long long ld_acquire_sys(const unsigned long long *p) {
@@ -1326,7 +1436,7 @@ __global__ void __launch_bounds__(512, PerSm) server_kernel(ServerArgs S) {
         A.out = S.results[rc] + slot;
         A.max_lag = S.max_lag;
         A.max_score = S.max_score;
-        align_one<P>(A, s, sh, 0);
+        align_one<P, false>(A, s, sh, 0);
         if (threadIdx.x == 0) {
             __threadfence_system();
             st_release_sys(S.done[rc] + slot, ticket + 1);
@@ -1382,15 +1492,16 @@ __global__ void slab_init_kernel(uint8_t *slabs, uint64_t slab_bytes, uint32_t n
 
 }  // namespace
 
+// the alignment kernel of a mode and CTA width
+static void (*align_entry(bool prune, bool traceback, uint32_t threads))(TierArgs) {
+    if (threads > kNarrow)
+        return !prune ? align_kernel_wide<false, false> : traceback ? align_kernel_wide<true, true> : align_kernel_wide<true, false>;
+    return !prune ? align_kernel<false, false> : traceback ? align_kernel<true, true> : align_kernel<true, false>;
+}
+
 cudaError_t launch_align(const TierArgs &a, bool prune, uint32_t ctas, uint32_t threads,
                          cudaStream_t st) {
-    if (threads > kNarrow) {
-        if (prune) align_kernel_wide<true><<<ctas, threads, 0, st>>>(a);
-        else align_kernel_wide<false><<<ctas, threads, 0, st>>>(a);
-    } else {
-        if (prune) align_kernel<true><<<ctas, threads, 0, st>>>(a);
-        else align_kernel<false><<<ctas, threads, 0, st>>>(a);
-    }
+    align_entry(prune, a.traceback != 0, threads)<<<ctas, threads, 0, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -1431,17 +1542,15 @@ cudaError_t launch_slab_init(uint8_t *slabs, uint64_t slab_bytes, uint32_t n_sla
 // beside tier 0), so it touches them all before the first one starts.
 cudaError_t preload_kernels() {
     cudaFuncAttributes fa;
-    cudaError_t e = cudaFuncGetAttributes(&fa, align_kernel<false>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, align_kernel<true>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, align_kernel_wide<false>);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, align_kernel_wide<true>);
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < 6 && e == cudaSuccess; ++i)
+        e = cudaFuncGetAttributes(&fa, align_entry(i % 3 > 0, i % 3 > 1, i < 3 ? kNarrow : 1024u));
     return e;
 }
 
 int align_occupancy(bool prune, uint32_t threads, int *blocks_per_sm) {
-    void (*k)(TierArgs) = threads > kNarrow ? (prune ? align_kernel_wide<true> : align_kernel_wide<false>)
-                                            : (prune ? align_kernel<true> : align_kernel<false>);
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, (int)threads, 0) == cudaSuccess ? 0 : -1;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, align_entry(prune, false, threads),
+                                                         (int)threads, 0) == cudaSuccess ? 0 : -1;
 }
 
 }  // namespace gwfa
