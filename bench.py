@@ -347,11 +347,11 @@ def kernel_counters():
 # each) and writes up to 3 frontier entries (12 B each) -- about 120 B -- plus 0.5 B
 # per aligned base (2 bits of query and label each).
 B_CELL = 120
-# The kernel's own minimum (its design keeps the diagonal, the vertex record and the
-# windows in registers and L1 and merges the frontier per 8-diagonal tile): the offset
-# read and written by GwfExtend (8 B), the snapshot read and up to three candidates
-# written by GwfExpand (16 B).
-B_CELL_KERNEL = 24
+# The kernel's own minimum (its design visits an 8-diagonal tile once a score and keeps the
+# diagonal, the vertex record and the windows in registers and L1): the offset read and
+# written (8 B), and a tile's side words, list entries and border words (56 B) over the 4.8
+# diagonals a visited tile has in Q on the benchmark graphs.
+B_CELL_KERNEL = 20
 
 
 def roofline(cells: int, aligned_bp: int, t_kernel: float, int_peak: dict | None, counters: dict | None,

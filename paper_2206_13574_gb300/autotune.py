@@ -1,7 +1,7 @@
 """Launch-shape autotuner for the batched engine.
 
 Grid search on held-out samples of queries over the CTA width (1 to 32 warps per
-query, i.e. 4 to 128 8-lane groups: threads / 8), CTAs per SM and tier-0 slab size, in
+query, i.e. 8 to 256 four-lane groups: threads / 4), CTAs per SM and tier-0 slab size, in
 two stages (every shape on a small sample, the fastest few again on a batch of the
 size the engine will run); every candidate must give the same results (they are
 compared), the fastest is kept.
@@ -9,10 +9,10 @@ Results are persisted as JSON keyed by (graph fingerprint, GPU name, mode), so l
 runs on the same graph and GPU reuse them without searching again (cache_path=None
 searches every time and persists nothing).
 
-The kernel is compiled for at most 32 registers per thread, so a CTA of T threads
-fits min(2048 / T, 32) times per SM (32 resident CTAs at most); candidate CTA counts
-are multiples of the SM count.  The frontier tile stays 8 diagonals: the expand
-step's neighbour exchange is a shuffle inside an 8-lane group.
+CTAs of up to 256 threads share an SM up to 1,536 threads (1,024 with pruning's 64-bit
+offsets), wider ones up to 1,024, and 32 CTAs at most; candidate CTA counts are multiples
+of the SM count.  The frontier tile stays 8 diagonals: the expand step's neighbour exchange
+is a shuffle among the four lanes that hold them.
 """
 from __future__ import annotations
 
@@ -107,7 +107,8 @@ def autotune(graph: Graph, sample, max_lag: int = 0, threads=(32, 64, 128, 256, 
     shapes = []
     for th in threads:
         for frac in per_sm_frac:
-            per_sm = max(1, int(min(2048 // th, 32) * frac))
+            resident = 1536 if th <= 256 and not prune else 1024
+            per_sm = max(1, int(min(resident // th, 32) * frac))
             for lg in log2_tiles:
                 lg = lg if not prune else lg - 1
                 shape = (th, per_sm, lg, sms * per_sm)

@@ -60,22 +60,71 @@ int ensure(uint8_t **buf, uint64_t *have, uint64_t need) {
 }
 
 // Host reachability v_s -> v_e (Def. 2 assumes it; the paper's loop never ends otherwise).
+// Breadth first: v_e is about as many vertices away as the query has, while depth first runs
+// to the far end of the graph before it looks beside its way.  `seen` holds the number of
+// the call that reached a vertex last, so nothing is cleared (both guarded by g->mu).
 bool reachable(const gwfa_graph *g, uint32_t vs, uint32_t ve) {
     if (vs == ve) return true;
-    std::vector<uint8_t> seen(g->nv, 0);
-    std::vector<uint32_t> st;
-    st.push_back(vs);
-    seen[vs] = 1;
-    while (!st.empty()) {
-        uint32_t v = st.back();
-        st.pop_back();
+    if (g->seen.size() != g->nv || ++g->seen_call == 0) {
+        g->seen.assign(g->nv, 0);
+        g->seen_call = 1;
+    }
+    std::vector<uint32_t> &q = g->bfs;
+    q.clear();
+    q.push_back(vs);
+    g->seen[vs] = g->seen_call;
+    for (size_t head = 0; head < q.size(); ++head) {
+        const uint32_t v = q[head];
         for (uint32_t a = g->h_arc_off[v]; a < g->h_arc_off[v + 1]; ++a) {
-            uint32_t u = g->h_arc_dst[a];
+            const uint32_t u = g->h_arc_dst[a];
             if (u == ve) return true;
-            if (!seen[u]) { seen[u] = 1; st.push_back(u); }
+            if (g->seen[u] != g->seen_call) {
+                g->seen[u] = g->seen_call;
+                q.push_back(u);
+            }
         }
     }
     return false;
+}
+
+// 2-bit packing of a query on the host, as pack_kernel does it; false for a base other
+// than A/C/G/T.  (n + 15) / 16 words.
+bool pack_host(const char *q, uint32_t n, uint32_t *w) {
+    static const struct Lut {
+        uint8_t c[256];
+        Lut() {
+            for (int i = 0; i < 256; ++i) c[i] = 4;
+            for (int i = 0; i < 4; ++i) c[(uint8_t)"ACGT"[i]] = c[(uint8_t)"acgt"[i]] = (uint8_t)i;
+        }
+    } lut;
+    uint32_t bad = 0;
+    for (uint32_t p = 0; p < n; p += 16) {
+        uint32_t x = 0;
+        const uint32_t e = std::min(n - p, 16u);
+        for (uint32_t i = 0; i < e; ++i) {
+            const uint32_t c = lut.c[(uint8_t)q[p + i]];
+            bad |= c;
+            x |= (c & 3u) << (2 * i);
+        }
+        w[p >> 4] = x;
+    }
+    return (bad & 4u) == 0;
+}
+
+// Grow-only pinned host buffer, mapped into the device's address space.
+int ensure_pinned(uint8_t **buf, uint64_t *have, uint64_t need) {
+    if (*have >= need) return GWFA_OK;
+    if (*buf) cudaFreeHost(*buf);
+    *buf = nullptr;
+    *have = 0;
+    const uint64_t want = std::max<uint64_t>(need, 64 << 10);
+    if (cudaHostAlloc((void **)buf, want, cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        *buf = nullptr;
+        return GWFA_ERR_OOM;
+    }
+    *have = want;
+    return GWFA_OK;
 }
 
 struct Carve {
@@ -91,22 +140,29 @@ struct Carve {
 // The default config's CTA width: the engine chooses it for each batch.
 constexpr uint32_t kAutoThreads = 512;
 
-// Width of tier 0's CTAs for n queries of `len` bases on average (0 = not known on the
-// host), where the configuration leaves it to the engine.  A wide CTA shortens a query, a
+// Host-buffer batches up to this many bytes of inputs go over in one copy.
+constexpr uint64_t kStagedBatch = 256 << 10;
+
+// Mean lengths from which n queries get 1024 and 512 threads each, see auto_threads.
+uint64_t wide_from(uint64_t n, int sms) { return 600 * n / (uint64_t)sms; }
+uint64_t mid_from(uint64_t n, int sms) { return 180 * n / (uint64_t)sms; }
+
+// Width of tier 0's CTAs for n queries of `len` bases on average, where the configuration
+// leaves it to the engine.  A wide CTA shortens a query, a
 // narrow one wastes fewer warps on small frontiers and at barriers: few queries are bound
 // by their longest, many by throughput, and a frontier grows with the length.  Measured
 // crossings, 1024 -> 512 -> 256 threads (ms at 1024 / 512 / 256): 1-20 kb reads, 6.4 kb on
-// average, n = 1000: 9.6 / 12.3 / 20.3, 1500: 13.9 / 14.6 / 25.7, 2500: 22.5 / 15.9 / 24.5,
-// 4000: 35.8 / 23.9 / 29.1, 7000: 62 / 41.7 / 37.7; 0.5-5 kb, 2.0 kb on average, n = 600:
-// 1.37 / 1.47 / 1.74, 1000: 1.94 / 1.51 / 1.88, 2500: 4.8 / 2.56 / 2.46.
+// average, n = 1000: 8.4 / 10.4 / 17.6, 1500: 12.1 / 12.3 / 21.0, 2500: 19.6 / 12.5 / 21.2,
+// 5000: 38.7 / 23.8 / 25.3, 7000: 54 / 33.5 / 28.2; 0.5-5 kb, 2.0 kb on average, n = 600:
+// 1.27 / 1.33 / 1.57, 1000: 1.84 / 1.40 / 1.64, 2500: 4.5 / 2.40 / 2.12; 1 kb, n = 1000:
+// 0.58 / 0.33 / 0.20.
 // Lag pruning keeps the frontier near 0.03 tiles per unit of lag, whatever the length
-// (lag 1000, 1024 / 256 / 128 threads, n = 150: 9.5 / 9.6 / 10.2, 400: 25.7 / 9.8 / 10.8,
-// 1000: 59 / 18.7 / 12.0; lag 4000: 15.6 / 19.5 / 27.2, 41.5 / 21.5 / 26.9, 95 / 39 / 33).
+// (lag 1000, 1024 / 256 / 128 threads, n = 150: 9.0 / 9.1 / 9.8, 400: 24.4 / 9.4 / 10.5,
+// 1000: 56 / 17.4 / 11.1; lag 4000: 15.3 / 20.1 / 25.7, 40.6 / 20.3 / 28.1, 93 / 38 / 32).
 uint32_t auto_threads(uint64_t n, uint64_t len, int sms, int max_lag) {
     const uint64_t m = (uint64_t)sms;
     if (max_lag > 0) return n <= m && max_lag > 2000 ? 1024u : n <= 4 * m ? 256u : 128u;
-    if (len == 0) len = 4000;
-    return n <= m * len / 600 ? 1024u : n <= m * len / 180 ? 512u : gwfa::kNarrow;
+    return len >= wide_from(n, sms) ? 1024u : len >= mid_from(n, sms) ? 512u : gwfa::kNarrow;
 }
 
 uint64_t words_for(uint32_t nq, uint64_t nbases) { return (nbases >> 4) + nq + 2; }
@@ -228,6 +284,7 @@ int gwfa_graph_destroy(gwfa_graph *g) {
     cudaFree(g->d_arc_dst);
     cudaFree(g->plain_slab);
     cudaFree(g->plain_stage);
+    if (g->plain_host) cudaFreeHost(g->plain_host);
     if (g->stream) cudaStreamDestroy(g->stream);
     delete g;
     return GWFA_OK;
@@ -287,31 +344,46 @@ static int align_plain(const gwfa_graph *g, const char *h_q, uint32_t n, uint32_
         out->status = GWFA_ERR_INVALID;
         return GWFA_ERR_INVALID;
     }
+    std::lock_guard<std::mutex> lk(g->mu);
     if (!reachable(g, vs, ve)) {
         out->status = GWFA_ERR_UNREACHABLE;
         return GWFA_OK;
     }
-    std::lock_guard<std::mutex> lk(g->mu);
     int st = cuda_status(cudaSetDevice(g->device));
     if (st) return st;
     const bool prune = o.max_lag > 0 || o.traceback;   // 64-bit values (walk base) and trace words
-    // staging: query bytes | q_off[2] | v_s | v_e | words | status | head | result | path
-    const uint64_t need = gwfa::align256(n + 16) + 256 * 6 + gwfa::align256(words_for(1, n) * 4) +
-                          gwfa::align256(sizeof(gwfa_result)) + gwfa::align256((uint64_t)path_cap * 4) + 1024;
-    st = ensure(&g->plain_stage, &g->plain_stage_bytes, need);
+    // A short call is bound by its launches and copies (one 1 kb read took 118 us with four copies
+    // in, a clear, a packing kernel and a copy out, of which the alignment is about 70), so the
+    // inputs go over in one copy from pinned memory, packed here, and the result comes back in
+    // pinned memory that the kernel writes itself: 97 us.
+    //   staged: q_off[2] | v_s | v_e | work counter | words;  pinned only: result, path_len
+    const uint64_t in_bytes = 64 + words_for(1, n) * 4;
+    const uint64_t res_off = gwfa::align256(in_bytes);
+    st = ensure_pinned(&g->plain_host, &g->plain_host_bytes, res_off + 256);
     if (st) return st;
-    Carve c{g->plain_stage};
-    char *d_q = c.take<char>(n + 16);
-    uint64_t *d_off = c.take<uint64_t>(16);
-    uint32_t *d_vs = c.take<uint32_t>(4);
-    uint32_t *d_ve = c.take<uint32_t>(4);
-    int32_t *d_status = c.take<int32_t>(4);
-    uint32_t *d_head = c.take<uint32_t>(4);
-    gwfa_result *d_res = c.take<gwfa_result>(sizeof(gwfa_result));
-    uint32_t *d_words = c.take<uint32_t>(words_for(1, n) * 4);
-    uint32_t *d_plen = c.take<uint32_t>(4);
-    uint32_t *d_path = c.take<uint32_t>((uint64_t)path_cap * 4);
-    uint64_t h_off[2] = {0, n};
+    struct In {
+        uint64_t off[2];
+        uint32_t vs, ve, head, pad;
+    };
+    static_assert(sizeof(In) <= 64, "words start at byte 64");
+    In *in = (In *)g->plain_host;
+    uint32_t *h_words = (uint32_t *)(g->plain_host + 64);
+    *in = In{{0, n}, vs, ve, 0u, 0u};
+    if (!pack_host(h_q, n, h_words)) {
+        out->status = GWFA_ERR_INVALID;
+        return GWFA_OK;
+    }
+    for (uint64_t w = ((uint64_t)n + 15) >> 4; w < words_for(1, n); ++w) h_words[w] = 0;
+    st = ensure(&g->plain_stage, &g->plain_stage_bytes, gwfa::align256(in_bytes) + (uint64_t)path_cap * 4);
+    if (st) return st;
+    In *d_in = (In *)g->plain_stage;
+    uint32_t *d_path = (uint32_t *)(g->plain_stage + gwfa::align256(in_bytes));
+    gwfa_result *h_res = (gwfa_result *)(g->plain_host + res_off);
+    uint32_t *h_plen = (uint32_t *)(h_res + 1);
+    void *d_res = nullptr, *d_plen = nullptr;
+    st = cuda_status(cudaHostGetDevicePointer(&d_res, h_res, 0));
+    if (!st) st = cuda_status(cudaHostGetDevicePointer(&d_plen, h_plen, 0));
+    if (st) return st;
     cudaStream_t s = g->stream;
     uint32_t log2 = g->plain_log2 && g->plain_prune == prune ? g->plain_log2 : (prune ? 15u : 16u);
     for (;;) {
@@ -326,27 +398,18 @@ static int align_plain(const gwfa_graph *g, const char *h_q, uint32_t n, uint32_
             g->plain_log2 = log2;
             g->plain_prune = prune;
         }
-        if (n) cudaMemcpyAsync(d_q, h_q, n, cudaMemcpyHostToDevice, s);
-        cudaMemcpyAsync(d_off, h_off, 16, cudaMemcpyHostToDevice, s);
-        cudaMemcpyAsync(d_vs, &vs, 4, cudaMemcpyHostToDevice, s);
-        cudaMemcpyAsync(d_ve, &ve, 4, cudaMemcpyHostToDevice, s);
-        cudaMemsetAsync(d_head, 0, 4, s);
-        st = cuda_status(gwfa::launch_pack(1, d_q, d_off, d_words, d_status, s));
+        st = cuda_status(cudaMemcpyAsync(g->plain_stage, g->plain_host, in_bytes, cudaMemcpyHostToDevice, s));
         if (st) return st;
+        *h_plen = 0;
         TierArgs a{};
         a.g = g->dev();
-        a.qwords = d_words;
-        a.q_off = d_off;
-        a.v_s = d_vs;
-        a.v_e = d_ve;
-        a.qstatus = d_status;
-        a.out = d_res;
-        a.list = nullptr;
-        a.list_count = nullptr;
+        a.qwords = (const uint32_t *)(g->plain_stage + 64);
+        a.q_off = d_in->off;
+        a.v_s = &d_in->vs;
+        a.v_e = &d_in->ve;
+        a.out = (gwfa_result *)d_res;
         a.count_val = 1;
-        a.retry = nullptr;
-        a.retry_count = nullptr;
-        a.head = d_head;
+        a.head = &d_in->head;
         a.slabs = g->plain_slab;
         a.slab_bytes = gwfa::slab_layout(log2, prune).total;
         a.log2cap = log2;
@@ -357,18 +420,19 @@ static int align_plain(const gwfa_graph *g, const char *h_q, uint32_t n, uint32_
         a.evict_lag = o.evict_lag;
         a.evict_every = o.evict_every ? o.evict_every : 64;
         a.paths = o.traceback ? d_path : nullptr;
-        a.path_len = o.traceback ? d_plen : nullptr;
+        a.path_len = o.traceback ? (uint32_t *)d_plen : nullptr;
         a.path_cap = path_cap;
-        if (o.traceback) cudaMemsetAsync(d_plen, 0, 4, s);
         st = cuda_status(gwfa::launch_align(a, prune, 1, o.max_lag > 0 ? 256 : n < 3000 ? 512 : 1024, s));
-        if (st) return st;
-        st = cuda_status(cudaMemcpyAsync(out, d_res, sizeof(gwfa_result), cudaMemcpyDeviceToHost, s));
-        if (!st && o.traceback) st = cuda_status(cudaMemcpyAsync(path_len, d_plen, 4, cudaMemcpyDeviceToHost, s));
         if (!st) st = cuda_status(cudaStreamSynchronize(s));
-        if (!st && o.traceback && path_cap && *path_len)
-            st = cuda_status(cudaMemcpy(h_path, d_path, (uint64_t)std::min(path_cap, *path_len) * 4,
-                                        cudaMemcpyDeviceToHost));
         if (st) return st;
+        *out = *h_res;
+        if (o.traceback) {
+            *path_len = *h_plen;
+            if (path_cap && *path_len)
+                st = cuda_status(cudaMemcpy(h_path, d_path, (uint64_t)std::min(path_cap, *path_len) * 4,
+                                            cudaMemcpyDeviceToHost));
+            if (st) return st;
+        }
         if (out->status == GWFA_ERR_CAPACITY && log2 + 3 <= gwfa::kMaxLog2Tiles) {
             log2 += 3;   // grow the workspace and run again
             continue;
@@ -416,6 +480,7 @@ int gwfa_engine_destroy(gwfa_engine *e) {
     cudaFree(e->counters);
     cudaFree(e->retry_lists);
     cudaFree(e->stage);
+    if (e->host) cudaFreeHost(e->host);
     if (e->stream) cudaStreamDestroy(e->stream);
     delete e;
     return GWFA_OK;
@@ -493,6 +558,7 @@ int gwfa_engine_create(const gwfa_graph *g, const gwfa_engine_config *cfg, gwfa_
     if (!st) st = cuda_status(cudaEventCreateWithFlags(&e->ev_fork, cudaEventDisableTiming));
     if (!st) st = cuda_status(cudaEventCreateWithFlags(&e->ev_join, cudaEventDisableTiming));
     if (!st) st = dmalloc(&e->counters, 256);
+    if (!st) st = ensure_pinned(&e->host, &e->host_bytes, kStagedBatch);
     if (!st) st = engine_retry_capacity(e, cfg->max_queries);
     if (!st) st = cuda_status(cudaStreamSynchronize(e->stream));
     if (st) { gwfa_engine_destroy(e); return st; }
@@ -630,13 +696,14 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
     // it): tier 0 gives up the room of the class CTAs it runs beside
     auto tier_threads = [&](const gwfa_tier &t, uint32_t count) {
         if (t.threads) return t.threads;
-        return e->cfg.threads != kAutoThreads ? e->cfg.threads : auto_threads(count, len, e->sms, o.max_lag);
+        return e->cfg.threads != kAutoThreads ? e->cfg.threads
+                                              : auto_threads(count, len ? len : 4000, e->sms, o.max_lag);
     };
     auto per_sm = [&](uint32_t threads) {
         int b = 1;
         return gwfa::align_occupancy(prune, threads, &b) || b < 1 ? 1u : (uint32_t)b;
     };
-    const uint32_t t0_threads = tier_threads(e->cfg.tiers[0], n - n_huge - n_wide), t0_per_sm = per_sm(t0_threads);
+    const uint32_t t0_threads = tier_threads(e->cfg.tiers[0], n - n_huge - n_wide);
     double yield_sms = 0;
     uint32_t cctas[2] = {0, 0};
     for (int c = 0; c < 2; ++c) {
@@ -644,9 +711,12 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
         cctas[c] = std::min(cls[c].tier->ctas, cls[c].count);
         yield_sms += (double)cctas[c] / per_sm(tier_threads(*cls[c].tier, cctas[c]));
     }
-    const uint32_t t0_max = std::min(e->cfg.tiers[0].ctas, (uint32_t)e->sms * t0_per_sm);
-    const uint32_t t0_yield = (uint32_t)std::ceil(yield_sms * t0_per_sm);
-    const uint32_t t0_ctas = t0_max > t0_yield ? t0_max - t0_yield : 1;
+    auto t0_ctas = [&](uint32_t threads) {
+        const uint32_t fit = per_sm(threads);
+        const uint32_t most = std::min(e->cfg.tiers[0].ctas, (uint32_t)e->sms * fit);
+        const uint32_t yield = (uint32_t)std::ceil(yield_sms * fit);
+        return most > yield ? most - yield : 1u;
+    };
     bool forked = false;
     for (int c = 0; c < 2; ++c) {
         if (!cls[c].count) continue;
@@ -696,10 +766,29 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
         a.slabs = e->slabs[t];
         a.slab_bytes = e->slab_bytes[t];
         a.log2cap = e->cfg.tiers[t].log2_tiles;
-        const uint32_t th = t == 0 ? t0_threads : tier_threads(e->cfg.tiers[t], e->cfg.tiers[t].ctas);
-        st = cuda_status(gwfa::launch_align(a, prune, t == 0 ? t0_ctas : e->cfg.tiers[t].ctas, th, s));
+        const uint32_t most = t == 0 ? a.count_val : n;   // no more CTAs than queries there can be
+        auto launch = [&](uint32_t th, uint32_t ctas) {
+            const int r = cuda_status(gwfa::launch_align(a, prune, std::max(std::min(ctas, most), 1u), th, s));
+            if (!r) e->last_launches++;
+            return r;
+        };
+        if (t > 0) {
+            st = launch(tier_threads(e->cfg.tiers[t], e->cfg.tiers[t].ctas), e->cfg.tiers[t].ctas);
+        } else if (len || e->cfg.tiers[0].threads || e->cfg.threads != kAutoThreads || o.max_lag > 0) {
+            st = launch(t0_threads, t0_ctas(t0_threads));
+        } else {
+            // lengths in device memory only: one launch per width, two of which leave at once
+            // (about 3 us each; the wrong width costs up to 3x, see auto_threads)
+            const uint64_t from[4] = {1ull << 32, wide_from(most, e->sms), mid_from(most, e->sms), 0};
+            const uint32_t width[3] = {1024u, 512u, gwfa::kNarrow};
+            a.n_all = n;
+            for (int w = 0; w < 3 && !st; ++w) {
+                a.len_lo = (uint32_t)std::min<uint64_t>(from[w + 1], 0xFFFFFFFFull);
+                a.len_hi = (uint32_t)std::min<uint64_t>(from[w], 0xFFFFFFFFull);
+                if (a.len_lo < a.len_hi) st = launch(width[w], t0_ctas(width[w]));
+            }
+        }
         if (st) return st;
-        e->last_launches++;
     }
     if (T == 1) return join_classes();
     return GWFA_OK;
@@ -752,15 +841,30 @@ int gwfa_align_batch(gwfa_engine *e, uint32_t n, const char *h_q, const uint64_t
     uint32_t *d_vs = c.take<uint32_t>((uint64_t)n * 4);
     uint32_t *d_ve = c.take<uint32_t>((uint64_t)n * 4);
     uint32_t *d_order = c.take<uint32_t>((uint64_t)n * 4);
+    const uint64_t in_bytes = c.off;   // the inputs come first
     int32_t *d_status = c.take<int32_t>((uint64_t)n * 4);
     uint32_t *d_words = c.take<uint32_t>(words_for(n, nb) * 4);
     gwfa_result *d_out = c.take<gwfa_result>((uint64_t)n * sizeof(gwfa_result));
     nvtxRangePushA("copy in + pack");
-    st = cuda_status(cudaMemcpyAsync(d_q, h_q, nb, cudaMemcpyHostToDevice, s));
-    if (!st) st = cuda_status(cudaMemcpyAsync(d_off, h_q_off, (uint64_t)(n + 1) * 8, cudaMemcpyHostToDevice, s));
-    if (!st) st = cuda_status(cudaMemcpyAsync(d_vs, h_vs, (uint64_t)n * 4, cudaMemcpyHostToDevice, s));
-    if (!st) st = cuda_status(cudaMemcpyAsync(d_ve, h_ve, (uint64_t)n * 4, cudaMemcpyHostToDevice, s));
-    if (!st && h_order) st = cuda_status(cudaMemcpyAsync(d_order, h_order, (uint64_t)n * 4, cudaMemcpyHostToDevice, s));
+    if (in_bytes <= kStagedBatch) {
+        // a small batch is bound by its copies and launches: its arrays are gathered in pinned
+        // memory (the call waits for the batch, so the buffer is free again when it returns)
+        auto put = [&](void *d, const void *h, uint64_t bytes) {
+            if (bytes) memcpy(e->host + ((uint8_t *)d - e->stage), h, bytes);
+        };
+        put(d_q, h_q, nb);
+        put(d_off, h_q_off, (uint64_t)(n + 1) * 8);
+        put(d_vs, h_vs, (uint64_t)n * 4);
+        put(d_ve, h_ve, (uint64_t)n * 4);
+        if (h_order) put(d_order, h_order, (uint64_t)n * 4);
+        st = cuda_status(cudaMemcpyAsync(e->stage, e->host, in_bytes, cudaMemcpyHostToDevice, s));
+    } else {
+        st = cuda_status(cudaMemcpyAsync(d_q, h_q, nb, cudaMemcpyHostToDevice, s));
+        if (!st) st = cuda_status(cudaMemcpyAsync(d_off, h_q_off, (uint64_t)(n + 1) * 8, cudaMemcpyHostToDevice, s));
+        if (!st) st = cuda_status(cudaMemcpyAsync(d_vs, h_vs, (uint64_t)n * 4, cudaMemcpyHostToDevice, s));
+        if (!st) st = cuda_status(cudaMemcpyAsync(d_ve, h_ve, (uint64_t)n * 4, cudaMemcpyHostToDevice, s));
+        if (!st && h_order) st = cuda_status(cudaMemcpyAsync(d_order, h_order, (uint64_t)n * 4, cudaMemcpyHostToDevice, s));
+    }
     if (!st) st = cuda_status(gwfa::launch_pack(n, d_q, d_off, d_words, d_status, s));
     nvtxRangePop();
     nvtxRangePushA("alignment tiers");

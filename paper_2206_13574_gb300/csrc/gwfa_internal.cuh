@@ -140,6 +140,10 @@ struct TierArgs {
     uint32_t *paths;            // traceback: path_cap vertex ids per query id
     uint32_t *path_len;         // traceback: walk length per query id (may exceed path_cap)
     uint32_t path_cap;
+    // run only if the mean length of the batch's n_all queries is in [len_lo, len_hi) (len_hi
+    // 0: always): where the host does not know the lengths it launches every width, and the
+    // device settles which one works
+    uint32_t n_all, len_lo, len_hi;
 };
 constexpr int kStatWords = 8;
 
@@ -203,8 +207,12 @@ struct gwfa_graph {
     mutable uint8_t *plain_slab = nullptr;
     mutable uint32_t plain_log2 = 0;
     mutable bool plain_prune = false;
-    mutable uint8_t *plain_stage = nullptr;   // query bytes + words + counters + result
+    mutable uint8_t *plain_stage = nullptr;   // offsets, ends, work counter, query words | path
     mutable uint64_t plain_stage_bytes = 0;
+    mutable uint8_t *plain_host = nullptr;    // pinned: inputs to copy over, result
+    mutable uint64_t plain_host_bytes = 0;
+    mutable std::vector<uint32_t> seen, bfs;  // host reachability
+    mutable uint32_t seen_call = 0;
     mutable cudaStream_t stream = nullptr;
     gwfa::DevGraph dev() const {
         return gwfa::DevGraph{d_words, d_vx, d_vinfo, d_arc_dst, nv};
@@ -226,6 +234,8 @@ struct gwfa_engine {
     // staging for the host-buffer entry point
     uint8_t *stage = nullptr;
     uint64_t stage_bytes = 0;
+    uint8_t *host = nullptr;        // pinned, for small batches
+    uint64_t host_bytes = 0;
     cudaStream_t stream = nullptr;
     uint64_t device_bytes = 0;
     uint32_t last_launches = 0;

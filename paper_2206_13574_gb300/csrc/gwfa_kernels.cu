@@ -1298,6 +1298,10 @@ __device__ __forceinline__ void align_queries(const TierArgs &A) {
     // were spilled to local memory and reloaded through L1/L2 in the hot phases);
     // visible to all threads after the first barrier of the loop below
     __shared__ Slab<P> s;
+    if (A.len_hi) {
+        const uint64_t len = (A.q_off[A.n_all] - A.q_off[0]) / A.n_all;
+        if (len < A.len_lo || len >= A.len_hi) return;   // the same for every thread of the grid
+    }
     if (threadIdx.x == 0) s = carve<P>(A.slabs + (uint64_t)blockIdx.x * A.slab_bytes, A.log2cap);
     const uint32_t count = A.list_count ? *A.list_count : A.count_val;
     for (;;) {
