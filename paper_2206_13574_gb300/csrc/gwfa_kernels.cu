@@ -128,6 +128,7 @@ struct Score {
     int found, err;
     uint32_t nlink;     // neighbours to be linked after the pass
     int err_next;       // out of room for a tile that only the next score needs
+    uint32_t nt0, nclaim0;   // exact mode: Sh::nt and nclaim when the score began
 };
 
 // CTA-shared state of the query being aligned.
@@ -137,6 +138,7 @@ struct Sh {
     uint32_t nclaim;    // tiles that hold a diagonal (the 3/4 load limit counts these)
     uint32_t nr[3];     // requests / insertions of the spill rounds, rotating
     uint32_t nins[2];
+    uint32_t held;      // see tiles_held
     int nfree;          // memory bound: records on the free list
     uint32_t tlen;      // traceback: entries of T
     uint32_t peak;
@@ -285,9 +287,28 @@ __device__ __forceinline__ uint32_t tile_hash(unsigned long long key, uint32_t m
     return (uint32_t)((key * 0x9E3779B97F4A7C15ull) >> 32) & mask;
 }
 
-// A tile came to hold a diagonal: the load limit of 3/4 of the slab's tiles.
-template <bool P> __device__ __forceinline__ void count_claim(const Slab<P> &s, Sh &sh, int *err) {
-    if (atomicAdd(&sh.nclaim, 1u) + 1 > (s.cap >> 1) + (s.cap >> 2)) atomicCAS(err, 0, GWFA_ERR_CAPACITY);
+// The load limit: 3/4 of the slab's tiles may come to hold a diagonal.
+template <bool P> __device__ __forceinline__ uint32_t load_limit(const Slab<P> &s) { return (s.cap >> 1) + (s.cap >> 2); }
+
+// Records from `first` on that hold a diagonal (or, pruning mode, held one since the last
+// eviction), counted by the whole CTA.  The tiles that the links of a score claim belong to
+// the next score, and a query that ends in this one does not need them; which of both
+// claimed a tile depends on timing, but only the spills have put a diagonal into it.
+template <bool P> __device__ __noinline__ uint32_t tiles_held(const Slab<P> &s, Sh &sh, uint32_t first) {
+    __syncthreads();
+    if (threadIdx.x == 0) sh.held = 0;
+    __syncthreads();
+    uint32_t c = 0;
+    for (uint32_t t = first + threadIdx.x; t < min(sh.nt, s.cap); t += blockDim.x) {
+        if (s.touched[t] == kNone) continue;
+        bool any = false;
+        if constexpr (P) any = s.recs[t].side[1].counted != 0;
+        for (int ln = 0; ln < kTile; ++ln) any = any || s.recs[t].vals[ln] >= 0;
+        c += any;
+    }
+    if (c) atomicAdd(&sh.held, c);
+    __syncthreads();
+    return sh.held;
 }
 
 // An empty record of a tile at kb, written by the thread that claims it, in whole lines:
@@ -331,7 +352,7 @@ __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsign
             if (e.key == kEmptyKey) {
                 s.touched[idx] = h;
                 if constexpr (P) s.tkey[idx] = key;
-                else count_claim<P>(s, sh, err);   // a claimed tile always gets a diagonal
+                else atomicAdd(&sh.nclaim, 1u);   // a claimed tile always gets a diagonal
                 return (int)idx;
             }
         }
@@ -667,7 +688,7 @@ __device__ __forceinline__ void offset_pass(const DevGraph &g, const Slab<P> &s,
             const unsigned has = __ballot_sync(full, inq[0] || inq[1] || raw[0] >= 0 || raw[1] >= 0);
             if (sub == 3 && !counted && on && ((has >> (lane & 28)) & 15u)) {
                 rec->side[1].counted = 1u;
-                count_claim<P>(s, sh, &S.err);
+                if (atomicAdd(&sh.nclaim, 1u) + 1 > load_limit(s)) atomicCAS(&S.err, 0, GWFA_ERR_CAPACITY);
             }
             if (on) {
                 longlong2 r2;
@@ -1133,6 +1154,8 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         Score &S = sh.score[d & 3];
         if (threadIdx.x == blockDim.x - 32) {   // the last warp: the first to run out of tiles
             sh.score[(d + 2) & 3] = Score{};
+            S.nt0 = sh.nt;
+            S.nclaim0 = sh.nclaim;
             sh.nr[0] = 0;
             sh.nins[0] = 0;
         }
@@ -1229,9 +1252,16 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         }
         if (A.stats && threadIdx.x == 0) sh.st[1] += globaltimer_ns() - sh.t_phase;
         if (S.err) { status = S.err; break; }
+        // the load limit, over the tiles that this score needs (rare: a query passes here
+        // once, or in pruning mode ends with most of the slab in use)
+        const bool over = !P && sh.nclaim > load_limit(s);
+        if (over || (P && S.found && sh.nt > load_limit(s))) {
+            const uint32_t held = (P ? 0u : S.nclaim0) + tiles_held<P>(s, sh, P ? 0u : S.nt0);
+            if (held > load_limit(s)) { status = GWFA_ERR_CAPACITY; break; }
+        }
         if (S.found) break;   // end test of Alg. 1
         if (A.max_score >= 0 && d >= A.max_score) { status = GWFA_ERR_SCORE_LIMIT; break; }
-        if (S.err_next) { status = S.err_next; ++d; break; }
+        if (over || S.err_next) { status = GWFA_ERR_CAPACITY; ++d; break; }
     }
     __syncthreads();
     const uint32_t n_tiles = sh.nclaim;

@@ -107,3 +107,25 @@ def test_freed_records_are_used_again():
     for i, w in enumerate(want):
         same(res[i], w, i)
         assert int(res[i]["evicted"]) == w["evicted"] and w["visited"] > 8 * 384
+
+
+@pytest.mark.parametrize("prune", [False, True])
+def test_the_load_limit_does_not_depend_on_timing(prune):
+    """Which queries a slab has room for is the same on CTAs of every width, also for those
+    that end in the very score that brings the tiles to the limit."""
+    g, _ = synth.make_config(2, n_queries=1)
+    graph = gw.Graph.from_synth(g)
+    for seed in range(3):
+        qs = synth.make_queries(g, 600, seed, synth._const(3000), synth._uniform(0.0, 0.08), (1, 1, 1), (1, 1))
+        first = None
+        for threads in (64, 256, 512 if prune else 1024):
+            cfg = gw.default_config(graph, prune=prune)
+            cfg.n_tiers, cfg.threads = 1, threads
+            cfg.tiers[0].log2_tiles = 10
+            eng = gw.Engine(graph, prune=prune, config=cfg)
+            for _ in range(2):
+                status = eng.align_batch(qs.seq, qs.off, qs.v_s, qs.v_e)["status"].copy()
+                first = status if first is None else first
+                assert np.array_equal(status, first), (seed, threads)
+            eng.close()
+        assert 0 < (first == 0).sum() < 600
