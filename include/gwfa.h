@@ -227,7 +227,7 @@ uint64_t gwfa_engine_device_bytes(const gwfa_engine *e);
 /*
  * Host-buffer batch (end to end).  Queries concatenated in h_q (ASCII) with
  * h_q_off[n_queries+1] byte offsets, per-query start/end vertices in
- * h_v_s / h_v_e.  h_order (may be NULL = input order) is the order in which the
+ * h_v_s / h_v_e.  h_order (may be NULL = longest first) is the order in which the
  * work queue hands queries to CTAs (a permutation of 0..n_queries-1), placed by
  * `sched` (NULL = all on tier 0).  The call
  * copies the inputs to the device, packs them (kernel), runs the tiers, copies
@@ -254,7 +254,8 @@ int gwfa_pack_queries_device(uint32_t n_queries, const char *d_q, const uint64_t
  * Device-resident batch (inputs already in HBM): d_words / d_q_off as written
  * by gwfa_pack_queries_device (d_status may be NULL, else queries with a
  * nonzero status are skipped and keep it), d_v_s / d_v_e start/end vertices,
- * d_order the queue order (NULL = 0..n-1) placed by `sched` (NULL = all on
+ * d_order the queue order (NULL = longest first; 0..n-1 with a
+ * `sched`), placed by `sched` (NULL = all on
  * tier 0; host memory), results into d_out[n_queries].
  * Asynchronous on `stream`; no host synchronisation inside.
  */

@@ -492,7 +492,7 @@ static int engine_retry_capacity(gwfa_engine *e, uint64_t n) {
     e->retry_lists = nullptr;
     e->retry_cap = 0;
     uint64_t want = std::max<uint64_t>(n, 1024);
-    if (dmalloc(&e->retry_lists, want * 4 * GWFA_MAX_TIERS)) return GWFA_ERR_OOM;
+    if (dmalloc(&e->retry_lists, want * 4 * (GWFA_MAX_TIERS + 1))) return GWFA_ERR_OOM;
     e->retry_cap = want;
     return GWFA_OK;
 }
@@ -567,7 +567,7 @@ int gwfa_engine_create(const gwfa_graph *g, const gwfa_engine_config *cfg, gwfa_
 }
 
 uint64_t gwfa_engine_device_bytes(const gwfa_engine *e) {
-    return e ? e->device_bytes + e->retry_cap * 4 * GWFA_MAX_TIERS + e->stage_bytes : 0;
+    return e ? e->device_bytes + e->retry_cap * 4 * (GWFA_MAX_TIERS + 1) + e->stage_bytes : 0;
 }
 
 uint32_t gwfa_engine_last_launches(const gwfa_engine *e) { return e ? e->last_launches : 0; }
@@ -677,6 +677,14 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
     // CTAs, concurrently with tier 0, and hand their overflows to the retry tiers
     uint32_t n_huge = sched && e->huge_slabs ? std::min(sched->n_huge, n) : 0;
     uint32_t n_wide = sched && e->wide_slabs ? std::min(sched->n_wide, n - n_huge) : 0;
+    // a batch without an order, and with more queries than the widest CTAs take at once
+    // (997 reads of 1-20 kb: 14.3 ms in input order, 9.4 longest first; the sort takes a few us)
+    if (!d_order && n_huge + n_wide == 0 && n > (uint32_t)e->sms) {
+        uint32_t *order = e->retry_lists + (uint64_t)GWFA_MAX_TIERS * e->retry_cap;
+        st = cuda_status(gwfa::launch_order(n, d_q_off, order, s));
+        if (st) return st;
+        d_order = order;
+    }
     struct Cls {
         const gwfa_tier *tier;
         uint8_t *slabs;
@@ -704,6 +712,11 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
         return gwfa::align_occupancy(prune, threads, &b) || b < 1 ? 1u : (uint32_t)b;
     };
     const uint32_t t0_threads = tier_threads(e->cfg.tiers[0], n - n_huge - n_wide);
+    // (an engine with classes has its own place for heavy queries)
+    const bool few = T > 1 && n <= 4u * (uint32_t)e->sms && !e->wide_slabs && !e->huge_slabs &&
+                     !e->cfg.tiers[0].threads && e->cfg.threads == kAutoThreads &&
+                     e->cfg.tiers[1].log2_tiles > e->cfg.tiers[0].log2_tiles &&
+                     e->cfg.tiers[1].ctas >= std::min(n, (uint32_t)e->sms);
     double yield_sms = 0;
     uint32_t cctas[2] = {0, 0};
     for (int c = 0; c < 2; ++c) {
@@ -768,7 +781,19 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
         a.log2cap = e->cfg.tiers[t].log2_tiles;
         const uint32_t most = t == 0 ? a.count_val : n;   // no more CTAs than queries there can be
         auto launch = [&](uint32_t th, uint32_t ctas) {
-            const int r = cuda_status(gwfa::launch_align(a, prune, std::max(std::min(ctas, most), 1u), th, s));
+            TierArgs b = a;
+            if (t == 0 && th == 1024 && few) {
+                // a few queries, one wide CTA an SM: they start on tier 1's slabs, so that the
+                // heaviest do not run a second time after the others (300 reads with a heavy
+                // tail, 15 to 20 of which overflow tier 0: 67 ms, 46 so)
+                b.slabs = e->slabs[1];
+                b.slab_bytes = e->slab_bytes[1];
+                b.log2cap = e->cfg.tiers[1].log2_tiles;
+                b.retry = T > 2 ? e->retry_lists + e->retry_cap : nullptr;
+                b.retry_count = rcount + 1;
+                ctas = std::min(ctas, e->cfg.tiers[1].ctas);   // (one slab a CTA)
+            }
+            const int r = cuda_status(gwfa::launch_align(b, prune, std::max(std::min(ctas, most), 1u), th, s));
             if (!r) e->last_launches++;
             return r;
         };

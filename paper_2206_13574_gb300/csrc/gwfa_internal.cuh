@@ -183,6 +183,7 @@ cudaError_t launch_align(const TierArgs &a, bool prune, uint32_t ctas, uint32_t 
                          cudaStream_t st);
 cudaError_t launch_pack(uint32_t nq, const char *d_q, const uint64_t *d_off, uint32_t *d_words,
                         int32_t *d_status, cudaStream_t st);
+cudaError_t launch_order(uint32_t n, const uint64_t *d_off, uint32_t *d_order, cudaStream_t st);
 cudaError_t launch_slab_init(uint8_t *slabs, uint64_t slab_bytes, uint32_t n_slabs, uint32_t log2cap,
                              bool prune, cudaStream_t st);
 int align_occupancy(bool prune, uint32_t threads, int *blocks_per_sm);
@@ -229,7 +230,7 @@ struct gwfa_engine {
     cudaStream_t side = nullptr, side2 = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr, ev_join2 = nullptr;
     uint32_t *counters = nullptr;   // per tier: head, retry_count; plus retry lists
-    uint32_t *retry_lists = nullptr;
+    uint32_t *retry_lists = nullptr;   // one per tier, then the order of a batch without one
     uint64_t retry_cap = 0;
     // staging for the host-buffer entry point
     uint8_t *stage = nullptr;

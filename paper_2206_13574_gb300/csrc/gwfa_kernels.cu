@@ -23,8 +23,8 @@
 // at a time fit L2 only while nothing else is fetched for them (10,000 reads 48.3 -> 35.3 ms).
 // Measured against the form with separate extend and expand passes that max-merged
 // candidates with atomics and probed the hash for each one leaving a tile (reads of
-// 1-20 kb): 10,000 reads 101 -> 32.2 ms, 997 reads 49 -> 12.9 ms, 300 with a heavy tail
-// 415 -> 64 ms, 400 pruned 50 kb reads 50.7 -> 23.2 ms, one 10 kb read 8.5 -> 2.1 ms.
+// 1-20 kb): 10,000 reads 101 -> 32 ms, 400 pruned 50 kb reads 50.7 -> 23 ms, one 10 kb
+// read 7.7 -> 1.9 ms.
 // What bounds it: of the ~13,000 cycles a score of one 10 kb read takes, the pass has 5,000
 // (one visit per warp, bound by issue), the second step 7,700: a few warps walk the code
 // of links and spills, one after the other, while the rest wait.  Memory is not it: with
@@ -1516,6 +1516,38 @@ __global__ void pack_kernel(uint32_t nq, const char *__restrict__ q, const uint6
     if (blockIdx.x == 0 && threadIdx.x < 2) words[(off[nq] >> 4) + nq + threadIdx.x] = 0;
 }
 
+// A queue order for a batch that comes without one: longest first, by the length's exponent
+// and five bits of its mantissa (a counting sort of one block; the order within a class of
+// lengths is left to the atomics, results do not depend on it).  A query that starts last
+// ends last, and the longest take a hundred times the median.
+__global__ void __launch_bounds__(1024) order_kernel(uint32_t n, const uint64_t *__restrict__ off,
+                                                     uint32_t *__restrict__ order) {
+    __shared__ uint32_t at[1024], warp_sum[32];
+    const uint32_t tid = threadIdx.x, lane = tid & 31;
+    auto cls = [&](uint32_t i) {
+        const uint32_t len = (uint32_t)min(off[i + 1] - off[i], (uint64_t)0x7FFFFFFF);
+        const uint32_t e = 31 - __clz(len | 1u);
+        return 1023u - (e << 5 | ((len << (31 - e)) >> 26 & 31u));   // longest: class 0
+    };
+    at[tid] = 0;
+    __syncthreads();
+    for (uint32_t i = tid; i < n; i += 1024) atomicAdd(&at[cls(i)], 1u);
+    __syncthreads();
+    const uint32_t mine = at[tid];
+    uint32_t x = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, o);
+        if (lane >= (uint32_t)o) x += y;
+    }
+    if (lane == 31) warp_sum[tid >> 5] = x;
+    __syncthreads();
+    uint32_t before = 0;
+    for (uint32_t w = 0; w < tid >> 5; ++w) before += warp_sum[w];
+    at[tid] = before + x - mine;
+    __syncthreads();
+    for (uint32_t i = tid; i < n; i += 1024) order[atomicAdd(&at[cls(i)], 1u)] = i;
+}
+
 // Slabs start with an empty hash (all ones); everything else is written before it is read.
 __global__ void slab_init_kernel(uint8_t *slabs, uint64_t slab_bytes, uint32_t n_slabs, uint64_t table_bytes) {
     const uint64_t per = table_bytes / 16, total = per * n_slabs;
@@ -1556,6 +1588,11 @@ cudaError_t launch_pack(uint32_t nq, const char *d_q, const uint64_t *d_off, uin
     if (blocks == 0) blocks = 1;
     if (blocks > 65535) blocks = 65535;
     pack_kernel<<<blocks, 256, 0, st>>>(nq, d_q, d_off, d_words, d_status);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_order(uint32_t n, const uint64_t *d_off, uint32_t *d_order, cudaStream_t st) {
+    order_kernel<<<1, 1024, 0, st>>>(n, d_off, d_order);
     return cudaGetLastError();
 }
 

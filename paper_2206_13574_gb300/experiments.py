@@ -170,7 +170,7 @@ def scheduler(n: int = 5000, n_train_c2: int = 3000, n_train_c3: int = 300, n_pl
            "time_coeffs_us": list(coeffs)}
     ref = None
     # (order, n_huge, n_wide, huge CTAs, wide CTAs, threads per huge CTA)
-    plans = {"plain_fifo": (None, 0, 0, 0, 0, 512),
+    plans = {"plain_fifo": (np.arange(len(q4)), 0, 0, 0, 0, 512),
              "plain_longest_first": (np.argsort(-q4.lengths(), kind="stable"), 0, 0, 0, 0, 512)}
     o2, _, nw2 = gw.plan_schedule(pred, int(0.75 * (1 << base.tiers[0].log2_tiles)))
     plans["learned_wide_only"] = (o2, 0, nw2, 0, costmodel.wide_ctas(pred, o2, nw2, total, coeffs), 512)

@@ -89,3 +89,51 @@ def test_single_calls(graph):
     assert (bad["status"], bad["edit_distance"], bad["cells"]) == (gw.GWFA_ERR_INVALID, -1, 0)
     assert gr.align(q, ve, vs)["status"] == gw.GWFA_ERR_UNREACHABLE
     assert gr.align(q, vs, ve)["edit_distance"] == r["edit_distance"]   # and the path works on
+
+
+# more queries than SMs run longest first when the batch brings no order: every length
+# class from empty on, classes of one query and of many, and one query over 1,024 of them
+@pytest.mark.parametrize("n", [153, 305, 1025, 4097])
+def test_batch_without_order(graph, n):
+    import torch
+    g, gr = graph
+    rng = np.random.default_rng(n)
+    lens = np.where(rng.random(n) < 0.1, rng.integers(0, 4, n), (2.0 ** rng.uniform(2, 11, n)).astype(np.int64))
+    qs = synth.make_queries(g, n, n, synth._const(2100), synth._uniform(0.0, 0.02), (1, 1, 1), (1, 1))
+    seq = np.concatenate([np.frombuffer(qs.query(i), np.uint8)[:lens[i]] for i in range(n)])
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.uint64)
+    cut = synth.Queries(seq, off, qs.v_s, qs.v_s, qs.edits, qs.divergence)
+    eng = gw.Engine(gr)
+    want = eng.align_batch(seq, off, cut.v_s, cut.v_e, order=np.arange(n, dtype=np.uint32))
+    batch = gw.DeviceBatch(cut)
+    batch.run(eng)
+    torch.cuda.synchronize()
+    for res in (batch.results(), eng.align_batch(seq, off, cut.v_s, cut.v_e)):
+        for f in FIELDS:
+            assert np.array_equal(res[f], want[f]), f
+
+
+# up to four queries an SM start on tier 1's slabs: tier 0's would overflow here, and some
+# queries leave tier 1's as well (or have no tier to go to)
+@pytest.mark.parametrize("n,tiers", [(20, 3), (152, 3), (300, 3), (300, 2), (300, 1)])
+def test_few_queries_start_on_tier_1(graph, n, tiers):
+    import torch
+    g, gr = graph
+    qs = synth.make_queries(g, n, 5, synth._const(5000), synth._uniform(0.0, 0.08), (1, 1, 1), (1, 1))
+    cfg = gw.default_config(gr)
+    cfg.n_tiers = tiers
+    cfg.tiers[0].log2_tiles, cfg.tiers[1].log2_tiles, cfg.tiers[2].log2_tiles = 8, 12, 17
+    fixed = gw.default_config(gr)
+    fixed.threads, fixed.n_tiers = 256, tiers
+    for t in range(3):
+        fixed.tiers[t].log2_tiles = cfg.tiers[t].log2_tiles
+    want = gw.Engine(gr, config=fixed).align_batch(qs.seq, qs.off, qs.v_s, qs.v_e)
+    eng = gw.Engine(gr, config=cfg)
+    batch = gw.DeviceBatch(qs)
+    batch.run(eng)
+    torch.cuda.synchronize()
+    assert (want["status"] == 0).all() == (tiers == 3)
+    for res in (batch.results(), eng.align_batch(qs.seq, qs.off, qs.v_s, qs.v_e)):
+        assert np.array_equal(res["status"], want["status"])
+        for f in FIELDS:   # a query that ends without room reports what it did until then
+            assert np.array_equal(res[f][want["status"] == 0], want[f][want["status"] == 0]), f
