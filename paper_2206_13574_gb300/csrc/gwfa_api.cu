@@ -717,12 +717,20 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
                      !e->cfg.tiers[0].threads && e->cfg.threads == kAutoThreads &&
                      e->cfg.tiers[1].log2_tiles > e->cfg.tiers[0].log2_tiles &&
                      e->cfg.tiers[1].ctas >= std::min(n, (uint32_t)e->sms);
+    // the classes leave tier 0 half of the SMs, or what their part of tier 0's CTAs (the
+    // measure by which plans size them) leaves it if that is less: a wide CTA takes up to
+    // half an SM (5,000 reads of 1-100 kb, 489 of them on 443 CTAs of 512 threads, two an
+    // SM: with one CTA left for tier 0 the batch takes 13 s, so 0.43)
     double yield_sms = 0;
+    const double part = (double)(std::min(e->cfg.huge.ctas, n_huge) + std::min(e->cfg.wide.ctas, n_wide)) / e->cfg.tiers[0].ctas;
+    const double room = e->sms * std::min(std::max(0.5, part), 0.9);
     uint32_t cctas[2] = {0, 0};
     for (int c = 0; c < 2; ++c) {
         if (!cls[c].count) continue;
         cctas[c] = std::min(cls[c].tier->ctas, cls[c].count);
-        yield_sms += (double)cctas[c] / per_sm(tier_threads(*cls[c].tier, cctas[c]));
+        const double fit = per_sm(tier_threads(*cls[c].tier, cctas[c]));
+        cctas[c] = std::max(std::min(cctas[c], (uint32_t)(std::max(room - yield_sms, 0.0) * fit)), 1u);
+        yield_sms += cctas[c] / fit;
     }
     auto t0_ctas = [&](uint32_t threads) {
         const uint32_t fit = per_sm(threads);

@@ -137,3 +137,23 @@ def test_few_queries_start_on_tier_1(graph, n, tiers):
         assert np.array_equal(res["status"], want["status"])
         for f in FIELDS:   # a query that ends without room reports what it did until then
             assert np.array_equal(res[f][want["status"] == 0], want[f][want["status"] == 0]), f
+
+
+@pytest.mark.parametrize("huge,wide", [(0, 700), (300, 400), (160, 0), (3, 2)])
+def test_more_class_ctas_than_fit(graph, huge, wide):
+    """Classes with more CTAs than the GPU holds beside tier 0 run on fewer."""
+    import torch
+    g, gr = graph
+    qs = synth.make_queries(g, 900, 17, synth._const(1500), synth._uniform(0.0, 0.05), (1, 1, 1), (1, 1))
+    order = np.argsort(-qs.edits, kind="stable").astype(np.uint32)
+    want = gw.Engine(gr).align_batch(qs.seq, qs.off, qs.v_s, qs.v_e)
+    cfg = gw.default_config(gr)
+    cfg.wide.ctas, cfg.wide.log2_tiles, cfg.wide.threads = wide, 14, 512
+    cfg.huge.ctas, cfg.huge.log2_tiles, cfg.huge.threads = huge, 15, 1024
+    eng = gw.Engine(gr, config=cfg)
+    batch = gw.DeviceBatch(qs, order=order)
+    batch.run(eng, n_wide=wide, n_huge=huge)
+    torch.cuda.synchronize()
+    res = batch.results()
+    for f in FIELDS:
+        assert np.array_equal(res[f], want[f]), f
