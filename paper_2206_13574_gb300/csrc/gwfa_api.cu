@@ -689,19 +689,14 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
         const gwfa_tier *tier;
         uint8_t *slabs;
         uint64_t slab_bytes;
-        cudaStream_t side;
-        cudaEvent_t join;
         uint32_t count, offset, *head, *retry, *retry_count;
     } cls[2] = {
-        {&e->cfg.huge, e->huge_slabs, e->huge_slab_bytes, e->side2, e->ev_join2, n_huge, 0,
+        {&e->cfg.huge, e->huge_slabs, e->huge_slab_bytes, n_huge, 0,
          e->counters + 2 * GWFA_MAX_TIERS + 1, T > 1 ? e->retry_lists + (uint64_t)(T - 2) * e->retry_cap : nullptr,
          rcount + (T > 1 ? T - 2 : 0)},
-        {&e->cfg.wide, e->wide_slabs, e->wide_slab_bytes, e->side, e->ev_join, n_wide, n_huge,
+        {&e->cfg.wide, e->wide_slabs, e->wide_slab_bytes, n_wide, n_huge,
          e->counters + 2 * GWFA_MAX_TIERS, T > 1 ? e->retry_lists : nullptr, rcount},
     };
-    // the classes' CTAs and tier 0's must be resident together (tier 0 would
-    // otherwise fill every SM slot and the heaviest queries would start only after
-    // it): tier 0 gives up the room of the class CTAs it runs beside
     auto tier_threads = [&](const gwfa_tier &t, uint32_t count) {
         if (t.threads) return t.threads;
         return e->cfg.threads != kAutoThreads ? e->cfg.threads
@@ -717,11 +712,13 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
                      !e->cfg.tiers[0].threads && e->cfg.threads == kAutoThreads &&
                      e->cfg.tiers[1].log2_tiles > e->cfg.tiers[0].log2_tiles &&
                      e->cfg.tiers[1].ctas >= std::min(n, (uint32_t)e->sms);
+    // the classes' CTAs and tier 0's must be resident together (tier 0 would otherwise fill
+    // every SM and the heaviest queries would start only after it, or the other way round):
     // the classes leave tier 0 half of the SMs, or what their part of tier 0's CTAs (the
     // measure by which plans size them) leaves it if that is less: a wide CTA takes up to
     // half an SM (5,000 reads of 1-100 kb, 489 of them on 443 CTAs of 512 threads, two an
     // SM: with one CTA left for tier 0 the batch takes 13 s, so 0.43)
-    double yield_sms = 0;
+    double taken = 0;   // SMs
     const double part = (double)(std::min(e->cfg.huge.ctas, n_huge) + std::min(e->cfg.wide.ctas, n_wide)) / e->cfg.tiers[0].ctas;
     const double room = e->sms * std::min(std::max(0.5, part), 0.9);
     uint32_t cctas[2] = {0, 0};
@@ -729,23 +726,33 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
         if (!cls[c].count) continue;
         cctas[c] = std::min(cls[c].tier->ctas, cls[c].count);
         const double fit = per_sm(tier_threads(*cls[c].tier, cctas[c]));
-        cctas[c] = std::max(std::min(cctas[c], (uint32_t)(std::max(room - yield_sms, 0.0) * fit)), 1u);
-        yield_sms += cctas[c] / fit;
+        cctas[c] = std::max(std::min(cctas[c], (uint32_t)(std::max(room - taken, 0.0) * fit)), 1u);
+        taken += cctas[c] / fit;
     }
     auto t0_ctas = [&](uint32_t threads) {
-        const uint32_t fit = per_sm(threads);
-        const uint32_t most = std::min(e->cfg.tiers[0].ctas, (uint32_t)e->sms * fit);
-        const uint32_t yield = (uint32_t)std::ceil(yield_sms * fit);
-        return most > yield ? most - yield : 1u;
+        return std::min(e->cfg.tiers[0].ctas, (uint32_t)e->sms * per_sm(threads));
     };
-    bool forked = false;
+    // A class is dispatched before tier 0, which would else leave no SM with room for a wide
+    // CTA until it ends: the first one in the caller's stream itself, the second one event
+    // later, tier 0 another event later.  Tier 0 has all its CTAs: those that
+    // find no room beside the classes start when a class CTA ends (10,000 reads of 1-20 kb,
+    // the longest 25 or 100 in a class of 512-thread CTAs: 44.5 / 50.3 ms with the classes on
+    // side streams and fewer CTAs for tier 0, 33.1 / 34.5 so, 32.7 without a class; a
+    // replayed graph with both classes may still take tier 0 first, 43.2).
+    cudaStream_t ts = s;   // tier 0's
+    const bool two = n_huge && n_wide;
+    if (n_huge || n_wide) {
+        ts = e->side;
+        st = cuda_status(cudaEventRecord(e->ev_fork, s));
+        if (two) {
+            if (!st) st = cuda_status(cudaStreamWaitEvent(e->side2, e->ev_fork, 0));
+            if (!st) st = cuda_status(cudaEventRecord(e->ev_join2, e->side2));
+        }
+        if (!st) st = cuda_status(cudaStreamWaitEvent(ts, two ? e->ev_join2 : e->ev_fork, 0));
+        if (st) return st;
+    }
     for (int c = 0; c < 2; ++c) {
         if (!cls[c].count) continue;
-        if (!forked) {
-            st = cuda_status(cudaEventRecord(e->ev_fork, s));
-            if (st) return st;
-            forked = true;
-        }
         TierArgs a = tier_args(e, d_words, d_q_off, d_vs, d_ve, d_status, o, d_out);
         a.list = d_order;
         a.count_val = cls[c].count;
@@ -757,23 +764,21 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
         a.slab_bytes = cls[c].slab_bytes;
         a.log2cap = cls[c].tier->log2_tiles;
         const uint32_t th = tier_threads(*cls[c].tier, cctas[c]);
-        st = cuda_status(cudaStreamWaitEvent(cls[c].side, e->ev_fork, 0));
-        if (!st) st = cuda_status(gwfa::launch_align(a, prune, cctas[c], th, cls[c].side));
-        if (!st) st = cuda_status(cudaEventRecord(cls[c].join, cls[c].side));
+        st = cuda_status(gwfa::launch_align(a, prune, cctas[c], th, c == 1 && two ? e->side2 : s));
         if (st) return st;
         e->last_launches++;
     }
-    auto join_classes = [&]() -> int {
-        for (int c = 0; c < 2; ++c)
-            if (cls[c].count) {
-                const int r = cuda_status(cudaStreamWaitEvent(s, cls[c].join, 0));
-                if (r) return r;
-            }
-        return GWFA_OK;
+    auto join = [&]() -> int {
+        if (ts == s) return GWFA_OK;
+        int r = cuda_status(cudaEventRecord(e->ev_join, ts));
+        if (!r) r = cuda_status(cudaStreamWaitEvent(s, e->ev_join, 0));
+        if (!r && two) r = cuda_status(cudaEventRecord(e->ev_join2, e->side2));
+        if (!r && two) r = cuda_status(cudaStreamWaitEvent(s, e->ev_join2, 0));
+        return r;
     };
     for (uint32_t t = 0; t < T; ++t) {
         if (t == 1) {
-            st = join_classes();   // the retry tiers also take the classes' overflows
+            st = join();   // the retry tiers also take the classes' overflows
             if (st) return st;
         }
         TierArgs a = tier_args(e, d_words, d_q_off, d_vs, d_ve, d_status, o, d_out);
@@ -801,7 +806,7 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
                 b.retry_count = rcount + 1;
                 ctas = std::min(ctas, e->cfg.tiers[1].ctas);   // (one slab a CTA)
             }
-            const int r = cuda_status(gwfa::launch_align(b, prune, std::max(std::min(ctas, most), 1u), th, s));
+            const int r = cuda_status(gwfa::launch_align(b, prune, std::max(std::min(ctas, most), 1u), th, t == 0 ? ts : s));
             if (!r) e->last_launches++;
             return r;
         };
@@ -823,7 +828,7 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
         }
         if (st) return st;
     }
-    if (T == 1) return join_classes();
+    if (T == 1) return join();
     return GWFA_OK;
 }
 
