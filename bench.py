@@ -299,6 +299,7 @@ def ncu_case(args):
     g, qs = synth.make_config(2, n_queries=args.queries or 2000)
     graph = gw.Graph.from_synth(g)
     c = gw.default_config(graph)
+    c.tiers[0].threads = 256      # the benchmark batch's CTA width: one launch per tier
     c.tiers[0].log2_tiles = 14
     c.tiers[1].ctas, c.tiers[1].log2_tiles = 16, 18
     c.tiers[2].ctas, c.tiers[2].log2_tiles = 1, 21
