@@ -70,8 +70,7 @@ struct FeatGraph {
 constexpr uint32_t kSetCap = 8192;          // table entries per search (power of two)
 constexpr uint32_t kSetLoad = kSetCap / 4 * 3;
 constexpr uint32_t kFeatWarps = 1216;       // warps of the features kernel (8 per SM on 152 SMs)
-// Shared-memory tables of the ordinary case: both searches of a warp in 18 KB.
-constexpr uint32_t kSmCap = 1024, kSmLoad = kSmCap / 4 * 3, kSmFront = 256;
+constexpr uint32_t kSmFront = 256;          // frontier slots of the searches in shared memory
 constexpr uint32_t kEmptyV = 0xFFFFFFFFu;
 
 __device__ __forceinline__ uint64_t feature_budget(uint64_t n) { return (5 * n + 3) / 4 + 64; }
@@ -177,10 +176,15 @@ __device__ void bounded_search(const FeatGraph &fg, const SetScratch &S, int t, 
 // a query); here the tables are in shared memory, frontiers hold table slots, a vertex and
 // its arcs are one 32-byte sector, the forward search runs on the warp's lower half beside
 // the backward one on its upper half, and the counts visit only the vertices reached.  A
-// search that outgrows the tables (about 70 kb of the benchmark's graphs) leaves it to the
-// global-memory form; the lengths, and so the counts, are the same by either.
+// search that outgrows the tables leaves it to the global-memory form; the lengths, and so
+// the counts, are the same by either.  1,024 entries a search (20 KB for both) hold reads of
+// 45 kb on the benchmark's graphs at eight warps an SM; batches of up to four queries an SM
+// get 2,048 and four warps.  Beyond that no search is begun that the graph's mean vertex
+// length says will not fit (60 reads of 50 kb: 3.40 ms in global memory, 0.73 in the
+// larger tables).
 // Measured on 2,000 reads of 1-20 kb (5 Mb graph), features and predictions: 3.37 ms -> 0.64 ms.
-struct SmSet {
+template <int LOG2> struct SmSet {
+    static constexpr uint32_t kSmCap = 1u << LOG2, kSmLoad = kSmCap / 4 * 3;
     uint32_t key[2][kSmCap], dist[2][kSmCap];
     uint16_t fr[2][2][kSmFront];   // per search, by step parity: slots
     uint16_t item[kSmLoad];        // forward search: slots in order of insertion
@@ -188,43 +192,43 @@ struct SmSet {
     uint32_t over;
 };
 
-__device__ __forceinline__ uint32_t sm_hash(uint32_t v) { return (v * 0x9E3779B1u) >> 22; }
-static_assert(kSmCap == 1u << 10, "sm_hash gives 10 bits");
+template <int LOG2> __device__ __forceinline__ uint32_t sm_hash(uint32_t v) { return (v * 0x9E3779B1u) >> (32 - LOG2); }
 
 // slot of v in table t, inserted when absent (-1: no room)
-__device__ __forceinline__ int sm_insert(SmSet &S, int t, uint32_t v) {
-    uint32_t h = sm_hash(v);
-    for (uint32_t p = 0; p < kSmCap; ++p) {
+template <int LOG2> __device__ __forceinline__ int sm_insert(SmSet<LOG2> &S, int t, uint32_t v) {
+    uint32_t h = sm_hash<LOG2>(v);
+    for (uint32_t p = 0; p < S.kSmCap; ++p) {
         uint32_t k = S.key[t][h];
         if (k == kEmptyV) {
             k = atomicCAS(&S.key[t][h], kEmptyV, v);
             if (k == kEmptyV) {
                 const uint32_t i = atomicAdd(&S.fill[t], 1u);
-                if (i >= kSmLoad) return -1;
+                if (i >= S.kSmLoad) return -1;
                 if (t == 0) S.item[i] = (uint16_t)h;
                 return (int)h;
             }
         }
         if (k == v) return (int)h;
-        h = (h + 1) & (kSmCap - 1);
+        h = (h + 1) & (S.kSmCap - 1);
     }
     return -1;
 }
-__device__ __forceinline__ uint32_t sm_find(const SmSet &S, int t, uint32_t v) {
-    uint32_t h = sm_hash(v);
-    for (uint32_t p = 0; p < kSmCap; ++p) {
+template <int LOG2> __device__ __forceinline__ uint32_t sm_find(const SmSet<LOG2> &S, int t, uint32_t v) {
+    uint32_t h = sm_hash<LOG2>(v);
+    for (uint32_t p = 0; p < S.kSmCap; ++p) {
         const uint32_t k = S.key[t][h];
         if (k == v) return S.dist[t][h];
         if (k == kEmptyV) break;
-        h = (h + 1) & (kSmCap - 1);
+        h = (h + 1) & (S.kSmCap - 1);
     }
     return kEmptyV;
 }
 
 // Both bounded searches of one warp; false if one outgrew the tables.
-__device__ __forceinline__ bool sm_search(const FeatGraph &fg, SmSet &S, uint32_t src, uint32_t dst, uint32_t budget) {
+template <int LOG2>
+__device__ __forceinline__ bool sm_search(const FeatGraph &fg, SmSet<LOG2> &S, uint32_t src, uint32_t dst, uint32_t budget) {
     const int lane = threadIdx.x & 31, t = lane >> 4, hl = lane & 15;
-    for (uint32_t i = lane; i < kSmCap; i += 32) {
+    for (uint32_t i = lane; i < S.kSmCap; i += 32) {
         S.key[0][i] = S.key[1][i] = kEmptyV;
         S.dist[0][i] = S.dist[1][i] = kEmptyV;
     }
@@ -306,6 +310,7 @@ __device__ __forceinline__ int kmers_absent(const uint32_t *a, uint64_t n, uint3
 //   3 log1p(arcs inside S)
 //   4 vertices of S with two or more arcs inside S, per kb of query
 //   5 log1p(arcs inside S that lie on a cycle)
+template <int LOG2>
 __global__ void features_kernel(FeatGraph fg, uint32_t nq, const uint32_t *__restrict__ words,
                                 const uint64_t *__restrict__ q_off, const uint32_t *__restrict__ vs,
                                 const uint32_t *__restrict__ ve, float *__restrict__ feat,
@@ -332,8 +337,15 @@ __global__ void features_kernel(FeatGraph fg, uint32_t nq, const uint32_t *__res
         const uint32_t a = min(vs[qi], fg.nv - 1), b = min(ve[qi], fg.nv - 1);
         const uint64_t budget = feature_budget(n);
         uint32_t nverts = 0, narcs = 0, nbub = 0, ncyc = 0;
-        SmSet &M = ((SmSet *)s_sets)[wib];
-        if (budget < 0x40000000ull && sm_search(fg, M, a, b, (uint32_t)budget)) {
+        SmSet<LOG2> &M = ((SmSet<LOG2> *)s_sets)[wib];
+        // a search reaches 1.4 to 1.55 vertices per mean vertex length of its budget (bubbles
+        // side by side; measured on the benchmark's graphs), and one that does not fit is
+        // made twice (700 reads of 50 kb 3.6 -> 4.0 ms)
+        const uint4 vl = __ldg(&fg.vinfo[fg.nv - 1]);
+        const bool fits = budget < 0x40000000ull &&
+                          (fg.nv <= M.kSmLoad ||
+                           budget * fg.nv < (uint64_t)(M.kSmCap * 15 / 32) * 16u * (vl.x + (vl.y + 15) / 16));
+        if (fits && sm_search(fg, M, a, b, (uint32_t)budget)) {
             const uint32_t lim = (uint32_t)budget;
             const uint32_t ni = M.fill[0];
             for (uint32_t i = lane; i < ni; i += 32) {
@@ -776,8 +788,10 @@ int gwfa_model_create(const gwfa_graph *g, uint64_t seed, gwfa_model **out) {
     if (st) { gwfa_model_destroy(m); return st; }
     m->fg = FeatGraph{m->d_kmers, kmers.size(), g->d_vinfo, g->d_arc_dst, m->d_in_off, m->d_in_src,
                       g->d_vx, m->d_vin, m->d_arc_cyc, g->nv};
-    if (cudaFuncSetAttribute(features_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(8 * sizeof(SmSet))) !=
-        cudaSuccess) {
+    if (cudaFuncSetAttribute(features_kernel<10>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(8 * sizeof(SmSet<10>))) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(features_kernel<11>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(4 * sizeof(SmSet<11>))) !=
+            cudaSuccess) {
         gwfa_model_destroy(m);
         return GWFA_ERR_CUDA;
     }
@@ -911,7 +925,10 @@ int gwfa_model_features_device(gwfa_model *m, uint32_t n, const uint32_t *d_word
     cudaStream_t s = (cudaStream_t)stream;   // NULL = the legacy default stream
     // kFeatWarps warps (8 per CTA), each with its own search tables in d_scratch
     const uint32_t blocks = std::min<uint32_t>((n + 7) / 8, kFeatWarps / 8);
-    features_kernel<<<blocks, 256, 8 * sizeof(SmSet), s>>>(m->fg, n, d_words, d_q_off, d_v_s, d_v_e, d_feat, m->d_scratch);
+    if (n <= kFeatWarps / 2)   // one query a warp either way
+        features_kernel<11><<<(n + 3) / 4, 128, 4 * sizeof(SmSet<11>), s>>>(m->fg, n, d_words, d_q_off, d_v_s, d_v_e, d_feat, m->d_scratch);
+    else
+        features_kernel<10><<<blocks, 256, 8 * sizeof(SmSet<10>), s>>>(m->fg, n, d_words, d_q_off, d_v_s, d_v_e, d_feat, m->d_scratch);
     return cstat(cudaGetLastError());
 }
 

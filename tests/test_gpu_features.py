@@ -121,6 +121,15 @@ def test_benchmark_graph(length, n, fits):
     assert (check(g, qs) <= 768) == fits
 
 
+# up to 608 queries get tables for 1,536 vertices a search, more than that 768; searches on
+# both sides of what fits, and some beyond what the mean vertex length says will fit
+@pytest.mark.parametrize("length,n", [(85_000, 12), (118_000, 12), (3000, 609), (52_000, 609)])
+def test_table_sizes(length, n):
+    g, _ = synth.make_config(2, n_queries=1)
+    qs = synth.make_queries(g, n, 77, synth._const(length), synth._const(0.03), (1, 1, 1), (1, 1))
+    check(g, qs)
+
+
 def test_cycles_and_many_arcs():
     rng = np.random.default_rng(5)
     labels = ["".join("ACGT"[c] for c in rng.integers(0, 4, int(rng.integers(1, 40)))) for _ in range(120)]
