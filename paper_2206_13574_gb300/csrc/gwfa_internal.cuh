@@ -102,7 +102,7 @@ __host__ __device__ inline SlabLayout slab_layout(uint32_t log2cap, bool prune) 
     L.list0 = o;   o = align256(o + cap * 8);                  // (record, vertex)
     L.list1 = o;   o = align256(o + cap * 8);
     L.links = o;   o = align256(o + 2 * cap * 8);              // neighbours to be linked
-    L.req = o;     o = align256(o + (prune ? cap * 16 : 4 * cap * 8));   // arc-spill requests of a score
+    L.req = o;     o = align256(o + (prune ? cap * 16 : 4 * cap * 8));   // arc-spill requests of a score (6 cap, see put_req)
     L.reqt = o;    o = align256(o + (prune ? cap * 4 : 0));    // trace index of each request
     L.ins = o;     o = align256(o + (prune ? 2 * cap * 16 : 0));   // diagonals a spill round inserted
     L.freel = o;   o = align256(o + (prune ? cap * 4 : 0));    // records the memory bound freed

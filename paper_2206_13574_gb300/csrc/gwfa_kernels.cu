@@ -466,14 +466,30 @@ __device__ __forceinline__ uint32_t push_trace(const Slab<true> &s, Sh &sh, uint
     return idx;
 }
 
-// Spill lists: the first entries in shared memory, the rest in the slab.
-__device__ __forceinline__ void put_req(const Slab<false> &s, Sh &sh, uint32_t i, uint32_t v, int ku, int *err) {
+// Spill lists: the first entries in shared memory, the rest in the slab.  Exact mode logs a
+// score's requests of all rounds, at most one a diagonal that the score extends, so the
+// 6 cap diagonals of the tiles that the load limit admits always fit (a run of one base can
+// bring them all to the end of their vertices in one score).  More than 2 cap requests are
+// so rare that those beyond are kept as the diagonal alone (record << 3 | diagonal), in half
+// the space; vertex and position are looked up when such a request is read.
+__device__ __forceinline__ uint32_t req_cap(const Slab<false> &s) { return 6 * s.cap; }
+
+__device__ __forceinline__ void put_req(const Slab<false> &s, Sh &sh, uint32_t i, uint32_t v, int ku, uint32_t diag,
+                                        int *err) {
     if (i < 4 * kSmall) ((uint2 *)sh.small)[i] = make_uint2(v, (uint32_t)ku);
-    else if (i < 4 * s.cap) s.req[i] = make_uint2(v, (uint32_t)ku);
+    else if (i < 2 * s.cap) s.req[i] = make_uint2(v, (uint32_t)ku);
+    else if (i < req_cap(s)) ((uint32_t *)s.req)[i + 2 * s.cap] = diag;
     else atomicCAS(err, 0, GWFA_ERR_CAPACITY);
 }
-__device__ __forceinline__ uint2 get_req(const Slab<false> &s, const Sh &sh, uint32_t i) {
-    return i < 4 * kSmall ? ((const uint2 *)sh.small)[i] : s.req[i];
+__device__ __noinline__ uint2 get_req_diag(const DevGraph &g, const Slab<false> &s, uint32_t i) {
+    const uint32_t x = ((const uint32_t *)s.req)[i + 2 * s.cap];
+    const unsigned long long key = ld_ent(&s.table[s.touched[x >> 3]]).key;
+    const uint32_t v = (uint32_t)(key >> 32);
+    return make_uint2(v, (uint32_t)((int)(uint32_t)key * kTile + (int)(x & 7)) + __ldg(&g.vx[2 * (uint64_t)v]).y);
+}
+__device__ __forceinline__ uint2 get_req(const DevGraph &g, const Slab<false> &s, const Sh &sh, uint32_t i) {
+    if (i < 4 * kSmall) return ((const uint2 *)sh.small)[i];
+    return i < 2 * s.cap ? s.req[i] : get_req_diag(g, s, i);
 }
 __device__ __forceinline__ int4 get_req4(const Slab<true> &s, const Sh &sh, uint32_t i) {
     return i < kSmall ? ((const int4 *)sh.small)[i] : s.req4[i];
@@ -722,7 +738,7 @@ __device__ __forceinline__ void offset_pass(const DevGraph &g, const Slab<P> &s,
             if (spill[u]) {
                 const uint32_t at = atomicAdd(&S.nreq, 1u);
                 if constexpr (P) request_spill(s, sh, at, vi.y, ent.y, k[u], base[u], trn[u], TB, &S.err);
-                else put_req(s, sh, at, ent.y, k[u] + (int)vi.y, &S.err);
+                else put_req(s, sh, at, ent.y, k[u] + (int)vi.y, ent.x << 3 | (uint32_t)(2 * sub + u), &S.err);
             }
         // the next score visits this tile if it has a diagonal in Q (lane 1 lists it), and
         // a neighbour that an edge diagonal's candidate enters (lanes 0 and 3)
@@ -799,7 +815,7 @@ __device__ __forceinline__ void spill_round(const DevGraph &g, const Slab<false>
     uint32_t won = 0;
     for (uint32_t b = (threadIdx.x >> 5) * 16; b < n; b += blockDim.x >> 1) {
         const uint32_t r = b + (uint32_t)(lane >> 1);
-        uint2 rq = r < n ? get_req(s, sh, r0 + r) : make_uint2(kNone, 0u);
+        uint2 rq = r < n ? get_req(g, s, sh, r0 + r) : make_uint2(kNone, 0u);
         uint2 wait = make_uint2(kNone, 0u);   // this lane's inserted diagonal that spills in turn
         for (;;) {
             if (rq.x != kNone) {
@@ -824,7 +840,8 @@ __device__ __forceinline__ void spill_round(const DevGraph &g, const Slab<false>
                     enter_next<false>(s, sh, q, (uint32_t)su, u, ku, l, 0u, ui.y, d, 0u, false);
                     if ((uint32_t)l == ui.y) {
                         if (wait.x == kNone) wait = make_uint2(u, (uint32_t)(ku + l));
-                        else put_req(s, sh, r0 + n + atomicAdd(next_count, 1u), u, ku + l, &S.err);
+                        else put_req(s, sh, r0 + n + atomicAdd(next_count, 1u), u, ku + l,
+                                     (uint32_t)su << 3 | (uint32_t)(ku & 7), &S.err);
                     }
                 }
             }
@@ -1228,7 +1245,9 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
             }
             if (solo && any) __syncthreads();
         } else {
+            // the log's end: more requests than it holds were refused, and end the score
             uint32_t r0 = 0;
+            n = min(n, req_cap(s));
             for (int round = 0; n; ++round) {
                 uint32_t *next_count = &sh.nr[round % 3];
                 if (threadIdx.x == 0) sh.nr[(round + 1) % 3] = 0;
@@ -1236,7 +1255,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
                 r0 += n;
                 __syncthreads();
                 n = *next_count;
-                n = min(n, r0 < 4 * s.cap ? 4 * s.cap - r0 : 0u);
+                n = min(n, req_cap(s) - r0);
                 if (A.stats && threadIdx.x == 0 && n) sh.st[2] += 1;
             }
             if (nl && !r0) __syncthreads();

@@ -1,0 +1,85 @@
+"""What a slab has room for, against the CPU oracle: queries that use most of the lists of a
+small slab end on it with the oracle's result, and those whose tiles exceed the load limit
+(3/4 of the slab's) are handed to the next tier."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2206_13574_gb300 as gw
+from paper_2206_13574_gb300 import _build, synth
+
+pytestmark = pytest.mark.gpu
+FIELDS = [("edit_distance", "distance"), ("n_scores", "n_scores"), ("cells", "cells"),
+          ("peak_frontier", "peak"), ("visited", "visited"), ("spills", "spills"),
+          ("pruned", "pruned"), ("is_upper_bound", "is_upper_bound")]
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import torch
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    _build.build()
+    oracle.build()
+
+
+def same(r, w, ctx):
+    assert int(r["status"]) == 0, (ctx, r, w)
+    for a, b in FIELDS:
+        assert int(r[a]) == w[b], (ctx, a, int(r[a]), w[b])
+
+
+def engine(graph, threads, log2, prune=False):
+    """One tier (or two) of four CTAs of `threads` threads."""
+    cfg = gw.default_config(graph, prune=prune)
+    log2 = (log2,) if isinstance(log2, int) else log2
+    cfg.n_tiers = len(log2)
+    for t, lg in enumerate(log2):
+        cfg.tiers[t].ctas, cfg.tiers[t].log2_tiles, cfg.tiers[t].threads = 4, lg, threads
+    return gw.Engine(graph, prune=prune, config=cfg)
+
+
+def batch(queries):
+    off = np.concatenate([[0], np.cumsum([len(q) for q in queries])]).astype(np.uint64)
+    return np.frombuffer(b"".join(queries), np.uint8), off
+
+
+# Score 0 fills 4 n diagonals, and at score 1 all of C, G and T reach the end of their vertex
+# at once: 3 n spill requests, over the 256 kept in shared memory, the 512 kept whole and the
+# 1,024 that half of the slab's diagonals make; 192 tiles are the load limit (n = 383)
+@pytest.mark.parametrize("threads", [64, 256, 1024])
+def test_every_diagonal_spills_in_one_score(threads):
+    g = synth.Graph.from_lists(["A", "C", "G", "T"], [(0, 0), (0, 1), (0, 2), (0, 3), (1, 2), (2, 3), (3, 0)])
+    graph = gw.Graph.from_synth(g)
+    lens = [84, 85, 86, 87, 170, 171, 172, 340, 341, 342, 343, 360, 383, 384, 500]
+    qs = [b"A" * n for n in lens]
+    seq, off = batch(qs)
+    zero, one = [0] * len(qs), [1] * len(qs)
+    want = [oracle.gwfa(g, q, 0, 1) for q in qs]
+    res = engine(graph, threads, 8).align_batch(seq, off, zero, one)
+    for n, r, w in zip(lens, res, want):
+        if n < 384:
+            same(r, w, n)
+        else:
+            assert int(r["status"]) == gw.GWFA_ERR_CAPACITY, n
+    for n, r, w in zip(lens, engine(graph, threads, (8, 11)).align_batch(seq, off, zero, one), want):
+        same(r, w, n)
+
+
+# A free start puts all diagonals of a run of one base on the wavefront at score 0, and every
+# one of them reaches the end of its vertex; 1,528 diagonals are what the load limit admits
+@pytest.mark.parametrize("threads", [64, 1024])
+@pytest.mark.parametrize("size", [255, 257, 511, 513, 1023, 1025, 1300, 1528, 1529])
+def test_free_start_on_a_run_of_one_base(threads, size):
+    g = synth.Graph.from_lists(["A" * size, "GC"], [])
+    graph = gw.Graph.from_synth(g)
+    qs = [b"A" * size, b"A" * size + b"T"]
+    seq, off = batch(qs)
+    res = engine(graph, threads, 8).align_batch(seq, off, [0, 0], [0, 0], ends=1)
+    wide = engine(graph, threads, (8, 11)).align_batch(seq, off, [0, 0], [0, 0], ends=1)
+    for q, a, b in zip(qs, res, wide):
+        w = oracle.gwfa(g, q, 0, 0, ends=1)
+        same(b, w, q[size:])
+        if size <= 1528:
+            same(a, w, q[size:])
+        else:
+            assert int(a["status"]) == gw.GWFA_ERR_CAPACITY
