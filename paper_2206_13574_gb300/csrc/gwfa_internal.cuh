@@ -81,6 +81,13 @@ struct alignas(64) TraceRec {
     uint32_t pad[4];
 };
 
+// Records of a slab of 2^log2 tiles.  A CTA has up to one more in use for each of its threads
+// (see find_or_insert); the quarter above the load limit has room for them but on the
+// smallest slabs.
+__host__ __device__ inline uint32_t slab_records(uint32_t log2cap) {
+    return (1u << log2cap) + (log2cap < 13 ? 1024u : 0u);
+}
+
 // Per-CTA slab layout (all arrays 256-byte aligned), cap = 2^log2 tiles: the hash (twice
 // as many entries as tiles, all ones = empty), the records, the hash position of each
 // record and its list stamp, then the two tile lists and the spill lists.
@@ -91,23 +98,23 @@ struct SlabLayout {
 __host__ __device__ inline uint64_t align256(uint64_t x) { return (x + 255) & ~255ull; }
 
 __host__ __device__ inline SlabLayout slab_layout(uint32_t log2cap, bool prune) {
-    const uint64_t cap = 1ull << log2cap;
+    const uint64_t cap = 1ull << log2cap, rcap = slab_records(log2cap);
     SlabLayout L;
     uint64_t o = 0;
     L.table = o;   o = align256(o + 2 * cap * sizeof(TabEnt));
-    L.recs = o;    o = align256(o + cap * (prune ? sizeof(RecT<long long>) : sizeof(RecT<int>)));
-    L.touched = o; o = align256(o + cap * 4);
-    L.stamp = o;   o = align256(o + cap * 4);
-    L.tkey = o;    o = align256(o + (prune ? cap * 8 : 0));    // keys by record (memory bound)
-    L.list0 = o;   o = align256(o + cap * 8);                  // (record, vertex)
-    L.list1 = o;   o = align256(o + cap * 8);
-    L.links = o;   o = align256(o + 2 * cap * 8);              // neighbours to be linked
+    L.recs = o;    o = align256(o + rcap * (prune ? sizeof(RecT<long long>) : sizeof(RecT<int>)));
+    L.touched = o; o = align256(o + rcap * 4);
+    L.stamp = o;   o = align256(o + rcap * 4);
+    L.tkey = o;    o = align256(o + (prune ? rcap * 8 : 0));    // keys by record (memory bound)
+    L.list0 = o;   o = align256(o + rcap * 8);                  // (record, vertex)
+    L.list1 = o;   o = align256(o + rcap * 8);
+    L.links = o;   o = align256(o + 2 * rcap * 8);              // neighbours to be linked
     L.req = o;     o = align256(o + (prune ? cap * 16 : 4 * cap * 8));   // arc-spill requests of a score (6 cap, see put_req)
     L.reqt = o;    o = align256(o + (prune ? cap * 4 : 0));    // trace index of each request
     L.ins = o;     o = align256(o + (prune ? 2 * cap * 16 : 0));   // diagonals a spill round inserted
-    L.freel = o;   o = align256(o + (prune ? cap * 4 : 0));    // records the memory bound freed
+    L.freel = o;   o = align256(o + (prune ? rcap * 4 : 0));    // records the memory bound freed
     L.trace = o;   o = align256(o + (prune ? cap * 2 * 8 : 0));   // Alg. 5's T: (v, t) pairs
-    L.trec = o;    o = align256(o + (prune ? cap * sizeof(TraceRec) : 0));
+    L.trec = o;    o = align256(o + (prune ? rcap * sizeof(TraceRec) : 0));
     L.total = o;
     return L;
 }

@@ -91,7 +91,7 @@ template <bool P> struct Slab {
     uint4 *ins;
     uint2 *trace;
     TraceRec *trec;
-    uint32_t cap, tmask;
+    uint32_t cap, rcap, tmask;
 };
 
 template <bool P>
@@ -114,6 +114,7 @@ __device__ __forceinline__ Slab<P> carve(uint8_t *base, uint32_t log2cap) {
     s.trace = (uint2 *)(base + L.trace);
     s.trec = (TraceRec *)(base + L.trec);
     s.cap = 1u << log2cap;
+    s.rcap = slab_records(log2cap);
     s.tmask = 2 * s.cap - 1;
     return s;
 }
@@ -128,7 +129,6 @@ struct Score {
     int found, err;
     uint32_t nlink;     // neighbours to be linked after the pass
     int err_next;       // out of room for a tile that only the next score needs
-    uint32_t nt0, nclaim0;   // exact mode: Sh::nt and nclaim when the score began
 };
 
 // CTA-shared state of the query being aligned.
@@ -155,6 +155,12 @@ struct Sh {
     uint2 link[kLink];            // (record | side << 31, vertex)
     uint32_t bits[2][kBitTiles / 32];
 };
+// With a record per thread behind it, see find_or_insert (a CTA's width is the kernel's).
+template <int Threads> struct ShOf {
+    Sh sh;
+    uint32_t spare[Threads];
+};
+__device__ __forceinline__ uint32_t &spare_record(Sh &sh) { return ((uint32_t *)(&sh + 1))[threadIdx.x]; }
 
 __device__ __forceinline__ unsigned long long globaltimer_ns() {
     unsigned long long t;
@@ -290,16 +296,16 @@ __device__ __forceinline__ uint32_t tile_hash(unsigned long long key, uint32_t m
 // The load limit: 3/4 of the slab's tiles may come to hold a diagonal.
 template <bool P> __device__ __forceinline__ uint32_t load_limit(const Slab<P> &s) { return (s.cap >> 1) + (s.cap >> 2); }
 
-// Records from `first` on that hold a diagonal (or, pruning mode, held one since the last
-// eviction), counted by the whole CTA.  The tiles that the links of a score claim belong to
-// the next score, and a query that ends in this one does not need them; which of both
-// claimed a tile depends on timing, but only the spills have put a diagonal into it.
-template <bool P> __device__ __noinline__ uint32_t tiles_held(const Slab<P> &s, Sh &sh, uint32_t first) {
+// Records that hold a diagonal (or, pruning mode, held one since the last eviction), counted
+// by the whole CTA.  The tiles that the links of a score claim belong to the next score, and
+// a query that ends in this one does not need them; which of both claimed a tile depends on
+// timing, but only the spills have put a diagonal into it.
+template <bool P> __device__ __noinline__ uint32_t tiles_held(const Slab<P> &s, Sh &sh) {
     __syncthreads();
     if (threadIdx.x == 0) sh.held = 0;
     __syncthreads();
     uint32_t c = 0;
-    for (uint32_t t = first + threadIdx.x; t < min(sh.nt, s.cap); t += blockDim.x) {
+    for (uint32_t t = threadIdx.x; t < min(sh.nt, s.rcap); t += blockDim.x) {
         if (s.touched[t] == kNone) continue;
         bool any = false;
         if constexpr (P) any = s.recs[t].side[1].counted != 0;
@@ -329,7 +335,15 @@ template <bool P> __device__ __forceinline__ void empty_record(const Slab<P> &s,
 }
 
 // Record of tile (v, kb), claimed if absent; -1 (and *err) when the slab is full.  The
-// first probe is inline, the rest (and the claim) is not.
+// first probe is inline, the rest (and the claim) is not.  A claim puts key and record into
+// the table at once, so it brings a record along, and where several threads meet at one new
+// tile (the eight diagonals of a neighbour do, and the two vertices of a bubble) all but one
+// are left with theirs.  Such a thread keeps it for its next claim: a slab then has at most
+// one record a thread in use beside its tiles, and what it has room for does not depend on
+// how often they meet (without, 255 spills at once into 32 tiles used 255 records, and a read
+// under the memory bound lost one at every bubble, for good).  It costs 0 to 1% (pruned
+// 22.8 -> 23.1 ms); to claim the key first and have the others wait for the record costs
+// them a poll (10,000 reads 32.5 -> 37.5 ms).
 template <bool P>
 __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsigned long long key, uint32_t h, Ent e,
                                                 int *err) {
@@ -338,13 +352,18 @@ __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsign
         if (probe > 0) e = ld_ent(&s.table[h]);
         if (e.key == kEmptyKey) {
             if (idx == kNone) {
-                if constexpr (P) {
-                    const int f = sh.nfree > 0 ? atomicSub(&sh.nfree, 1) : 0;
-                    idx = f > 0 ? s.freel[f - 1] : atomicAdd(&sh.nt, 1u);
+                idx = spare_record(sh);
+                if (idx != kNone) {
+                    spare_record(sh) = kNone;
                 } else {
-                    idx = atomicAdd(&sh.nt, 1u);
+                    if constexpr (P) {
+                        const int f = sh.nfree > 0 ? atomicSub(&sh.nfree, 1) : 0;
+                        idx = f > 0 ? s.freel[f - 1] : atomicAdd(&sh.nt, 1u);
+                    } else {
+                        idx = atomicAdd(&sh.nt, 1u);
+                    }
+                    if (idx >= s.rcap) break;
                 }
-                if (idx >= s.cap) break;
                 empty_record<P>(s, idx, (int)(uint32_t)key);
                 __threadfence_block();   // before the key that leads others to it
             }
@@ -357,8 +376,9 @@ __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsign
             }
         }
         if (e.key == key) {
+            if (idx != kNone) spare_record(sh) = idx;
             __threadfence_block();
-            return (int)e.idx;   // a record taken for a lost race stays unused
+            return (int)e.idx;
         }
         h = (h + 1) & s.tmask;
     }
@@ -1011,7 +1031,7 @@ __device__ __forceinline__ void extend_spilled(const DevGraph &g, const Slab<tru
 // Empty the hash entries of a query; in exact mode, which never removes a diagonal from
 // H~, also count the diagonals its records hold (the visited ones).
 template <bool P> __device__ void wipe(const Slab<P> &s, Sh &sh) {
-    const uint32_t nt = min(sh.nt, s.cap);
+    const uint32_t nt = min(sh.nt, s.rcap);
     for (uint32_t t = threadIdx.x; t < nt; t += blockDim.x) {
         const uint32_t h = s.touched[t];
         if (h != kNone) *(uint4 *)&s.table[h] = make_uint4(~0u, ~0u, ~0u, ~0u);
@@ -1037,7 +1057,7 @@ template <bool P> __device__ void wipe(const Slab<P> &s, Sh &sh) {
 // freed record, are dropped and found again on use.  A removed diagonal may be inserted
 // again later, like any absent one.
 __device__ void evict_behind(const Slab<true> &s, Sh &sh, long long amax, int lag, int d) {
-    const uint32_t nt = min(sh.nt, s.cap);
+    const uint32_t nt = min(sh.nt, s.rcap);
     for (uint32_t t = threadIdx.x; t < nt; t += blockDim.x) {
         const uint32_t h = s.touched[t];
         if (h != kNone) *(uint4 *)&s.table[h] = make_uint4(~0u, ~0u, ~0u, ~0u);
@@ -1050,7 +1070,7 @@ __device__ void evict_behind(const Slab<true> &s, Sh &sh, long long amax, int la
     uint32_t ev = 0;
     for (uint32_t t = threadIdx.x; t < nt; t += blockDim.x) {
         const unsigned long long key = s.tkey[t];
-        if (key == kEmptyKey) continue;   // free, or never used
+        if (key == kEmptyKey) continue;   // free, or some thread's spare
         const int kb = (int)(uint32_t)(key & 0xFFFFFFFFull);
         bool any = false;
 #pragma unroll
@@ -1110,6 +1130,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         return;
     }
     // Alg. 1 initialisation: H~_{v_s,0} <- 0, Q <- [(v_s, 0)], d <- 0
+    spare_record(sh) = kNone;
     if (threadIdx.x == 0) {
         sh.t_start = globaltimer_ns();
         for (int i = 0; i < 6; ++i) sh.st[i] = 0;
@@ -1171,8 +1192,6 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         Score &S = sh.score[d & 3];
         if (threadIdx.x == blockDim.x - 32) {   // the last warp: the first to run out of tiles
             sh.score[(d + 2) & 3] = Score{};
-            S.nt0 = sh.nt;
-            S.nclaim0 = sh.nclaim;
             sh.nr[0] = 0;
             sh.nins[0] = 0;
         }
@@ -1275,8 +1294,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         // once, or in pruning mode ends with most of the slab in use)
         const bool over = !P && sh.nclaim > load_limit(s);
         if (over || (P && S.found && sh.nt > load_limit(s))) {
-            const uint32_t held = (P ? 0u : S.nclaim0) + tiles_held<P>(s, sh, P ? 0u : S.nt0);
-            if (held > load_limit(s)) { status = GWFA_ERR_CAPACITY; break; }
+            if (tiles_held<P>(s, sh) > load_limit(s)) { status = GWFA_ERR_CAPACITY; break; }
         }
         if (S.found) break;   // end test of Alg. 1
         if (A.max_score >= 0 && d >= A.max_score) { status = GWFA_ERR_SCORE_LIMIT; break; }
@@ -1339,9 +1357,10 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
 }
 
 // The persistent loop of a CTA: pull a query id, run its score loop, repeat.
-template <bool P, bool TB>
+template <bool P, bool TB, int Threads>
 __device__ __forceinline__ void align_queries(const TierArgs &A) {
-    __shared__ Sh sh;
+    __shared__ ShOf<Threads> shared;
+    Sh &sh = shared.sh;
     // the slab's array pointers are the same for every thread: held once in shared
     // memory rather than in each thread's registers (where, at 32 registers, they
     // were spilled to local memory and reloaded through L1/L2 in the hot phases);
@@ -1375,14 +1394,14 @@ __device__ __forceinline__ void align_queries(const TierArgs &A) {
 // with spill_step).
 template <bool P, bool TB>
 __global__ void __launch_bounds__(kNarrow, P ? 4 : 6) align_kernel(TierArgs A) {
-    align_queries<P, TB>(A);
+    align_queries<P, TB, kNarrow>(A);
 }
 
 // Up to 1024 threads, 64 registers: more groups on one query, for batches and queries
 // whose own latency is the bound.
 template <bool P, bool TB>
 __global__ void __launch_bounds__(1024, 1) align_kernel_wide(TierArgs A) {
-    align_queries<P, TB>(A);
+    align_queries<P, TB, 1024>(A);
 }
 
 __device__ __forceinline__ unsigned long long ld_acquire_sys(const unsigned long long *p) {
@@ -1408,7 +1427,8 @@ __device__ __forceinline__ void st_release_sys(unsigned long long *p, unsigned l
 template <bool P, int PerSm>
 __global__ void __launch_bounds__(512, PerSm) server_kernel(ServerArgs S) {
     uint32_t *const qst = S.stage + (uint64_t)blockIdx.x * S.slot_words;   // the request's packed words
-    __shared__ Sh sh;
+    __shared__ ShOf<512> shared;
+    Sh &sh = shared.sh;
     __shared__ unsigned long long s_ticket;
     __shared__ uint64_t s_qoff[2];
     __shared__ uint32_t s_vs, s_ve;

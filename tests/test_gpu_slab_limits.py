@@ -83,3 +83,55 @@ def test_free_start_on_a_run_of_one_base(threads, size):
             same(a, w, q[size:])
         else:
             assert int(a["status"]) == gw.GWFA_ERR_CAPACITY
+
+
+def bubble_chain(rng, sites, seg):
+    """Segments of `seg` bases with a bubble of two single bases after each, and a walk through."""
+    labels, arcs, walk = [], [], []
+    for _ in range(sites):
+        at = len(labels)
+        labels.append("".join("ACGT"[c] for c in rng.integers(0, 4, seg)))
+        a, b = rng.permutation(4)[:2]
+        labels += ["ACGT"[a], "ACGT"[b]]
+        arcs += [(at, at + 1), (at, at + 2), (at + 1, at + 3), (at + 2, at + 3)]
+        walk += [at, at + 1 + int(rng.integers(2))]
+    labels.append("ACGTTGCA")
+    return synth.Graph.from_lists(labels, arcs), walk + [len(labels) - 1]
+
+
+def noisy(rng, text, rate):
+    q = np.searchsorted(np.frombuffer(b"ACGT", np.uint8), np.frombuffer(text, np.uint8))
+    q = np.where(rng.random(len(q)) < rate, rng.integers(0, 4, len(q)), q)
+    q = np.repeat(q, rng.choice([0, 1, 2], len(q), p=[rate / 2, 1 - rate, rate / 2]))
+    return bytes(np.frombuffer(b"ACGT", np.uint8)[q])
+
+
+# The eight diagonals of a tile of the run spill into one tile each, many at once: a tile uses
+# up one record however many threads meet there (192 are the load limit)
+@pytest.mark.parametrize("threads", [64, 256, 1024])
+@pytest.mark.parametrize("size", [255, 257, 511, 513, 755])
+def test_spills_that_meet_at_one_tile(threads, size):
+    g = synth.Graph.from_lists(["A" * size, "GC"], [(0, 1)])
+    qs = [b"A" * size + t for t in (b"GC", b"TC", b"C")]
+    seq, off = batch(qs)
+    res = engine(gw.Graph.from_synth(g), threads, 8).align_batch(seq, off, [0] * 3, [1] * 3, ends=1)
+    for q, r in zip(qs, res):
+        same(r, oracle.gwfa(g, q, 0, 1, ends=1), q[size:])
+
+
+# Behind a bubble both of its vertices spill into the same tiles in the same round.  Under the
+# memory bound a long query passes thousands of bubbles on a slab of 256 tiles.
+@pytest.mark.parametrize("threads", [32, 256])
+def test_bubbles_under_the_memory_bound(threads):
+    rng = np.random.default_rng(threads)
+    g, walk = bubble_chain(rng, 1500, 12)
+    text = b"".join(g.label(v) for v in walk)
+    qs = [noisy(rng, text, e) for e in (0.01, 0.02, 0.03, 0.03)]
+    seq, off = batch(qs)
+    opts = dict(evict_lag=60, evict_every=4)
+    res = engine(gw.Graph.from_synth(g), threads, 8, prune=True).align_batch(
+        seq, off, [0] * 4, [walk[-1]] * 4, max_lag=60, **opts)
+    for i, (q, r) in enumerate(zip(qs, res)):
+        w = oracle.gwfa(g, q, 0, walk[-1], a_diff=60, **opts)
+        same(r, w, i)
+        assert int(r["evicted"]) == w["evicted"]
