@@ -111,7 +111,7 @@ __host__ __device__ inline SlabLayout slab_layout(uint32_t log2cap, bool prune) 
     L.links = o;   o = align256(o + 2 * rcap * 8);              // neighbours to be linked
     L.req = o;     o = align256(o + (prune ? cap * 16 : 4 * cap * 8));   // arc-spill requests of a score (6 cap, see put_req)
     L.reqt = o;    o = align256(o + (prune ? cap * 4 : 0));    // trace index of each request
-    L.ins = o;     o = align256(o + (prune ? 2 * cap * 16 : 0));   // diagonals a spill round inserted
+    L.ins = o;     o = align256(o + (prune ? 6 * cap * 4 : 0));   // diagonals a spill round inserted
     L.freel = o;   o = align256(o + (prune ? rcap * 4 : 0));    // records the memory bound freed
     L.trace = o;   o = align256(o + (prune ? cap * 2 * 8 : 0));   // Alg. 5's T: (v, t) pairs
     L.trec = o;    o = align256(o + (prune ? rcap * sizeof(TraceRec) : 0));

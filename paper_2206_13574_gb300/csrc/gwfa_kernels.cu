@@ -88,7 +88,7 @@ template <bool P> struct Slab {
     unsigned long long *tkey;   // the rest: pruning mode only
     uint32_t *freel, *reqt;
     int4 *req4;
-    uint4 *ins;
+    uint32_t *ins;
     uint2 *trace;
     TraceRec *trec;
     uint32_t cap, rcap, tmask;
@@ -110,7 +110,7 @@ __device__ __forceinline__ Slab<P> carve(uint8_t *base, uint32_t log2cap) {
     s.freel = (uint32_t *)(base + L.freel);
     s.reqt = (uint32_t *)(base + L.reqt);
     s.req4 = (int4 *)(base + L.req);
-    s.ins = (uint4 *)(base + L.ins);
+    s.ins = (uint32_t *)(base + L.ins);
     s.trace = (uint2 *)(base + L.trace);
     s.trec = (TraceRec *)(base + L.trec);
     s.cap = 1u << log2cap;
@@ -325,7 +325,6 @@ template <bool P> __device__ __forceinline__ void empty_record(const Slab<P> &s,
     if constexpr (P) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) p[i] = i == 5 || i == 7 ? make_uint4(o, (uint32_t)kb, 0u, 0u) : make_uint4(o, o, o, o);
-        s.tkey[idx] = kEmptyKey;
     } else {
         p[0] = p[1] = make_uint4(o - 1, o - 1, o - 1, o - 1);   // kAbsent
         p[2] = p[3] = make_uint4(o, o, o, (uint32_t)kb);
@@ -365,18 +364,21 @@ __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsign
                     if (idx >= s.rcap) break;
                 }
                 empty_record<P>(s, idx, (int)(uint32_t)key);
+                if constexpr (P) s.tkey[idx] = key;
                 __threadfence_block();   // before the key that leads others to it
             }
             e = cas_ent(&s.table[h], key, idx);
             if (e.key == kEmptyKey) {
                 s.touched[idx] = h;
-                if constexpr (P) s.tkey[idx] = key;
-                else atomicAdd(&sh.nclaim, 1u);   // a claimed tile always gets a diagonal
+                if constexpr (!P) atomicAdd(&sh.nclaim, 1u);   // a claimed tile always gets a diagonal
                 return (int)idx;
             }
         }
         if (e.key == key) {
-            if (idx != kNone) spare_record(sh) = idx;
+            if (idx != kNone) {
+                spare_record(sh) = idx;
+                if constexpr (P) s.tkey[idx] = kEmptyKey;
+            }
             __threadfence_block();
             return (int)e.idx;
         }
@@ -510,6 +512,20 @@ __device__ __noinline__ uint2 get_req_diag(const DevGraph &g, const Slab<false> 
 __device__ __forceinline__ uint2 get_req(const DevGraph &g, const Slab<false> &s, const Sh &sh, uint32_t i) {
     if (i < 4 * kSmall) return ((const uint2 *)sh.small)[i];
     return i < 2 * s.cap ? s.req[i] : get_req_diag(g, s, i);
+}
+// Pruning mode: insertion i of a round, (record, vertex, diagonal).  There is room for the
+// 6 cap diagonals that the load limit admits (a vertex with many arcs inserts more than it
+// requests); beyond the first ones an entry is record << 3 | diagonal.
+__device__ __forceinline__ void put_ins(const Slab<true> &s, Sh &sh, uint32_t i, uint32_t rec, uint32_t v, int k, int *err) {
+    if (i < kSmall) sh.small[kSmall + i] = make_uint4(rec, v, (uint32_t)k, 0u);
+    else if (i < 6 * s.cap) s.ins[i] = rec << 3 | (uint32_t)(k & 7);
+    else atomicCAS(err, 0, GWFA_ERR_CAPACITY);
+}
+__device__ __forceinline__ uint4 get_ins(const Slab<true> &s, const Sh &sh, uint32_t i) {
+    if (i < kSmall) return sh.small[kSmall + i];
+    const uint32_t x = s.ins[i];
+    const unsigned long long key = s.tkey[x >> 3];
+    return make_uint4(x >> 3, (uint32_t)(key >> 32), (uint32_t)key * kTile + (x & 7), 0u);
 }
 __device__ __forceinline__ int4 get_req4(const Slab<true> &s, const Sh &sh, uint32_t i) {
     return i < kSmall ? ((const int4 *)sh.small)[i] : s.req4[i];
@@ -903,9 +919,7 @@ __device__ __forceinline__ void apply_spills(const DevGraph &g, const Slab<true>
             if (g_max(&s.recs[su].vals[ku & 7], cand) >= 0) continue;
             ++won;
             if (traceback) s.trec[su].tr[ku & 7] = 0u;   // set by resolve_spill_traces
-            const uint32_t i = atomicAdd(n_ins, 1u);
-            if (i < 2 * s.cap) *(i < kSmall ? &sh.small[kSmall + i] : &s.ins[i]) = make_uint4((uint32_t)su, u, (uint32_t)ku, 0u);
-            else atomicCAS(&S.err, 0, GWFA_ERR_CAPACITY);
+            put_ins(s, sh, atomicAdd(n_ins, 1u), (uint32_t)su, u, ku, &S.err);
         }
     }
     if (won) {
@@ -1009,8 +1023,8 @@ __device__ __forceinline__ bool spill_step(const DevGraph &g, const Slab<true> &
 __device__ __forceinline__ void extend_spilled(const DevGraph &g, const Slab<true> &s, Sh &sh, const QCtx &q, int d,
                                                uint32_t n, uint32_t *n_req, uint32_t nthr, bool traceback) {
     Score &S = sh.score[d & 3];
-    for (uint32_t r = threadIdx.x; r < min(n, 2 * s.cap); r += nthr) {
-        const uint4 in = r < kSmall ? sh.small[kSmall + r] : s.ins[r];
+    for (uint32_t r = threadIdx.x; r < min(n, 6 * s.cap); r += nthr) {
+        const uint4 in = get_ins(s, sh, r);
         const int k = (int)in.z;
         const uint2 vi = __ldg((const uint2 *)&g.vx[2 * (uint64_t)in.y]);
         const uint32_t base = pbase(s.recs[in.x].vals[k & 7]);

@@ -135,3 +135,28 @@ def test_bubbles_under_the_memory_bound(threads):
         w = oracle.gwfa(g, q, 0, walk[-1], a_diff=60, **opts)
         same(r, w, i)
         assert int(r["evicted"]) == w["evicted"]
+
+
+# A round of spills into a vertex with many arcs inserts more diagonals than it has requests:
+# over the 64 kept in shared memory, and over twice the tiles of the slab (traceback runs on
+# the pruning kernel).  160 bases make 1,288 insertions into 189 tiles.
+@pytest.mark.parametrize("threads", [32, 256, 1024])
+@pytest.mark.parametrize("size", [1, 7, 8, 31, 32, 63, 64, 65, 120, 160])
+def test_insertions_of_a_vertex_with_many_arcs(threads, size):
+    import torch
+    ends = ["ACG", "CAT", "CGT", "GCA", "GTT", "TAC", "TCC", "TGA"]
+    g = synth.Graph.from_lists(["A" * size] + ends, [(0, 1 + i) for i in range(8)])
+    qs = [b"A" * size + t for t in ((b"CGT", b"CT", b"CAGT") if size < 64 else (b"CGT",))]   # (T holds 512 requests)
+    n = len(qs)
+    seq, off = batch(qs)
+    vs, ve = np.zeros(n, np.uint32), np.full(n, 3, np.uint32)
+    b = gw.DeviceBatch(synth.Queries(seq.copy(), off, vs, ve, np.zeros(n, np.int64), np.zeros(n)))
+    eng = engine(gw.Graph.from_synth(g), threads, 8, prune=True)
+    paths = torch.zeros(n * 8, dtype=torch.int32, device="cuda")
+    plen = torch.zeros(n, dtype=torch.int32, device="cuda")
+    eng.set_paths(paths.data_ptr(), 8, plen.data_ptr())
+    b.run(eng, traceback=True, ends=1)
+    torch.cuda.synchronize()
+    for i, (q, r) in enumerate(zip(qs, b.results())):
+        same(r, oracle.gwfa(g, q, 0, 3, ends=1), q[size:])
+        assert plen[i].item() == 2 and paths[8 * i:8 * i + 2].tolist() == [0, 3]
