@@ -246,8 +246,11 @@ __device__ __forceinline__ bool sm_search(const FeatGraph &fg, SmSet<LOG2> &S, u
     }
     __syncwarp();
     for (int cur = 0;; cur ^= 1) {
+        // `over` is read before the vote, the same by every lane, as none has gone on to the
+        // body, which may set it
         const uint32_t nf = S.nf[t][cur];
-        if (!__any_sync(0xFFFFFFFFu, nf > 0) || S.over) break;
+        const bool over = S.over != 0;
+        if (!__any_sync(0xFFFFFFFFu, nf > 0 && !over)) return !over;
         for (uint32_t i = hl; i < nf; i += 16) {
             const uint32_t h = S.fr[t][cur][i], v = S.key[t][h];
             const uint4 *rec = (t ? fg.vin : fg.vx) + 2 * (uint64_t)v;
@@ -276,7 +279,6 @@ __device__ __forceinline__ bool sm_search(const FeatGraph &fg, SmSet<LOG2> &S, u
         if (hl == 0) S.nf[t][cur] = 0;
         __syncwarp();
     }
-    return S.over == 0;
 }
 
 __device__ __forceinline__ uint32_t qwindow16(const uint32_t *w, uint64_t p) {

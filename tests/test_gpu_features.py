@@ -143,3 +143,23 @@ def test_cycles_and_many_arcs():
     ve[0] = 119
     qs = synth.Queries(seq, np.arange(m + 1, dtype=np.uint64) * 100, vs, ve, np.zeros(m, np.int64), np.zeros(m))
     check(g, qs)
+
+
+# A vertex with more arcs than the 256 frontier slots of a search (forward, backward, both)
+# sends it to the global-memory form in the middle of a step; with 1,300 queries some warps
+# run two of them, one of each form
+@pytest.mark.parametrize("out,back", [(255, 1), (257, 1), (1, 257), (400, 400)])
+@pytest.mark.parametrize("n", [5, 1300])
+def test_frontier_overflow(out, back, n):
+    rng = np.random.default_rng(out + back)
+    labels = ["".join("ACGT"[c] for c in rng.integers(0, 4, int(rng.integers(1, 20)))) for _ in range(60 + out + back)]
+    arcs = [(v, v + 1) for v in range(59)]
+    arcs += [(10, 60 + i) for i in range(out)] + [(60 + i, 11) for i in range(out)]
+    arcs += [(40, 60 + out + i) for i in range(back)] + [(60 + out + i, 41) for i in range(back)]
+    arcs += [(30, 29)]
+    g = synth.Graph.from_lists(labels, arcs)
+    lens = rng.integers(20, 400, n)
+    seq = np.frombuffer(b"ACGT", np.uint8)[rng.integers(0, 4, int(lens.sum()))]
+    vs, ve = rng.integers(0, 30, n).astype(np.uint32), rng.integers(20, 60, n).astype(np.uint32)
+    off = np.concatenate([[0], np.cumsum(lens)]).astype(np.uint64)
+    check(g, synth.Queries(seq, off, vs, ve, np.zeros(n, np.int64), np.zeros(n)))
