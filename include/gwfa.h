@@ -184,13 +184,14 @@ typedef struct gwfa_engine gwfa_engine;
  *                  queries start at once on slabs that fit them instead of forming a
  *                  tail of overflow re-runs; their overflows go to the retry tiers
  *   threads        threads per CTA (multiple of 32, 32..1024; a wide CTA shortens
- *                  its query, narrow ones run more of them); 0 = 128; 512 (the
- *                  default configuration) lets the engine choose the width of
- *                  each batch's CTAs from its queries
+ *                  its query, narrow ones run more of them); 0 = 128;
+ *                  GWFA_THREADS_AUTO (the default configuration) lets the engine
+ *                  choose the width of each batch's CTAs from its queries
  *   max_queries, max_bases  sizes of the engine's staging buffers for the
  *                  host-buffer entry point (grown on demand)
  */
 #define GWFA_MAX_TIERS 4
+#define GWFA_THREADS_AUTO 0xFFFFFFFFu
 typedef struct {
     uint32_t ctas;
     uint32_t log2_tiles;
@@ -216,8 +217,7 @@ typedef struct {
     uint32_t n_wide;
 } gwfa_schedule;
 
-/* fills a default configuration for this GPU (3 tiers, 512 threads = width chosen for
- * each batch, no classes) */
+/* fills a default configuration for this GPU (3 tiers, GWFA_THREADS_AUTO, no classes) */
 int gwfa_engine_default_config(const gwfa_graph *g, int prune, gwfa_engine_config *cfg);
 int gwfa_engine_create(const gwfa_graph *g, const gwfa_engine_config *cfg, gwfa_engine **out);
 int gwfa_engine_destroy(gwfa_engine *e);

@@ -50,6 +50,7 @@ class gwfa_opts(ctypes.Structure):
 
 # formulation variants (gwfa_opts.ends flags)
 GWFA_FREE_START, GWFA_FREE_END, GWFA_EXTEND = 1, 2, 4
+GWFA_THREADS_AUTO = 0xFFFFFFFF   # gwfa_engine_config.threads: width chosen for each batch
 
 
 class gwfa_result(ctypes.Structure):

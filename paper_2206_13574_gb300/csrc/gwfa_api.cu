@@ -137,9 +137,6 @@ struct Carve {
     }
 };
 
-// The default config's CTA width: the engine chooses it for each batch.
-constexpr uint32_t kAutoThreads = 512;
-
 // Host-buffer batches up to this many bytes of inputs go over in one copy.
 constexpr uint64_t kStagedBatch = 256 << 10;
 
@@ -451,8 +448,8 @@ int gwfa_engine_default_config(const gwfa_graph *g, int prune, gwfa_engine_confi
     int sms = 0, bps = 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device) != cudaSuccess)
         return GWFA_ERR_CUDA;
-    // width chosen for each batch (tier0_threads); as many narrow CTAs as fit on an SM
-    cfg->threads = kAutoThreads;
+    // width chosen for each batch (auto_threads); as many narrow CTAs as fit on an SM
+    cfg->threads = GWFA_THREADS_AUTO;
     if (gwfa::align_occupancy(prune != 0, prune ? gwfa::kNarrow / 2 : gwfa::kNarrow, &bps) || bps < 1) bps = 1;
     cfg->wide = {0u, prune ? 18u : 19u, 512u, 0u};   // no concurrent classes by default
     cfg->huge = {0u, 22u, 512u, 0u};
@@ -503,7 +500,7 @@ int gwfa_engine_create(const gwfa_graph *g, const gwfa_engine_config *cfg, gwfa_
     *out = nullptr;
     if (cfg->n_tiers < 1 || cfg->n_tiers > GWFA_MAX_TIERS) return GWFA_ERR_INVALID;
     const uint32_t threads = cfg->threads ? cfg->threads : 128;
-    if (threads % 32 || threads < 32 || threads > 1024) return GWFA_ERR_INVALID;
+    if (threads != GWFA_THREADS_AUTO && (threads % 32 || threads < 32 || threads > 1024)) return GWFA_ERR_INVALID;
     for (uint32_t t = 0; t < cfg->n_tiers + 2; ++t) {
         const gwfa_tier &tt = t < cfg->n_tiers ? cfg->tiers[t] : (t == cfg->n_tiers ? cfg->wide : cfg->huge);
         if (t >= cfg->n_tiers && tt.ctas == 0) continue;   // class not used
@@ -699,7 +696,7 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
     };
     auto tier_threads = [&](const gwfa_tier &t, uint32_t count) {
         if (t.threads) return t.threads;
-        return e->cfg.threads != kAutoThreads ? e->cfg.threads
+        return e->cfg.threads != GWFA_THREADS_AUTO ? e->cfg.threads
                                               : auto_threads(count, len ? len : 4000, e->sms, o.max_lag);
     };
     auto per_sm = [&](uint32_t threads) {
@@ -709,7 +706,7 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
     const uint32_t t0_threads = tier_threads(e->cfg.tiers[0], n - n_huge - n_wide);
     // (an engine with classes has its own place for heavy queries)
     const bool few = T > 1 && n <= 4u * (uint32_t)e->sms && !e->wide_slabs && !e->huge_slabs &&
-                     !e->cfg.tiers[0].threads && e->cfg.threads == kAutoThreads &&
+                     !e->cfg.tiers[0].threads && e->cfg.threads == GWFA_THREADS_AUTO &&
                      e->cfg.tiers[1].log2_tiles > e->cfg.tiers[0].log2_tiles &&
                      e->cfg.tiers[1].ctas >= std::min(n, (uint32_t)e->sms);
     // the classes' CTAs and tier 0's must be resident together (tier 0 would otherwise fill
@@ -812,7 +809,7 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
         };
         if (t > 0) {
             st = launch(tier_threads(e->cfg.tiers[t], e->cfg.tiers[t].ctas), e->cfg.tiers[t].ctas);
-        } else if (len || e->cfg.tiers[0].threads || e->cfg.threads != kAutoThreads || o.max_lag > 0) {
+        } else if (len || e->cfg.tiers[0].threads || e->cfg.threads != GWFA_THREADS_AUTO || o.max_lag > 0) {
             st = launch(t0_threads, t0_ctas(t0_threads));
         } else {
             // lengths in device memory only: one launch per width, two of which leave at once

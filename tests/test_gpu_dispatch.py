@@ -55,6 +55,26 @@ def test_chosen_width(graph, n, length, mode):
         assert (int(want[i]["edit_distance"]), int(want[i]["cells"])) == (w["distance"], w["cells"])
 
 
+# a width that the configuration names is the one that runs: one launch a tier, while the
+# engine's own choice for a device batch is settled there, among three launches of tier 0
+@pytest.mark.parametrize("threads", [0, 128, 256, 512, 1024, None])
+def test_configured_width(graph, threads):
+    import torch
+    g, gr = graph
+    qs = synth.make_queries(g, 100, 3, synth._const(900), synth._const(0.02), (1, 1, 1), (1, 1))
+    cfg = gw.default_config(gr)
+    assert cfg.threads == gw.GWFA_THREADS_AUTO
+    if threads is not None:
+        cfg.threads = threads
+    eng = gw.Engine(gr, config=cfg)
+    batch = gw.DeviceBatch(qs)
+    batch.run(eng)
+    torch.cuda.synchronize()
+    assert eng.last_launches == (3 if threads is not None else 5)
+    want = gr.align(qs.query(0), int(qs.v_s[0]), int(qs.v_e[0]))
+    assert int(batch.results()[0]["cells"]) == want["cells"]
+
+
 @pytest.mark.parametrize("kb", [2, 250, 260, 700])   # one copy up to 256 KB of inputs
 def test_host_batch_inputs(graph, kb):
     g, gr = graph
