@@ -680,6 +680,7 @@ static int run_tiers(gwfa_engine *e, uint32_t n, const uint32_t *d_words, const 
         uint32_t *order = e->retry_lists + (uint64_t)GWFA_MAX_TIERS * e->retry_cap;
         st = cuda_status(gwfa::launch_order(n, d_q_off, order, s));
         if (st) return st;
+        e->last_launches++;
         d_order = order;
     }
     struct Cls {

@@ -133,6 +133,24 @@ def test_batch_without_order(graph, n):
             assert np.array_equal(res[f], want[f]), f
 
 
+def test_launches_of_a_batch_without_order(graph):
+    import torch
+    g, gr = graph
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    for n, sort in ((sms, 0), (sms + 1, 1)):
+        qs = synth.make_queries(g, n, 3, synth._const(300), synth._const(0.01), (1, 1, 1), (1, 1))
+        cfg = gw.default_config(gr)
+        cfg.threads = 128
+        eng = gw.Engine(gr, config=cfg)
+        batch = gw.DeviceBatch(qs)
+        batch.run(eng)
+        assert eng.last_launches == 3 + sort                # three tiers
+        eng.align_batch(qs.seq, qs.off, qs.v_s, qs.v_e)
+        assert eng.last_launches == 3 + 1 + sort            # and the packing
+        eng.align_batch(qs.seq, qs.off, qs.v_s, qs.v_e, order=np.arange(n))
+        assert eng.last_launches == 3 + 1
+
+
 # up to four queries an SM start on tier 1's slabs: tier 0's would overflow here, and some
 # queries leave tier 1's as well (or have no tier to go to)
 @pytest.mark.parametrize("n,tiers", [(20, 3), (152, 3), (300, 3), (300, 2), (300, 1)])
