@@ -10,8 +10,8 @@ runs on the same graph and GPU reuse them without searching again (cache_path=No
 searches every time and persists nothing).
 
 CTAs of up to 256 threads share an SM up to 1,536 threads (1,024 with pruning's 64-bit
-offsets), wider ones up to 1,024, and 32 CTAs at most; candidate CTA counts are multiples
-of the SM count.  The frontier tile stays 8 diagonals: the expand step's neighbour exchange
+offsets), wider ones up to 1,024, and 14 CTAs at most (15 KB of shared memory each);
+candidate CTA counts are multiples of the SM count.  The frontier tile stays 8 diagonals: the expand step's neighbour exchange
 is a shuffle among the four lanes that hold them.
 """
 from __future__ import annotations
@@ -54,9 +54,9 @@ def _time(engine: Engine, batch: DeviceBatch, max_lag: int, reps: int) -> float:
 def _tier0_bytes(threads_ctas: int, log2: int, prune: bool) -> int:
     """Approximate device bytes of a tier of CTAs with 2^log2-tile slabs: per tile a
     record (64 / 128 bytes), two hash entries, its hash position and stamp, two list
-    entries and the spill requests (32 bytes); pruning adds the keys, trace words, T and
-    the insertion and free lists."""
-    per_tile = 152 if not prune else 328
+    entries, two neighbours to be linked and the spill requests (32 bytes); pruning adds
+    the keys, trace words, T and the insertion and free lists."""
+    per_tile = 168 if not prune else 336
     return threads_ctas * (per_tile << log2)
 
 
@@ -108,7 +108,7 @@ def autotune(graph: Graph, sample, max_lag: int = 0, threads=(32, 64, 128, 256, 
     for th in threads:
         for frac in per_sm_frac:
             resident = 1536 if th <= 256 and not prune else 1024
-            per_sm = max(1, int(min(resident // th, 32) * frac))
+            per_sm = max(1, int(min(resident // th, 14) * frac))
             for lg in log2_tiles:
                 lg = lg if not prune else lg - 1
                 shape = (th, per_sm, lg, sms * per_sm)

@@ -151,6 +151,19 @@ def test_launches_of_a_batch_without_order(graph):
         assert eng.last_launches == 3 + 1
 
 
+@pytest.mark.parametrize("prune", [False, True])
+def test_autotuner_knows_the_size_of_a_slab(graph, prune):
+    from paper_2206_13574_gb300 import autotune
+    g, gr = graph
+    size = []
+    for ctas in (8, 24):
+        cfg = gw.default_config(gr, prune=prune)
+        cfg.n_tiers, cfg.tiers[0].ctas, cfg.tiers[0].log2_tiles = 1, ctas, 14
+        size.append(gw.Engine(gr, prune=prune, config=cfg).device_bytes)
+    estimate = autotune._tier0_bytes(16, 14, prune)
+    assert abs(size[1] - size[0] - estimate) < 0.001 * estimate
+
+
 # up to four queries an SM start on tier 1's slabs: tier 0's would overflow here, and some
 # queries leave tier 1's as well (or have no tier to go to)
 @pytest.mark.parametrize("n,tiers", [(20, 3), (152, 3), (300, 3), (300, 2), (300, 1)])
