@@ -160,3 +160,25 @@ def test_insertions_of_a_vertex_with_many_arcs(threads, size):
     for i, (q, r) in enumerate(zip(qs, b.results())):
         same(r, oracle.gwfa(g, q, 0, 3, ends=1), q[size:])
         assert plen[i].item() == 2 and paths[8 * i:8 * i + 2].tolist() == [0, 3]
+
+
+# Which lag-pruned reads a slab has room for is the same on CTAs of every width
+@pytest.mark.parametrize("lag", [400, 1000])
+def test_the_load_limit_with_pruning_does_not_depend_on_timing(lag):
+    rng = np.random.default_rng(lag)
+    g, walk = bubble_chain(rng, 300, 12)
+    graph = gw.Graph.from_synth(g)
+    text = b"".join(g.label(v) for v in walk)
+    qs = [noisy(rng, text, e) for e in rng.uniform(0, 0.1, 200)]
+    seq, off = batch(qs)
+    first = None
+    for threads in (32, 256, 512, 1024):
+        eng = engine(graph, threads, 11, prune=True)
+        for _ in range(2):
+            res = eng.align_batch(seq, off, [0] * len(qs), [walk[-1]] * len(qs), max_lag=lag)
+            first = res if first is None else first
+            assert np.array_equal(res["status"], first["status"]), threads
+    fit = np.nonzero(first["status"] == 0)[0]
+    assert 0 < len(fit) < len(qs)
+    for i in fit[:8]:
+        same(first[i], oracle.gwfa(g, qs[i], 0, walk[-1], a_diff=lag), i)
