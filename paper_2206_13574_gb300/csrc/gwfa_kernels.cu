@@ -1429,15 +1429,17 @@ __device__ __forceinline__ void st_release_sys(unsigned long long *p, unsigned l
 
 // Serving: a persistent kernel whose CTAs take requests from host-published rings
 // (continuous batching: a CTA starts a new request as soon as it finishes one).
-// CTAs [0, n_small) serve class 0 (small hash slabs), the rest class 1 (large
-// slabs), which also take class-0 requests whenever no class-1 request waits, so
-// large slabs are never left idle while small requests queue.  Every
+// The first CTAs serve class 1 (large slabs) and also take class-0 requests whenever no
+// class-1 request waits, so large slabs are never left idle while small requests queue; the
+// last n_small serve class 0 (small hash slabs).  So where a configuration has more CTAs
+// than the GPU holds (14 an SM by their shared memory), those that wait for room are of the
+// class that others serve too.  Every
 // wait is bounded: a CTA idle for wait_limit polls votes idle (and withdraws the
 // vote if work comes); the CTAs leave together once every CTA has voted, or after
 // 16 x wait_limit polls in any case, and the host relaunches the kernel when work
 // comes.  Leaving together keeps the full set of CTAs whenever the kernel runs.
-// CTAs per SM are a template parameter: all CTAs must be resident, and with fewer of them
-// a thread has more registers (64, 40 or 32 at 2, 3 or 4).
+// CTAs per SM are a template parameter: with fewer of them a thread has more registers (64,
+// 40 or 32 at 2, 3 or 4).
 template <bool P, int PerSm>
 __global__ void __launch_bounds__(512, PerSm) server_kernel(ServerArgs S) {
     uint32_t *const qst = S.stage + (uint64_t)blockIdx.x * S.slot_words;   // the request's packed words
@@ -1447,9 +1449,10 @@ __global__ void __launch_bounds__(512, PerSm) server_kernel(ServerArgs S) {
     __shared__ uint64_t s_qoff[2];
     __shared__ uint32_t s_vs, s_ve;
     __shared__ int s_go, s_ring;
-    const int cls = blockIdx.x < S.n_small ? 0 : 1;
-    uint8_t *base = cls == 0 ? S.slabs + (uint64_t)blockIdx.x * S.slab_bytes[0]
-                             : S.slabs + S.big_offset + (uint64_t)(blockIdx.x - S.n_small) * S.slab_bytes[1];
+    const uint32_t n_big = S.n_ctas - S.n_small;
+    const int cls = blockIdx.x < n_big ? 1 : 0;
+    uint8_t *base = cls == 0 ? S.slabs + (uint64_t)(blockIdx.x - n_big) * S.slab_bytes[0]
+                             : S.slabs + S.big_offset + (uint64_t)blockIdx.x * S.slab_bytes[1];
     __shared__ Slab<P> s;   // as in align_queries; visible after the first poll barrier
     if (threadIdx.x == 0) s = carve<P>(base, S.log2cap[cls]);
     for (;;) {

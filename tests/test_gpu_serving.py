@@ -140,3 +140,25 @@ def test_poisson_stream_latency(c2):
     assert all(r["status"] == 0 for r in res)
     assert summ["p99_ms"] >= summ["p50_ms"] > 0
     srv.close()
+
+
+def test_more_ctas_than_are_resident(c2):
+    """Requests for the large slabs are served at once also where a server has more CTAs than
+    the GPU holds together, whose small-slab ones stay as long as the server waits for work."""
+    import torch
+    g, qs, graph = c2
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    cfg = gw.gwfa_server_config()
+    gw.load().gwfa_server_default_config(graph.handle, cfg)
+    cfg.threads, cfg.ctas_small, cfg.ctas_big = 64, 22 * sms, 2 * sms
+    cfg.log2_small, cfg.log2_big, cfg.ring_slots, cfg.max_query_len = 8, 12, 64, 2000
+    cfg.idle_us, cfg.big_length = 4_000_000, 100
+    srv = gw.Server(graph, cfg)
+    try:
+        for n, vs in ((50, 0), (300, 0), (400, 3), (80, 1)):   # small, large, large, small
+            q = qs.query(0)[:n]
+            r = srv.wait(srv.submit(q, vs, vs), timeout_ms=5000)
+            want = oracle.gwfa(g, q, vs, vs)
+            assert (r["status"], r["edit_distance"], r["cells"]) == (0, want["distance"], want["cells"]), n
+    finally:
+        srv.close()
