@@ -117,57 +117,6 @@ __device__ uint32_t set_find(const SetScratch &S, int t, uint32_t v) {
     return kEmptyV;
 }
 
-// Bounded search of one warp: t = 0 forward from `src` over out-arcs, t = 1
-// backward over in-arcs; lengths are spelled bases strictly before (forward) or
-// after (backward) a vertex.
-__device__ void bounded_search(const FeatGraph &fg, const SetScratch &S, int t, uint32_t src, uint64_t budget,
-                               uint32_t *cnt /* shared: fill, frontier sizes [2] */) {
-    const int lane = threadIdx.x & 31;
-    for (uint32_t i = lane; i < kSetCap; i += 32) {
-        __stcg(&S.key[t][i], kEmptyV);
-        __stcg(&S.dist[t][i], kEmptyV);
-    }
-    if (lane == 0) {
-        cnt[0] = 0;
-        cnt[1] = 1;
-        cnt[2] = 0;
-    }
-    __syncwarp();
-    if (lane == 0) {
-        const int h = set_insert(S, t, src, &cnt[0]);
-        if (h >= 0) __stcg(&S.dist[t][h], 0u);
-        __stcg(&S.fr[0][0], src);
-    }
-    __syncwarp();
-    for (int cur = 0;; cur ^= 1) {
-        const uint32_t nf = min(cnt[1 + cur], kSetCap);
-        if (nf == 0) break;
-        for (uint32_t i = lane; i < nf; i += 32) {
-            const uint32_t v = __ldcg(&S.fr[cur][i]);
-            const uint32_t dv = set_find(S, t, v);
-            const uint4 vi = __ldg(&fg.vinfo[v]);
-            // forward: a successor starts |v| bases later; backward: a predecessor u
-            // ends where v starts, so its length after it is b(v) + |v|
-            const uint64_t cand = (uint64_t)dv + vi.y;
-            if (cand > budget) continue;
-            const uint32_t a0 = t == 0 ? vi.z : __ldg(&fg.in_off[v]);
-            const uint32_t a1 = t == 0 ? vi.w : __ldg(&fg.in_off[v + 1]);
-            for (uint32_t a = a0; a < a1; ++a) {
-                const uint32_t u = t == 0 ? __ldg(&fg.arc_dst[a]) : __ldg(&fg.in_src[a]);
-                const int h = set_insert(S, t, u, &cnt[0]);
-                if (h < 0) continue;
-                if (atomicMin(&S.dist[t][h], (uint32_t)cand) > (uint32_t)cand) {
-                    const uint32_t k = atomicAdd(&cnt[2 - cur], 1u);
-                    if (k < kSetCap) __stcg(&S.fr[cur ^ 1][k], u);
-                }
-            }
-        }
-        __syncwarp();
-        if (lane == 0) cnt[1 + cur] = 0;
-        __syncwarp();
-    }
-}
-
 // ---- the same searches in shared memory
 //
 // The searches walk a chain of sites, one or a few vertices a step, so a query is bound by
@@ -176,12 +125,11 @@ __device__ void bounded_search(const FeatGraph &fg, const SetScratch &S, int t, 
 // a query); here the tables are in shared memory, frontiers hold table slots, a vertex and
 // its arcs are one 32-byte sector, the forward search runs on the warp's lower half beside
 // the backward one on its upper half, and the counts visit only the vertices reached.  A
-// search that outgrows the tables leaves it to the global-memory form; the lengths, and so
-// the counts, are the same by either.  1,024 entries a search (20 KB for both) hold reads of
+// search that outgrows the tables goes on in global memory where it stopped (50 reads of 8 kb
+// on a graph with a bubble every 9 bases, 2,700 vertices: 13.7 ms all there, 14.6 begun
+// again, 9.0 continued); the lengths, and so the counts, are the same.  1,024 entries a search (20 KB for both) hold reads of
 // 45 kb on the benchmark's graphs at eight warps an SM; batches of up to four queries an SM
-// get 2,048 and four warps.  Beyond that no search is begun that the graph's mean vertex
-// length says will not fit (60 reads of 50 kb: 3.40 ms in global memory, 0.73 in the
-// larger tables).
+// get 2,048 and four warps.
 // Measured on 2,000 reads of 1-20 kb (5 Mb graph), features and predictions: 3.37 ms -> 0.64 ms.
 template <int LOG2> struct SmSet {
     static constexpr uint32_t kSmCap = 1u << LOG2, kSmLoad = kSmCap / 4 * 3;
@@ -224,9 +172,10 @@ template <int LOG2> __device__ __forceinline__ uint32_t sm_find(const SmSet<LOG2
     return kEmptyV;
 }
 
-// Both bounded searches of one warp; false if one outgrew the tables.
+// Both bounded searches of one warp; -1 when they are done, or the parity of the frontier
+// whose step outgrew the tables.
 template <int LOG2>
-__device__ __forceinline__ bool sm_search(const FeatGraph &fg, SmSet<LOG2> &S, uint32_t src, uint32_t dst, uint32_t budget) {
+__device__ __forceinline__ int sm_search(const FeatGraph &fg, SmSet<LOG2> &S, uint32_t src, uint32_t dst, uint32_t budget) {
     const int lane = threadIdx.x & 31, t = lane >> 4, hl = lane & 15;
     for (uint32_t i = lane; i < S.kSmCap; i += 32) {
         S.key[0][i] = S.key[1][i] = kEmptyV;
@@ -245,12 +194,19 @@ __device__ __forceinline__ bool sm_search(const FeatGraph &fg, SmSet<LOG2> &S, u
         S.fr[t][0][0] = (uint16_t)h;
     }
     __syncwarp();
+    uint32_t before = 0;   // frontier of the step before
     for (int cur = 0;; cur ^= 1) {
         // `over` is read before the vote, the same by every lane, as none has gone on to the
         // body, which may set it
         const uint32_t nf = S.nf[t][cur];
         const bool over = S.over != 0;
-        if (!__any_sync(0xFFFFFFFFu, nf > 0 && !over)) return !over;
+        if (!__any_sync(0xFFFFFFFFu, nf > 0 && !over)) {
+            if (!over) return -1;
+            if (hl == 0) S.nf[t][cur ^ 1] = before;
+            __syncwarp();
+            return cur ^ 1;
+        }
+        before = nf;
         for (uint32_t i = hl; i < nf; i += 16) {
             const uint32_t h = S.fr[t][cur][i], v = S.key[t][h];
             const uint4 *rec = (t ? fg.vin : fg.vx) + 2 * (uint64_t)v;
@@ -277,6 +233,73 @@ __device__ __forceinline__ bool sm_search(const FeatGraph &fg, SmSet<LOG2> &S, u
         }
         __syncwarp();
         if (hl == 0) S.nf[t][cur] = 0;
+        __syncwarp();
+    }
+}
+
+// Bounded search of one warp: t = 0 forward from `src` over out-arcs, t = 1
+// backward over in-arcs; lengths are spelled bases strictly before (forward) or
+// after (backward) a vertex.  With `from`, it goes on where the search in shared memory
+// stopped, in a step that outgrew its tables: it takes over what was reached and the
+// frontier of that step and makes the step again.  A vertex that the step had
+// lowered already is found by its length being the one offered; one that had that
+// length before comes along for nothing, its successors being there.
+template <int LOG2>
+__device__ void bounded_search(const FeatGraph &fg, const SetScratch &S, int t, uint32_t src, uint64_t budget,
+                               uint32_t *cnt /* shared: fill, frontier sizes [2] */, const SmSet<LOG2> *from, int from_cur) {
+    const int lane = threadIdx.x & 31;
+    for (uint32_t i = lane; i < kSetCap; i += 32) {
+        __stcg(&S.key[t][i], kEmptyV);
+        __stcg(&S.dist[t][i], kEmptyV);
+    }
+    if (lane == 0) {
+        cnt[0] = 0;
+        cnt[1] = from ? from->nf[t][from_cur] : 1;
+        cnt[2] = 0;
+    }
+    __syncwarp();
+    if (from) {
+        for (uint32_t i = lane; i < from->kSmCap; i += 32) {
+            const uint32_t v = from->key[t][i], d = from->dist[t][i];
+            if (v == kEmptyV || d == kEmptyV) continue;
+            const int h = set_insert(S, t, v, &cnt[0]);
+            if (h >= 0) __stcg(&S.dist[t][h], d);
+        }
+        for (uint32_t i = lane; i < from->nf[t][from_cur]; i += 32) __stcg(&S.fr[0][i], from->key[t][from->fr[t][from_cur][i]]);
+    } else if (lane == 0) {
+        const int h = set_insert(S, t, src, &cnt[0]);
+        if (h >= 0) __stcg(&S.dist[t][h], 0u);
+        __stcg(&S.fr[0][0], src);
+    }
+    __syncwarp();
+    bool again = from != nullptr;
+    for (int cur = 0;; cur ^= 1) {
+        const uint32_t nf = min(cnt[1 + cur], kSetCap);
+        if (nf == 0) break;
+        for (uint32_t i = lane; i < nf; i += 32) {
+            const uint32_t v = __ldcg(&S.fr[cur][i]);
+            const uint32_t dv = set_find(S, t, v);
+            const uint4 vi = __ldg(&fg.vinfo[v]);
+            // forward: a successor starts |v| bases later; backward: a predecessor u
+            // ends where v starts, so its length after it is b(v) + |v|
+            const uint64_t cand = (uint64_t)dv + vi.y;
+            if (cand > budget) continue;
+            const uint32_t a0 = t == 0 ? vi.z : __ldg(&fg.in_off[v]);
+            const uint32_t a1 = t == 0 ? vi.w : __ldg(&fg.in_off[v + 1]);
+            for (uint32_t a = a0; a < a1; ++a) {
+                const uint32_t u = t == 0 ? __ldg(&fg.arc_dst[a]) : __ldg(&fg.in_src[a]);
+                const int h = set_insert(S, t, u, &cnt[0]);
+                if (h < 0) continue;
+                const uint32_t old = atomicMin(&S.dist[t][h], (uint32_t)cand);
+                if (old > (uint32_t)cand || (again && old == (uint32_t)cand)) {
+                    const uint32_t k = atomicAdd(&cnt[2 - cur], 1u);
+                    if (k < kSetCap) __stcg(&S.fr[cur ^ 1][k], u);
+                }
+            }
+        }
+        again = false;
+        __syncwarp();
+        if (lane == 0) cnt[1 + cur] = 0;
         __syncwarp();
     }
 }
@@ -340,14 +363,9 @@ __global__ void features_kernel(FeatGraph fg, uint32_t nq, const uint32_t *__res
         const uint64_t budget = feature_budget(n);
         uint32_t nverts = 0, narcs = 0, nbub = 0, ncyc = 0;
         SmSet<LOG2> &M = ((SmSet<LOG2> *)s_sets)[wib];
-        // a search reaches 1.4 to 1.55 vertices per mean vertex length of its budget (bubbles
-        // side by side; measured on the benchmark's graphs), and one that does not fit is
-        // made twice (700 reads of 50 kb 3.6 -> 4.0 ms)
-        const uint4 vl = __ldg(&fg.vinfo[fg.nv - 1]);
-        const bool fits = budget < 0x40000000ull &&
-                          (fg.nv <= M.kSmLoad ||
-                           budget * fg.nv < (uint64_t)(M.kSmCap * 15 / 32) * 16u * (vl.x + (vl.y + 15) / 16));
-        if (fits && sm_search(fg, M, a, b, (uint32_t)budget)) {
+        const bool fits = budget < 0x40000000ull;   // (lengths have 32 bits there)
+        const int stop = fits ? sm_search(fg, M, a, b, (uint32_t)budget) : 0;
+        if (stop < 0) {
             const uint32_t lim = (uint32_t)budget;
             const uint32_t ni = M.fill[0];
             for (uint32_t i = lane; i < ni; i += 32) {
@@ -370,8 +388,8 @@ __global__ void features_kernel(FeatGraph fg, uint32_t nq, const uint32_t *__res
                 nbub += deg > 1 ? 1u : 0u;
             }
         } else {
-        bounded_search(fg, S, 0, a, budget, s_cnt[wib]);
-        bounded_search(fg, S, 1, b, budget, s_cnt[wib]);
+        bounded_search<LOG2>(fg, S, 0, a, budget, s_cnt[wib], fits ? &M : nullptr, stop);
+        bounded_search<LOG2>(fg, S, 1, b, budget, s_cnt[wib], fits ? &M : nullptr, stop);
         for (uint32_t i = lane; i < kSetCap; i += 32) {
             const uint32_t v = __ldcg(&S.key[0][i]);
             if (v == kEmptyV) continue;

@@ -163,3 +163,31 @@ def test_frontier_overflow(out, back, n):
     vs, ve = rng.integers(0, 30, n).astype(np.uint32), rng.integers(20, 60, n).astype(np.uint32)
     off = np.concatenate([[0], np.cumsum(lens)]).astype(np.uint64)
     check(g, synth.Queries(seq, off, vs, ve, np.zeros(n, np.int64), np.zeros(n)))
+
+
+# A dense stretch (a bubble every 9 bases) beside long vertices: searches of 1,300 and 3,400
+# vertices that begin in shared memory and go on in global memory
+@pytest.mark.parametrize("n,length", [(12, 3000), (620, 3000), (12, 8000), (620, 8000)])
+def test_search_goes_on_in_global_memory(n, length):
+    rng = np.random.default_rng(n + length)
+    labels, arcs, walk = [], [], []
+    for _ in range(1000):
+        at = len(labels)
+        labels.append("".join("ACGT"[c] for c in rng.integers(0, 4, 8)))
+        a, b = rng.permutation(4)[:2]
+        labels += ["ACGT"[a], "ACGT"[b]]
+        arcs += [(at, at + 1), (at, at + 2), (at + 1, at + 3), (at + 2, at + 3)]
+        walk += [at, at + 1 + int(rng.integers(2))]
+    labels += ["ACGTTGCA", "".join("ACGT"[c] for c in rng.integers(0, 4, 300_000))]
+    arcs += [(len(labels) - 2, len(labels) - 1), (len(labels) - 2, len(labels) - 3)]
+    g = synth.Graph.from_lists(labels, arcs)
+    qs, vs, ve = [], [], []
+    for i in range(n):
+        first = 2 * int(rng.integers(0, 650 if length < 5000 else 100))
+        last = min(first + length * 2 // 9, len(walk) - 1)
+        qs.append("".join(labels[v] for v in walk[first:last + 1])[:length])
+        vs.append(walk[first])
+        ve.append(walk[last])
+    off = np.concatenate([[0], np.cumsum([len(q) for q in qs])]).astype(np.uint64)
+    seq = np.frombuffer("".join(qs).encode(), np.uint8).copy()
+    check(g, synth.Queries(seq, off, np.array(vs, np.uint32), np.array(ve, np.uint32), np.zeros(n, np.int64), np.zeros(n)))
