@@ -313,7 +313,7 @@ uint32_t gwfa_engine_last_launches(const gwfa_engine *e);
  * GwfExpand and GwfExtend along vertices, and in the arc spills of GwfExtend (ns,
  * measured by the CTA), extension rounds, tiles visited, tiles listed for the next
  * score, largest tile count of a score, tiles
- * claimed in the hash, and the number of scores.  These are the wavefront sizes
+ * that hold a diagonal at the end, and the number of scores.  These are the wavefront sizes
  * the learned cost model trains on.
  */
 int gwfa_engine_set_stats(gwfa_engine *e, uint64_t *d_stats);

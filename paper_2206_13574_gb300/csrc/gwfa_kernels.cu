@@ -1315,7 +1315,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         if (over || S.err_next) { status = GWFA_ERR_CAPACITY; ++d; break; }
     }
     __syncthreads();
-    const uint32_t n_tiles = sh.nclaim;
+    const uint32_t n_tiles = A.stats ? tiles_held<P>(s, sh) : 0u;
     if constexpr (P) {
         if (threadIdx.x == 0) {
             const Score &S = sh.score[d & 3];

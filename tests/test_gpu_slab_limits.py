@@ -182,3 +182,30 @@ def test_the_load_limit_with_pruning_does_not_depend_on_timing(lag):
     assert 0 < len(fit) < len(qs)
     for i in fit[:8]:
         same(first[i], oracle.gwfa(g, qs[i], 0, walk[-1], a_diff=lag), i)
+
+
+# The tiles of the statistics are those that hold a diagonal when the query ends: with the
+# spills of its last score, without the neighbours that only a next score would need
+@pytest.mark.parametrize("lag", [0, 500])
+def test_tiles_in_the_statistics(lag):
+    import torch
+    g = synth.Graph.from_lists(["A", "C", "G", "T"], [(0, 0), (0, 1), (0, 2), (0, 3), (1, 2), (2, 3), (3, 0)])
+    lens = [0, 1, 6, 7, 8, 100, 343, 1000]
+    seq, off = batch([b"A" * n for n in lens])
+    stats = torch.zeros(len(lens) * 8, dtype=torch.int64, device="cuda")
+    eng = engine(gw.Graph.from_synth(g), 64, 11, prune=lag > 0)
+    eng.set_stats(stats.data_ptr())
+    for ve, first in ((0, 0), (1, 1)):   # distance 0 and 1; diagonals 0..n of A, 1..n of the others
+        res = eng.align_batch(seq, off, [0] * len(lens), [ve] * len(lens), max_lag=lag)
+        for n, r, t in zip(lens, res, stats.view(-1, 8)[:, 6].tolist()):
+            w = oracle.gwfa(g, b"A" * n, 0, ve, a_diff=lag)
+            if n > 0:
+                assert (int(r["edit_distance"]), int(r["visited"])) == (w["distance"], w["visited"])
+                assert w["visited"] not in (4 * n + 1, 4 * n + 4) or t == 4 * (n // 8 + 1), (n, t)
+    rng = np.random.default_rng(3)
+    ends = ["".join("ACGT"[c] for c in rng.integers(0, 4, 12)) for _ in range(50)]
+    eng = engine(gw.Graph.from_synth(synth.Graph.from_lists(["ACGTTGCA"] + ends, [(0, 1 + i) for i in range(50)])), 64, 11, prune=lag > 0)
+    eng.set_stats(stats.data_ptr())
+    seq, off = batch([("ACGTTGCA" + ends[20]).encode()])
+    assert eng.align_batch(seq, off, [0], [21], max_lag=lag)[0]["edit_distance"] == 0
+    assert stats[6].item() == 51   # the first vertex and its successors, (u, 8) each
