@@ -81,11 +81,10 @@ struct alignas(64) TraceRec {
     uint32_t pad[4];
 };
 
-// Records of a slab of 2^log2 tiles.  A CTA has up to one more in use for each of its threads
-// (see find_or_insert); the quarter above the load limit has room for them but on the
-// smallest slabs.
+// Records of a slab of 2^log2 tiles.  A CTA has up to two more in use for each of its threads
+// (see link_stop); the quarter above the load limit has room for them but on small slabs.
 __host__ __device__ inline uint32_t slab_records(uint32_t log2cap) {
-    return (1u << log2cap) + (log2cap < 13 ? 1024u : 0u);
+    return (1u << log2cap) + (log2cap < 14 ? 1024u : 0u);
 }
 
 // Per-CTA slab layout (all arrays 256-byte aligned), cap = 2^log2 tiles: the hash (twice

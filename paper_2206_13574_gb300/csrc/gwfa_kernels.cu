@@ -128,7 +128,8 @@ struct Score {
     uint32_t amax;      // largest i + W~ (fits: i < 2^31, W~ < 2^31)
     int found, err;
     uint32_t nlink;     // neighbours to be linked after the pass
-    int err_next;       // out of room for a tile that only the next score needs
+    int err_next;       // out of room for a tile that only the next score needs, or kLinksWait
+    uint32_t link_stop; // with this many records in use links wait (kNone: they don't)
 };
 
 // CTA-shared state of the query being aligned.
@@ -333,8 +334,23 @@ template <bool P> __device__ __forceinline__ void empty_record(const Slab<P> &s,
     if (idx >= kBitTiles) s.stamp[idx] = kNone;
 }
 
-// Record of tile (v, kb), claimed if absent; -1 (and *err) when the slab is full.  The
-// first probe is inline, the rest (and the claim) is not.  A claim puts key and record into
+// Links claim tiles beside the spills of a score.  Such a tile belongs to the next score, which
+// a query that ends in this one does not need, and with pruning it often stays empty, while a
+// spill must find room as long as the tiles that hold a diagonal are within the load limit.
+// So links leave the records that the spills may still ask for, and two a thread: one that a
+// race has left over, and one that it takes right now.  The rest of the links follows after
+// the spills (check_room).
+constexpr int kLinksWait = 1;
+template <bool P> __device__ __forceinline__ uint32_t records_in_use(const Slab<P> &s, const Sh &sh) {
+    return min(sh.nt, s.rcap) - (P ? max(sh.nfree, 0) : 0);
+}
+template <bool P> __device__ __forceinline__ uint32_t link_stop(const Slab<P> &s, const Sh &sh) {
+    return (uint32_t)max((int)(s.rcap - load_limit(s) + sh.nclaim) - 2 * (int)blockDim.x, 0);
+}
+
+// Record of tile (v, kb), claimed if absent, for score `who` & 3 (| kForLink); -1 (and an
+// error) when the slab is full or a link has to wait.  The first probe is inline, the rest
+// (and the claim) is not.  A claim puts key and record into
 // the table at once, so it brings a record along, and where several threads meet at one new
 // tile (the eight diagonals of a neighbour do, and the two vertices of a bubble) all but one
 // are left with theirs.  Such a thread keeps it for its next claim: a slab then has at most
@@ -343,16 +359,26 @@ template <bool P> __device__ __forceinline__ void empty_record(const Slab<P> &s,
 // under the memory bound lost one at every bubble, for good).  It costs 0 to 1% (pruned
 // 22.8 -> 23.1 ms); to claim the key first and have the others wait for the record costs
 // them a poll (10,000 reads 32.5 -> 37.5 ms).
+constexpr uint32_t kForLink = 4;
 template <bool P>
 __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsigned long long key, uint32_t h, Ent e,
-                                                int *err) {
+                                                uint32_t who) {
+    Score &S = sh.score[who & 3];
     uint32_t idx = kNone;
     for (int probe = 0; probe < 256; ++probe) {
         if (probe > 0) e = ld_ent(&s.table[h]);
         if (e.key == kEmptyKey) {
             if (idx == kNone) {
+                // (exact mode looks at the number it gets instead, which costs no load: 10,000
+                // reads 33.9 -> 33.3 ms; a link that waits keeps the record, and none of its
+                // thread's later ones takes it)
+                if (P && (who & kForLink) && records_in_use<P>(s, sh) >= S.link_stop) {
+                    atomicCAS(&S.err_next, 0, kLinksWait);
+                    return -1;
+                }
                 idx = spare_record(sh);
                 if (idx != kNone) {
+                    if (!P && (who & kForLink) && S.err_next == kLinksWait) return -1;
                     spare_record(sh) = kNone;
                 } else {
                     if constexpr (P) {
@@ -364,6 +390,11 @@ __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsign
                     if (idx >= s.rcap) break;
                 }
                 empty_record<P>(s, idx, (int)(uint32_t)key);
+                if (!P && (who & kForLink) && idx >= S.link_stop) {
+                    spare_record(sh) = idx;
+                    atomicCAS(&S.err_next, 0, kLinksWait);
+                    return -1;
+                }
                 if constexpr (P) s.tkey[idx] = key;
                 __threadfence_block();   // before the key that leads others to it
             }
@@ -384,15 +415,15 @@ __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsign
         }
         h = (h + 1) & s.tmask;
     }
-    atomicCAS(err, 0, GWFA_ERR_CAPACITY);
+    *(who & kForLink ? &S.err_next : &S.err) = GWFA_ERR_CAPACITY;
     return -1;
 }
 template <bool P>
-__device__ __forceinline__ int find_or_insert(const Slab<P> &s, Sh &sh, uint32_t v, int kb, int *err) {
+__device__ __forceinline__ int find_or_insert(const Slab<P> &s, Sh &sh, uint32_t v, int kb, uint32_t who) {
     const unsigned long long key = tile_key(v, kb);
     const uint32_t h = tile_hash(key, s.tmask);
     const Ent e = ld_ent(&s.table[h]);
-    if (e.key != key) return find_or_insert_slow<P>(s, sh, key, h, e, err);
+    if (e.key != key) return find_or_insert_slow<P>(s, sh, key, h, e, who);
     __threadfence_block();   // see empty_record
     return (int)e.idx;
 }
@@ -410,8 +441,8 @@ __device__ __forceinline__ bool list_once(const Slab<P> &s, Sh &sh, uint32_t idx
 // The neighbour tile on side sd (0 left, 1 right), linked on first use.
 template <bool P>
 __device__ __noinline__ uint32_t link_neighbour(const Slab<P> &s, Sh &sh, uint32_t idx, uint32_t v, int kb, int sd,
-                                                int *err) {
-    const int t = find_or_insert<P>(s, sh, v, sd ? kb + 1 : kb - 1, err);
+                                                uint32_t who) {
+    const int t = find_or_insert<P>(s, sh, v, sd ? kb + 1 : kb - 1, who);
     if (t < 0) return kNone;
     s.recs[idx].side[sd].link = (uint32_t)t;
     s.recs[t].side[sd ^ 1].link = idx;
@@ -444,7 +475,7 @@ __device__ void enter_next(const Slab<P> &s, Sh &sh, const QCtx &q, uint32_t idx
     const int sd = ln == 7;
     if ((ln == 0 && (uint32_t)j < lv) || (ln == 7 && k + j < q.n)) {
         uint32_t t = s.recs[idx].side[sd].link;
-        if (t == kNone) t = link_neighbour<P>(s, sh, idx, v, k >> 3, sd, &sh.score[d & 3].err_next);
+        if (t == kNone) t = link_neighbour<P>(s, sh, idx, v, k >> 3, sd, ((uint32_t)d & 3u) | kForLink);
         if (t == kNone) return;
         leave_border<P>(s, t, sd, j, base, d, tr, traceback);
         if (list_once<P>(s, sh, t, d)) next[atomicAdd(nq, 1u)] = make_uint2(t, v);
@@ -462,7 +493,7 @@ __device__ __forceinline__ void link_pending(const Slab<P> &s, Sh &sh, int d, ui
         const uint2 rq = i < kLink ? sh.link[i] : s.links[i];
         const uint32_t idx = rq.x & 0x7FFFFFFFu;
         const int sd = (int)(rq.x >> 31), ln = sd ? 7 : 0;
-        const uint32_t t = link_neighbour<P>(s, sh, idx, rq.y, s.recs[idx].side[0].kb, sd, &sh.score[d & 3].err_next);
+        const uint32_t t = link_neighbour<P>(s, sh, idx, rq.y, s.recs[idx].side[0].kb, sd, ((uint32_t)d & 3u) | kForLink);
         if (t == kNone) continue;
         if constexpr (P) {
             const long long v = s.recs[idx].vals[ln];
@@ -862,7 +893,7 @@ __device__ __forceinline__ void spill_round(const DevGraph &g, const Slab<false>
                 for (uint32_t o = (uint32_t)arc; ar.x + o < ar.y; o += 2) {
                     if (o >= 2) u = arc_target(g, rq.x, ar.x + o, o);
                     const uint2 ui = ld_early(&g.vx[2 * (uint64_t)u], 0);
-                    const int su = find_or_insert<false>(s, sh, u, ku >> 3, &S.err);
+                    const int su = find_or_insert<false>(s, sh, u, ku >> 3, (uint32_t)d & 3u);
                     if (su < 0) break;
                     // the offset and the first windows together; most spills end here, the
                     // diagonal being there already
@@ -914,7 +945,7 @@ __device__ __forceinline__ void apply_spills(const DevGraph &g, const Slab<true>
         const uint2 ar = __ldg((const uint2 *)&g.vx[2 * (uint64_t)(uint32_t)rq.z].z);
         for (uint32_t o = threadIdx.x & 3; ar.x + o < ar.y; o += 4) {
             const uint32_t u = arc_target(g, (uint32_t)rq.z, ar.x + o, o);
-            const int su = find_or_insert<true>(s, sh, u, ku >> 3, &S.err);
+            const int su = find_or_insert<true>(s, sh, u, ku >> 3, (uint32_t)d & 3u);
             if (su < 0) break;
             if (g_max(&s.recs[su].vals[ku & 7], cand) >= 0) continue;
             ++won;
@@ -942,7 +973,7 @@ __device__ __forceinline__ void resolve_spill_traces(const DevGraph &g, const Sl
         const uint2 ar = __ldg((const uint2 *)&g.vx[2 * (uint64_t)(uint32_t)rq.z].z);
         for (uint32_t o = threadIdx.x & 3; ar.x + o < ar.y; o += 4) {
             const uint32_t u = arc_target(g, (uint32_t)rq.z, ar.x + o, o);
-            const int su = find_or_insert<true>(s, sh, u, ku >> 3, &sh.score[d & 3].err);
+            const int su = find_or_insert<true>(s, sh, u, ku >> 3, (uint32_t)d & 3u);
             if (su < 0) return;
             if (s.recs[su].vals[ku & 7] == cand) g_max32(&s.trec[su].tr[ku & 7], s.reqt[r]);
         }
@@ -976,7 +1007,7 @@ __device__ __forceinline__ bool spill_step(const DevGraph &g, const Slab<true> &
     bool want = ar.x + arc < ar.y;
     if (want) {
         ui = ld_early(&g.vx[2 * (uint64_t)u], 0);
-        su = find_or_insert<true>(s, sh, u, ku >> 3, &S.err);
+        su = find_or_insert<true>(s, sh, u, ku >> 3, (uint32_t)d & 3u);
         want = su >= 0;
         if (want) {
             const long long raw = s.recs[su].vals[ln];
@@ -1070,7 +1101,7 @@ template <bool P> __device__ void wipe(const Slab<P> &s, Sh &sh) {
 // flags and border words stay valid; the links between neighbours, which could point to a
 // freed record, are dropped and found again on use.  A removed diagonal may be inserted
 // again later, like any absent one.
-__device__ void evict_behind(const Slab<true> &s, Sh &sh, long long amax, int lag, int d) {
+__device__ __noinline__ void evict_behind(const Slab<true> &s, Sh &sh, long long amax, long long lag, int d) {
     const uint32_t nt = min(sh.nt, s.rcap);
     for (uint32_t t = threadIdx.x; t < nt; t += blockDim.x) {
         const uint32_t h = s.touched[t];
@@ -1092,7 +1123,7 @@ __device__ void evict_behind(const Slab<true> &s, Sh &sh, long long amax, int la
             const long long v = s.recs[t].vals[ln];
             if (v < 0) continue;
             const long long a = (long long)(kb * kTile + ln) + 2ll * pj(v) + (long long)pbase(v);
-            if (((v >> 30) & 3) == kTagLive || amax - a < (long long)lag) {
+            if (((v >> 30) & 3) == kTagLive || amax - a < lag) {
                 any = true;
             } else {
                 s.recs[t].vals[ln] = -1ll;
@@ -1117,6 +1148,57 @@ __device__ void evict_behind(const Slab<true> &s, Sh &sh, long long amax, int la
     ev = __reduce_add_sync(0xFFFFFFFFu, ev);
     if ((threadIdx.x & 31) == 0 && ev) atomicAdd(&sh.evicted, (unsigned long long)ev);
     __syncthreads();
+    if (threadIdx.x == 0) sh.score[d & 3].link_stop = link_stop<true>(s, sh);
+    __syncthreads();
+}
+
+// Whether the slab has room for score d, over the tiles that it needs, and for the next one,
+// unless this is the last.  The links that waited for the spills get their turn here: every
+// diagonal in Q at an edge of its tile (all such tiles are listed by now) hands its candidate
+// over, to most neighbours for the second time, which does nothing.  In pruning mode the empty
+// tiles are cleared away first if the records might not do.
+enum Room { kRoom, kNoRoom, kNoRoomNext };
+template <bool P>
+__device__ __noinline__ Room check_room(const uint4 *vx, const Slab<P> &s, Sh &sh, int n, int d, bool last, bool traceback) {
+    Score &S = sh.score[d & 3];
+    uint32_t *nq = &sh.score[(d + 1) & 3].nq;
+    const bool over = !P && sh.nclaim > load_limit(s);
+    if ((over || (P && S.found)) && tiles_held<P>(s, sh) > load_limit(s)) return kNoRoom;
+    if (last) return kRoom;
+    if (over || S.err_next != kLinksWait) return kNoRoomNext;
+    const uint32_t listed = *nq;
+    if constexpr (P) {
+        if (s.rcap - records_in_use<P>(s, sh) < 2 * listed + blockDim.x) evict_behind(s, sh, 0, 1ll << 62, d);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        S.err_next = P && sh.nclaim > load_limit(s) ? GWFA_ERR_CAPACITY : 0;
+        S.link_stop = kNone;
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < 2 * listed; i += blockDim.x) {
+        const uint2 ent = s.list[(d + 1) & 1][i >> 1];
+        const int sd = (int)(i & 1), ln = sd ? 7 : 0, kb = s.recs[ent.x].side[0].kb;
+        const auto v = s.recs[ent.x].vals[ln];
+        bool live;
+        int j;
+        uint32_t base = 0u;
+        if constexpr (P) {
+            live = v >= 0 && ((v >> 30) & 3) == kTagLive;
+            j = pj(v);
+            base = pbase(v);
+        } else {
+            live = v & 1;
+            j = v >> 1;
+        }
+        if (!live || (sd ? kb * kTile + 7 + j >= n : j >= (int)__ldg(&vx[2 * (uint64_t)ent.y]).y)) continue;
+        const uint32_t t = link_neighbour<P>(s, sh, ent.x, ent.y, kb, sd, ((uint32_t)d & 3u) | kForLink);
+        if (t == kNone) continue;
+        leave_border<P>(s, t, sd, j, base, d, traceback ? s.trec[ent.x].tr[ln] : 0u, traceback);
+        if (list_once<P>(s, sh, t, d)) s.list[(d + 1) & 1][atomicAdd(nq, 1u)] = make_uint2(t, ent.y);
+    }
+    __syncthreads();
+    return S.err_next || (!P && sh.nclaim > load_limit(s)) ? kNoRoomNext : kRoom;
 }
 
 template <bool P, bool TB>
@@ -1155,7 +1237,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         sh.peak = 0;
         sh.tlen = 0;
         sh.end_vp = ((unsigned long long)q.ve << 32) | kNoTrace;
-        const int t = find_or_insert<P>(s, sh, vs, 0, &sh.score[0].err);
+        const int t = find_or_insert<P>(s, sh, vs, 0, 0u);
         if (t >= 0) {
             if constexpr (P) {
                 s.recs[t].vals[0] = pk(0, kTagLive, 0u);
@@ -1179,7 +1261,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         const int ntile = (lvs + kTile - 1) / kTile;   // tiles kb = -1 .. -ntile
         for (int i = threadIdx.x; i < ntile; i += blockDim.x) {
             const int kb = -1 - i;
-            const int t = find_or_insert<P>(s, sh, vs, kb, &sh.score[0].err);
+            const int t = find_or_insert<P>(s, sh, vs, kb, 0u);
             if (t < 0) continue;
             uint32_t cnt = 0;
             for (int ln = 0; ln < kTile; ++ln) {
@@ -1206,6 +1288,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         Score &S = sh.score[d & 3];
         if (threadIdx.x == blockDim.x - 32) {   // the last warp: the first to run out of tiles
             sh.score[(d + 2) & 3] = Score{};
+            S.link_stop = link_stop<P>(s, sh);
             sh.nr[0] = 0;
             sh.nins[0] = 0;
         }
@@ -1304,15 +1387,14 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         }
         if (A.stats && threadIdx.x == 0) sh.st[1] += globaltimer_ns() - sh.t_phase;
         if (S.err) { status = S.err; break; }
-        // the load limit, over the tiles that this score needs (rare: a query passes here
-        // once, or in pruning mode ends with most of the slab in use)
-        const bool over = !P && sh.nclaim > load_limit(s);
-        if (over || (P && S.found && sh.nt > load_limit(s))) {
-            if (tiles_held<P>(s, sh) > load_limit(s)) { status = GWFA_ERR_CAPACITY; break; }
-        }
+        // rare: a query passes here once, or in pruning mode ends with most of the slab in use
+        Room room = kRoom;
+        if (S.err_next || (P ? S.found && sh.nt > load_limit(s) : sh.nclaim > load_limit(s)))
+            room = check_room<P>(g.vx, s, sh, q.n, d, S.found || (A.max_score >= 0 && d >= A.max_score), TB);
+        if (room == kNoRoom) { status = GWFA_ERR_CAPACITY; break; }
         if (S.found) break;   // end test of Alg. 1
         if (A.max_score >= 0 && d >= A.max_score) { status = GWFA_ERR_SCORE_LIMIT; break; }
-        if (over || S.err_next) { status = GWFA_ERR_CAPACITY; ++d; break; }
+        if (room == kNoRoomNext) { status = GWFA_ERR_CAPACITY; ++d; break; }
     }
     __syncthreads();
     const uint32_t n_tiles = A.stats ? tiles_held<P>(s, sh) : 0u;

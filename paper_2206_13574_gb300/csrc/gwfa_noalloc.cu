@@ -127,6 +127,8 @@ extern "C" int gwfa_align_noalloc(const gwfa_graph *g, uint32_t n_queries, const
     a.log2cap = log2_tiles;
     a.max_lag = o.max_lag;
     a.max_score = o.max_score;
-    // a handful of CTAs: as wide as their frontiers are worth
-    return gwfa::launch_align(a, prune, ctas, prune ? 256 : 1024, s) == cudaSuccess ? GWFA_OK : GWFA_ERR_CUDA;
+    // a handful of CTAs: as wide as their frontiers are worth (on slabs below 2^13 tiles the
+    // links of 1,024 threads would wait for the spills, see link_stop)
+    const uint32_t threads = prune ? 256 : log2_tiles >= 13 ? 1024 : 512;
+    return gwfa::launch_align(a, prune, ctas, threads, s) == cudaSuccess ? GWFA_OK : GWFA_ERR_CUDA;
 }

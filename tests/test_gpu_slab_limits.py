@@ -195,7 +195,7 @@ def test_tiles_in_the_statistics(lag):
     stats = torch.zeros(len(lens) * 8, dtype=torch.int64, device="cuda")
     eng = engine(gw.Graph.from_synth(g), 64, 11, prune=lag > 0)
     eng.set_stats(stats.data_ptr())
-    for ve, first in ((0, 0), (1, 1)):   # distance 0 and 1; diagonals 0..n of A, 1..n of the others
+    for ve in (0, 1):   # distance 0 and 1; diagonals 0..n of A, 1..n of the others
         res = eng.align_batch(seq, off, [0] * len(lens), [ve] * len(lens), max_lag=lag)
         for n, r, t in zip(lens, res, stats.view(-1, 8)[:, 6].tolist()):
             w = oracle.gwfa(g, b"A" * n, 0, ve, a_diff=lag)
@@ -209,3 +209,61 @@ def test_tiles_in_the_statistics(lag):
     seq, off = batch([("ACGTTGCA" + ends[20]).encode()])
     assert eng.align_batch(seq, off, [0], [21], max_lag=lag)[0]["edit_distance"] == 0
     assert stats[6].item() == 51   # the first vertex and its successors, (u, 8) each
+
+
+# A score whose spills bring the tiles to most of the slab may leave border words for as many
+# tiles again (here each of 5,000 diagonals for the tile on its left).  They belong to the
+# next score: a query that ends in this one does not need them, and has room.
+@pytest.mark.parametrize("threads", [64, 256, 1024])
+@pytest.mark.parametrize("mode", ["exact", "lag", "traceback"])
+def test_tiles_of_the_next_score_leave_room_for_spills(threads, mode):
+    import torch
+    rng = np.random.default_rng(threads)
+    ends = ["".join("ACGT"[c] for c in rng.integers(0, 4, 12)) for _ in range(5000)]
+    g = synth.Graph.from_lists(["ACGTTGCA"] + ends, [(0, 1 + i) for i in range(5000)])
+    qs = [("ACGTTGCA" + ends[i]).encode() for i in (0, 2500, 4999)] + [("ACGTTGCT" + ends[7]).encode()]
+    ve = np.array([1, 2501, 5000, 8], np.uint32)
+    n, vs = len(qs), np.zeros(4, np.uint32)
+    seq, off = batch(qs)
+    prune, lag = mode != "exact", 500 if mode == "lag" else 0
+    b = gw.DeviceBatch(synth.Queries(seq.copy(), off, vs, ve, np.zeros(n, np.int64), np.zeros(n)))
+    graph = gw.Graph.from_synth(g)
+    for log2, fit in ((13, 3), (15, 4)):   # 6,144 tiles are the load limit; the last query needs 10,000
+        eng = engine(graph, threads, log2, prune=prune)
+        for _ in range(3):
+            b.run(eng, traceback=mode == "traceback", max_lag=lag)
+            torch.cuda.synchronize()
+            res = b.results()
+            for i in range(n):
+                if i < fit:
+                    same(res[i], oracle.gwfa(g, qs[i], 0, int(ve[i]), a_diff=lag), i)
+                else:
+                    assert int(res[i]["status"]) == gw.GWFA_ERR_CAPACITY
+
+
+# With pruning a border word's candidate may be dropped, its tile staying empty: such tiles
+# give way to those that hold a diagonal.  Reads with few errors leave many.
+@pytest.mark.parametrize("threads", [64, 256, 1024])
+def test_empty_tiles_give_way(threads):
+    import torch
+    rng = np.random.default_rng(11)
+    g, walk = bubble_chain(rng, 1500, 3)
+    graph = gw.Graph.from_synth(g)
+    text = b"".join(g.label(v) for v in walk)
+    qs = [noisy(rng, text, e) for e in rng.uniform(0.0005, 0.012, 120)]
+    seq, off = batch(qs)
+    n, end = len(qs), [walk[-1]] * len(qs)
+    held = torch.zeros(n * 8, dtype=torch.int64, device="cuda")
+    eng = engine(graph, threads, 17, prune=True)
+    eng.set_stats(held.data_ptr())
+    want = eng.align_batch(seq, off, [0] * n, end, max_lag=200)
+    held = held.view(n, 8)[:, 6].cpu().numpy()
+    res = engine(graph, threads, 13, prune=True).align_batch(seq, off, [0] * n, end, max_lag=200)
+    assert (want["status"] == 0).all() and ((held > 5000) & (held <= 6144)).sum() > 5 and (held > 6144).any()
+    for i in range(n):
+        if held[i] <= 6144:
+            assert int(res[i]["status"]) == 0, (i, held[i])
+            for f in ("edit_distance", "cells", "visited", "pruned", "spills"):
+                assert res[i][f] == want[i][f], (i, f)
+        else:
+            assert int(res[i]["status"]) == gw.GWFA_ERR_CAPACITY
