@@ -348,22 +348,20 @@ template <bool P> __device__ __forceinline__ uint32_t link_stop(const Slab<P> &s
     return (uint32_t)max((int)(s.rcap - load_limit(s) + sh.nclaim) - 2 * (int)blockDim.x, 0);
 }
 
-// Record of tile (v, kb), claimed if absent, for score `who` & 3 (| kForLink); -1 (and an
-// error) when the slab is full or a link has to wait.  The first probe is inline, the rest
-// (and the claim) is not.  A claim puts key and record into
-// the table at once, so it brings a record along, and where several threads meet at one new
-// tile (the eight diagonals of a neighbour do, and the two vertices of a bubble) all but one
-// are left with theirs.  Such a thread keeps it for its next claim: a slab then has at most
-// one record a thread in use beside its tiles, and what it has room for does not depend on
-// how often they meet (without, 255 spills at once into 32 tiles used 255 records, and a read
-// under the memory bound lost one at every bubble, for good).  It costs 0 to 1% (pruned
-// 22.8 -> 23.1 ms); to claim the key first and have the others wait for the record costs
-// them a poll (10,000 reads 32.5 -> 37.5 ms).
-constexpr uint32_t kForLink = 4;
-template <bool P>
+// Record of tile (v, kb), claimed if absent; -1 (and an error) when the slab is full or a link
+// has to wait.  The first probe is inline, the rest (and the claim) is not, in one function
+// for spills and one for links (with a switch 10,000 reads take 33.5 ms, so 32.7).  A claim
+// puts key and record into the table at once, so it brings a record along, and where several
+// threads meet at one new tile (the eight diagonals of a neighbour do, and the two vertices of
+// a bubble) all but one are left with theirs.  Such a thread keeps it for its next claim: a
+// slab then has at most one record a thread in use beside its tiles, and what it has room for
+// does not depend on how often they meet (without, 255 spills at once into 32 tiles used 255
+// records, and a read under the memory bound lost one at every bubble, for good).  To claim
+// the key first and have the others wait for the record costs them a poll (10,000 reads 32.5
+// -> 37.5 ms).
+template <bool P, bool Link>
 __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsigned long long key, uint32_t h, Ent e,
-                                                uint32_t who) {
-    Score &S = sh.score[who & 3];
+                                                Score &S) {
     uint32_t idx = kNone;
     for (int probe = 0; probe < 256; ++probe) {
         if (probe > 0) e = ld_ent(&s.table[h]);
@@ -372,13 +370,13 @@ __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsign
                 // (exact mode looks at the number it gets instead, which costs no load: 10,000
                 // reads 33.9 -> 33.3 ms; a link that waits keeps the record, and none of its
                 // thread's later ones takes it)
-                if (P && (who & kForLink) && records_in_use<P>(s, sh) >= S.link_stop) {
+                if (P && Link && records_in_use<P>(s, sh) >= S.link_stop) {
                     atomicCAS(&S.err_next, 0, kLinksWait);
                     return -1;
                 }
                 idx = spare_record(sh);
                 if (idx != kNone) {
-                    if (!P && (who & kForLink) && S.err_next == kLinksWait) return -1;
+                    if (!P && Link && S.err_next == kLinksWait) return -1;
                     spare_record(sh) = kNone;
                 } else {
                     if constexpr (P) {
@@ -390,7 +388,7 @@ __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsign
                     if (idx >= s.rcap) break;
                 }
                 empty_record<P>(s, idx, (int)(uint32_t)key);
-                if (!P && (who & kForLink) && idx >= S.link_stop) {
+                if (!P && Link && idx >= S.link_stop) {
                     spare_record(sh) = idx;
                     atomicCAS(&S.err_next, 0, kLinksWait);
                     return -1;
@@ -415,15 +413,15 @@ __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsign
         }
         h = (h + 1) & s.tmask;
     }
-    *(who & kForLink ? &S.err_next : &S.err) = GWFA_ERR_CAPACITY;
+    *(Link ? &S.err_next : &S.err) = GWFA_ERR_CAPACITY;
     return -1;
 }
-template <bool P>
-__device__ __forceinline__ int find_or_insert(const Slab<P> &s, Sh &sh, uint32_t v, int kb, uint32_t who) {
+template <bool P, bool Link = false>
+__device__ __forceinline__ int find_or_insert(const Slab<P> &s, Sh &sh, uint32_t v, int kb, Score &S) {
     const unsigned long long key = tile_key(v, kb);
     const uint32_t h = tile_hash(key, s.tmask);
     const Ent e = ld_ent(&s.table[h]);
-    if (e.key != key) return find_or_insert_slow<P>(s, sh, key, h, e, who);
+    if (e.key != key) return find_or_insert_slow<P, Link>(s, sh, key, h, e, S);
     __threadfence_block();   // see empty_record
     return (int)e.idx;
 }
@@ -441,8 +439,8 @@ __device__ __forceinline__ bool list_once(const Slab<P> &s, Sh &sh, uint32_t idx
 // The neighbour tile on side sd (0 left, 1 right), linked on first use.
 template <bool P>
 __device__ __noinline__ uint32_t link_neighbour(const Slab<P> &s, Sh &sh, uint32_t idx, uint32_t v, int kb, int sd,
-                                                uint32_t who) {
-    const int t = find_or_insert<P>(s, sh, v, sd ? kb + 1 : kb - 1, who);
+                                                Score &S) {
+    const int t = find_or_insert<P, true>(s, sh, v, sd ? kb + 1 : kb - 1, S);
     if (t < 0) return kNone;
     s.recs[idx].side[sd].link = (uint32_t)t;
     s.recs[t].side[sd ^ 1].link = idx;
@@ -475,7 +473,7 @@ __device__ void enter_next(const Slab<P> &s, Sh &sh, const QCtx &q, uint32_t idx
     const int sd = ln == 7;
     if ((ln == 0 && (uint32_t)j < lv) || (ln == 7 && k + j < q.n)) {
         uint32_t t = s.recs[idx].side[sd].link;
-        if (t == kNone) t = link_neighbour<P>(s, sh, idx, v, k >> 3, sd, ((uint32_t)d & 3u) | kForLink);
+        if (t == kNone) t = link_neighbour<P>(s, sh, idx, v, k >> 3, sd, sh.score[d & 3]);
         if (t == kNone) return;
         leave_border<P>(s, t, sd, j, base, d, tr, traceback);
         if (list_once<P>(s, sh, t, d)) next[atomicAdd(nq, 1u)] = make_uint2(t, v);
@@ -493,7 +491,7 @@ __device__ __forceinline__ void link_pending(const Slab<P> &s, Sh &sh, int d, ui
         const uint2 rq = i < kLink ? sh.link[i] : s.links[i];
         const uint32_t idx = rq.x & 0x7FFFFFFFu;
         const int sd = (int)(rq.x >> 31), ln = sd ? 7 : 0;
-        const uint32_t t = link_neighbour<P>(s, sh, idx, rq.y, s.recs[idx].side[0].kb, sd, ((uint32_t)d & 3u) | kForLink);
+        const uint32_t t = link_neighbour<P>(s, sh, idx, rq.y, s.recs[idx].side[0].kb, sd, sh.score[d & 3]);
         if (t == kNone) continue;
         if constexpr (P) {
             const long long v = s.recs[idx].vals[ln];
@@ -893,7 +891,7 @@ __device__ __forceinline__ void spill_round(const DevGraph &g, const Slab<false>
                 for (uint32_t o = (uint32_t)arc; ar.x + o < ar.y; o += 2) {
                     if (o >= 2) u = arc_target(g, rq.x, ar.x + o, o);
                     const uint2 ui = ld_early(&g.vx[2 * (uint64_t)u], 0);
-                    const int su = find_or_insert<false>(s, sh, u, ku >> 3, (uint32_t)d & 3u);
+                    const int su = find_or_insert<false>(s, sh, u, ku >> 3, sh.score[d & 3]);
                     if (su < 0) break;
                     // the offset and the first windows together; most spills end here, the
                     // diagonal being there already
@@ -945,7 +943,7 @@ __device__ __forceinline__ void apply_spills(const DevGraph &g, const Slab<true>
         const uint2 ar = __ldg((const uint2 *)&g.vx[2 * (uint64_t)(uint32_t)rq.z].z);
         for (uint32_t o = threadIdx.x & 3; ar.x + o < ar.y; o += 4) {
             const uint32_t u = arc_target(g, (uint32_t)rq.z, ar.x + o, o);
-            const int su = find_or_insert<true>(s, sh, u, ku >> 3, (uint32_t)d & 3u);
+            const int su = find_or_insert<true>(s, sh, u, ku >> 3, sh.score[d & 3]);
             if (su < 0) break;
             if (g_max(&s.recs[su].vals[ku & 7], cand) >= 0) continue;
             ++won;
@@ -973,7 +971,7 @@ __device__ __forceinline__ void resolve_spill_traces(const DevGraph &g, const Sl
         const uint2 ar = __ldg((const uint2 *)&g.vx[2 * (uint64_t)(uint32_t)rq.z].z);
         for (uint32_t o = threadIdx.x & 3; ar.x + o < ar.y; o += 4) {
             const uint32_t u = arc_target(g, (uint32_t)rq.z, ar.x + o, o);
-            const int su = find_or_insert<true>(s, sh, u, ku >> 3, (uint32_t)d & 3u);
+            const int su = find_or_insert<true>(s, sh, u, ku >> 3, sh.score[d & 3]);
             if (su < 0) return;
             if (s.recs[su].vals[ku & 7] == cand) g_max32(&s.trec[su].tr[ku & 7], s.reqt[r]);
         }
@@ -1007,7 +1005,7 @@ __device__ __forceinline__ bool spill_step(const DevGraph &g, const Slab<true> &
     bool want = ar.x + arc < ar.y;
     if (want) {
         ui = ld_early(&g.vx[2 * (uint64_t)u], 0);
-        su = find_or_insert<true>(s, sh, u, ku >> 3, (uint32_t)d & 3u);
+        su = find_or_insert<true>(s, sh, u, ku >> 3, sh.score[d & 3]);
         want = su >= 0;
         if (want) {
             const long long raw = s.recs[su].vals[ln];
@@ -1192,7 +1190,7 @@ __device__ __noinline__ Room check_room(const uint4 *vx, const Slab<P> &s, Sh &s
             j = v >> 1;
         }
         if (!live || (sd ? kb * kTile + 7 + j >= n : j >= (int)__ldg(&vx[2 * (uint64_t)ent.y]).y)) continue;
-        const uint32_t t = link_neighbour<P>(s, sh, ent.x, ent.y, kb, sd, ((uint32_t)d & 3u) | kForLink);
+        const uint32_t t = link_neighbour<P>(s, sh, ent.x, ent.y, kb, sd, sh.score[d & 3]);
         if (t == kNone) continue;
         leave_border<P>(s, t, sd, j, base, d, traceback ? s.trec[ent.x].tr[ln] : 0u, traceback);
         if (list_once<P>(s, sh, t, d)) s.list[(d + 1) & 1][atomicAdd(nq, 1u)] = make_uint2(t, ent.y);
@@ -1237,7 +1235,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         sh.peak = 0;
         sh.tlen = 0;
         sh.end_vp = ((unsigned long long)q.ve << 32) | kNoTrace;
-        const int t = find_or_insert<P>(s, sh, vs, 0, 0u);
+        const int t = find_or_insert<P>(s, sh, vs, 0, sh.score[0]);
         if (t >= 0) {
             if constexpr (P) {
                 s.recs[t].vals[0] = pk(0, kTagLive, 0u);
@@ -1261,7 +1259,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         const int ntile = (lvs + kTile - 1) / kTile;   // tiles kb = -1 .. -ntile
         for (int i = threadIdx.x; i < ntile; i += blockDim.x) {
             const int kb = -1 - i;
-            const int t = find_or_insert<P>(s, sh, vs, kb, 0u);
+            const int t = find_or_insert<P>(s, sh, vs, kb, sh.score[0]);
             if (t < 0) continue;
             uint32_t cnt = 0;
             for (int ln = 0; ln < kTile; ++ln) {
