@@ -275,7 +275,7 @@ int gwfa_align_batch_device(gwfa_engine *e, uint32_t n_queries, const uint32_t *
  * but its scratch is one fixed 32 MiB device array inside the library (present
  * on every GPU that loads it, until the process exits), carved into
  * floor((32 MiB - 256 B) / slab) CTA slabs of 2^log2_tiles hash tiles each
- * (log2_tiles 0 = 15: six CTAs in exact mode, two with pruning).  There is
+ * (log2_tiles 0 = 15: six CTAs in exact mode, three with pruning).  There is
  * no overflow tier: a query needing more than 3/4 of its slab gets status
  * GWFA_ERR_CAPACITY.  log2_tiles outside [8, 24] (other than 0) is
  * GWFA_ERR_INVALID; a valid log2_tiles whose slab does not fit the array is
