@@ -376,7 +376,8 @@ int gwfa_server_get_stats(gwfa_server *sv, gwfa_server_stats *o) {
     o->requeued = sv->n_requeued;
     o->launches = sv->n_launches;
     o->in_flight = sv->n_submitted - sv->n_completed;
-    o->device_bytes = sv->big_offset + sv->slab_bytes[1] * sv->cfg.ctas_big;
+    o->device_bytes = sv->big_offset + sv->slab_bytes[1] * sv->cfg.ctas_big +
+                      (uint64_t)sv->slot_words * 4 * (sv->cfg.ctas_small + sv->cfg.ctas_big);   // slabs, request words
     return GWFA_OK;
 }
 

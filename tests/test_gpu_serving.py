@@ -162,3 +162,17 @@ def test_more_ctas_than_are_resident(c2):
             assert (r["status"], r["edit_distance"], r["cells"]) == (0, want["distance"], want["cells"]), n
     finally:
         srv.close()
+
+
+def test_device_bytes_count_the_request_words(c2):
+    g, qs, graph = c2
+    size = []
+    for longest in (16_000, 1_600_000):
+        cfg = gw.gwfa_server_config()
+        gw.load().gwfa_server_default_config(graph.handle, cfg)
+        cfg.ctas_small, cfg.ctas_big, cfg.log2_small, cfg.log2_big = 20, 4, 10, 12
+        cfg.ring_slots, cfg.max_query_len = 4, longest
+        srv = gw.Server(graph, cfg)
+        size.append(srv.stats()["device_bytes"])
+        srv.close()
+    assert size[1] - size[0] == (1_600_000 - 16_000) // 16 * 4 * 24   # a CTA keeps its request's packed words
