@@ -22,8 +22,8 @@ struct Range {
 };
 
 // A tile groups the 8 diagonals k = 8*kb .. 8*kb+7 of one vertex: its 8 offsets
-// H~_{v,k} are one 32-byte sector (exact mode) and are processed by 8 adjacent
-// lanes of a warp, so that the expand step (Alg. 3) is a shuffle inside the tile.
+// H~_{v,k} are one 32-byte sector (exact mode) and are processed by four adjacent lanes
+// of a warp, two each, so that the expand step (Alg. 3) is a shuffle inside the tile.
 constexpr int kTile = 8;
 constexpr uint64_t kEmptyKey = ~0ull;
 
@@ -104,14 +104,14 @@ __host__ __device__ inline SlabLayout slab_layout(uint32_t log2cap, bool prune) 
     L.recs = o;    o = align256(o + rcap * (prune ? sizeof(RecT<long long>) : sizeof(RecT<int>)));
     L.touched = o; o = align256(o + rcap * 4);
     L.stamp = o;   o = align256(o + rcap * 4);
-    L.tkey = o;    o = align256(o + (prune ? rcap * 8 : 0));    // keys by record (memory bound)
-    L.list0 = o;   o = align256(o + rcap * 8);                  // (record, vertex)
+    L.tkey = o;    o = align256(o + (prune ? rcap * 8 : 0));   // keys by record
+    L.list0 = o;   o = align256(o + rcap * 8);                 // (record, vertex)
     L.list1 = o;   o = align256(o + rcap * 8);
-    L.links = o;   o = align256(o + 2 * rcap * 8);              // neighbours to be linked
-    L.req = o;     o = align256(o + (prune ? cap * 16 : 4 * cap * 8));   // arc-spill requests of a score (6 cap, see put_req)
+    L.links = o;   o = align256(o + 2 * rcap * 8);             // neighbours to be linked
+    L.req = o;     o = align256(o + (prune ? cap * 16 : 4 * cap * 8));   // arc-spill requests: of a round, or 6 cap of a score (put_req)
     L.reqt = o;    o = align256(o + (prune ? cap * 4 : 0));    // trace index of each request
-    L.ins = o;     o = align256(o + (prune ? 6 * cap * 4 : 0));   // diagonals a spill round inserted
-    L.freel = o;   o = align256(o + (prune ? rcap * 4 : 0));    // records the memory bound freed
+    L.ins = o;     o = align256(o + (prune ? 6 * cap * 4 : 0));   // diagonals a spill round inserted (put_ins)
+    L.freel = o;   o = align256(o + (prune ? rcap * 4 : 0));   // records freed by evict_behind
     L.trace = o;   o = align256(o + (prune ? cap * 2 * 8 : 0));   // Alg. 5's T: (v, t) pairs
     L.trec = o;    o = align256(o + (prune ? rcap * sizeof(TraceRec) : 0));
     L.total = o;

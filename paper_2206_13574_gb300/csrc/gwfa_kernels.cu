@@ -7,14 +7,15 @@
 //
 // A score d is two steps with a barrier after each:
 //   offset_pass   visits every tile (the 8 diagonals 8 kb .. 8 kb + 7 of one vertex) that
-//                 may change, by an 8-lane group: GwfExpand of score d - 1 gathered into
-//                 the tile (a lane's own source and its neighbours' by shuffle, the two
-//                 edge lanes' from border words that the neighbour tiles left), GwfPrune on
-//                 those sources, GwfExtend of the diagonals that improved, and the tile's
-//                 own border words and list entries for score d + 1;
+//                 may change, by four lanes with two diagonals each: GwfExpand of score
+//                 d - 1 gathered into the tile (a lane's own sources and its neighbours' by
+//                 shuffle, the two edge diagonals' from border words that the neighbour
+//                 tiles left), GwfPrune on those sources, GwfExtend of the diagonals that
+//                 improved, and the tile's own border words and list entries for score d + 1;
 //   spill rounds  the arcs of the diagonals that reached |v| (rare: about 1% of the
 //                 diagonals, none in many scores).  They come after the pass because a
-//                 spill only fills a diagonal that GwfExpand left absent.
+//                 spill only fills a diagonal that GwfExpand left absent.  Neighbour tiles
+//                 that a border word meets for the first time are looked up beside them.
 // A tile is read and written once a score, by one thread group, with plain loads and
 // stores: no offset is merged by an atomic, and all the data of a query live in one CTA,
 // so they stay in L1 (39 cycles a load there, 275 from L2, 477 for an atomic, which also
@@ -35,7 +36,7 @@
 //          (v << 32 | kb) to them.  The hash is probed for spills and when two
 //          neighbouring tiles meet for the first time (they then hold each other's record
 //          index).  Entries persist for the whole query (an entry blocks re-spilling,
-//          Alg. 2); records and hash are emptied when it ends.
+//          Alg. 2); the hash is emptied when it ends, a record when it is claimed.
 //   lists  (record, vertex) of the tiles to visit in this score and in the next: the tiles
 //          with a diagonal in Q and those a border word was left for.  A flag per tile and
 //          parity keeps them without repeats.
