@@ -55,3 +55,13 @@ def test_roofline_arithmetic():
     r = bench.roofline(10 ** 9, 10 ** 8, 0.5, peak, counters, 6000.0, "measured", 1)
     assert abs(r["int_frac"] - 10.0 * 10 ** 9 / 0.5 / 6.0e11) < 1e-12
     assert abs(r["traffic"] - 27.5e9) < 1e-3 and abs(r["l2_frac"] - 0.15) < 1e-12
+
+
+def test_roofline_headline_follows_the_counters():
+    counters = {"dram_bytes_per_cell": 5.0, "l2_throughput_pct": 13.0, "warp_inst_per_cell": 11.5,
+                "alu_warp_inst_per_cell": 5.0, "source": "test"}
+    peak = {"warp_inst_per_s": 6.0e11}
+    r = bench.roofline(10 ** 9, 10 ** 8, 0.015, peak, counters, 6000.0, "measured", 1)
+    assert r["bound"] == "int" and r["frac"] == r["int_frac"] == r["achieved"] / r["peak"] < 1
+    assert r["hbm_frac"] == r["hbm_achieved_gbs"] / 6000.0 > 1   # work units, not traffic
+    assert bench.roofline(10 ** 9, 10 ** 8, 0.015, peak, None, 6000.0, "measured", 1)["bound"] == "hbm"
