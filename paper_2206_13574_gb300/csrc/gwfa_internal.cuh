@@ -44,6 +44,7 @@ struct DevGraph {
 
 constexpr uint32_t kMaxLog2Tiles = 24;
 constexpr uint32_t kNarrow = 256;   // threads per CTA up to which the narrow kernel runs
+constexpr uint32_t kMaxThreads = 1024;
 
 
 // Hash entry: the tile's key (v << 32 | kb, all ones = empty) and its record.
@@ -81,10 +82,12 @@ struct alignas(64) TraceRec {
     uint32_t pad[4];
 };
 
-// Records of a slab of 2^log2 tiles.  A CTA has up to two more in use for each of its threads
-// (see link_stop); the quarter above the load limit has room for them but on small slabs.
-__host__ __device__ inline uint32_t slab_records(uint32_t log2cap) {
-    return (1u << log2cap) + (log2cap < 14 ? 1024u : 0u);
+// Records of a slab of 2^log2 tiles for CTAs of up to `threads` threads.  A CTA has up to two
+// more in use for each of them (see link_stop): the quarter above the load limit has room for
+// these, and a sixteenth for links, but on small slabs.
+__host__ __device__ inline uint32_t slab_records(uint32_t log2cap, uint32_t threads) {
+    const uint32_t cap = 1u << log2cap, need = 2 * threads + cap / 16;
+    return cap + (need > cap / 4 ? need - cap / 4 : 0u);
 }
 
 // Per-CTA slab layout (all arrays 256-byte aligned), cap = 2^log2 tiles: the hash (twice
@@ -96,8 +99,8 @@ struct SlabLayout {
 
 __host__ __device__ inline uint64_t align256(uint64_t x) { return (x + 255) & ~255ull; }
 
-__host__ __device__ inline SlabLayout slab_layout(uint32_t log2cap, bool prune) {
-    const uint64_t cap = 1ull << log2cap, rcap = slab_records(log2cap);
+__host__ __device__ inline SlabLayout slab_layout(uint32_t log2cap, bool prune, uint32_t threads = kMaxThreads) {
+    const uint64_t cap = 1ull << log2cap, rcap = slab_records(log2cap, threads);
     SlabLayout L;
     uint64_t o = 0;
     L.table = o;   o = align256(o + 2 * cap * sizeof(TabEnt));
@@ -146,6 +149,7 @@ struct TierArgs {
     uint32_t *paths;            // traceback: path_cap vertex ids per query id
     uint32_t *path_len;         // traceback: walk length per query id (may exceed path_cap)
     uint32_t path_cap;
+    uint32_t slab_threads = kMaxThreads;   // widest CTA that the slabs are laid out for
     // run only if the mean length of the batch's n_all queries is in [len_lo, len_hi) (len_hi
     // 0: always): where the host does not know the lengths it launches every width, and the
     // device settles which one works

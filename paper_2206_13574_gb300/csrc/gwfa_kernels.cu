@@ -96,8 +96,8 @@ template <bool P> struct Slab {
 };
 
 template <bool P>
-__device__ __forceinline__ Slab<P> carve(uint8_t *base, uint32_t log2cap) {
-    SlabLayout L = slab_layout(log2cap, P);
+__device__ __forceinline__ Slab<P> carve(uint8_t *base, uint32_t log2cap, uint32_t threads) {
+    SlabLayout L = slab_layout(log2cap, P, threads);
     Slab<P> s;
     s.table = (TabEnt *)(base + L.table);
     s.recs = (RecT<typename VT<P>::T> *)(base + L.recs);
@@ -115,7 +115,7 @@ __device__ __forceinline__ Slab<P> carve(uint8_t *base, uint32_t log2cap) {
     s.trace = (uint2 *)(base + L.trace);
     s.trec = (TraceRec *)(base + L.trec);
     s.cap = 1u << log2cap;
-    s.rcap = slab_records(log2cap);
+    s.rcap = slab_records(log2cap, threads);
     s.tmask = 2 * s.cap - 1;
     return s;
 }
@@ -1465,7 +1465,7 @@ __device__ __forceinline__ void align_queries(const TierArgs &A) {
         const uint64_t len = (A.q_off[A.n_all] - A.q_off[0]) / A.n_all;
         if (len < A.len_lo || len >= A.len_hi) return;   // the same for every thread of the grid
     }
-    if (threadIdx.x == 0) s = carve<P>(A.slabs + (uint64_t)blockIdx.x * A.slab_bytes, A.log2cap);
+    if (threadIdx.x == 0) s = carve<P>(A.slabs + (uint64_t)blockIdx.x * A.slab_bytes, A.log2cap, A.slab_threads);
     const uint32_t count = A.list_count ? *A.list_count : A.count_val;
     for (;;) {
         if (threadIdx.x == 0) {
@@ -1535,7 +1535,7 @@ __global__ void __launch_bounds__(512, PerSm) server_kernel(ServerArgs S) {
     uint8_t *base = cls == 0 ? S.slabs + (uint64_t)(blockIdx.x - n_big) * S.slab_bytes[0]
                              : S.slabs + S.big_offset + (uint64_t)blockIdx.x * S.slab_bytes[1];
     __shared__ Slab<P> s;   // as in align_queries; visible after the first poll barrier
-    if (threadIdx.x == 0) s = carve<P>(base, S.log2cap[cls]);
+    if (threadIdx.x == 0) s = carve<P>(base, S.log2cap[cls], kMaxThreads);
     for (;;) {
         if (threadIdx.x == 0) {
             int go = 0;

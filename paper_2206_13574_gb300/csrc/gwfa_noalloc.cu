@@ -99,7 +99,13 @@ extern "C" int gwfa_align_noalloc(const gwfa_graph *g, uint32_t n_queries, const
     if (log2_tiles == 0) log2_tiles = 15;
     const bool prune = o.max_lag > 0;
     if (log2_tiles < 8 || log2_tiles > gwfa::kMaxLog2Tiles) return GWFA_ERR_INVALID;
-    const uint64_t slab = gwfa::slab_layout(log2_tiles, prune).total;
+    // as wide as the frontiers of a slab are worth (with pruning they stay small): a narrow CTA
+    // needs fewer records beside the slab's tiles, so more of them fit.  2,000 reads of 1 kb on
+    // 2^8, 2^10, 2^12 tiles: 1.52, 1.51, 4.22 ms with 1,024 threads, 0.74, 1.40, 4.30 ms so; on
+    // slabs laid out for 1,024 threads 1.09, 1.79, 4.69 ms.
+    const uint32_t threads = prune ? (log2_tiles < 10 ? 64 : log2_tiles < 11 ? 128 : 256)
+                                   : (log2_tiles < 10 ? 128 : log2_tiles < 12 ? 256 : log2_tiles < 14 ? 512 : 1024);
+    const uint64_t slab = gwfa::slab_layout(log2_tiles, prune, threads).total;
     if (slab + kHeadBytes > kNoallocScratchBytes) return GWFA_ERR_CAPACITY;   // does not fit the array
     if (n_queries == 0) return GWFA_OK;
     if (cudaSetDevice(g->device) != cudaSuccess) return GWFA_ERR_CUDA;
@@ -125,10 +131,8 @@ extern "C" int gwfa_align_noalloc(const gwfa_graph *g, uint32_t n_queries, const
     a.slabs = base + kHeadBytes;
     a.slab_bytes = slab;
     a.log2cap = log2_tiles;
+    a.slab_threads = threads;
     a.max_lag = o.max_lag;
     a.max_score = o.max_score;
-    // a handful of CTAs: as wide as their frontiers are worth (on slabs below 2^13 tiles the
-    // links of 1,024 threads would wait for the spills, see link_stop)
-    const uint32_t threads = prune ? 256 : log2_tiles >= 13 ? 1024 : 512;
     return gwfa::launch_align(a, prune, ctas, threads, s) == cudaSuccess ? GWFA_OK : GWFA_ERR_CUDA;
 }
