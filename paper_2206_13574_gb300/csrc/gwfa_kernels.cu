@@ -349,35 +349,25 @@ template <bool P> __device__ __forceinline__ uint32_t link_stop(const Slab<P> &s
     return (uint32_t)max((int)(s.rcap - load_limit(s) + sh.nclaim) - 2 * (int)blockDim.x, 0);
 }
 
-// Record of tile (v, kb), claimed if absent; -1 (and an error) when the slab is full or a link
-// has to wait.  The first probe is inline, the rest (and the claim) is not, in one function
-// for spills and one for links (with a switch 10,000 reads take 33.5 ms, so 32.7).  A claim
-// puts key and record into the table at once, so it brings a record along, and where several
-// threads meet at one new tile (the eight diagonals of a neighbour do, and the two vertices of
-// a bubble) all but one are left with theirs.  Such a thread keeps it for its next claim: a
-// slab then has at most one record a thread in use beside its tiles, and what it has room for
-// does not depend on how often they meet (without, 255 spills at once into 32 tiles used 255
-// records, and a read under the memory bound lost one at every bubble, for good).  To claim
-// the key first and have the others wait for the record costs them a poll (10,000 reads 32.5
-// -> 37.5 ms).
-template <bool P, bool Link>
+// Record of tile (v, kb), claimed if absent; -1 (and *err) when the slab is full.  The first
+// probe is inline, the rest (and the claim) is not.  A claim puts key and record into the table
+// at once, so it brings a record along, and where several threads meet at one new tile (the
+// eight diagonals of a neighbour do, and the two vertices of a bubble) all but one are left
+// with theirs.  Such a thread keeps it for its next claim: a slab then has at most one record a
+// thread in use beside its tiles, and what it has room for does not depend on how often they
+// meet (without, 255 spills at once into 32 tiles used 255 records, and a read under the memory
+// bound lost one at every bubble, for good).  To claim the key first and have the others wait
+// for the record costs them a poll (10,000 reads 32.5 -> 37.5 ms).
+template <bool P>
 __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsigned long long key, uint32_t h, Ent e,
-                                                Score &S) {
+                                                int *err) {
     uint32_t idx = kNone;
     for (int probe = 0; probe < 256; ++probe) {
         if (probe > 0) e = ld_ent(&s.table[h]);
         if (e.key == kEmptyKey) {
             if (idx == kNone) {
-                // (exact mode looks at the number it gets instead, which costs no load: 10,000
-                // reads 33.9 -> 33.3 ms; a link that waits keeps the record, and none of its
-                // thread's later ones takes it)
-                if (P && Link && records_in_use<P>(s, sh) >= S.link_stop) {
-                    atomicCAS(&S.err_next, 0, kLinksWait);
-                    return -1;
-                }
                 idx = spare_record(sh);
                 if (idx != kNone) {
-                    if (!P && Link && S.err_next == kLinksWait) return -1;
                     spare_record(sh) = kNone;
                 } else {
                     if constexpr (P) {
@@ -389,11 +379,6 @@ __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsign
                     if (idx >= s.rcap) break;
                 }
                 empty_record<P>(s, idx, (int)(uint32_t)key);
-                if (!P && Link && idx >= S.link_stop) {
-                    spare_record(sh) = idx;
-                    atomicCAS(&S.err_next, 0, kLinksWait);
-                    return -1;
-                }
                 if constexpr (P) s.tkey[idx] = key;
                 __threadfence_block();   // before the key that leads others to it
             }
@@ -414,15 +399,15 @@ __device__ __noinline__ int find_or_insert_slow(const Slab<P> &s, Sh &sh, unsign
         }
         h = (h + 1) & s.tmask;
     }
-    *(Link ? &S.err_next : &S.err) = GWFA_ERR_CAPACITY;
+    *err = GWFA_ERR_CAPACITY;
     return -1;
 }
-template <bool P, bool Link = false>
-__device__ __forceinline__ int find_or_insert(const Slab<P> &s, Sh &sh, uint32_t v, int kb, Score &S) {
+template <bool P>
+__device__ __forceinline__ int find_or_insert(const Slab<P> &s, Sh &sh, uint32_t v, int kb, int *err) {
     const unsigned long long key = tile_key(v, kb);
     const uint32_t h = tile_hash(key, s.tmask);
     const Ent e = ld_ent(&s.table[h]);
-    if (e.key != key) return find_or_insert_slow<P, Link>(s, sh, key, h, e, S);
+    if (e.key != key) return find_or_insert_slow<P>(s, sh, key, h, e, err);
     __threadfence_block();   // see empty_record
     return (int)e.idx;
 }
@@ -441,8 +426,22 @@ __device__ __forceinline__ bool list_once(const Slab<P> &s, Sh &sh, uint32_t idx
 template <bool P>
 __device__ __noinline__ uint32_t link_neighbour(const Slab<P> &s, Sh &sh, uint32_t idx, uint32_t v, int kb, int sd,
                                                 Score &S) {
-    const int t = find_or_insert<P, true>(s, sh, v, sd ? kb + 1 : kb - 1, S);
-    if (t < 0) return kNone;
+    // (the look at the room stands where a tile is claimed: in the claiming function, which
+    // spills use too, it cost 10,000 reads 33.5 ms, 33.1 so; a second copy of that function for
+    // links 32.9, but 100 reads of 1 kb 170.6 us instead of 167.7, in code to fetch)
+    const unsigned long long key = tile_key(v, sd ? kb + 1 : kb - 1);
+    const uint32_t h = tile_hash(key, s.tmask);
+    const Ent e = ld_ent(&s.table[h]);
+    int t = (int)e.idx;
+    if (e.key != key) {
+        if ((P ? records_in_use<P>(s, sh) : sh.nt) >= S.link_stop) {
+            atomicCAS(&S.err_next, 0, kLinksWait);
+            return kNone;
+        }
+        t = find_or_insert_slow<P>(s, sh, key, h, e, &S.err_next);
+        if (t < 0) return kNone;
+    }
+    __threadfence_block();   // see empty_record
     s.recs[idx].side[sd].link = (uint32_t)t;
     s.recs[t].side[sd ^ 1].link = idx;
     return (uint32_t)t;
@@ -892,7 +891,7 @@ __device__ __forceinline__ void spill_round(const DevGraph &g, const Slab<false>
                 for (uint32_t o = (uint32_t)arc; ar.x + o < ar.y; o += 2) {
                     if (o >= 2) u = arc_target(g, rq.x, ar.x + o, o);
                     const uint2 ui = ld_early(&g.vx[2 * (uint64_t)u], 0);
-                    const int su = find_or_insert<false>(s, sh, u, ku >> 3, sh.score[d & 3]);
+                    const int su = find_or_insert<false>(s, sh, u, ku >> 3, &S.err);
                     if (su < 0) break;
                     // the offset and the first windows together; most spills end here, the
                     // diagonal being there already
@@ -944,7 +943,7 @@ __device__ __forceinline__ void apply_spills(const DevGraph &g, const Slab<true>
         const uint2 ar = __ldg((const uint2 *)&g.vx[2 * (uint64_t)(uint32_t)rq.z].z);
         for (uint32_t o = threadIdx.x & 3; ar.x + o < ar.y; o += 4) {
             const uint32_t u = arc_target(g, (uint32_t)rq.z, ar.x + o, o);
-            const int su = find_or_insert<true>(s, sh, u, ku >> 3, sh.score[d & 3]);
+            const int su = find_or_insert<true>(s, sh, u, ku >> 3, &sh.score[d & 3].err);
             if (su < 0) break;
             if (g_max(&s.recs[su].vals[ku & 7], cand) >= 0) continue;
             ++won;
@@ -972,7 +971,7 @@ __device__ __forceinline__ void resolve_spill_traces(const DevGraph &g, const Sl
         const uint2 ar = __ldg((const uint2 *)&g.vx[2 * (uint64_t)(uint32_t)rq.z].z);
         for (uint32_t o = threadIdx.x & 3; ar.x + o < ar.y; o += 4) {
             const uint32_t u = arc_target(g, (uint32_t)rq.z, ar.x + o, o);
-            const int su = find_or_insert<true>(s, sh, u, ku >> 3, sh.score[d & 3]);
+            const int su = find_or_insert<true>(s, sh, u, ku >> 3, &sh.score[d & 3].err);
             if (su < 0) return;
             if (s.recs[su].vals[ku & 7] == cand) g_max32(&s.trec[su].tr[ku & 7], s.reqt[r]);
         }
@@ -1006,7 +1005,7 @@ __device__ __forceinline__ bool spill_step(const DevGraph &g, const Slab<true> &
     bool want = ar.x + arc < ar.y;
     if (want) {
         ui = ld_early(&g.vx[2 * (uint64_t)u], 0);
-        su = find_or_insert<true>(s, sh, u, ku >> 3, sh.score[d & 3]);
+        su = find_or_insert<true>(s, sh, u, ku >> 3, &sh.score[d & 3].err);
         want = su >= 0;
         if (want) {
             const long long raw = s.recs[su].vals[ln];
@@ -1236,7 +1235,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         sh.peak = 0;
         sh.tlen = 0;
         sh.end_vp = ((unsigned long long)q.ve << 32) | kNoTrace;
-        const int t = find_or_insert<P>(s, sh, vs, 0, sh.score[0]);
+        const int t = find_or_insert<P>(s, sh, vs, 0, &sh.score[0].err);
         if (t >= 0) {
             if constexpr (P) {
                 s.recs[t].vals[0] = pk(0, kTagLive, 0u);
@@ -1260,7 +1259,7 @@ __device__ __forceinline__ void align_one(const TierArgs &A, const Slab<P> &s, S
         const int ntile = (lvs + kTile - 1) / kTile;   // tiles kb = -1 .. -ntile
         for (int i = threadIdx.x; i < ntile; i += blockDim.x) {
             const int kb = -1 - i;
-            const int t = find_or_insert<P>(s, sh, vs, kb, sh.score[0]);
+            const int t = find_or_insert<P>(s, sh, vs, kb, &sh.score[0].err);
             if (t < 0) continue;
             uint32_t cnt = 0;
             for (int ln = 0; ln < kTile; ++ln) {
